@@ -333,6 +333,7 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
 
 // Combines the chunk partials of one (request, KV head): grid = n_req * n_kv.
 __global__ void __launch_bounds__(ATT_THREADS) attn_merge_kernel(const AttnArgs a) {
+  pdl_launch_dependents();    // the next call's first kernel may set itself up; it waits for this grid before it reads anything
   pdl_wait();
   const int i = blockIdx.x / a.n_kv, h = blockIdx.x % a.n_kv;
   const int4 info = a.req_info[i];

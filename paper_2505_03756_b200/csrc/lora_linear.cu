@@ -20,6 +20,7 @@
 #include <string.h>
 #include <algorithm>
 #include "lora_plan.cuh"
+#include "lora_skinny.cuh"
 #include "mma_utils.cuh"
 #include "pool.cuh"
 #include "sgmv.cuh"
@@ -520,7 +521,8 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
   // Segments of a few tokens each (a decode batch): a 128-token tile would take one LoRA stage per segment, each
   // for a handful of rows, and y is small next to W.  Then the GEMM computes x W alone (no LoRA stages in the plan)
   // and the segmented projection adds the LoRA term to y afterwards.
-  const bool hybrid = n_seg > 0 && n_tokens <= 16 * n_seg;
+  const bool few = n_tokens <= skinny::MAX_TOKENS;      // W streamed once for all tokens: a kernel of its own
+  const bool hybrid = !few && n_seg > 0 && n_tokens <= 16 * n_seg;
   if (hybrid) a.n_seg = 0;
   for (int j = 0; j < MAX_LIN; ++j) a.kv_side[j] = -1;
   if (kv) {
@@ -530,9 +532,9 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
     for (int side = 0; side < 2; ++side) {
       const int slot = side ? kv->v_slot : kv->k_slot;
       if (slot < 0 || slot >= n_mats || a.d_out[slot] != kv->n_kv * FL_HEAD_DIM) return FL_EINVAL;
+      if (n_seg > 0 && n_tokens <= 16 * n_seg && !(side ? kv->tmp_v : kv->tmp_k)) return FL_EINVAL;   // whichever kernel serves the batch
       if (hybrid) {      // x W goes to a scratch row first; the segmented projection then stores base + LoRA term in the pool
         fl_bf16* tmp = side ? kv->tmp_v : kv->tmp_k;
-        if (!tmp) return FL_EINVAL;
         ys[slot] = tmp;
         a.y[slot] = reinterpret_cast<__nv_bfloat16*>(tmp);
       } else {
@@ -576,6 +578,40 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
   const cudaStream_t st = (cudaStream_t)stream;
   int rc = FL_OK;
   do {
+    if (few) {
+      skinny::Args k;
+      memset(&k, 0, sizeof(k));
+      k.pv = a.pv;
+      k.v = reinterpret_cast<const __nv_bfloat16*>(a.v);
+      k.seg_indptr = seg_indptr;
+      k.lora_ids = lora_ids;
+      k.n_seg = n_seg;
+      k.n_tokens = n_tokens;
+      k.d_in = a.d_in;
+      k.n_mats = n_mats;
+      for (int j = 0; j < n_mats; ++j) {
+        k.y[j] = a.y[j];
+        k.d_out[j] = a.d_out[j];
+        k.mat_index[j] = a.mat_index[j];
+        k.kv_side[j] = a.kv_side[j];
+      }
+      k.req_indptr = a.req_indptr;
+      k.tbl_indptr = a.tbl_indptr;
+      k.tbl = a.tbl;
+      k.prefix_lens = a.prefix_lens;
+      k.n_req = a.n_req;
+      k.n_kv = a.n_kv;
+      k.bt = a.bt;
+      sgmv::ShrinkInfo info = {1, 16};
+      if (n_seg > 0) {
+        rc = sgmv::shrink_scaled(p, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, scale, wsb + lw.v,
+                                 fl_lora_sgmv_workspace(n_tokens, n_mats), stream, &info);
+        if (rc != FL_OK) break;
+      }
+      k.rmax = info.rmax;
+      rc = skinny::launch(p, k, x, reinterpret_cast<const void* const*>(ws), st);
+      break;
+    }
     alignas(64) LinMaps maps;
     {
       const uint64_t dims[2] = {(uint64_t)a.d_in, (uint64_t)n_tokens};

@@ -1,0 +1,555 @@
+// y = x W + scale * (x A_i) B_i (Eq. 1, Eq. 2) for batches of at most 256 tokens: decode steps and short prompts.
+//
+// Such a call is bound by streaming W once and, with many adapters, their B rows.  One CTA owns 128 output columns for
+// ALL tokens (one or two row tiles of 128) and a slice of d_in; the CTAs of a column tile form a cluster that adds its
+// partial sums through distributed shared memory, so that narrow projections still use every SM and no partial sum goes
+// through global memory.
+//   warp 0      TMA producer: x tile [tokens x 64] and W tile [64 x 128] per stage, ring of as many stages as fit
+//   warp 1      MMA issuer of x W
+//   warp 6      MMA issuer of the LoRA term, into an accumulator of its own
+//   warps 2-5   LoRA stages, then the epilogue (thread = token row)
+// The LoRA term is one more product over a long, sparse k: the rank-rows of every adapter of the batch one after the
+// other, 64 to a stage, against a matrix that holds in row t the shrink result of token t at the ranks of its own adapter
+// and zeros elsewhere.  A stage has the layout of a main stage: B rows through the block table in place of W rows,
+// shrink results in place of x, both by cp.async (a masked copy writes the zeros).  A batch whose every token uses
+// another adapter is thus no special case, and since the two accumulators have one issuer each, the order of either's
+// sums does not depend on which stage is ready first.
+// Launched behind the shrink, the kernel streams W and B rows while the shrink still runs: the shrink lets it start only
+// after everything before the shrink is done, and only v is waited for.
+// Tokens are the tensor core's rows although most of its 128 rows may be empty: with W as the row operand and the tokens
+// as columns an MMA step took about 170 cycles however few the tokens, against 64 here.
+// What bounds it: W.  Of one 7B layer's projections the W stream alone takes 18.6 us (q, k, v) and 8.3 us (o) when nothing
+// is computed, the calls take 25 and 17 us; before, with the GEMM for long batches followed by the segmented projection,
+// they took 44 and 32 us.  The rest is the shrink's chain of look-ups in front and the sum over the cluster behind.
+// Every mbarrier wait is bounded; a wait that gives up raises a sticky flag and the CTA still meets its cluster's
+// barriers, drains its copies and frees its TMEM.  No multicast.
+#include <cuda.h>
+#include <string.h>
+#include <algorithm>
+#include "lora_skinny.cuh"
+#include "mma_utils.cuh"
+#include "tc_ptx.cuh"
+#include "tmap.cuh"
+
+namespace {
+
+using namespace tc;
+
+constexpr int THREADS = 224;
+constexpr int BN = 128, BK = 64;                   // columns per CTA; d_in (or rank-rows) per stage
+constexpr uint32_t W_BYTES = BK * BN * 2, W_GROUP = BK * 128;      // two groups of 64 columns
+constexpr int MAX_NS = 12, MAX_NE = 3;
+constexpr int UNIT = 16;                           // rank-rows per entry of the LoRA list: one k-step
+constexpr int UNITS_PER_TOKEN = FL_MAX_RANK / UNIT;      // every token its own adapter of the highest rank
+constexpr int GROUP = 8;                           // LoRA stages whose row addresses are looked up together
+constexpr int MAX_SPLIT = 8;
+// Not all of an SM's 227 KB: what is left lets the CTA start beside CTAs of the shrink before it (a decode step of one token:
+// 57 us a layer at 180 KB, 61 at 227 KB, 59 at 113 KB; of 48 tokens the same at 180 and 227 KB, 2 % more at 113 KB).
+constexpr uint32_t SMEM_LIMIT = 180 * 1024;
+
+struct LoraUnit {        // 16 rank-rows of one segment's adapter
+  uint16_t lo, hi;       // the segment's tokens
+  uint16_t r0, nr;       // first rank, rank-rows (1..16; 0 = padding of the last stage)
+  uint32_t tab, row0;    // first table entry of the stream the B rows are in, row of rank r0 inside it
+};
+
+struct KArgs {
+  skinny::Args s;
+  int tile_base[skinny::MAX_LIN + 1];
+  int npad, ns, ne, split;        // tokens rounded up to 16, stages of the two rings, CTAs per column tile
+  uint32_t tmem_cols;
+};
+struct Maps {
+  CUtensorMap x;
+  CUtensorMap w[skinny::MAX_LIN];
+};
+
+enum { B_FULL = 0, B_EMPTY = MAX_NS, B_EFULL = 2 * MAX_NS, B_EEMPTY = B_EFULL + MAX_NE, B_LIST = B_EEMPTY + MAX_NE, B_ACC, B_COUNT };
+// behind the two rings: barriers and bookkeeping | B row addresses of two groups of stages | list of LoRA units
+constexpr uint32_t BOOK_BYTES = 384, ROWS_BYTES = 2 * GROUP * BK * 8;
+static_assert(8 * B_COUNT + 48 <= BOOK_BYTES, "bookkeeping area too small");
+static_assert(sizeof(LoraUnit) == 16, "one 16-byte shared-memory access per unit");
+
+__global__ void __launch_bounds__(THREADS, 1) lora_skinny_kernel(const __grid_constant__ KArgs ka, const __grid_constant__ Maps maps) {
+  const skinny::Args& a = ka.s;
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  const uint32_t sbase = smem_u32(smem);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int ns = ka.ns, ne = ka.ne, npad = ka.npad, split = ka.split;
+  const int mt = npad > 128 ? 2 : 1;                                // row tiles
+  const uint32_t x_bytes = (uint32_t)npad * 128, stage_bytes = x_bytes + W_BYTES;      // [x rows][W rows]
+  const uint32_t off_ext = ns * stage_bytes, off_book = off_ext + ne * stage_bytes;
+  const uint32_t bar0 = sbase + off_book;
+  auto bar = [&](int k) { return bar0 + 8u * k; };
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + off_book + 8 * B_COUNT);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + off_book + 8 * B_COUNT + 4);
+  volatile int* n_stage_slot = reinterpret_cast<volatile int*>(smem + off_book + 8 * B_COUNT + 8);
+  int* scan = reinterpret_cast<int*>(smem + off_book + 8 * B_COUNT + 16);      // [4], one per filler warp
+  unsigned long long* row_ptr = reinterpret_cast<unsigned long long*>(smem + off_book + BOOK_BYTES);     // [2][GROUP * BK], 0 = no row
+  LoraUnit* list = reinterpret_cast<LoraUnit*>(smem + off_book + BOOK_BYTES + ROWS_BYTES);
+  const int max_units = npad * UNITS_PER_TOKEN;
+
+  const int crank = blockIdx.x % split;            // clusters are `split` consecutive CTAs
+  const int tile = blockIdx.x / split;
+  int j = 0;
+  while (j + 1 < a.n_mats && tile >= ka.tile_base[j + 1]) ++j;
+  const int n0 = (tile - ka.tile_base[j]) * BN;
+  const int d_out = a.d_out[j];
+  const int nk = (a.d_in + BK - 1) / BK;
+  const int k0 = crank * nk / split, k1 = (crank + 1) * nk / split;
+
+  if (tid == 0) {
+    for (int s = 0; s < ns; ++s) {
+      mbar_init(bar(B_FULL + s), 1);
+      mbar_init(bar(B_EMPTY + s), 1);
+    }
+    for (int e = 0; e < ne; ++e) {
+      mbar_init(bar(B_EFULL + e), 128);
+      mbar_init(bar(B_EEMPTY + e), 1);
+    }
+    mbar_init(bar(B_LIST), 1);
+    mbar_init(bar(B_ACC), 2);            // both issuers
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void*)tmem_slot)), "r"(ka.tmem_cols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem_lora = tmem + mt * BN;
+  // Behind the shrink everything but v was finished before this kernel could start (the shrink lets it start after its own
+  // wait); without one, the kernel before may still be writing x.
+  if (a.n_seg == 0) pdl_wait();
+
+  constexpr uint32_t IDESC = instr_desc(BN, true);       // A (x, v) K-major, B (W, adapter rows) N-contiguous
+  constexpr uint32_t HI = desc_hi(1024);
+  // four k-steps of one stage into the accumulators at d
+  auto issue_stage = [&](uint32_t stage, uint32_t d, bool first, int steps) {
+    const uint32_t a_lo = desc_lo(stage, 16), b_lo = desc_lo(stage + x_bytes, W_GROUP);
+    for (int m = 0; m < mt; ++m) {
+#pragma unroll
+      for (int q = 0; q < BK / 16; ++q)
+        if (q < steps)
+          umma_ss_elect(d + m * BN, a_lo + m * (128 * 128 / 16) + q * 2, HI, b_lo + q * (16 * 128 / 16), HI, IDESC, first && q == 0 ? 0u : 1u);
+    }
+  };
+  auto wait_all = [&](uint32_t b, uint32_t parity) {
+    if (__all_sync(0xffffffffu, mbar_try(b, parity))) return true;       // the common case: one test
+    return __all_sync(0xffffffffu, mbar_wait(b, parity, abort_flag)) != 0;
+  };
+
+  bool ok = true;
+  int n_stages = 0;                        // LoRA stages of this CTA (known to the LoRA roles)
+  const int et = tid - 64;                 // filler / epilogue thread 0..127
+  if (warp == 0) {
+    // ------------------------------------------------ TMA producer
+    if (lane == 0) {
+      const CUtensorMap* wm = &maps.w[j];
+      int s = 0;
+      uint32_t ph = 1;
+      for (int ks = k0; ks < k1; ++ks) {
+        if (ks - k0 >= ns && !mbar_wait(bar(B_EMPTY + s), ph, abort_flag)) break;
+        mbar_expect_tx(bar(B_FULL + s), stage_bytes);
+        const uint32_t dst = sbase + s * stage_bytes;
+        tma_load_2d(dst + x_bytes, wm, bar(B_FULL + s), n0, ks * BK);
+        tma_load_2d(dst + x_bytes + W_GROUP, wm, bar(B_FULL + s), n0 + 64, ks * BK);
+        tma_load_2d(dst, &maps.x, bar(B_FULL + s), ks * BK, 0);
+        if (++s == ns) { s = 0; ph ^= 1u; }
+      }
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------ MMA issuer of x W
+    int s = 0;
+    uint32_t ph = 0;
+    for (int ks = k0; ks < k1; ++ks) {
+      if (!(ok = wait_all(bar(B_FULL + s), ph))) break;
+      tc_fence_after();
+      issue_stage(sbase + s * stage_bytes, tmem, ks == k0, BK / 16);
+      umma_commit_elect(bar(B_EMPTY + s));
+      if (++s == ns) { s = 0; ph ^= 1u; }
+    }
+    if (ok) umma_commit_elect(bar(B_ACC));
+  } else if (warp == 6) {
+    // ------------------------------------------------ MMA issuer of the LoRA term
+    ok = wait_all(bar(B_LIST), 0);
+    if (ok) n_stages = *n_stage_slot;
+    int s = 0;
+    uint32_t ph = 0;
+    for (int i = 0; ok && i < n_stages; ++i) {
+      if (!(ok = wait_all(bar(B_EFULL + s), ph))) break;
+      tc_fence_after();
+      issue_stage(sbase + off_ext + s * stage_bytes, tmem_lora, i == 0, BK / 16);
+      umma_commit_elect(bar(B_EEMPTY + s));
+      if (++s == ne) { s = 0; ph ^= 1u; }
+    }
+    if (ok) umma_commit_elect(bar(B_ACC));
+  } else {
+    // ------------------------------------------------ list of the LoRA units, in segment order
+    int n_units = 0;
+    uint32_t rpb = 1;
+    for (int s0 = 0; s0 < a.n_seg; s0 += 128) {
+      const int s = s0 + et;
+      int lo = 0, hi = 0, rank = 0;
+      uint32_t tab = 0, row0 = 0;
+      if (s < a.n_seg) {
+        lo = max(a.seg_indptr[s], 0);
+        hi = min(a.seg_indptr[s + 1], a.n_tokens);
+        const int lid = a.lora_ids[s];
+        if (lid >= 0 && hi > lo) {
+          if ((uint32_t)lid >= a.pv.dir_cap || a.pv.dir[lid].rank <= 0 || a.mat_index[j] >= a.pv.dir[lid].n_mats) {
+            atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_LORA);
+          } else {
+            const LoraEntry* en = a.pv.dir + lid;
+            rank = min(en->rank, a.rmax);
+            const LoraMat lm = en->mats[a.mat_index[j]];
+            tab = en->table_off + lm.b_tab;
+            row0 = lm.b_row0;
+            rpb = lm.b_rpb;          // the same for every adapter: they share the projection's shape
+          }
+        }
+      }
+      const int cnt = (rank + UNIT - 1) / UNIT;
+      int incl = cnt;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int o = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += o;
+      }
+      if (lane == 31) scan[warp - 2] = incl;
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      int at = n_units + incl - cnt;
+      for (int w = 0; w < 4; ++w) {
+        const int t = scan[w];
+        if (w < warp - 2) at += t;
+        n_units += t;
+      }
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      for (int r0 = 0; r0 < rank; r0 += UNIT, ++at)
+        if (at < max_units) {
+          LoraUnit u;
+          u.lo = (uint16_t)lo;
+          u.hi = (uint16_t)hi;
+          u.r0 = (uint16_t)r0;
+          u.nr = (uint16_t)min(UNIT, rank - r0);
+          u.tab = tab;
+          u.row0 = row0 + r0;
+          list[at] = u;
+        }
+    }
+    n_units = min(n_units, max_units);           // (overlapping segments, which the interface rules out, could exceed it)
+    const int all_stages = (n_units + 3) / 4;
+    if (et < all_stages * 4 - n_units) {
+      LoraUnit none = {};
+      list[n_units + et] = none;
+    }
+    {
+      const uint32_t m = __reduce_max_sync(0xffffffffu, rpb);
+      if (lane == 0) scan[warp - 2] = (int)m;
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      for (int w = 0; w < 4; ++w) rpb = max(rpb, (uint32_t)scan[w]);
+    }
+    // stages are dealt round robin over the cluster
+    n_stages = all_stages > crank ? (all_stages - crank + split - 1) / split : 0;
+    if (et == 0) {
+      *n_stage_slot = n_stages;
+      mbar_arrive(bar(B_LIST));
+    }
+    // ------------------------------------------------ fill the LoRA stages
+    // Addresses of a group's B rows, looked up side by side a group ahead of their use, and their 256 bytes asked into L2:
+    // under the stream of W a load takes 2 us, and a stage that had to wait for its table entry and then for its rows took
+    // 3.5 us (decode step of 48 tokens and 35 adapters of rank 32, d_out 15360).
+    auto find_rows = [&](int g) {
+      for (int i = et; i < GROUP * BK; i += 128) {
+        const int st = g * GROUP + i / BK, r = i % BK;
+        unsigned long long at = 0;
+        if (st < n_stages) {
+          const LoraUnit x = list[4 * (crank + st * split) + r / UNIT];
+          if (r % UNIT < x.nr) {
+            const uint32_t gr = x.row0 + r % UNIT;
+            const uint32_t blk = a.pv.tables[x.tab + gr / rpb];
+            if (blk >= a.pv.n_blocks) {
+              atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_BLOCK);
+            } else {
+              const unsigned char* p = a.pv.slab + (size_t)blk * a.pv.block_bytes + ((size_t)(gr % rpb) * d_out + n0) * 2;
+              at = reinterpret_cast<unsigned long long>(p);
+              asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+              if (n0 + 64 < d_out) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + 128));
+            }
+          }
+        }
+        row_ptr[(g & 1) * GROUP * BK + i] = at;
+      }
+    };
+    const int row = et >> 4, ch = et & 15;               // B rows row + 8 i, 16-byte chunk ch of the 128 columns
+    const int vrow = et >> 3, vch = et & 7;              // v rows vrow + 16 i, ranks 8 vch .. of the stage's 64
+    const bool col_ok = n0 + ch * 8 < d_out;
+    auto landed = [&](int pending) {                     // all but this thread's newest `pending` stages have landed
+      if (pending == 0) cp_async_wait<0>();
+      else if (pending == 1) cp_async_wait<1>();
+      else cp_async_wait<2>();
+      fence_async_smem();
+    };
+    if (n_stages > 0) {
+      find_rows(0);
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+    }
+    int s = 0, done = 0, ds = 0;
+    uint32_t ph = 1;
+    for (int i = 0; i < n_stages; ++i) {
+      // (the barrier also makes the addresses of a group visible that were looked up some stages ago)
+      if (i >= ne) ok = group_and(mbar_wait(bar(B_EEMPTY + s), ph, abort_flag), 1, 128);
+      if (!ok) break;
+      const LoraUnit* u = list + 4 * (crank + i * split);
+      const unsigned long long* rp = row_ptr + (i % (2 * GROUP)) * BK;
+      const uint32_t vb = sbase + off_ext + s * stage_bytes, bb = vb + x_bytes;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int r = row + 8 * q;
+        const unsigned long long at = rp[r];
+        cp_async16(bb + (ch >> 3) * W_GROUP + r * 128 + (((ch & 7) ^ (r & 7)) << 4),
+                   at ? reinterpret_cast<const unsigned char*>(at) + ch * 16 : a.pv.slab, at && col_ok);
+      }
+      if (i == 0) pdl_wait();                            // v is the shrink's output
+      {
+        const LoraUnit x = u[vch >> 1];
+        const int r = x.r0 + 8 * (vch & 1);
+        const bool live = 8 * (vch & 1) < x.nr;
+        const __nv_bfloat16* src = a.v + ((size_t)j * a.n_tokens) * a.rmax + r;
+        for (int t = vrow; t < npad; t += 16) {
+          const bool mine = live && t >= x.lo && t < x.hi;
+          cp_async16(vb + t * 128 + ((vch ^ (t & 7)) << 4), mine ? src + (size_t)t * a.rmax : a.v, mine);
+        }
+      }
+      cp_async_commit();
+      if (++s == ne) { s = 0; ph ^= 1u; }
+      if (i % GROUP == 0 && i + GROUP < n_stages) find_rows(i / GROUP + 1);
+      if (i + 1 >= ne) {
+        landed(ne - 1);
+        mbar_arrive(bar(B_EFULL + ds));
+        if (++ds == ne) ds = 0;
+        ++done;
+      }
+    }
+    if (ok && done < n_stages) {
+      landed(0);
+      for (; done < n_stages; ++done) {
+        mbar_arrive(bar(B_EFULL + ds));
+        if (++ds == ne) ds = 0;
+      }
+    }
+    cp_async_wait<0>();
+    if (n_stages == 0) pdl_wait();
+  }
+
+  // ------------------------------------------------ epilogue: this thread's token row(s)
+  const int quarter = warp & 3;
+  const int lrow = quarter * 32 + lane;                       // row of the tile = TMEM lane
+  const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
+  const bool epi = warp >= 2 && warp < 6;
+  const int side = a.kv_side[j];
+  uint32_t kv_blk[2] = {0, 0};
+  int kv_slot[2] = {-1, -1};
+  bool kv_last[2] = {false, false};
+  if (epi) {
+    if (side >= 0) {                                          // where K / V rows go
+      for (int m = 0; m < mt; ++m) {
+        const int t = m * 128 + lrow;
+        if (t >= a.n_tokens) continue;
+        int lo = 0, hi = a.n_req;
+        while (hi - lo > 1) {
+          const int mid = (lo + hi) >> 1;
+          if (a.req_indptr[mid] <= t) lo = mid; else hi = mid;
+        }
+        const int pos = a.prefix_lens[lo] + (t - a.req_indptr[lo]);
+        const int entry = pos / a.bt, slot = pos - entry * a.bt;
+        if (pos < 0 || t < a.req_indptr[lo] || t >= a.req_indptr[lo + 1] || entry >= a.tbl_indptr[lo + 1] - a.tbl_indptr[lo]) {
+          atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_POS);
+          continue;
+        }
+        const uint32_t b = a.tbl[a.tbl_indptr[lo] + entry];
+        if (b >= a.pv.n_blocks) {
+          atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_BLOCK);
+          continue;
+        }
+        kv_blk[m] = b;
+        kv_slot[m] = slot;
+        kv_last[m] = t == a.req_indptr[lo + 1] - 1;
+      }
+    }
+    if (ok) ok = mbar_wait(bar(B_ACC), 0, abort_flag);
+    ok = group_and(ok, 1, 128);
+    tc_fence_after();
+  }
+  __syncwarp();
+  pdl_launch_dependents();
+  // columns of the tile that each CTA of the cluster finishes; partial sums as [sender][token][share + 4] floats
+  const int share = split > 1 ? (BN / 16 + split - 1) / split * 16 : BN;
+  const int pitch = share + 4;
+  const int c0 = min(crank * share, BN), c1 = min(c0 + share, BN);
+  if (split > 1) {
+    cluster_sync();                                           // every CTA of the cluster is done with its rings
+    if (epi && ok) {
+      for (int p = 0; p < split; ++p) {
+        if (p == crank) continue;
+        const uint32_t slot = (uint32_t)(crank < p ? crank : crank - 1);
+        const uint32_t dst = map_cluster_rank(sbase + slot * (uint32_t)(npad * pitch) * 4u, (uint32_t)p);
+        const int p0 = min(p * share, BN), p1 = min(p0 + share, BN);
+        for (int m = 0; m < mt; ++m)
+          for (int c = p0; c < p1; c += 16) {
+            uint32_t o[16], l[16];
+            __syncwarp();
+            tmem_ld16(tmem + m * BN + lane_addr + c, o);
+            if (n_stages > 0) tmem_ld16(tmem_lora + m * BN + lane_addr + c, l);
+            tmem_wait_ld();
+            const int t = m * 128 + lrow;
+            if (t < a.n_tokens) {
+              const uint32_t at = dst + (uint32_t)(t * pitch + c - p0) * 4u;
+#pragma unroll
+              for (int q = 0; q < 16; q += 4) {
+                float4 f = make_float4(__uint_as_float(o[q]), __uint_as_float(o[q + 1]), __uint_as_float(o[q + 2]), __uint_as_float(o[q + 3]));
+                if (n_stages > 0) {
+                  f.x += __uint_as_float(l[q]); f.y += __uint_as_float(l[q + 1]);
+                  f.z += __uint_as_float(l[q + 2]); f.w += __uint_as_float(l[q + 3]);
+                }
+                st_cluster_f32x4(at + 4 * q, f);
+              }
+            }
+          }
+      }
+    }
+    __syncwarp();
+    cluster_sync();
+  }
+  if (epi && ok) {
+    for (int m = 0; m < mt; ++m) {
+      const int t = m * 128 + lrow;
+      for (int c = c0; c < c1; c += 16) {
+        uint32_t o[16], l[16];
+        __syncwarp();
+        tmem_ld16(tmem + m * BN + lane_addr + c, o);
+        if (n_stages > 0) tmem_ld16(tmem_lora + m * BN + lane_addr + c, l);
+        tmem_wait_ld();
+        if (t >= a.n_tokens) continue;
+        float f[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) f[q] = __uint_as_float(o[q]) + (n_stages > 0 ? __uint_as_float(l[q]) : 0.f);
+        for (int p = 0; p + 1 < split; ++p) {
+          const float4* part = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(smem) + (size_t)(p * npad + t) * pitch + (c - c0));
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const float4 v = part[q];
+            f[4 * q] += v.x; f[4 * q + 1] += v.y; f[4 * q + 2] += v.z; f[4 * q + 3] += v.w;
+          }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int col = n0 + c + 8 * h;
+          if (col >= d_out) continue;
+          const uint4 q = make_uint4(pack_bf16(f[8 * h], f[8 * h + 1]), pack_bf16(f[8 * h + 2], f[8 * h + 3]),
+                                     pack_bf16(f[8 * h + 4], f[8 * h + 5]), pack_bf16(f[8 * h + 6], f[8 * h + 7]));
+          if (side < 0) {
+            *reinterpret_cast<uint4*>(a.y[j] + (size_t)t * d_out + col) = q;
+          } else if (kv_slot[m] >= 0) {
+            // [K|V][kv head][slot][128] inside the block
+            unsigned char* dst = a.pv.slab + (size_t)kv_blk[m] * a.pv.block_bytes +
+                                 ((size_t)(side * a.n_kv + col / FL_HEAD_DIM) * a.bt + kv_slot[m]) * (FL_HEAD_DIM * 2) + (col % FL_HEAD_DIM) * 2;
+            *reinterpret_cast<uint4*>(dst) = q;
+            if (side == 1 && kv_last[m])       // V of a request's last token: clear the slots behind it
+              for (int z = kv_slot[m] + 1; z < a.bt; ++z)
+                *reinterpret_cast<uint4*>(dst + (size_t)(z - kv_slot[m]) * (FL_HEAD_DIM * 2)) = make_uint4(0u, 0u, 0u, 0u);
+          }
+        }
+      }
+    }
+    tc_fence_before();
+  }
+  // ------------------------------------------------ teardown
+  __syncthreads();
+  if (*abort_flag) {
+    if (tid == 0) atomicOr(a.pv.flags, (uint32_t)FLAG_WAIT_GAVE_UP);
+    // copies still in flight target this CTA's shared memory: give every armed barrier a bounded chance to complete
+    if (warp == 0 && lane == 0) {
+      for (int s = 0; s < ns; ++s)
+        for (uint32_t i = 0; i < (1u << 16); ++i)
+          if (mbar_try(bar(B_FULL + s), 0) || mbar_try(bar(B_FULL + s), 1)) break;
+    }
+    __syncthreads();
+  }
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ka.tmem_cols) : "memory");
+  }
+}
+
+// Tiles, split of d_in, rings and shared memory of a call.
+void layout(const fl_pool* p, const skinny::Args& a, KArgs* out, uint32_t* smem) {
+  KArgs& ka = *out;
+  memset(&ka, 0, sizeof(ka));
+  ka.s = a;
+  ka.npad = (a.n_tokens + 15) / 16 * 16;
+  int tiles = 0;
+  for (int j = 0; j < a.n_mats; ++j) {
+    ka.tile_base[j] = tiles;
+    tiles += (a.d_out[j] + BN - 1) / BN;
+  }
+  for (int j = a.n_mats; j <= skinny::MAX_LIN; ++j) ka.tile_base[j] = tiles;
+  ka.tmem_cols = ka.npad > 128 ? 512 : 256;
+  const uint32_t fixed = BOOK_BYTES + ROWS_BYTES + ka.npad * UNITS_PER_TOKEN * sizeof(LoraUnit) + 1024;
+  const uint32_t stage = W_BYTES + (uint32_t)ka.npad * 128;
+  const int fit = (int)((SMEM_LIMIT - fixed) / stage);
+  ka.ne = fit >= 9 ? 3 : fit >= 6 ? 2 : 1;
+  ka.ns = std::min(MAX_NS, fit - ka.ne);
+  // As many CTAs per column tile as the SMs hold at once (clusters above two do not fill every SM), every one with at least
+  // four stages of d_in, as long as the partial sums fit in the ring that they reuse.
+  const int nk = (a.d_in + BK - 1) / BK;
+  ka.split = 1;
+  for (int s = 2; s <= MAX_SPLIT; ++s) {
+    const int share = (BN / 16 + s - 1) / s * 16;
+    if (tiles * s <= (s == 2 ? p->sm_count : p->sm_count * 9 / 10) && nk / s >= 4 &&
+        (uint32_t)((s - 1) * ka.npad * (share + 4) * 4) <= ka.ns * stage)
+      ka.split = s;
+  }
+  *smem = fixed + (ka.ns + ka.ne) * stage;
+}
+
+}  // namespace
+
+namespace skinny {
+
+int launch(fl_pool* p, const Args& a, const void* x, const void* const* w, cudaStream_t st) {
+  KArgs ka;
+  uint32_t smem;
+  layout(p, a, &ka, &smem);
+  const unsigned ctas = (unsigned)(ka.tile_base[a.n_mats] * ka.split);
+  Maps maps;
+  {
+    const uint64_t dims[2] = {(uint64_t)a.d_in, (uint64_t)a.n_tokens};
+    const uint64_t strides[1] = {(uint64_t)a.d_in * 2};
+    const uint32_t box[2] = {BK, (uint32_t)ka.npad};
+    const int rc = tmap::encode_bf16(&maps.x, x, 2, dims, strides, box);
+    if (rc != FL_OK) return rc;
+  }
+  for (int j = 0; j < MAX_LIN; ++j) {
+    if (j >= a.n_mats) { maps.w[j] = maps.w[0]; continue; }
+    const uint64_t dims[2] = {(uint64_t)a.d_out[j], (uint64_t)a.d_in};
+    const uint64_t strides[1] = {(uint64_t)a.d_out[j] * 2};
+    const uint32_t box[2] = {64, BK};
+    const int rc = tmap::encode_bf16(&maps.w[j], w[j], 2, dims, strides, box);
+    if (rc != FL_OK) return rc;
+  }
+  static bool configured[16] = {};
+  if (!configured[p->device & 15]) {
+    FL_CUDA(p, cudaFuncSetAttribute(lora_skinny_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT));
+    configured[p->device & 15] = true;
+  }
+  FL_CUDA(p, launch_pdl_cluster(lora_skinny_kernel, dim3(ctas), dim3((unsigned)ka.split), dim3(THREADS), smem, st, ka, maps));
+  FL_CUDA(p, cudaGetLastError());
+  return FL_OK;
+}
+
+}  // namespace skinny

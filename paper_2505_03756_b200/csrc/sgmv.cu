@@ -38,6 +38,7 @@ struct SgmvArgs {
   int n_seg, n_tokens;
   float scale;
   float* v;        // [n_mats][ksplit][n_tokens][RMAX]
+  __nv_bfloat16* v16;   // where the scaled bf16 sum goes instead, [n_mats][n_tokens][RMAX] (tiles of 16 tokens only), or null
   int ksplit;
   int tc_ksplit;     // slices of d_in for the tcgen05 shrink of long segments (0 = not applicable)
   int expand_cols;   // y columns one expand CTA covers
@@ -64,6 +65,9 @@ __device__ __forceinline__ uint4 add_bf16x8(uint4 a, uint4 b) {
   return r;
 }
 
+// the pipeline's stages, and for short tiles (which reuse it) the sums of the four warps
+__host__ __device__ constexpr int shrink_pipe_bytes(int tm, int rmax) { return SH_STAGES * (tm + rmax) * 128; }
+
 template <int TM, int RMAX>
 __global__ void __launch_bounds__(SG_THREADS) sgmv_shrink_kernel(const SgmvArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -88,6 +92,8 @@ __global__ void __launch_bounds__(SG_THREADS) sgmv_shrink_kernel(const SgmvArgs 
   // into a graph): its extra rank-rows are left out, and the status word says so
   if (e->rank > RMAX && tid == 0) atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_LORA);
   const uint32_t table_off = e->table_off;
+  const bool clustered = TM == 16 && a.v16 && a.ksplit > 1;
+  if (clustered) cluster_arrive();       // "this CTA is running"; the others wait for it before they store into its memory
   const int d_in = lm.d_in;
   const int kchunk = ((d_in + a.ksplit * KS - 1) / (a.ksplit * KS)) * KS;
   const int kb = split * kchunk, ke = min(d_in, kb + kchunk);
@@ -159,9 +165,9 @@ __global__ void __launch_bounds__(SG_THREADS) sgmv_shrink_kernel(const SgmvArgs 
       }
     }
   }
-  float* vout = a.v + ((size_t)(j * a.ksplit + split) * a.n_tokens) * RMAX;
   const int g = lane >> 2, t4 = lane & 3;
   if (TM == 64) {
+    float* vout = a.v + ((size_t)(j * a.ksplit + split) * a.n_tokens) * RMAX;
 #pragma unroll
     for (int n = 0; n < RMAX / 8; ++n) {
       const int r0 = tok0 + warp * 16 + g;
@@ -178,12 +184,41 @@ __global__ void __launch_bounds__(SG_THREADS) sgmv_shrink_kernel(const SgmvArgs 
       r[0] = acc[n][0]; r[1] = acc[n][1];
       r[8 * RMAX] = acc[n][2]; r[8 * RMAX + 1] = acc[n][3];
     }
+    if (!a.v16) {
+      __syncthreads();
+      float* vout = a.v + ((size_t)(j * a.ksplit + split) * a.n_tokens) * RMAX;
+      for (int i = tid; i < 16 * RMAX; i += SG_THREADS) {
+        const int row = i / RMAX;
+        if (tok0 + row < tok1)
+          vout[(size_t)(tok0 + row) * RMAX + (i % RMAX)] =
+              red[i] + red[16 * RMAX + i] + red[32 * RMAX + i] + red[48 * RMAX + i];
+      }
+      return;
+    }
+    // The final form is wanted: the slices of d_in are the CTAs of one cluster, and each hands its sums to the first one
+    // through distributed shared memory.  The slices are added in order: the result does not depend on timing.  (Where an
+    // expand of the same few microseconds follows, it adds the slices itself: the cluster's barrier costs 1 to 2 us more than
+    // it saves there.)
+    float* all = reinterpret_cast<float*>(smem + shrink_pipe_bytes(TM, RMAX));      // first CTA: [slice][16 rows][RMAX]
     __syncthreads();
+    if (clustered) cluster_wait();
+    const uint32_t dst = clustered ? map_cluster_rank(smem_u32(all + split * 16 * RMAX), 0) : 0;
     for (int i = tid; i < 16 * RMAX; i += SG_THREADS) {
-      const int row = i / RMAX;
-      if (tok0 + row < tok1)
-        vout[(size_t)(tok0 + row) * RMAX + (i % RMAX)] =
-            red[i] + red[16 * RMAX + i] + red[32 * RMAX + i] + red[48 * RMAX + i];
+      const float sum = red[i] + red[16 * RMAX + i] + red[32 * RMAX + i] + red[48 * RMAX + i];
+      if (clustered) st_cluster_f32(dst + 4u * i, sum);
+      else all[i] = sum;
+    }
+    if (clustered) cluster_sync(); else __syncthreads();
+    if (split == 0) {
+      const size_t vout = (size_t)j * a.n_tokens * RMAX;
+      for (int i = tid; i < 16 * RMAX; i += SG_THREADS) {
+        const int row = i / RMAX;
+        if (tok0 + row < tok1) {
+          float sum = 0.f;
+          for (int sp = 0; sp < a.ksplit; ++sp) sum += all[sp * 16 * RMAX + i];
+          a.v16[vout + (size_t)(tok0 + row) * RMAX + (i % RMAX)] = __float2bfloat16_rn(sum * a.scale);
+        }
+      }
     }
   }
 }
@@ -555,10 +590,11 @@ template <int TM, int RMAX>
 int launch_pair(fl_pool* p, SgmvArgs& a, int tiles, int d_out_max, cudaStream_t st, bool shrink_only) {
   a.expand_cols = pick_expand_cols(a, tiles);
   static bool configured[16] = {};
-  const int shrink_smem = SH_STAGES * (TM + RMAX) * 128;
+  const int shrink_smem_max = shrink_pipe_bytes(TM, RMAX) + (TM == 16 ? KSPLIT_MAX * 16 * RMAX * 4 : 0);
+  const int shrink_smem = a.v16 ? shrink_smem_max : shrink_pipe_bytes(TM, RMAX);      // + every slice's sums
   const int expand_smem = expand_smem_bytes(TM, RMAX);     // two stages of (y, B) + the LoRA-term tile
   if (!configured[p->device & 15]) {
-    FL_CUDA(p, cudaFuncSetAttribute(sgmv_shrink_kernel<TM, RMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, shrink_smem));
+    FL_CUDA(p, cudaFuncSetAttribute(sgmv_shrink_kernel<TM, RMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, shrink_smem_max));
     FL_CUDA(p, cudaFuncSetAttribute(sgmv_expand_kernel<TM, RMAX, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, expand_smem));
     FL_CUDA(p, cudaFuncSetAttribute(sgmv_expand_kernel<TM, RMAX, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, expand_smem));
     configured[p->device & 15] = true;
@@ -588,7 +624,8 @@ int launch_pair(fl_pool* p, SgmvArgs& a, int tiles, int d_out_max, cudaStream_t 
     }
     FL_CUDA(p, launch_pdl(sgmv_shrink3_kernel<RMAX>, dim3(tiles, a.ksplit), dim3(SG_THREADS), smem3, st, a));
   } else {
-    FL_CUDA(p, launch_pdl(sgmv_shrink_kernel<TM, RMAX>, dim3(tiles * a.n_mats, a.ksplit), dim3(SG_THREADS), shrink_smem, st, a));
+    FL_CUDA(p, launch_pdl_cluster(sgmv_shrink_kernel<TM, RMAX>, dim3(tiles * a.n_mats, a.ksplit), dim3(1, a.v16 ? a.ksplit : 1),
+                                  dim3(SG_THREADS), shrink_smem, st, a));
   }
   if (shrink_only) return FL_OK;       // the caller consumes the partial sums itself
   const dim3 egrid(tiles * a.n_mats, (d_out_max + a.expand_cols - 1) / a.expand_cols);
@@ -626,7 +663,7 @@ struct KvDest {      // where K and V results go when they are appended to the p
 int sgmv_common(fl_pool* p, fl_bf16* const* ys, const fl_bf16* x, const int* mat_indices, int n_mats,
                 const int32_t* seg_indptr, const int32_t* lora_ids, int n_seg, int n_tokens,
                 float scale, void* workspace, size_t workspace_bytes, fl_stream stream, const KvDest* kv,
-                sgmv::ShrinkInfo* shrink_only = nullptr) {
+                sgmv::ShrinkInfo* shrink_only = nullptr, bool scaled = false) {
   if (!p || n_mats < 1 || n_mats > FL_MAX_MATS || n_seg < 0 || n_tokens < 0 || !ys || !mat_indices) return FL_EINVAL;
   if (n_seg == 0 || n_tokens == 0) return FL_OK;
   if (!x || !seg_indptr || !lora_ids || !workspace) return FL_EINVAL;
@@ -683,7 +720,8 @@ int sgmv_common(fl_pool* p, fl_bf16* const* ys, const fl_bf16* x, const int* mat
   int prev = -1;
   cudaGetDevice(&prev);
   if (prev != p->device) cudaSetDevice(p->device);
-  const bool small = n_tokens <= 16 * n_seg;   // average segment of at most 16 tokens: decode-like
+  a.v16 = scaled ? reinterpret_cast<__nv_bfloat16*>(workspace) : nullptr;
+  const bool small = scaled || n_tokens <= 16 * n_seg;   // average segment of at most 16 tokens: decode-like
   const int rmax = rmax_of(p);
   const cudaStream_t st = (cudaStream_t)stream;
   if (!small && rmax == 16 && a.ksplit == 1) {
@@ -716,6 +754,8 @@ int sgmv_common(fl_pool* p, fl_bf16* const* ys, const fl_bf16* x, const int* mat
   }
   if (small) {
     const int tiles = n_seg + n_tokens / 16;
+    // slices of d_in so that all CTAs run at once: at rank 64 three of them fit on an SM, below that at least five
+    if (scaled) a.ksplit = std::max(1, std::min(KSPLIT_MAX, (rmax == 64 ? 3 : 4) * p->sm_count / (tiles * n_mats)));
     rc = rmax == 16 ? launch_pair<16, 16>(p, a, tiles, d_out_max, st, so)
        : rmax == 32 ? launch_pair<16, 32>(p, a, tiles, d_out_max, st, so)
                     : launch_pair<16, 64>(p, a, tiles, d_out_max, st, so);
@@ -738,6 +778,13 @@ int shrink(fl_pool* p, const fl_bf16* x, const int* mat_indices, int n_mats, con
   fl_bf16* none[FL_MAX_MATS] = {};
   return sgmv_common(p, none, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, 1.f, workspace,
                      workspace_bytes, stream, nullptr, info);
+}
+int shrink_scaled(fl_pool* p, const fl_bf16* x, const int* mat_indices, int n_mats, const int32_t* seg_indptr,
+                  const int32_t* lora_ids, int n_seg, int n_tokens, float scale, void* workspace, size_t workspace_bytes,
+                  fl_stream stream, ShrinkInfo* info) {
+  fl_bf16* none[FL_MAX_MATS] = {};
+  return sgmv_common(p, none, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace,
+                     workspace_bytes, stream, nullptr, info, true);
 }
 }  // namespace sgmv
 

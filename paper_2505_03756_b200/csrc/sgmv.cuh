@@ -15,7 +15,11 @@ struct ShrinkInfo {
 int shrink(fl_pool* p, const fl_bf16* x, const int* mat_indices, int n_mats, const int32_t* seg_indptr,
            const int32_t* lora_ids, int n_seg, int n_tokens, void* workspace, size_t workspace_bytes, fl_stream stream,
            ShrinkInfo* info);
-
+// The same in its final form: slices added, scaled, rounded to bf16 as the expand product takes them, [projection][token][rmax].
+// Tiles of 16 tokens whatever the segments' lengths: meant for batches of a few hundred tokens.
+int shrink_scaled(fl_pool* p, const fl_bf16* x, const int* mat_indices, int n_mats, const int32_t* seg_indptr,
+                  const int32_t* lora_ids, int n_seg, int n_tokens, float scale, void* workspace, size_t workspace_bytes,
+                  fl_stream stream, ShrinkInfo* info);
 
 #ifdef __CUDACC__
 // Token tile `tile` (tiles of TM tokens, counted over segments that carry an adapter, or over all segments) -> segment and

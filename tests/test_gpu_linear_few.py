@@ -1,0 +1,77 @@
+"""fl_lora_linear* on batches of at most 256 tokens (W streamed once for all of them), at the sizes where its tiles end:
+token counts around multiples of 16, 128 and 256 and the two ends of the range, ranks that end inside a 16-row step or a
+64-row stage, widths that end inside a column tile or a k-stage, one CTA per column tile up to a cluster of eight."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from oracle.lora import lora_linear
+from paper_2505_03756_b200 import synth
+
+from _util import assert_close, oracle_adapters
+
+RANKS = [1, 8, 5, 24, 32, 33, 64, 16]
+
+
+def _workload(T, shape, per_req, n_adapters):
+    """T tokens in requests of `per_req` tokens (the last one takes the rest), ranks from RANKS, every fifth request without
+    an adapter."""
+    n = max(1, T // per_req)
+    wl = synth.make_workload("decode13b", n_req=n, len_range=(3, 40), n_adapters=n_adapters, shape=shape)
+    wl.ranks[:] = [RANKS[i % len(RANKS)] for i in range(n_adapters)]
+    wl.new_lens[:] = per_req
+    wl.new_lens[-1] += T - n * per_req
+    wl.lora_of_req[2::5] = -1
+    wl.lora_of_req.sort()
+    wl.pool_blocks = int(np.sum((wl.prefix_lens + wl.new_lens + 15) // 16)) + 130 * n_adapters + 64
+    return wl
+
+
+@pytest.mark.parametrize("T,per_req,hidden,heads", [
+    (1, 1, 1024, (8, 8)), (2, 1, 4096, (32, 32)), (15, 1, 328, (3, 1)), (16, 16, 328, (3, 1)), (17, 1, 1024, (8, 8)),
+    (33, 11, 200, (2, 1)), (127, 1, 1024, (8, 8)), (129, 43, 328, (3, 1)), (200, 100, 1024, (8, 2)), (255, 1, 328, (3, 1)),
+    (256, 256, 1024, (8, 8)), (256, 1, 2048, (4, 1)), (257, 1, 328, (3, 1))])
+def test_linear_of_few_tokens(T, per_req, hidden, heads):
+    from paper_2505_03756_b200 import binding as fl, harness as H
+    wl = _workload(T, synth.LayerShape(hidden, *heads), per_req, 12)
+    assert wl.n_tokens == T
+    s = H.Session(wl)
+    try:
+        s.load_adapters()
+        s.build_batch()
+        s.fill_prefix_kv()
+        dims = dict((n, o) for n, _, o in wl.shape.mats)
+        seg, ids = wl.segments()
+        x = wl.x("q")
+        tx = H.f32_to_dev(x, s.dev)
+        tw = {m: H.f32_to_dev(wl.weight(m), s.dev) for m in "qkvo"}
+        want = {m: lora_linear(x, wl.weight(m), seg, ids, oracle_adapters(wl, m), wl.scale) for m in "qkv"}
+        # q, k, v into y, with K and V stored afterwards; then the fused call, bit for bit the same
+        ty = [torch.full((T, dims[m]), 7.0, dtype=torch.bfloat16, device=s.dev) for m in "qkv"]
+        s.lora_linear(ty, tx, [tw[m] for m in "qkv"], ["q", "k", "v"])
+        for m, t in zip("qkv", ty):
+            assert_close(H.dev_to_f32(t), want[m], f"few tokens {T} {m}")
+        blocks = sorted({int(b) for t in s.kv_tables for b in t})
+        s.kv_append(ty[1], ty[2])
+        torch.cuda.synchronize()
+        stored = fl.device_block_bytes(s.pool, s.block_bytes, blocks)
+        junk = torch.full_like(ty[1], 5.0)
+        s.kv_append(junk, junk)
+        y_q = torch.full_like(ty[0], -5.0)
+        s.lora_linear_qkv_append(y_q, tx, tw["q"], tw["k"], tw["v"])
+        torch.cuda.synchronize()
+        assert torch.equal(y_q, ty[0])
+        assert np.array_equal(fl.device_block_bytes(s.pool, s.block_bytes, blocks), stored)
+        # one projection (narrow: more CTAs per column tile), and the LoRA term alone against its own size
+        xo = wl.x("o")
+        y_o = torch.full((T, hidden), 3.0, dtype=torch.bfloat16, device=s.dev)
+        s.lora_linear([y_o], H.f32_to_dev(xo, s.dev), [tw["o"]], ["o"])
+        assert_close(H.dev_to_f32(y_o), lora_linear(xo, wl.weight("o"), seg, ids, oracle_adapters(wl, "o"), wl.scale), f"few tokens {T} o")
+        s.lora_linear([y_o], H.f32_to_dev(xo, s.dev), [torch.zeros_like(tw["o"])], ["o"])
+        assert_close(H.dev_to_f32(y_o), lora_linear(xo, np.zeros_like(wl.weight("o")), seg, ids, oracle_adapters(wl, "o"), wl.scale),
+                     f"few tokens {T} LoRA term")
+        assert s.status()["device_flags"] == 0
+    finally:
+        s.close()
