@@ -52,12 +52,6 @@ enum { C_QFULL = 0, C_QEMPTY = 1, C_FULL = 2, C_EMPTY = C_FULL + NSLOT, C_SFULL 
        C_ODONE = C_PFULL + 2, C_UFULL = C_ODONE + 2, C_UEMPTY = C_UFULL + 2, C_COUNT = C_UEMPTY + 2 };
 constexpr int UNIT_READERS = 9;                        // MMA issuer + 8 softmax warps
 
-// 32 bytes to a 32-byte aligned global address in one instruction.
-__device__ __forceinline__ void st_global_v8(void* dst, const uint32_t* r) {
-  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]),
-               "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
-}
-
 struct Unit {           // what a CTA works on at one time
   int tok0[2];          // first token row (in the packed q / out tensors) of each tile
   int hq[2];            // query head of each tile

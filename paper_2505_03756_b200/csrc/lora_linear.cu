@@ -1,25 +1,28 @@
 // Base projection with the LoRA branch folded in: y = x W + scale * (x A_i) B_i per segment (Eq. 1: W' = W + A B;
 // Eq. 2: the same branch on the K/V projections), written once, never read back.
 //
-// A persistent tcgen05 GEMM.  One CTA per SM walks tiles of 128 tokens x BN output columns; the accumulator of a
-// tile lives in TMEM (two buffers, so the epilogue of one tile overlaps the MMAs of the next).  The LoRA branch is a
-// few extra k-steps into the same accumulator: for every segment that overlaps the tile, the shrink result
-// v = x A_i of the tile's tokens (rows outside the segment zeroed, scaled, rounded to bf16) times the adapter's B
-// rank-rows of the tile's columns, fetched through the adapter's block table out of the pool blocks.  A tile thus
-// needs no alignment with the segments, and a decode batch whose every token uses another adapter is the same
-// code path (one extra 16..64-deep k-block per token's adapter).
-//   warp 0      TMA producer: x tile [128 x 64] (K-major) and W tile [64 x BN] (N contiguous, as stored) per stage
-//   warp 1      MMA issuer: per tile first the LoRA stages, then the d_in / 64 main stages, 128 x BN x 16 MMAs
-//   warps 2-5   LoRA stage filler (v rows and B rows into a ring slot, by hand, in the swizzled operand layout),
-//               then epilogue of the tile: TMEM -> bf16 -> y
-// Main stages and LoRA stages (32 ranks each) have rings of their own, each with one producer and one consumer, so a
-// parity wait never has to tell phases two apart; a plan kernel lists, per 128-token tile, the LoRA stages it needs.
-// Every mbarrier wait is bounded; a wait that gives up raises a sticky flag, the CTA drains its copies and frees
-// its TMEM.  No cluster launch, no multicast.
+// A persistent tcgen05 GEMM.  A pair of CTAs on two neighbouring SMs (cta_group::2) walks tiles of 256 tokens x BN output
+// columns: each CTA holds 128 token rows of x and half of the tile's columns of W, and the pair's tensor cores read both
+// halves, so a k-step costs each SM two thirds of the shared-memory fill that a 128 x BN tile of its own would.  The
+// accumulator lives in TMEM (each CTA its own rows, two buffers, so the epilogue of one tile overlaps the MMAs of the next).
+// The LoRA branch is a few more k-steps into the same accumulator: the rank-rows of every adapter that overlaps the tile, 16
+// to a unit and two units to a LoRA stage, against a matrix that holds in row t the shrink result of token t (slices
+// summed, scaled, rounded to bf16) at the ranks of its own adapter and zeros elsewhere.  A tile thus needs no alignment with
+// the segments.  The stages are spread over the second half of the tile's main stages: their place in the order of the
+// sums is fixed, and a tile of many one-token segments fills its stages while the tensor cores work on.
+//   warp 0       TMA producer: x tile [128 x 64] (K-major) and W tile [64 x BN/2] (N contiguous, as stored) per stage
+//   warp 1       MMA issuer (of the pair's first CTA, for both)
+//   warps 2-5    epilogue: TMEM -> bf16 -> y, or K and V rows straight into each token's pool block
+//   warps 6-13   LoRA stages, warps 6-9 the even ones, 10-13 the odd ones
+// What bounds it: the tensor cores, and above them the power limit.  A layer step of 16 prompts (4907 tokens, 7B) went 737
+// -> 665 us, of 4 prompts of 1024 new tokens (34B, rank 64) 1727 -> 1507 us against the tiles of 128 tokens per CTA before;
+// with 28 one-token segments next to 4 prompts (7B, ranks 8 to 64) 734 -> 453 us, because a stage now takes the rank-rows of
+// two to four segments and is filled side by side instead of one by one.
+// Every mbarrier wait is bounded; a wait that gives up raises a sticky flag, the CTA drains its copies, meets its partner
+// and frees its TMEM.  No multicast.
 #include <cuda.h>
 #include <string.h>
 #include <algorithm>
-#include "lora_plan.cuh"
 #include "lora_skinny.cuh"
 #include "mma_utils.cuh"
 #include "pool.cuh"
@@ -31,32 +34,34 @@ namespace {
 
 using namespace tc;
 
-using lora_plan::BM;
-using lora_plan::ER;
-using lora_plan::EXT_CAP;
-
-constexpr int LT_THREADS = 192;
+constexpr int LT_THREADS = 448;
+constexpr int BM = 128;                          // token rows per CTA; a pair's tile has twice as many
 constexpr int BK = 64;
 constexpr int MAX_LIN = 3;                       // projections per launch (q, k, v share x)
+constexpr int UNIT = 16;                         // rank-rows per entry of a tile's LoRA list: one k-step
+constexpr int ER = 2 * UNIT;                     // rank-rows per LoRA stage
+constexpr int MAX_UNITS = 2 * BM * (FL_MAX_RANK / UNIT);
+constexpr int GROUP = 8;                         // LoRA stages whose row addresses are looked up together
+constexpr int RASTER = 8;                        // token tiles that are walked together over a projection's columns
 constexpr uint32_t A_BYTES = BM * BK * 2;        // x tile, K-major: 128 rows of 128 bytes
 constexpr uint32_t B_GROUP = BK * 128;           // one 64-column group of a W tile: 64 k-rows of 128 bytes
 
 template <int BN>
 struct Cfg {
-  static constexpr uint32_t B_BYTES = (BN / 64) * B_GROUP;
+  static constexpr int BH = BN / 2;                           // columns of W this CTA loads
+  static constexpr uint32_t B_BYTES = (BH / 64) * B_GROUP;
   static constexpr uint32_t STAGE = A_BYTES + B_BYTES;
-  static constexpr int NS = BN == 256 ? 4 : BN == 128 ? 5 : 6;
-  // a LoRA stage: v tile [128 x 32 ranks] in 128-byte rows (half of each row used) + B rows [32 x BN]
-  static constexpr uint32_t EB_GROUP = ER * 128;
-  static constexpr uint32_t EXT = A_BYTES + (BN / 64) * EB_GROUP;
-  static constexpr int NE = BN == 256 ? 1 : BN == 128 ? 2 : 4;
+  static constexpr int NS = BN == 256 ? 5 : 7;
+  // two LoRA stages side by side in one buffer of a main stage's layout: ranks 0-31 and 32-63 of every row
   static constexpr uint32_t OFF_EXT = NS * STAGE;
-  static constexpr uint32_t OFF_BAR = OFF_EXT + NE * EXT;
-  static constexpr uint32_t SMEM = OFF_BAR + 256 + 1024;      // barriers and bookkeeping; slack for 1024-byte alignment
+  static constexpr uint32_t OFF_ROWS = OFF_EXT + STAGE;       // B row addresses of two groups of LoRA stages
+  static constexpr uint32_t OFF_LIST = OFF_ROWS + 2 * GROUP * ER * 8;
+  static constexpr uint32_t OFF_BAR = OFF_LIST + MAX_UNITS * 8;
+  static constexpr uint32_t SMEM = OFF_BAR + 512 + 1024;      // barriers and bookkeeping; slack for 1024-byte alignment
   static constexpr uint32_t TMEM_COLS = 2 * BN;               // two accumulators
-  static_assert(TMEM_COLS == 512 || TMEM_COLS == 256 || TMEM_COLS == 128, "TMEM allocations are powers of two");
+  static_assert(TMEM_COLS == 512 || TMEM_COLS == 256, "TMEM allocations are powers of two");
   static_assert(SMEM <= 227 * 1024, "shared memory");
-  static_assert(EXT % 1024 == 0 && STAGE % 1024 == 0, "operand tiles start on 1024-byte boundaries");
+  static_assert(STAGE % 1024 == 0, "operand tiles start on 1024-byte boundaries");
 };
 
 struct LinArgs {
@@ -69,10 +74,9 @@ struct LinArgs {
   int n_seg, n_tokens, d_in;
   int n_mats;
   __nv_bfloat16* y[MAX_LIN];
+  int wide[MAX_LIN];           // rows of y start on 32-byte boundaries
   int d_out[MAX_LIN], mat_index[MAX_LIN], n_tiles_n[MAX_LIN], tile_base[MAX_LIN + 1];
   int m_tiles;
-  const int* ext_count;        // per 128-token tile: LoRA stages (32 ranks of one overlapping segment's adapter)
-  const int* ext_list;         // [m_tiles][EXT_CAP]: segment << 1 | which half of the ranks
   // K / V projections whose rows go straight into the requests' pool blocks (kv_side: -1 = rows go to y, 0 = K, 1 = V)
   int kv_side[MAX_LIN];
   const int32_t* req_indptr;
@@ -90,241 +94,176 @@ struct LinMaps {
 struct Tile {
   int j, m, n;       // projection, token tile, column tile
 };
+// Tiles run over the tokens first, RASTER token tiles at a time, then over the columns: the pairs' tiles in flight (74 on a
+// B200) share about nine column slices of W and eight x tiles, and W is read from memory once per RASTER token tiles.
 __device__ __forceinline__ Tile decode_tile(const LinArgs& a, int idx) {
   Tile t;
   t.j = 0;
   while (t.j + 1 < a.n_mats && idx >= a.tile_base[t.j + 1]) ++t.j;
-  const int local = idx - a.tile_base[t.j];
-  t.m = local / a.n_tiles_n[t.j];
-  t.n = local - t.m * a.n_tiles_n[t.j];
+  const int local = idx - a.tile_base[t.j], nt = a.n_tiles_n[t.j];
+  const int g = local / (RASTER * nt), r = local - g * RASTER * nt;
+  const int gm = min(RASTER, a.m_tiles - g * RASTER);
+  t.n = r / gm;
+  t.m = g * RASTER + (r - t.n * gm);
   return t;
 }
 
+// A LoRA unit: adapter (20 bits) | first rank / 16 (2) | rank-rows (5) | first token of the tile (9) | behind the last one (9)
+__device__ __forceinline__ unsigned long long pack_unit(int lid, int q, int nr, int lo, int hi) {
+  return (unsigned long long)lid << 25 | (unsigned long long)((uint32_t)q << 23 | (uint32_t)nr << 18 | (uint32_t)lo << 9 | (uint32_t)hi);
+}
+static_assert(FL_MAX_LORA_ID <= 1 << 20 && FL_MAX_RANK / UNIT <= 4 && 2 * BM < 512, "fields of a LoRA unit");
+
 template <int BN, int RMAX>
-__global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const LinArgs a, const __grid_constant__ LinMaps maps) {
+__global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid_constant__ LinArgs a, const __grid_constant__ LinMaps maps) {
   using C = Cfg<BN>;
-  constexpr int NS = C::NS;
+  constexpr int NS = C::NS, BH = C::BH;
   extern __shared__ unsigned char smem_raw[];
   // the swizzled operand tiles need 1024-byte alignment
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const uint32_t sbase = smem_u32(smem);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  constexpr int NE = C::NE;
-  enum { B_FULL = 0, B_EMPTY = NS, B_ACC_FULL = 2 * NS, B_ACC_EMPTY = 2 * NS + 2, B_EFULL = 2 * NS + 4,
-         B_EEMPTY = B_EFULL + NE, B_COUNT = B_EEMPTY + NE };
+  const int crank = (int)cluster_ctarank();
+  const bool leader = crank == 0;
+  enum { B_FULL = 0, B_EMPTY = NS, B_ACC_FULL = 2 * NS, B_ACC_EMPTY = B_ACC_FULL + 2, B_EFULL = B_ACC_EMPTY + 2, B_EEMPTY = B_EFULL + 2,
+         B_LFULL = B_EEMPTY + 2, B_LEMPTY = B_LFULL + 2, B_COUNT = B_LEMPTY + 2 };
   const uint32_t bar0 = sbase + C::OFF_BAR;
   auto bar = [&](int k) { return bar0 + 8u * k; };
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + C::OFF_BAR + 8 * B_COUNT);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_BAR + 8 * B_COUNT + 4);
-  volatile int* ext_ksteps = reinterpret_cast<volatile int*>(smem + C::OFF_BAR + 8 * B_COUNT + 8);   // [NE]
-  static_assert(8 * B_COUNT + 8 + 4 * NE <= 256, "bookkeeping area too small");
+  volatile int* n_ext_slot = reinterpret_cast<volatile int*>(smem + C::OFF_BAR + 8 * B_COUNT + 8);   // [2] LoRA stages of a tile
+  int* scan = reinterpret_cast<int*>(smem + C::OFF_BAR + 8 * B_COUNT + 16);                          // [8] per filler warp
+  static_assert(8 * B_COUNT + 16 + 32 <= 512, "bookkeeping area too small");
 
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) {
       mbar_init(bar(B_FULL + s), 1);
       mbar_init(bar(B_EMPTY + s), 1);
     }
-    for (int e = 0; e < NE; ++e) {
-      mbar_init(bar(B_EFULL + e), 1);
-      mbar_init(bar(B_EEMPTY + e), 1);
-    }
     for (int b = 0; b < 2; ++b) {
       mbar_init(bar(B_ACC_FULL + b), 1);
-      mbar_init(bar(B_ACC_EMPTY + b), 4);
+      mbar_init(bar(B_ACC_EMPTY + b), 8);      // the epilogue warps of both CTAs
+      mbar_init(bar(B_EFULL + b), 2);          // both CTAs' fillers
+      mbar_init(bar(B_EEMPTY + b), 1);
+      mbar_init(bar(B_LFULL + b), 1);
+      mbar_init(bar(B_LEMPTY + b), 1);
     }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void*)tmem_slot)), "r"(C::TMEM_COLS) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void*)tmem_slot)), "r"(C::TMEM_COLS) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync();          // both CTAs' barriers exist
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  pdl_wait();     // x, the shrink's partial sums and the plan are the work of the kernels before this one
+  // Behind the shrink everything but v was finished before this kernel could start (the shrink lets it start after its own
+  // wait); without one, the kernel before may still be writing x.
+  if (a.n_seg == 0) pdl_wait();
 
   const int total = a.tile_base[a.n_mats];
   const int nk = (a.d_in + BK - 1) / BK;
+  const int first = blockIdx.x >> 1, step = gridDim.x >> 1;      // pairs
 
   if (warp == 0) {
-    // ------------------------------------------------ TMA producer (one lane)
+    // ------------------------------------------------ TMA producer (one lane): this CTA's halves; both CTAs' bytes are counted
+    // on the first CTA's barrier
     if (lane == 0) {
-      long long f = 0;       // main stages so far
-      bool ok = true;
-      for (int idx = blockIdx.x; ok && idx < total; idx += gridDim.x) {
+      const uint32_t full0 = map_cluster_rank(bar(B_FULL), 0);
+      int s = 0;
+      uint32_t ph = 1;
+      bool wrapped = false, ok = true;
+      for (int idx = first; ok && idx < total; idx += step) {
         const Tile t = decode_tile(a, idx);
         const CUtensorMap* wm = &maps.w[t.j];
-        for (int ks = 0; ks < nk; ++ks, ++f) {
-          const int s = (int)(f % NS);
-          const long long use = f / NS;
-          if (use > 0) ok = mbar_wait(bar(B_EMPTY + s), (uint32_t)((use - 1) & 1), abort_flag);
+        const int row0 = t.m * (2 * BM) + crank * BM, col0 = t.n * BN + crank * BH;
+        for (int ks = 0; ks < nk; ++ks) {
+          if (wrapped) ok = mbar_wait(bar(B_EMPTY + s), ph, abort_flag);
           if (!ok) break;
-          mbar_expect_tx(bar(B_FULL + s), C::STAGE);
-          const uint32_t dst = sbase + s * C::STAGE;
-          tma_load_2d(dst, &maps.x, bar(B_FULL + s), ks * BK, t.m * BM);
+          if (leader) mbar_expect_tx(bar(B_FULL + s), 2 * C::STAGE);
+          const uint32_t dst = sbase + s * C::STAGE, fb = full0 + 8u * s;
+          tma_load_2d_pair(dst, &maps.x, fb, ks * BK, row0);
 #pragma unroll
-          for (int g = 0; g < BN / 64; ++g)
-            tma_load_2d(dst + A_BYTES + g * B_GROUP, wm, bar(B_FULL + s), t.n * BN + g * 64, ks * BK);
+          for (int g = 0; g < BH / 64; ++g) tma_load_2d_pair(dst + A_BYTES + g * B_GROUP, wm, fb, col0 + g * 64, ks * BK);
+          if (++s == NS) { s = 0; ph ^= 1u; wrapped = true; }
         }
       }
     }
   } else if (warp == 1) {
-    // ------------------------------------------------ MMA issuer (one lane)
-    if (lane == 0) {
-      constexpr uint32_t IDESC = instr_desc(BN, true);     // A (x, v) K-major, B (W, adapter rows) N-contiguous
-      long long f = 0, g = 0;      // main stages and LoRA stages so far
+    // ------------------------------------------------ MMA issuer: the whole warp runs converged, an elected lane issues
+    if (leader) {
+      constexpr uint32_t IDESC = instr_desc_pair(BN, true);     // A (x, v) K-major, B (W, adapter rows) N-contiguous
+      constexpr uint32_t HI = desc_hi(1024);
+      auto wait_all = [&](uint32_t b, uint32_t parity) {
+        if (__all_sync(0xffffffffu, mbar_try_cluster(b, parity))) return true;       // the common case: one test
+        return __all_sync(0xffffffffu, mbar_wait_cluster(b, parity, abort_flag)) != 0;
+      };
+      const uint32_t a_lo0 = desc_lo(sbase, 16), b_lo0 = desc_lo(sbase + A_BYTES, B_GROUP);
+      const uint32_t ea_lo0 = desc_lo(sbase + C::OFF_EXT, 16), eb_lo0 = desc_lo(sbase + C::OFF_EXT + A_BYTES, B_GROUP);
+      int s = 0, es = 0;
+      uint32_t ph = 0, eph = 0;
       bool ok = true;
-      int k = 0;             // tiles of this CTA so far
-      for (int idx = blockIdx.x; ok && idx < total; idx += gridDim.x, ++k) {
-        const Tile t = decode_tile(a, idx);
-        const int n_ext = a.ext_count[t.m];
+      int k = 0;             // tiles of this pair so far
+      const int half = nk / 2;
+      for (int idx = first; ok && idx < total; idx += step, ++k) {
         const int buf = k & 1;
-        if (k >= 2) ok = mbar_wait(bar(B_ACC_EMPTY + buf), (uint32_t)(((k >> 1) - 1) & 1), abort_flag);
+        if (k >= 2) ok = wait_all(bar(B_ACC_EMPTY + buf), (uint32_t)(((k >> 1) - 1) & 1));
         if (!ok) break;
         tc_fence_after();
-        const uint32_t d_tmem = tmem + buf * BN;
-        uint32_t acc = 0;
-        for (int e = 0; e < n_ext; ++e, ++g) {
-          const int s = (int)(g % NE);
-          ok = mbar_wait(bar(B_EFULL + s), (uint32_t)((g / NE) & 1), abort_flag);
+        const uint32_t d = tmem + buf * BN;
+        int n_ext = 0, e = 0;
+        for (int st = 0; st < nk; ++st) {
+          ok = wait_all(bar(B_FULL + s), ph);
           if (!ok) break;
           tc_fence_after();
-          const int steps = min(ext_ksteps[s], ER / 16);
-          const uint32_t ab = sbase + C::OFF_EXT + s * C::EXT, bb = ab + A_BYTES;
-          for (int ks = 0; ks < steps; ++ks) {
-            umma_bf16(d_tmem, smem_desc(ab + ks * 32, 16, 1024), smem_desc(bb + ks * (16 * 128), C::EB_GROUP, 1024), IDESC, acc);
-            acc = 1;
-          }
-          umma_commit(bar(B_EEMPTY + s));
-        }
-        if (!ok) break;
-        for (int st = 0; st < nk; ++st, ++f) {
-          const int s = (int)(f % NS);
-          ok = mbar_wait(bar(B_FULL + s), (uint32_t)((f / NS) & 1), abort_flag);
-          if (!ok) break;
-          tc_fence_after();
-          const uint32_t ab = sbase + s * C::STAGE, bb = ab + A_BYTES;
+          const uint32_t a_lo = a_lo0 + s * (C::STAGE >> 4), b_lo = b_lo0 + s * (C::STAGE >> 4);
 #pragma unroll
-          for (int ks = 0; ks < BK / 16; ++ks) {
-            umma_bf16(d_tmem, smem_desc(ab + ks * 32, 16, 1024), smem_desc(bb + ks * (16 * 128), B_GROUP, 1024), IDESC, acc);
-            acc = 1;
+          for (int q = 0; q < BK / 16; ++q)
+            umma_ss_pair_elect(d, a_lo + q * 2, HI, b_lo + q * (16 * 128 / 16), HI, IDESC, st > 0 || q > 0 ? 1u : 0u);
+          umma_commit_pair_elect(bar(B_EMPTY + s));
+          if (++s == NS) { s = 0; ph ^= 1u; }
+          if (st >= half) {
+            if (st == half && a.n_seg > 0) {
+              ok = wait_all(bar(B_LFULL + buf), (uint32_t)((k >> 1) & 1));
+              if (!ok) break;
+              n_ext = n_ext_slot[buf];
+              __syncwarp();
+              if (lane == 0) mbar_arrive(bar(B_LEMPTY + buf));
+            }
+            const int due = (st - half + 1) * n_ext / (nk - half);
+            for (; e < due; ++e) {
+              ok = wait_all(bar(B_EFULL + es), eph);
+              if (!ok) break;
+              tc_fence_after();
+#pragma unroll
+              for (int q = 0; q < ER / 16; ++q)
+                umma_ss_pair_elect(d, ea_lo0 + es * (ER * 2 / 16) + q * 2, HI, eb_lo0 + es * (ER * 128 / 16) + q * (16 * 128 / 16), HI, IDESC, 1u);
+              umma_commit_pair_elect(bar(B_EEMPTY + es));
+              es ^= 1;
+              if (es == 0) eph ^= 1u;
+            }
+            if (!ok) break;
           }
-          umma_commit(bar(B_EMPTY + s));
         }
-        if (ok) umma_commit(bar(B_ACC_FULL + buf));
+        if (ok) umma_commit_pair_elect(bar(B_ACC_FULL + buf));
       }
     }
-  } else {
-    // ------------------------------------------------ LoRA stage filler + epilogue (128 threads; thread = token row = TMEM lane)
-    const int et = tid - 64;                 // 0..127
+  } else if (warp < 6) {
+    // ------------------------------------------------ epilogue (128 threads; thread = token row = TMEM lane)
     const int quarter = warp & 3;            // the TMEM lanes this warp may touch
     const int row = quarter * 32 + lane;
     const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16);
-    long long g = 0;                         // LoRA stages so far
+    const uint32_t acc_empty0 = map_cluster_rank(bar(B_ACC_EMPTY), 0);
     bool ok = true;
     int k = 0;
-    // fills the LoRA stages of tile `idx`
-    auto fill_ext = [&](int idx) {
+    pdl_wait();
+    for (int idx = first; idx < total; idx += step, ++k) {
       const Tile t = decode_tile(a, idx);
-      const int n_ext = a.ext_count[t.m];
-      const int tok = t.m * BM + row;
-      const int n0 = t.n * BN;
-      const int d_out = a.d_out[t.j];
-      for (int e = 0; ok && e < n_ext; ++e, ++g) {
-        const int entry = a.ext_list[(size_t)t.m * EXT_CAP + e];
-        const int sg = entry >> 1, r0 = (entry & 1) * ER;
-        const int lid = a.lora_ids[sg];
-        const LoraEntry* en = a.pv.dir + lid;
-        const int rank = min(en->rank, RMAX);
-        const int nr = max(0, min(ER, rank - r0));       // ranks of this stage
-        const int steps = (nr + 15) >> 4;
-        const LoraMat lm = en->mats[a.mat_index[t.j]];
-        const uint32_t table_off = en->table_off;
-        const bool mine = tok >= a.seg_indptr[sg] && tok < a.seg_indptr[sg + 1] && tok < a.n_tokens;
-        // this row of v (ranks r0 ..): slices summed; everything is in registers before the slot is waited for
-        constexpr int VR = RMAX < ER ? RMAX : ER;
-        float vr[VR];
-#pragma unroll
-        for (int c = 0; c < VR; ++c) vr[c] = 0.f;
-        if (mine) {
-          for (int sp = 0; sp < a.ksplit; ++sp) {
-            const float4* src = reinterpret_cast<const float4*>(
-                a.v + ((size_t)(t.j * a.ksplit + sp) * a.n_tokens + tok) * RMAX + r0);
-#pragma unroll
-            for (int c = 0; c < VR / 4; ++c) {
-              if (4 * c < 16 * steps) {
-                const float4 p4 = src[c];
-                vr[4 * c] += p4.x; vr[4 * c + 1] += p4.y; vr[4 * c + 2] += p4.z; vr[4 * c + 3] += p4.w;
-              }
-            }
-          }
-        }
-        // the adapter's B rows r0 .. of this tile's columns: 16-byte chunk c of the [32 x BN] tile, c = et + 128 i
-        constexpr int BCH = ER * BN / 8 / 128;      // chunks per thread
-        constexpr int CPR = BN / 8;                 // chunks per row
-        uint4 bq[BCH];
-#pragma unroll
-        for (int i = 0; i < BCH; ++i) {
-          const int c = et + 128 * i;
-          const int r = c / CPR, cc = c % CPR;
-          bq[i] = make_uint4(0u, 0u, 0u, 0u);
-          if (r < nr && n0 + cc * 8 < d_out) {
-            const uint32_t gr = lm.b_row0 + (uint32_t)(r0 + r);
-            const uint32_t blk = a.pv.tables[table_off + lm.b_tab + gr / lm.b_rpb];
-            if (blk >= a.pv.n_blocks) {
-              atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_BLOCK);
-            } else {
-              const unsigned char* rp = a.pv.slab + (size_t)blk * a.pv.block_bytes + (size_t)(gr % lm.b_rpb) * 2 * (size_t)d_out;
-              bq[i] = __ldg(reinterpret_cast<const uint4*>(rp + (size_t)(n0 + cc * 8) * 2));
-            }
-          }
-        }
-        const int s = (int)(g % NE);
-        const long long use = g / NE;
-        // the 128 threads decide together (a wait that gave up in one of them ends the loop for all: they meet at a
-        // named barrier further down)
-        if (use > 0) ok = group_and(mbar_wait(bar(B_EEMPTY + s), (uint32_t)((use - 1) & 1), abort_flag), 1, 128);
-        if (!ok) break;
-        unsigned char* as = smem + C::OFF_EXT + s * C::EXT;
-        unsigned char* bs = as + A_BYTES;
-#pragma unroll
-        for (int c8 = 0; c8 < VR / 8; ++c8) {
-          if (c8 < 2 * steps) {
-            uint4 q;
-            q.x = pack_bf16(vr[8 * c8] * a.scale, vr[8 * c8 + 1] * a.scale);
-            q.y = pack_bf16(vr[8 * c8 + 2] * a.scale, vr[8 * c8 + 3] * a.scale);
-            q.z = pack_bf16(vr[8 * c8 + 4] * a.scale, vr[8 * c8 + 5] * a.scale);
-            q.w = pack_bf16(vr[8 * c8 + 6] * a.scale, vr[8 * c8 + 7] * a.scale);
-            *reinterpret_cast<uint4*>(as + row * 128 + ((c8 ^ (row & 7)) << 4)) = q;
-          }
-        }
-#pragma unroll
-        for (int i = 0; i < BCH; ++i) {
-          const int c = et + 128 * i;
-          const int r = c / CPR, cc = c % CPR;
-          if (r < 16 * steps)
-            *reinterpret_cast<uint4*>(bs + (cc >> 3) * C::EB_GROUP + r * 128 + (((cc & 7) ^ (r & 7)) << 4)) = bq[i];
-        }
-        fence_async_smem();                            // the tensor core reads shared memory through the async proxy
-        asm volatile("bar.sync 1, 128;" ::: "memory");
-        if (et == 0) {
-          ext_ksteps[s] = steps;
-          mbar_arrive(bar(B_EFULL + s));
-        }
-      }
-    };
-    int idx = blockIdx.x;
-    if (idx < total) fill_ext(idx);
-    for (; ok && idx < total; idx += gridDim.x, ++k) {
-      const Tile t = decode_tile(a, idx);
-      // the next tile's LoRA stages go in before this tile's epilogue: the issuer needs them the moment this
-      // tile's last MMA is out
-      if (idx + (int)gridDim.x < total) fill_ext(idx + gridDim.x);
-      if (!ok) break;
       const int buf = k & 1;
-      const int tok = t.m * BM + row;
+      const int tok = t.m * (2 * BM) + crank * BM + row;
       const int d_out = a.d_out[t.j];
       const int n0 = t.n * BN;
       const int side = a.kv_side[t.j];
@@ -353,29 +292,32 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const LinArg
           }
         }
       }
-      ok = group_and(mbar_wait(bar(B_ACC_FULL + buf), (uint32_t)((k >> 1) & 1), abort_flag), 1, 128);
+      ok = group_and(mbar_wait_cluster(bar(B_ACC_FULL + buf), (uint32_t)((k >> 1) & 1), abort_flag), 1, 128);
       if (!ok) break;
       tc_fence_after();
       __nv_bfloat16* yrow = side < 0 ? a.y[t.j] + (size_t)tok * d_out + n0 : nullptr;
+      const bool wide = side < 0 && a.wide[t.j];
 #pragma unroll 2
       for (int cb = 0; cb < BN; cb += 32) {
         uint32_t o[32];
+        __syncwarp();
         tmem_ld32(lane_addr + buf * BN + cb, o);
         tmem_wait_ld();
         if (tok < a.n_tokens) {
+          uint32_t pk[16];
+#pragma unroll
+          for (int c = 0; c < 16; ++c) pk[c] = pack_bf16(__uint_as_float(o[2 * c]), __uint_as_float(o[2 * c + 1]));
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
-            if (n0 + cb + 8 * c < d_out) {
-              uint4 q;
-              q.x = pack_bf16(__uint_as_float(o[8 * c + 0]), __uint_as_float(o[8 * c + 1]));
-              q.y = pack_bf16(__uint_as_float(o[8 * c + 2]), __uint_as_float(o[8 * c + 3]));
-              q.z = pack_bf16(__uint_as_float(o[8 * c + 4]), __uint_as_float(o[8 * c + 5]));
-              q.w = pack_bf16(__uint_as_float(o[8 * c + 6]), __uint_as_float(o[8 * c + 7]));
-              if (side < 0) {
+            const int colg = n0 + cb + 8 * c;
+            if (colg < d_out) {
+              const uint4 q = make_uint4(pk[4 * c], pk[4 * c + 1], pk[4 * c + 2], pk[4 * c + 3]);
+              if (wide) {                     // two chunks at a time: rows are whole multiples of 32 bytes
+                if (!(c & 1)) st_global_v8(yrow + cb + 8 * c, pk + 4 * c);
+              } else if (side < 0) {
                 *reinterpret_cast<uint4*>(yrow + cb + 8 * c) = q;
               } else if (kv_slot >= 0) {
                 // [K|V][kv head][slot][128] inside the block
-                const int colg = n0 + cb + 8 * c;
                 unsigned char* dst = a.pv.slab + (size_t)kv_blk * a.pv.block_bytes +
                                      ((size_t)(side * a.n_kv + colg / FL_HEAD_DIM) * a.bt + kv_slot) * (FL_HEAD_DIM * 2) +
                                      (colg % FL_HEAD_DIM) * 2;
@@ -390,10 +332,170 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const LinArg
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar(B_ACC_EMPTY + buf));
+      if (lane == 0) mbar_arrive_cluster(acc_empty0 + 8u * buf);
     }
+  } else {
+    // ------------------------------------------------ LoRA stages
+    const int ft = tid - 192;                // 0..255
+    const int et = ft & 127, slot = ft >> 7; // the buffer half (and the stages) of this group of four warps
+    const uint32_t efull0 = map_cluster_rank(bar(B_EFULL), 0);
+    unsigned long long* row_ptr = reinterpret_cast<unsigned long long*>(smem + C::OFF_ROWS);     // [2][GROUP * ER], 0 = no row
+    unsigned long long* list = reinterpret_cast<unsigned long long*>(smem + C::OFF_LIST);
+    unsigned char* as = smem + C::OFF_EXT;
+    const uint32_t bs = sbase + C::OFF_EXT + A_BYTES;
+    uint32_t ph = 1;                         // parity of this slot's B_EEMPTY
+    bool used = false, ok = true;
+    int count = 0;                           // LoRA stages of all tiles so far
+    int k = 0;
+    if (a.n_seg > 0) pdl_wait();             // v is the shrink's output
+    for (int idx = first; a.n_seg > 0 && ok && idx < total; idx += step, ++k) {
+      const Tile t = decode_tile(a, idx);
+      const int tok0 = t.m * (2 * BM), tok1 = min(a.n_tokens, tok0 + 2 * BM);
+      // ---- the tile's units, in segment order
+      int lo_s = 0, hi_s = a.n_seg;          // first segment that ends behind tok0
+      while (lo_s < hi_s) {
+        const int mid = (lo_s + hi_s) >> 1;
+        if (a.seg_indptr[mid + 1] > tok0) hi_s = mid; else lo_s = mid + 1;
+      }
+      int n_units = 0;
+      for (int s0 = lo_s;; s0 += 256) {
+        const int s = s0 + ft;
+        int lo = tok1, hi = tok1, rank = 0, lid = -1;
+        if (s < a.n_seg) {
+          lo = max(a.seg_indptr[s], tok0);
+          hi = min(a.seg_indptr[s + 1], tok1);
+          if (lo < hi) {
+            lid = a.lora_ids[s];
+            if (lid >= 0) {
+              if ((uint32_t)lid >= a.pv.dir_cap || a.pv.dir[lid].rank <= 0 || a.mat_index[t.j] >= a.pv.dir[lid].n_mats) {
+                atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_LORA);
+              } else {
+                rank = min(a.pv.dir[lid].rank, RMAX);
+              }
+            }
+          }
+        }
+        const int cnt = (rank + UNIT - 1) / UNIT;
+        int incl = cnt;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const int o = __shfl_up_sync(0xffffffffu, incl, d);
+          if (lane >= d) incl += o;
+        }
+        if (lane == 31) scan[warp - 6] = incl;
+        // (this barrier also keeps a new list from the old one's last readers)
+        const bool last = group_and(s >= a.n_seg || lo >= tok1, 2, 256) || s0 + 256 >= a.n_seg;
+        int at = n_units + incl - cnt;
+        for (int w = 0; w < 8; ++w) {
+          const int v = scan[w];
+          if (w < warp - 6) at += v;
+          n_units += v;
+        }
+        for (int q = 0; q < cnt; ++q, ++at)
+          if (at < MAX_UNITS) list[at] = pack_unit(lid, q, min(UNIT, rank - UNIT * q), lo - tok0, hi - tok0);
+        asm volatile("bar.sync 2, 256;" ::: "memory");
+        if (last) break;
+      }
+      n_units = min(n_units, MAX_UNITS);      // (overlapping segments, which the interface rules out, could exceed it)
+      const int n_ext = (n_units + 1) / 2;
+      if (leader && ft == 0) {
+        if (k >= 2) mbar_wait(bar(B_LEMPTY + (k & 1)), (uint32_t)(((k >> 1) - 1) & 1), abort_flag);
+        n_ext_slot[k & 1] = n_ext;
+        mbar_arrive(bar(B_LFULL + (k & 1)));
+      }
+      const int d_out = a.d_out[t.j], col0 = t.n * BN + crank * BH;
+      const int mat = a.mat_index[t.j];
+      // Addresses of a group's B rows, looked up side by side a group ahead of their use, and their columns asked into L2.
+      auto find_rows = [&](int g) {
+        for (int i = ft; i < GROUP * ER; i += 256) {
+          const int u = 2 * (g * GROUP + i / ER) + (i % ER) / UNIT, r = i % UNIT;
+          unsigned long long at = 0;
+          if (u < n_units) {
+            const unsigned long long x = list[u];
+            if (r < (int)(x >> 18 & 31)) {
+              const LoraEntry* en = a.pv.dir + (x >> 25);
+              const LoraMat lm = en->mats[mat];
+              const uint32_t gr = lm.b_row0 + (uint32_t)(x >> 23 & 3) * UNIT + r;
+              const uint32_t blk = a.pv.tables[en->table_off + lm.b_tab + gr / lm.b_rpb];
+              if (blk >= a.pv.n_blocks) {
+                atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_BLOCK);
+              } else if (col0 < d_out) {
+                const unsigned char* p = a.pv.slab + (size_t)blk * a.pv.block_bytes + ((size_t)(gr % lm.b_rpb) * d_out + col0) * 2;
+                at = reinterpret_cast<unsigned long long>(p);
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+                if (BH > 64 && col0 + 64 < d_out) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + 128));
+              }
+            }
+          }
+          row_ptr[(g & 1) * GROUP * ER + i] = at;
+        }
+      };
+      if (n_ext > 0) find_rows(0);
+      const int vrow = et >> 2, vch = et & 3;            // rows vrow + 32 i, ranks 8 vch .. of the stage's 32
+      for (int e = 0; e < n_ext; ++e) {
+        if (e % GROUP == 0) {
+          // rows of this group are there (and nobody reads the other buffer any more)
+          asm volatile("bar.sync 2, 256;" ::: "memory");
+          if (e + GROUP < n_ext) find_rows(e / GROUP + 1);
+        }
+        if (((count + e) & 1) != slot) continue;
+        if (used) ok = mbar_wait_cluster(bar(B_EEMPTY + slot), ph, abort_flag) && ok;
+        used = true;
+        ph ^= 1u;
+        ok = group_and(ok, 3 + slot, 128);
+        const unsigned long long* rp = row_ptr + (e % (2 * GROUP)) * ER;
+        constexpr int CPR = BH / 8;                      // 16-byte chunks per row
+#pragma unroll
+        for (int i = 0; i < ER * CPR / 128; ++i) {
+          const int c = et + 128 * i, r = c / CPR, ch = c % CPR;
+          const unsigned long long at = ok ? rp[r] : 0ull;
+          const bool have = at && col0 + ch * 8 < d_out;
+          cp_async16(bs + (ch >> 3) * B_GROUP + (ER * slot + r) * 128 + (((ch & 7) ^ (r & 7)) << 4),
+                     have ? reinterpret_cast<const unsigned char*>(at) + ch * 16 : a.pv.slab, have);
+        }
+        cp_async_commit();
+        // shrink results of this CTA's 128 rows at the stage's ranks
+        const int u = 2 * e + (vch >> 1);
+        const unsigned long long x = u < n_units ? list[u] : 0ull;
+        const int lo = (int)(x >> 9 & 511), hi = (int)(x & 511), r0 = (int)(x >> 23 & 3) * UNIT + 8 * (vch & 1);
+        const bool live = 8 * (vch & 1) < (int)(x >> 18 & 31);
+        float4 f[4][2];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) f[i][0] = f[i][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int sp = 0; sp < a.ksplit; ++sp) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int rt = crank * BM + vrow + 32 * i;
+            if (live && rt >= lo && rt < hi) {
+              const float4* src = reinterpret_cast<const float4*>(
+                  a.v + ((size_t)(t.j * a.ksplit + sp) * a.n_tokens + tok0 + rt) * RMAX + r0);
+              const float4 p = src[0], q = src[1];
+              f[i][0].x += p.x; f[i][0].y += p.y; f[i][0].z += p.z; f[i][0].w += p.w;
+              f[i][1].x += q.x; f[i][1].y += q.y; f[i][1].z += q.z; f[i][1].w += q.w;
+            }
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int row = vrow + 32 * i;
+          uint4 q;
+          q.x = pack_bf16(f[i][0].x * a.scale, f[i][0].y * a.scale);
+          q.y = pack_bf16(f[i][0].z * a.scale, f[i][0].w * a.scale);
+          q.z = pack_bf16(f[i][1].x * a.scale, f[i][1].y * a.scale);
+          q.w = pack_bf16(f[i][1].z * a.scale, f[i][1].w * a.scale);
+          *reinterpret_cast<uint4*>(as + row * 128 + (((4 * slot + vch) ^ (row & 7)) << 4)) = q;
+        }
+        cp_async_wait<0>();
+        fence_async_smem();                              // the tensor core reads shared memory through the async proxy
+        asm volatile("bar.sync %0, 128;" ::"r"(3 + slot) : "memory");
+        if (et == 0 && ok) mbar_arrive_cluster(efull0 + 8u * slot);
+      }
+      count += n_ext;
+      ok = group_and(ok, 2, 256);
+    }
+    cp_async_wait<0>();
   }
-  // ------------------------------------------------ teardown
+  // ------------------------------------------------ teardown: neither CTA leaves while the other's MMAs or arrivals need it
   tc_fence_before();
   __syncthreads();
   if (*abort_flag) {
@@ -406,27 +508,11 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const LinArg
     }
     __syncthreads();
   }
+  cluster_sync();
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::TMEM_COLS) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::TMEM_COLS) : "memory");
   }
-}
-
-size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
-
-struct LinWs {
-  size_t v, ext_count, ext_list, total;
-  int m_tiles;
-};
-LinWs lin_ws(int n_tokens, int n_mats) {
-  LinWs w;
-  w.m_tiles = (n_tokens + BM - 1) / BM;
-  size_t off = 0;
-  w.v = off; off = align256(off + fl_lora_sgmv_workspace(n_tokens, n_mats));
-  w.ext_count = off; off = align256(off + sizeof(int) * (size_t)w.m_tiles);
-  w.ext_list = off; off = align256(off + sizeof(int) * (size_t)w.m_tiles * EXT_CAP);
-  w.total = off;
-  return w;
 }
 
 template <int BN, int RMAX>
@@ -438,8 +524,8 @@ int launch_linear(fl_pool* p, const LinArgs& a, const LinMaps& maps, cudaStream_
     configured[p->device & 15] = true;
   }
   const int total = a.tile_base[a.n_mats];
-  const unsigned grid = (unsigned)std::min(total, p->sm_count);
-  FL_CUDA(p, launch_pdl(lora_linear_kernel<BN, RMAX>, dim3(grid), dim3(LT_THREADS), C::SMEM, st, a, maps));
+  const unsigned pairs = (unsigned)std::min(total, p->sm_count / 2);
+  FL_CUDA(p, launch_pdl_cluster(lora_linear_kernel<BN, RMAX>, dim3(2 * pairs), dim3(2), dim3(LT_THREADS), C::SMEM, st, a, maps));
   FL_CUDA(p, cudaGetLastError());
   return FL_OK;
 }
@@ -448,11 +534,8 @@ int launch_width(fl_pool* p, const LinArgs& a, const LinMaps& maps, cudaStream_t
   if (bn == 256)
     return rmax == 16 ? launch_linear<256, 16>(p, a, maps, st)
          : rmax == 32 ? launch_linear<256, 32>(p, a, maps, st) : launch_linear<256, 64>(p, a, maps, st);
-  if (bn == 128)
-    return rmax == 16 ? launch_linear<128, 16>(p, a, maps, st)
-         : rmax == 32 ? launch_linear<128, 32>(p, a, maps, st) : launch_linear<128, 64>(p, a, maps, st);
-  return rmax == 16 ? launch_linear<64, 16>(p, a, maps, st)
-       : rmax == 32 ? launch_linear<64, 32>(p, a, maps, st) : launch_linear<64, 64>(p, a, maps, st);
+  return rmax == 16 ? launch_linear<128, 16>(p, a, maps, st)
+       : rmax == 32 ? launch_linear<128, 32>(p, a, maps, st) : launch_linear<128, 64>(p, a, maps, st);
 }
 
 }  // namespace
@@ -461,7 +544,7 @@ extern "C" {
 
 size_t fl_lora_linear_workspace(int n_tokens, int n_mats) {
   if (n_tokens <= 0 || n_mats <= 0) return 256;
-  return lin_ws(n_tokens, n_mats).total;
+  return fl_lora_sgmv_workspace(n_tokens, n_mats);      // the shrink's results
 }
 
 }  // extern "C"
@@ -488,12 +571,11 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
   if (n_tokens == 0) return FL_OK;
   if (!x || !workspace || (n_seg > 0 && (!seg_indptr || !lora_ids))) return FL_EINVAL;
   if (p->n_mats == 0) return FL_EBADID;           // the projection shapes come with the first registered adapter
-  const LinWs lw = lin_ws(n_tokens, n_mats);
-  if (workspace_bytes < lw.total) return FL_ENOMEM;
+  const size_t v_bytes = fl_lora_linear_workspace(n_tokens, n_mats);
+  if (workspace_bytes < v_bytes) return FL_ENOMEM;
   LinArgs a;
   memset(&a, 0, sizeof(a));
   a.pv = p->view();
-  int d_out_min = 1 << 30;
   for (int j = 0; j < n_mats; ++j) {
     const int mi = mat_indices[j];
     const bool to_pool = kv && (j == kv->k_slot || j == kv->v_slot);
@@ -502,7 +584,6 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
     a.y[j] = reinterpret_cast<__nv_bfloat16*>(ys[j]);
     a.mat_index[j] = mi;
     a.d_out[j] = p->mats[mi].d_out;
-    d_out_min = std::min(d_out_min, a.d_out[j]);
   }
   a.d_in = p->mats[mat_indices[0]].d_in;
   a.n_mats = n_mats;
@@ -511,16 +592,10 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
   a.n_seg = n_seg;
   a.n_tokens = n_tokens;
   a.scale = scale;
-  unsigned char* wsb = reinterpret_cast<unsigned char*>(workspace);
-  a.v = reinterpret_cast<const float*>(wsb + lw.v);
-  int* ext_count = reinterpret_cast<int*>(wsb + lw.ext_count);
-  int* ext_list = reinterpret_cast<int*>(wsb + lw.ext_list);
-  a.ext_count = ext_count;
-  a.ext_list = ext_list;
-  a.m_tiles = lw.m_tiles;
-  // Segments of a few tokens each (a decode batch): a 128-token tile would take one LoRA stage per segment, each
-  // for a handful of rows, and y is small next to W.  Then the GEMM computes x W alone (no LoRA stages in the plan)
-  // and the segmented projection adds the LoRA term to y afterwards.
+  a.v = reinterpret_cast<const float*>(workspace);
+  a.m_tiles = (n_tokens + 2 * BM - 1) / (2 * BM);
+  // Segments of a few tokens each (a large decode batch): a tile would take a LoRA stage per segment or two, each for a
+  // handful of rows.  Then the GEMM computes x W alone and the segmented projection adds the LoRA term to y afterwards.
   const bool few = n_tokens <= skinny::MAX_TOKENS;      // W streamed once for all tokens: a kernel of its own
   const bool hybrid = !few && n_seg > 0 && n_tokens <= 16 * n_seg;
   if (hybrid) a.n_seg = 0;
@@ -549,28 +624,23 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
     a.n_kv = kv->n_kv;
     a.bt = (int)(p->block_bytes / per_tok);
   }
-  // few token tiles: narrower column tiles, so that every SM streams a slice of W.  Among 256, 128 and 64 columns the
-  // width with the least bytes through the busiest SM wins: rounds of tiles over the SMs times what a tile pulls per
-  // k-stage (its W slice and its x rows).
+  // Columns per tile, 256 or 128: the width whose rounds over the pairs of SMs cost less.  A tile of 128 columns costs more
+  // than half of one of 256 (three quarters of the shared-memory fill for half the product).
   int bn = 256;
   {
-    auto tiles = [&](int w) {
+    auto cost = [&](int w) {
       long t = 0;
-      for (int j = 0; j < n_mats; ++j) t += (long)lw.m_tiles * ((a.d_out[j] + w - 1) / w);
-      return t;
+      for (int j = 0; j < n_mats; ++j) t += (long)a.m_tiles * ((a.d_out[j] + w - 1) / w);
+      const long pairs = std::max(1, p->sm_count / 2);
+      return (t + pairs - 1) / pairs * (w + 48);
     };
-    if (tiles(256) < p->sm_count || hybrid) {
-      long best = -1;
-      for (int w = 256; w >= 64; w /= 2) {
-        const long cost = ((tiles(w) + p->sm_count - 1) / p->sm_count) * (w + BM);
-        if (best < 0 || cost < best) { best = cost; bn = w; }
-      }
-    }
+    if (cost(128) < cost(256)) bn = 128;
   }
+  for (int j = 0; j < n_mats; ++j) a.wide[j] = (reinterpret_cast<uintptr_t>(a.y[j]) & 31) == 0 && a.d_out[j] % 16 == 0;
   a.tile_base[0] = 0;
   for (int j = 0; j < n_mats; ++j) {
     a.n_tiles_n[j] = (a.d_out[j] + bn - 1) / bn;
-    a.tile_base[j + 1] = a.tile_base[j] + lw.m_tiles * a.n_tiles_n[j];
+    a.tile_base[j + 1] = a.tile_base[j] + a.m_tiles * a.n_tiles_n[j];
   }
   int prev = -1;
   cudaGetDevice(&prev);
@@ -604,8 +674,8 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
       k.bt = a.bt;
       sgmv::ShrinkInfo info = {1, 16};
       if (n_seg > 0) {
-        rc = sgmv::shrink_scaled(p, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, scale, wsb + lw.v,
-                                 fl_lora_sgmv_workspace(n_tokens, n_mats), stream, &info);
+        rc = sgmv::shrink_scaled(p, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace,
+                                 v_bytes, stream, &info);
         if (rc != FL_OK) break;
       }
       k.rmax = info.rmax;
@@ -628,20 +698,6 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
     }
     for (int j = n_mats; j < MAX_LIN; ++j) maps.w[j] = maps.w[0];
     if (rc != FL_OK) break;
-    lora_plan::PlanArgs pa;
-    pa.pv = a.pv;
-    pa.seg_indptr = a.seg_indptr;
-    pa.lora_ids = a.lora_ids;
-    pa.n_seg = a.n_seg;
-    pa.n_tokens = n_tokens;
-    pa.m_tiles = lw.m_tiles;
-    pa.n_mats = n_mats;
-    for (int j = 0; j < FL_MAX_MATS; ++j) pa.mat_index[j] = j < n_mats ? a.mat_index[j] : 0;
-    if (lora_plan::launch_plan(pa, ext_count, ext_list, st) != cudaSuccess) {
-      p->last_cuda = (int)cudaGetLastError();
-      rc = FL_ECUDA;
-      break;
-    }
     sgmv::ShrinkInfo info = {1, p->max_rank <= 16 ? 16 : (p->max_rank <= 32 ? 32 : 64)};
     if (hybrid) {
       // y = x W from the GEMM alone, then the segmented projection adds the LoRA term to it
@@ -652,18 +708,18 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
       if (kv && n_mats == 3 && kv->k_slot == 1 && kv->v_slot == 2)
         rc = fl_lora_sgmv_qkv_append(p, ys[0], ys[1], ys[2], x, mat_indices[0], mat_indices[1], mat_indices[2], seg_indptr,
                                      lora_ids, n_seg, n_tokens, scale, kv->req_indptr, kv->tbl_indptr, kv->tbl,
-                                     kv->prefix_lens, kv->n_req, kv->n_kv, wsb + lw.v,
-                                     fl_lora_sgmv_workspace(n_tokens, n_mats), stream);
+                                     kv->prefix_lens, kv->n_req, kv->n_kv, workspace,
+                                     v_bytes, stream);
       else if (kv)
         rc = FL_EINVAL;
       else
-        rc = fl_lora_sgmv_multi(p, ys, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, scale, wsb + lw.v,
-                                fl_lora_sgmv_workspace(n_tokens, n_mats), stream);
+        rc = fl_lora_sgmv_multi(p, ys, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace,
+                                v_bytes, stream);
       break;
     }
     if (n_seg > 0) {
-      rc = sgmv::shrink(p, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, wsb + lw.v,
-                        fl_lora_sgmv_workspace(n_tokens, n_mats), stream, &info);
+      rc = sgmv::shrink(p, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, workspace,
+                        v_bytes, stream, &info);
       if (rc != FL_OK) break;
     }
     a.ksplit = info.ksplit;

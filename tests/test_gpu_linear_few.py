@@ -75,3 +75,40 @@ def test_linear_of_few_tokens(T, per_req, hidden, heads):
         assert s.status()["device_flags"] == 0
     finally:
         s.close()
+
+
+@pytest.mark.parametrize("long_tokens,n_one,hidden,heads,n_adapters", [
+    (258, 0, 328, (3, 1), 3), (382, 1, 1024, (8, 8), 3), (500, 12, 328, (3, 1), 20), (513, 0, 4096, (3, 1), 2),
+    (1024, 40, 200, (2, 1), 60), (2300, 17, 1024, (8, 2), 24)])
+def test_linear_of_long_segments_next_to_one_token_segments(long_tokens, n_one, hidden, heads, n_adapters):
+    """The GEMM for longer batches: tiles of 256 tokens that end in the middle of a segment, tiles with more LoRA stages than
+    are looked up together, tiles without any, both column widths."""
+    from paper_2505_03756_b200 import harness as H
+    wl = synth.make_workload("decode13b", n_req=n_one + 2, len_range=(3, 40), n_adapters=n_adapters,
+                             shape=synth.LayerShape(hidden, *heads))
+    wl.ranks[:] = [RANKS[i % len(RANKS)] for i in range(n_adapters)]
+    wl.lora_of_req[:] = np.sort(np.arange(n_one + 2) % n_adapters)
+    wl.lora_of_req[0] = -1
+    wl.new_lens[-1] = long_tokens // 3
+    wl.new_lens[n_one // 2] = long_tokens - long_tokens // 3
+    wl.pool_blocks = int(np.sum((wl.prefix_lens + wl.new_lens + 15) // 16)) + 130 * n_adapters + 64
+    s = H.Session(wl)
+    try:
+        s.load_adapters()
+        s.build_batch()
+        T = wl.n_tokens
+        assert T > 256 and T > 16 * s.n_seg
+        dims = dict((n, o) for n, _, o in wl.shape.mats)
+        seg, ids = wl.segments()
+        x = wl.x("q")
+        tx = H.f32_to_dev(x, s.dev)
+        for scale_w in (1.0, 0.0):           # with W, and the LoRA term alone against its own size
+            tw = [H.f32_to_dev(wl.weight(m), s.dev) * scale_w for m in "qkv"]
+            ty = [torch.full((T, dims[m]), 7.0, dtype=torch.bfloat16, device=s.dev) for m in "qkv"]
+            s.lora_linear(ty, tx, tw, ["q", "k", "v"])
+            for m, t in zip("qkv", ty):
+                want = lora_linear(x, wl.weight(m) * scale_w, seg, ids, oracle_adapters(wl, m), wl.scale)
+                assert_close(H.dev_to_f32(t), want, f"long and one-token segments {T} {m} {scale_w}")
+        assert s.status()["device_flags"] == 0
+    finally:
+        s.close()
