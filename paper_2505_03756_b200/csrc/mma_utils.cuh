@@ -41,6 +41,16 @@ __device__ __forceinline__ float2 unpack_bf16(uint32_t u) {
   return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xFFFF0000u));
 }
 
+// Four 8 x 8 bf16 matrices in accumulator layout -> shared memory rows of 16 bytes (lane l gives the address of row l % 8 of matrix l / 8).
+__device__ __forceinline__ void stmatrix_x4(uint32_t addr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1,%2,%3,%4};\n" ::"r"(addr), "r"(r0), "r"(r1), "r"(r2), "r"(r3) : "memory");
+}
+__device__ __forceinline__ uint4 ld_shared_v4(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];\n" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+
 // Byte offset of 16-byte chunk `chunk` of row `row` in a shared tile whose rows hold `row_chunks`
 // chunks (8 or 16); chunk index is XOR-swizzled with the row so ldmatrix reads are conflict-free.
 __device__ __forceinline__ uint32_t swz(int row, int chunk, int row_chunks) {

@@ -52,6 +52,7 @@ struct SgmvArgs {
   const uint32_t* tbl;
   const int32_t* prefix_lens;
   int n_req, n_kv, bt;
+  uint32_t bt_inv;     // 2^32 / bt, rounded up
 };
 
 // Eight bf16 sums (round to nearest even each) of two 16-byte chunks.
@@ -226,10 +227,9 @@ __global__ void __launch_bounds__(SG_THREADS) sgmv_shrink_kernel(const SgmvArgs 
 // The shrink of three projections that share x (q, k, v) for long segments and ranks up to 16: one CTA stages each x tile once and
 // multiplies it by the three adapters' rank-rows, instead of three CTAs reading the same x rows.  With long
 // segments the shrink is bound by the traffic from L2 into shared memory, and x is most of it.
-template <int RMAX>
+template <int RMAX, int STAGES>
 __global__ void __launch_bounds__(SG_THREADS) sgmv_shrink3_kernel(const SgmvArgs a) {
   constexpr int TM = 64, NM = 3;
-  constexpr int STAGES = RMAX == 64 ? 3 : 4;
   extern __shared__ __align__(128) unsigned char smem[];
   pdl_wait();                 // x may come from the kernel right before this one
   pdl_launch_dependents();    // the expand may start its look-ups and first loads while this grid drains
@@ -351,17 +351,16 @@ __global__ void __launch_bounds__(SG_THREADS) sgmv_shrink3_kernel(const SgmvArgs
   }
 }
 
+// The expand of short segments (a decode step): tiles of 16 tokens.
 // KV: some projections of the call write their result rows into pool blocks (SgmvArgs::kv_side).
-// CTAs per SM the register budget is sized for (the kernel is bound by memory latency: occupancy matters more
-// than a few spilled values)
-constexpr int expand_min_ctas(int tm, int rmax, bool) { return tm == 16 ? 5 : (rmax == 16 ? 4 : 3); }
+// whether the LoRA-term tile reuses the adapter-row buffer of the stage
+__host__ __device__ constexpr bool expand_alias(int rmax) { return rmax >= 64; }
+constexpr int expand_smem_bytes(int rmax) { return 2 * (16 + rmax) * 256 + (expand_alias(rmax) ? 0 : 16 * 256); }
 
-// whether the LoRA-term tile reuses the adapter-row buffer of the stage (it has to fit there)
-__host__ __device__ constexpr bool expand_alias(int tm, int rmax) { return rmax >= 64 && rmax >= tm; }
-constexpr int expand_smem_bytes(int tm, int rmax) { return 2 * (tm + rmax) * 256 + (expand_alias(tm, rmax) ? 0 : tm * 256); }
-
-template <int TM, int RMAX, bool KV>
-__global__ void __launch_bounds__(SG_THREADS, expand_min_ctas(TM, RMAX, KV)) sgmv_expand_kernel(const SgmvArgs a) {
+// Five CTAs per SM: the kernel is bound by memory latency, occupancy matters more than a few spilled values.
+template <int RMAX, bool KV>
+__global__ void __launch_bounds__(SG_THREADS, 5) sgmv_expand_kernel(const SgmvArgs a) {
+  constexpr int TM = 16;
   extern __shared__ __align__(128) unsigned char smem[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int j = blockIdx.x % a.n_mats;
@@ -518,7 +517,7 @@ __global__ void __launch_bounds__(SG_THREADS, expand_min_ctas(TM, RMAX, KV)) sgm
     // the LoRA term of this sub-tile as bf16 pairs into a tile of its own (each element is owned by exactly one
     // thread); at rank 64 that tile takes the place of the adapter rows the MMAs have just consumed, which brings
     // the CTA to 64 KB and a third CTA onto the SM
-    constexpr bool ALIAS = expand_alias(TM, RMAX);
+    constexpr bool ALIAS = expand_alias(RMAX);
     unsigned char* dsm = ALIAS ? smem + st * STAGE_BYTES + TM * 256 : smem + 2 * STAGE_BYTES;
     if (ALIAS) __syncthreads();
 #pragma unroll
@@ -550,8 +549,9 @@ __global__ void __launch_bounds__(SG_THREADS, expand_min_ctas(TM, RMAX, KV)) sgm
               const uint32_t loc = kvloc[KV ? i : 0];
               const int slot = (loc >> 1) & 127;
               unsigned char* dst = a.pv.slab + (size_t)(loc >> 8) * a.pv.block_bytes + head_off + slot * (FL_HEAD_DIM * 2);
-              *reinterpret_cast<uint4*>(dst) = add_bf16x8(*reinterpret_cast<const uint4*>(ysm + swz(crow + 8 * i, cchunk, 16)),
-                                                          *reinterpret_cast<const uint4*>(dsm + swz(crow + 8 * i, cchunk, 16)));
+              const uint4 base = *reinterpret_cast<const uint4*>(ysm + swz(crow + 8 * i, cchunk, 16));
+              *reinterpret_cast<uint4*>(dst) =
+                  lid < 0 ? base : add_bf16x8(base, *reinterpret_cast<const uint4*>(dsm + swz(crow + 8 * i, cchunk, 16)));
               if (side == 1 && (loc & 1u))     // V of a request's last token: clear the slots behind it
                 for (int z = slot + 1; z < a.bt; ++z)
                   *reinterpret_cast<uint4*>(dst + (z - slot) * (FL_HEAD_DIM * 2)) = make_uint4(0u, 0u, 0u, 0u);
@@ -562,6 +562,255 @@ __global__ void __launch_bounds__(SG_THREADS, expand_min_ctas(TM, RMAX, KV)) sgm
     }
     __syncthreads();
   }
+}
+
+// The expand of long segments: a stream over y in which no warp waits for another.
+// A CTA takes up to `tm` tokens of one segment and 256 columns, a warp 64 of them.  The adapter's B rows of those columns go
+// through shared memory once and stay in registers as MMA fragments (64 at rank 64); then each warp walks the tokens 16 at a
+// time.  A thread copies ahead (cp.async, EX_DEPTH tiles) exactly the 16-byte pieces of y that it will add to itself, and
+// the LoRA term gets into that layout through 2 KB of shared memory of the warp's own (stmatrix), so the loop has no CTA
+// barrier but one per 96 to 128 tokens, when their shrink results are brought in.
+// What bounds it: reading and writing y; on the way there the instructions per piece of y and the latency of the prologue's
+// look-ups, which is why all 64 row addresses are found at once (a lane each), and so are the places of all the CTA's K / V
+// rows (a thread each; looked up tile by tile in the loop they cost 24 of 223 us for the q, k, v call of 64 prompts on 7B).
+// Shrink and expand of 16384 tokens on 34B (rank 64): o 217 -> 179 us, q, k, v with the KV store 271 -> 240 us; of 19770
+// tokens on 7B (rank 16): 98 -> 93 us and 232 -> 205 us; before, tiles of 64 tokens and 128 columns with three barriers
+// each had one tile of y per CTA in flight and read the B rows again for every 64 tokens.
+constexpr int EX_COLS = 256, EX_DEPTH = 4;
+constexpr int EX_TILE = 16 * 128;                  // bytes of a tile of 16 tokens x 64 columns
+constexpr int EX_RING = EX_TILE * EX_DEPTH;
+constexpr int EX_TM = 256;                         // tokens per CTA, at most
+// tokens whose v is in shared memory at a time: at rank 64 what leaves room for four CTAs per SM, at rank 16 for five
+__host__ __device__ constexpr int ex_vt(int rmax) { return rmax == 64 ? 112 : rmax == 32 ? 128 : 96; }
+__host__ __device__ constexpr int ex_smem(int rmax) { return ex_vt(rmax) * rmax * 2 + 4 * (EX_RING + EX_TILE) + EX_TM * 4; }
+static_assert(FL_MAX_RANK * EX_COLS * 2 <= 4 * EX_RING, "the B rows are staged where the y tiles go later");
+// 16-byte piece `chunk` of row `row` of the v tile; rows of 32, 64 or 128 bytes, conflict-free for ldmatrix
+template <int RMAX>
+__device__ __forceinline__ uint32_t ex_vswz(int row, int chunk) {
+  constexpr int CH = RMAX / 8, SH = RMAX == 64 ? 0 : RMAX == 32 ? 1 : 2;
+  return (uint32_t)((row * CH + (chunk ^ ((row >> SH) & (CH - 1)))) * 16);
+}
+
+// Request of a token, for tokens taken in ascending order, and where its K / V row lives in the pool.
+struct KvCursor {
+  int r, beg, end, pos0, tab, n_tab;
+  __device__ __forceinline__ void load(const SgmvArgs& a) {
+    beg = a.req_indptr[r];
+    end = a.req_indptr[r + 1];
+    pos0 = a.prefix_lens[r] - beg;
+    tab = a.tbl_indptr[r];
+    n_tab = a.tbl_indptr[r + 1] - tab;
+  }
+  // request of token t (the whole warp takes part with the same t): the first that ends behind it, 32 at a time
+  __device__ __forceinline__ void init(const SgmvArgs& a, int t) {
+    const int lane = threadIdx.x & 31;
+    r = a.n_req - 1;
+    for (int r0 = 0; r0 < a.n_req; r0 += 32) {
+      const bool behind = r0 + lane < a.n_req && a.req_indptr[r0 + lane + 1] > t;
+      const uint32_t m = __ballot_sync(0xffffffffu, behind);
+      if (m) {
+        r = r0 + __ffs(m) - 1;
+        break;
+      }
+    }
+    load(a);
+  }
+  // block << 8 | slot << 1 | "last token of its request", or ~0 when the token has no place (flag raised)
+  __device__ __forceinline__ uint32_t find(const SgmvArgs& a, int t) {
+    while (t >= end && r + 1 < a.n_req) {
+      ++r;
+      load(a);
+    }
+    const int pos = pos0 + t;
+    // pos / bt by the rounded-up reciprocal 2^32 / bt: exact below 2^25 for bt <= 128
+    const int entry = pos >= 0 && pos < (1 << 25) ? (a.bt == 1 ? pos : (int)__umulhi((uint32_t)pos, a.bt_inv)) : pos / a.bt;
+    const int slot = pos - entry * a.bt;
+    if (pos < 0 || t < beg || t >= end || entry >= n_tab) {
+      atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_POS);
+      return 0xffffffffu;
+    }
+    const uint32_t blk = a.tbl[tab + entry];
+    if (blk >= a.pv.n_blocks || blk >= (1u << 24)) {
+      atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_BLOCK);
+      return 0xffffffffu;
+    }
+    return blk << 8 | (uint32_t)slot << 1 | (t == end - 1 ? 1u : 0u);
+  }
+};
+
+template <int RMAX, bool KV>
+__global__ void __launch_bounds__(SG_THREADS, RMAX == 16 ? 5 : 4) sgmv_expand_long_kernel(const __grid_constant__ SgmvArgs a, int tm, int n_ranges) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  constexpr int KN = RMAX / 16, EX_VT = ex_vt(RMAX);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tile = blockIdx.x / n_ranges;
+  int range = blockIdx.x - tile * n_ranges, j = 0;       // column ranges of all projections, one after the other
+  for (; j + 1 < a.n_mats; ++j) {
+    const int n = (a.d_out[j] + EX_COLS - 1) / EX_COLS;
+    if (range < n) break;
+    range -= n;
+  }
+  int seg, tok0, tok1;
+  if (!find_tile(tm, a.seg_indptr, a.lora_ids, a.n_seg, tile, seg, tok0, tok1, a.all_segments != 0)) return;
+  const int lid = a.lora_ids[seg];
+  const int side = KV ? a.kv_side[j] : -1;   // >= 0: the result rows go into the requests' pool blocks
+  const int d_out = a.d_out[j], c0 = range * EX_COLS;
+  int rank = 0;
+  const uint32_t sbase = smem_u32(smem), ring0 = sbase + EX_VT * RMAX * 2;
+  // ---- B rows of the CTA's columns: shared memory, then fragments
+  const unsigned char* rowp[RMAX <= 32 ? 1 : 2];         // row lane (and lane + 32)
+  rowp[0] = nullptr;
+  if (RMAX > 32) rowp[RMAX > 32 ? 1 : 0] = nullptr;
+  if (lid >= 0) {
+    if ((uint32_t)lid >= a.pv.dir_cap || a.pv.dir[lid].rank <= 0 || a.mat_index[j] >= a.pv.dir[lid].n_mats) return;
+    const LoraEntry* e = a.pv.dir + lid;
+    const LoraMat lm = e->mats[a.mat_index[j]];
+    rank = min(e->rank, RMAX);
+#pragma unroll
+    for (int i = 0; i < (RMAX <= 32 ? 1 : 2); ++i) {
+      const int r = lane + 32 * i;
+      bool ok = false;
+      if (r < rank) rowp[i] = lora_row(a.pv, e->table_off, lm.b_tab, lm.b_row0, lm.b_rpb, d_out, r, ok);
+      if (!ok) rowp[i] = nullptr;
+    }
+  } else if (side < 0) {
+    return;                                // no adapter and y stays where it is: nothing to do
+  }
+  {
+    const int col = c0 + lane * 8;         // a warp copies whole rows of 512 bytes: rows warp, warp + 4, ...
+#pragma unroll
+    for (int i = 0; i < RMAX / 4; ++i) {
+      const int r = warp + 4 * i;
+      const unsigned char* src = reinterpret_cast<const unsigned char*>(
+          __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(rowp[RMAX > 32 && i >= 8 ? 1 : 0]), r & 31));
+      const bool have = src && col < d_out;
+      cp_async16(ring0 + swz(r, lane, 32), have ? src + col * 2 : a.pv.slab, have);
+    }
+  }
+  cp_async_commit();
+  const int rows = tok1 - tok0, n_tiles = (rows + 15) / 16;
+  uint32_t* const loc = reinterpret_cast<uint32_t*>(smem + EX_VT * RMAX * 2 + 4 * (EX_RING + EX_TILE));
+  if (KV && side >= 0) {                   // where each row goes
+    KvCursor cur;
+    cur.init(a, tok0);
+    for (int r = tid; r < rows; r += SG_THREADS) loc[r] = cur.find(a, tok0 + r);
+  }
+  cp_async_wait<0>();
+  __syncthreads();
+  uint32_t bf[KN][8][2];
+#pragma unroll
+  for (int ks = 0; ks < KN; ++ks)
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      uint32_t f[4];
+      ldmatrix_x4_trans(f, ring0 + swz(16 * ks + (lane & 7) + 8 * ((lane >> 3) & 1), warp * 8 + 2 * p + (lane >> 4), 32));
+      bf[ks][2 * p][0] = f[0]; bf[ks][2 * p][1] = f[1];
+      bf[ks][2 * p + 1][0] = f[2]; bf[ks][2 * p + 1][1] = f[3];
+    }
+  __syncthreads();
+  // ---- y ahead: this thread's pieces are rows pr + 4 k of a tile, 16-byte chunk pc of the warp's 64 columns
+  const int pr = lane >> 3, pc = lane & 7;
+  const int wc = c0 + warp * 64 + pc * 8;
+  const bool cok = wc < d_out;
+  const uint32_t ring = ring0 + warp * EX_RING + lane * 16;
+  const uint32_t term = ring0 + 4 * EX_RING + warp * EX_TILE;
+  __nv_bfloat16* const ycol = a.y[j] + (size_t)(tok0 + pr) * d_out + (cok ? wc : 0);
+  const size_t step4 = (size_t)4 * d_out;
+  auto load_y = [&](int i) {
+    const uint32_t dst = ring + (i % EX_DEPTH) * EX_TILE;
+    const __nv_bfloat16* src = ycol + (size_t)(16 * i) * d_out;
+    const int left = rows - 16 * i - pr;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) cp_async16(dst + k * 512, 4 * k < left ? src + k * step4 : ycol, cok && 4 * k < left);
+  };
+#pragma unroll
+  for (int i = 0; i < EX_DEPTH - 1; ++i) {
+    if (i < n_tiles) load_y(i);
+    cp_async_commit();
+  }
+  // Everything above reads only what was in memory before the shrink started; v is the shrink's output, so this is where a
+  // dependent launch waits.
+  pdl_wait();
+  const size_t head_off = KV && side >= 0 ? ((size_t)(side * a.n_kv + wc / FL_HEAD_DIM) * a.bt) * (FL_HEAD_DIM * 2) + (wc % FL_HEAD_DIM) * 2 : 0;
+  for (int i = 0; i < n_tiles; ++i) {
+    if (i % (EX_VT / 16) == 0) {
+      // ---- v of the next tokens: as the shrink left it in its final form, or slices summed, scaled, rounded to bf16
+      if (i > 0) __syncthreads();
+      const int v0 = 16 * i, vn = min(EX_VT, (n_tiles - i) * 16);
+      for (int c = tid; c < vn * (RMAX / 8); c += SG_THREADS) {
+        const int r = c / (RMAX / 8), ch = c % (RMAX / 8);
+        uint4 q = make_uint4(0u, 0u, 0u, 0u);
+        if (v0 + r < rows && 8 * ch < rank) {
+          if (a.v16) {
+            q = *reinterpret_cast<const uint4*>(a.v16 + ((size_t)j * a.n_tokens + tok0 + v0 + r) * RMAX + 8 * ch);
+          } else {
+            float4 s0 = make_float4(0.f, 0.f, 0.f, 0.f), s1 = s0;
+            for (int sp = 0; sp < a.ksplit; ++sp) {
+              const float4* src = reinterpret_cast<const float4*>(a.v + ((size_t)(j * a.ksplit + sp) * a.n_tokens + tok0 + v0 + r) * RMAX + 8 * ch);
+              const float4 p0 = src[0], p1 = src[1];
+              s0.x += p0.x; s0.y += p0.y; s0.z += p0.z; s0.w += p0.w;
+              s1.x += p1.x; s1.y += p1.y; s1.z += p1.z; s1.w += p1.w;
+            }
+            q = make_uint4(pack_bf16(s0.x * a.scale, s0.y * a.scale), pack_bf16(s0.z * a.scale, s0.w * a.scale),
+                           pack_bf16(s1.x * a.scale, s1.y * a.scale), pack_bf16(s1.z * a.scale, s1.w * a.scale));
+          }
+        }
+        *reinterpret_cast<uint4*>(smem + ex_vswz<RMAX>(r, ch)) = q;
+      }
+      __syncthreads();
+    }
+    if (i + EX_DEPTH - 1 < n_tiles) load_y(i + EX_DEPTH - 1);
+    cp_async_commit();
+    const int vr = 16 * (i % (EX_VT / 16));
+    uint32_t af[KN][4];
+#pragma unroll
+    for (int ks = 0; ks < KN; ++ks)
+      ldmatrix_x4(af[ks], sbase + ex_vswz<RMAX>(vr + (lane & 7) + 8 * ((lane >> 3) & 1), 2 * ks + (lane >> 4)));
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {          // 32 columns at a time
+      float acc[4][4];
+#pragma unroll
+      for (int n = 0; n < 4; ++n) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
+#pragma unroll
+      for (int ks = 0; ks < KN; ++ks)
+        if (KN == 1 || 16 * ks < rank) {
+#pragma unroll
+          for (int n = 0; n < 4; ++n) mma_bf16(acc[n], af[ks], bf[ks][4 * q + n][0], bf[ks][4 * q + n][1]);
+        }
+#pragma unroll
+      for (int n = 0; n < 4; n += 2)       // 16 rows x 2 tiles of 8 columns: rows of 128 bytes, chunks swizzled
+        stmatrix_x4(term + swz((lane & 7) + 8 * ((lane >> 3) & 1), 4 * q + n + (lane >> 4), 8), pack_bf16(acc[n][0], acc[n][1]),
+                    pack_bf16(acc[n][2], acc[n][3]), pack_bf16(acc[n + 1][0], acc[n + 1][1]), pack_bf16(acc[n + 1][2], acc[n + 1][3]));
+    }
+    cp_async_wait<EX_DEPTH - 1>();
+    __syncwarp();
+    const uint32_t yp = ring + (i % EX_DEPTH) * EX_TILE;
+    __nv_bfloat16* const yr = ycol + (size_t)(16 * i) * d_out;
+    const int left = rows - 16 * i - pr;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int r = pr + 4 * k;
+      const uint4 base = ld_shared_v4(yp + k * 512);
+      const uint4 sum = KV && lid < 0 ? base : add_bf16x8(base, ld_shared_v4(term + swz(r, pc, 8)));     // (a sum would turn -0 into 0)
+      if (cok && 4 * k < left) {
+        if (!KV || side < 0) {
+          *reinterpret_cast<uint4*>(yr + k * step4) = sum;
+        } else {
+          const uint32_t l = loc[16 * i + r];
+          if (l != 0xffffffffu) {
+            const int slot = (l >> 1) & 127;
+            unsigned char* dst = a.pv.slab + (size_t)(l >> 8) * a.pv.block_bytes + head_off + slot * (FL_HEAD_DIM * 2);
+            *reinterpret_cast<uint4*>(dst) = sum;
+            if (side == 1 && (l & 1u))     // V of a request's last token: clear the slots behind it
+              for (int z = slot + 1; z < a.bt; ++z)
+                *reinterpret_cast<uint4*>(dst + (z - slot) * (FL_HEAD_DIM * 2)) = make_uint4(0u, 0u, 0u, 0u);
+          }
+        }
+      }
+    }
+    __syncwarp();
+  }
+  cp_async_wait<0>();
 }
 
 int pick_ksplit(int n_tokens) {
@@ -586,17 +835,55 @@ int pick_expand_cols(const SgmvArgs& a, int tiles) {
   return cols;
 }
 
+template <int RMAX>
+int launch_expand_long(fl_pool* p, const SgmvArgs& a, cudaStream_t st) {
+  static bool configured[16] = {};
+  if (!configured[p->device & 15]) {
+    FL_CUDA(p, cudaFuncSetAttribute(sgmv_expand_long_kernel<RMAX, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ex_smem(RMAX)));
+    FL_CUDA(p, cudaFuncSetAttribute(sgmv_expand_long_kernel<RMAX, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ex_smem(RMAX)));
+    configured[p->device & 15] = true;
+  }
+  int n_ranges = 0;
+  for (int j = 0; j < a.n_mats; ++j) n_ranges += (a.d_out[j] + EX_COLS - 1) / EX_COLS;
+  // Tokens per CTA: the rounds of CTAs over the SMs times what a CTA costs, its prologue being worth about 48 tokens (of 256,
+  // 128 and 64 tokens, q of 8747 tokens on 7B takes 67, 69 and 71 us in one, two and four rounds; q of 4391 tokens 31 us at
+  // 128 in one round and 35 us at 64 in two).
+  const long slots = (RMAX == 16 ? 5L : 4L) * p->sm_count;
+  int tm = EX_TM;
+  long best = -1;
+  for (int t = EX_TM; t >= 64; t /= 2) {
+    const long cost = ((long)(a.n_tokens / t + 1) * n_ranges + slots - 1) / slots * (t + 48);
+    if (best < 0 || cost < best) { best = cost; tm = t; }
+  }
+  const unsigned grid = (unsigned)((a.n_seg + a.n_tokens / tm) * n_ranges);
+  if (a.all_segments) FL_CUDA(p, launch_pdl(sgmv_expand_long_kernel<RMAX, true>, dim3(grid), dim3(SG_THREADS), ex_smem(RMAX), st, a, tm, n_ranges));
+  else FL_CUDA(p, launch_pdl(sgmv_expand_long_kernel<RMAX, false>, dim3(grid), dim3(SG_THREADS), ex_smem(RMAX), st, a, tm, n_ranges));
+  return FL_OK;
+}
+
+template <int RMAX>
+int launch_expand_short(fl_pool* p, SgmvArgs& a, int tiles, int d_out_max, cudaStream_t st) {
+  const int smem = expand_smem_bytes(RMAX);     // two stages of (y, B) + the LoRA-term tile
+  static bool configured[16] = {};
+  if (!configured[p->device & 15]) {
+    FL_CUDA(p, cudaFuncSetAttribute(sgmv_expand_kernel<RMAX, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    FL_CUDA(p, cudaFuncSetAttribute(sgmv_expand_kernel<RMAX, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    configured[p->device & 15] = true;
+  }
+  a.expand_cols = pick_expand_cols(a, tiles);
+  const dim3 grid(tiles * a.n_mats, (d_out_max + a.expand_cols - 1) / a.expand_cols);
+  if (a.all_segments) FL_CUDA(p, launch_pdl(sgmv_expand_kernel<RMAX, true>, grid, dim3(SG_THREADS), smem, st, a));
+  else FL_CUDA(p, launch_pdl(sgmv_expand_kernel<RMAX, false>, grid, dim3(SG_THREADS), smem, st, a));
+  return FL_OK;
+}
+
 template <int TM, int RMAX>
 int launch_pair(fl_pool* p, SgmvArgs& a, int tiles, int d_out_max, cudaStream_t st, bool shrink_only) {
-  a.expand_cols = pick_expand_cols(a, tiles);
   static bool configured[16] = {};
   const int shrink_smem_max = shrink_pipe_bytes(TM, RMAX) + (TM == 16 ? KSPLIT_MAX * 16 * RMAX * 4 : 0);
   const int shrink_smem = a.v16 ? shrink_smem_max : shrink_pipe_bytes(TM, RMAX);      // + every slice's sums
-  const int expand_smem = expand_smem_bytes(TM, RMAX);     // two stages of (y, B) + the LoRA-term tile
   if (!configured[p->device & 15]) {
     FL_CUDA(p, cudaFuncSetAttribute(sgmv_shrink_kernel<TM, RMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, shrink_smem_max));
-    FL_CUDA(p, cudaFuncSetAttribute(sgmv_expand_kernel<TM, RMAX, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, expand_smem));
-    FL_CUDA(p, cudaFuncSetAttribute(sgmv_expand_kernel<TM, RMAX, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, expand_smem));
     configured[p->device & 15] = true;
   }
   if (TM == 64 && p->sgmv_shrink_kind == 0 && a.n_mats <= 3 && a.tc_ksplit > 0) {
@@ -613,27 +900,31 @@ int launch_pair(fl_pool* p, SgmvArgs& a, int tiles, int d_out_max, cudaStream_t 
     t.n_seg = a.n_seg;
     t.n_tokens = a.n_tokens;
     t.d_in = p->mats[a.mat_index[0]].d_in;
+    t.scale = a.scale;
+    t.v16 = nullptr;
+    if (!shrink_only && a.ksplit == 1) t.v16 = a.v16 = reinterpret_cast<__nv_bfloat16*>(a.v);      // one slice: v in its final form
     const int rc = sgmv::shrink_tc(p, t, a.x, RMAX, st);
     if (rc != FL_OK) return rc;
   } else if (TM == 64 && RMAX == 16 && a.n_mats == 3) {      // at higher ranks the three accumulators cost too many registers
+    // three stages (43 KB) put five CTAs on an SM, four stages three: 46 against 57 us for 19770 tokens on 7B, where 340 tiles
+    // in two slices are one round of five per SM and two rounds of three; with fewer CTAs the deeper pipeline is the better one
     static bool configured3[16] = {};
-    const int smem3 = (RMAX == 64 ? 3 : 4) * (64 + 3 * RMAX) * 128;
+    const int smem_of[2] = {3 * (64 + 3 * RMAX) * 128, 4 * (64 + 3 * RMAX) * 128};
     if (!configured3[p->device & 15]) {
-      FL_CUDA(p, cudaFuncSetAttribute(sgmv_shrink3_kernel<RMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem3));
+      FL_CUDA(p, cudaFuncSetAttribute(sgmv_shrink3_kernel<RMAX, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_of[0]));
+      FL_CUDA(p, cudaFuncSetAttribute(sgmv_shrink3_kernel<RMAX, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_of[1]));
       configured3[p->device & 15] = true;
     }
-    FL_CUDA(p, launch_pdl(sgmv_shrink3_kernel<RMAX>, dim3(tiles, a.ksplit), dim3(SG_THREADS), smem3, st, a));
+    if (tiles * a.ksplit > 3 * p->sm_count)
+      FL_CUDA(p, launch_pdl(sgmv_shrink3_kernel<RMAX, 3>, dim3(tiles, a.ksplit), dim3(SG_THREADS), smem_of[0], st, a));
+    else
+      FL_CUDA(p, launch_pdl(sgmv_shrink3_kernel<RMAX, 4>, dim3(tiles, a.ksplit), dim3(SG_THREADS), smem_of[1], st, a));
   } else {
     FL_CUDA(p, launch_pdl_cluster(sgmv_shrink_kernel<TM, RMAX>, dim3(tiles * a.n_mats, a.ksplit), dim3(1, a.v16 ? a.ksplit : 1),
                                   dim3(SG_THREADS), shrink_smem, st, a));
   }
   if (shrink_only) return FL_OK;       // the caller consumes the partial sums itself
-  const dim3 egrid(tiles * a.n_mats, (d_out_max + a.expand_cols - 1) / a.expand_cols);
-  // the expand may start while the shrink drains (it waits for the shrink's output inside the kernel)
-  FL_CUDA(p, cudaGetLastError());
-  if (a.all_segments) FL_CUDA(p, launch_pdl(sgmv_expand_kernel<TM, RMAX, true>, egrid, dim3(SG_THREADS), expand_smem, st, a));
-  else FL_CUDA(p, launch_pdl(sgmv_expand_kernel<TM, RMAX, false>, egrid, dim3(SG_THREADS), expand_smem, st, a));
-  return FL_OK;
+  return TM == 64 ? launch_expand_long<RMAX>(p, a, st) : launch_expand_short<RMAX>(p, a, tiles, d_out_max, st);
 }
 
 int rmax_of(const fl_pool* p) { return p->max_rank <= 16 ? 16 : (p->max_rank <= 32 ? 32 : 64); }
@@ -688,6 +979,7 @@ int sgmv_common(fl_pool* p, fl_bf16* const* ys, const fl_bf16* x, const int* mat
   a.req_indptr = a.tbl_indptr = a.prefix_lens = nullptr;
   a.tbl = nullptr;
   a.n_req = a.n_kv = a.bt = 0;
+  a.bt_inv = 0;
   if (kv) {
     const size_t per_tok = (size_t)2 * kv->n_kv * FL_HEAD_DIM * 2;
     if (kv->n_kv < 1 || kv->n_req < 1 || p->block_bytes % per_tok != 0 || kv->k_slot == kv->v_slot) return FL_EINVAL;
@@ -705,6 +997,7 @@ int sgmv_common(fl_pool* p, fl_bf16* const* ys, const fl_bf16* x, const int* mat
     a.n_req = kv->n_req;
     a.n_kv = kv->n_kv;
     a.bt = (int)(p->block_bytes / per_tok);
+    a.bt_inv = (uint32_t)(((1ull << 32) + a.bt - 1) / a.bt);
     // the expand packs a token's destination into one word: 7 bits of slot, 24 bits of block id
     if (a.bt > 128 || p->n_blocks > (1u << 24)) return FL_EINVAL;
   }

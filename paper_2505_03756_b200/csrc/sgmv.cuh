@@ -22,10 +22,9 @@ int shrink_scaled(fl_pool* p, const fl_bf16* x, const int* mat_indices, int n_ma
                   fl_stream stream, ShrinkInfo* info);
 
 #ifdef __CUDACC__
-// Token tile `tile` (tiles of TM tokens, counted over segments that carry an adapter, or over all segments) -> segment and
+// Token tile `tile` (tiles of tm tokens, counted over segments that carry an adapter, or over all segments) -> segment and
 // token range.  Every warp evaluates it redundantly with a warp scan over 32 segments at a time.
-template <int TM>
-__device__ __forceinline__ bool find_tile(const int32_t* __restrict__ seg_indptr, const int32_t* __restrict__ lora_ids,
+__device__ __forceinline__ bool find_tile(const int tm, const int32_t* __restrict__ seg_indptr, const int32_t* __restrict__ lora_ids,
                                           int n_seg, int tile, int& seg, int& tok0, int& tok1, bool all_segments = false) {
   const int lane = threadIdx.x & 31;
   int base = 0;
@@ -35,7 +34,7 @@ __device__ __forceinline__ bool find_tile(const int32_t* __restrict__ seg_indptr
     if (s < n_seg) {
       lo = seg_indptr[s];
       hi = seg_indptr[s + 1];
-      if ((all_segments || lora_ids[s] >= 0) && hi > lo) nt = (hi - lo + TM - 1) / TM;
+      if ((all_segments || lora_ids[s] >= 0) && hi > lo) nt = (hi - lo + tm - 1) / tm;
     }
     int incl = nt;
 #pragma unroll
@@ -50,13 +49,19 @@ __device__ __forceinline__ bool find_tile(const int32_t* __restrict__ seg_indptr
       const int src = __ffs(__ballot_sync(0xffffffffu, mine)) - 1;
       const int k = tile - __shfl_sync(0xffffffffu, first, src);
       seg = s0 + src;
-      tok0 = __shfl_sync(0xffffffffu, lo, src) + k * TM;
-      tok1 = min(tok0 + TM, __shfl_sync(0xffffffffu, hi, src));
+      tok0 = __shfl_sync(0xffffffffu, lo, src) + k * tm;
+      tok1 = min(tok0 + tm, __shfl_sync(0xffffffffu, hi, src));
       return true;
     }
     base += total;
   }
   return false;
+}
+
+template <int TM>
+__device__ __forceinline__ bool find_tile(const int32_t* __restrict__ seg_indptr, const int32_t* __restrict__ lora_ids,
+                                          int n_seg, int tile, int& seg, int& tok0, int& tok1, bool all_segments = false) {
+  return find_tile(TM, seg_indptr, lora_ids, n_seg, tile, seg, tok0, tok1, all_segments);
 }
 
 // Start of rank-row `row` of a stream (class table entry tab, first row row0, rows per block rpb, row width).
@@ -81,6 +86,8 @@ __device__ __forceinline__ const unsigned char* lora_row(const PoolView& pv, uin
 struct TcShrinkArgs {
   PoolView pv;
   float* v;
+  __nv_bfloat16* v16;      // one slice only: the scaled sum in bf16, [projection][token][rmax], instead of v
+  float scale;
   int ksplit, n_mats;
   int mat_index[3];
   const int32_t* seg_indptr;

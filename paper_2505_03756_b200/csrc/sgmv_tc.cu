@@ -249,7 +249,17 @@ __global__ void __launch_bounds__(ST_THREADS, 1) sgmv_shrink_tc_kernel(const sgm
         tmem_ld16(lane_addr + buf * N + c0, o);
         tmem_wait_ld();
         const int j = c0 / RMAX, col = c0 % RMAX;
-        if (mine && j < a.n_mats) {
+        if (mine && j < a.n_mats && a.v16) {
+          uint4* dst = reinterpret_cast<uint4*>(a.v16 + ((size_t)j * a.n_tokens + tok) * RMAX + col);
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            const uint32_t* q = o + 8 * c;
+            dst[c] = make_uint4(pack_bf16(__uint_as_float(q[0]) * a.scale, __uint_as_float(q[1]) * a.scale),
+                                pack_bf16(__uint_as_float(q[2]) * a.scale, __uint_as_float(q[3]) * a.scale),
+                                pack_bf16(__uint_as_float(q[4]) * a.scale, __uint_as_float(q[5]) * a.scale),
+                                pack_bf16(__uint_as_float(q[6]) * a.scale, __uint_as_float(q[7]) * a.scale));
+          }
+        } else if (mine && j < a.n_mats) {
           float4* dst = reinterpret_cast<float4*>(a.v + ((size_t)(j * a.ksplit + t.split) * a.n_tokens + tok) * RMAX + col);
 #pragma unroll
           for (int c = 0; c < 4; ++c)
