@@ -6,8 +6,9 @@
 // through global memory.
 //   warp 0      TMA producer: x tile [tokens x 64] and W tile [64 x 128] per stage, ring of as many stages as fit
 //   warp 1      MMA issuer of x W
-//   warp 6      MMA issuer of the LoRA term, into an accumulator of its own
-//   warps 2-5   LoRA stages, then the epilogue (thread = token row)
+//   warps 2-5   list of the LoRA stages, a share of them, then the epilogue (thread = token row)
+//   up to 8 more the other LoRA stages, four warps to a stage
+//   last warp   MMA issuer of the LoRA term, into an accumulator of its own
 // The LoRA term is one more product over a long, sparse k: the rank-rows of every adapter of the batch one after the
 // other, 64 to a stage, against a matrix that holds in row t the shrink result of token t at the ranks of its own adapter
 // and zeros elsewhere.  A stage has the layout of a main stage: B rows through the block table in place of W rows,
@@ -35,17 +36,21 @@ namespace {
 
 using namespace tc;
 
-constexpr int THREADS = 224;
+constexpr int FILLERS = 3;                         // groups of four warps that fill LoRA stages
+constexpr int MAX_THREADS = 96 + 128 * FILLERS;    // a launch brings one group per slot of the LoRA ring and no more: fewer
+                                                   // registers let the CTA start beside CTAs of the shrink
+
 constexpr int BN = 128, BK = 64;                   // columns per CTA; d_in (or rank-rows) per stage
 constexpr uint32_t W_BYTES = BK * BN * 2, W_GROUP = BK * 128;      // two groups of 64 columns
-constexpr int MAX_NS = 12, MAX_NE = 3;
+constexpr int MAX_NS = 12, MAX_NE = FILLERS;
 constexpr int UNIT = 16;                           // rank-rows per entry of the LoRA list: one k-step
 constexpr int UNITS_PER_TOKEN = FL_MAX_RANK / UNIT;      // every token its own adapter of the highest rank
-constexpr int GROUP = 8;                           // LoRA stages whose row addresses are looked up together
+constexpr int GROUP = 4;                           // LoRA stages whose row addresses a group of warps looks up together
 constexpr int MAX_SPLIT = 8;
 // Not all of an SM's 227 KB: what is left lets the CTA start beside CTAs of the shrink before it (a decode step of one token:
 // 57 us a layer at 180 KB, 61 at 227 KB, 59 at 113 KB; of 48 tokens the same at 180 and 227 KB, 2 % more at 113 KB).
-constexpr uint32_t SMEM_LIMIT = 180 * 1024;
+// Above 128 tokens a stage is mostly x, and the ring needs all of it.
+constexpr uint32_t SMEM_LIMIT = 180 * 1024, SMEM_MAX = 227 * 1024;
 
 struct LoraUnit {        // 16 rank-rows of one segment's adapter
   uint16_t lo, hi;       // the segment's tokens
@@ -65,12 +70,12 @@ struct Maps {
 };
 
 enum { B_FULL = 0, B_EMPTY = MAX_NS, B_EFULL = 2 * MAX_NS, B_EEMPTY = B_EFULL + MAX_NE, B_LIST = B_EEMPTY + MAX_NE, B_ACC, B_COUNT };
-// behind the two rings: barriers and bookkeeping | B row addresses of two groups of stages | list of LoRA units
-constexpr uint32_t BOOK_BYTES = 384, ROWS_BYTES = 2 * GROUP * BK * 8;
+// behind the two rings: barriers and bookkeeping | B row addresses, two sets of stages per group of warps | list of LoRA units
+constexpr uint32_t BOOK_BYTES = 512, ROWS_BYTES = FILLERS * 2 * GROUP * BK * 8;
 static_assert(8 * B_COUNT + 48 <= BOOK_BYTES, "bookkeeping area too small");
 static_assert(sizeof(LoraUnit) == 16, "one 16-byte shared-memory access per unit");
 
-__global__ void __launch_bounds__(THREADS, 1) lora_skinny_kernel(const __grid_constant__ KArgs ka, const __grid_constant__ Maps maps) {
+__global__ void __launch_bounds__(MAX_THREADS, 1) lora_skinny_kernel(const __grid_constant__ KArgs ka, const __grid_constant__ Maps maps) {
   const skinny::Args& a = ka.s;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -86,7 +91,8 @@ __global__ void __launch_bounds__(THREADS, 1) lora_skinny_kernel(const __grid_co
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + off_book + 8 * B_COUNT + 4);
   volatile int* n_stage_slot = reinterpret_cast<volatile int*>(smem + off_book + 8 * B_COUNT + 8);
   int* scan = reinterpret_cast<int*>(smem + off_book + 8 * B_COUNT + 16);      // [4], one per filler warp
-  unsigned long long* row_ptr = reinterpret_cast<unsigned long long*>(smem + off_book + BOOK_BYTES);     // [2][GROUP * BK], 0 = no row
+  volatile int* rpb_slot = reinterpret_cast<volatile int*>(smem + off_book + 8 * B_COUNT + 12);
+  unsigned long long* row_ptr = reinterpret_cast<unsigned long long*>(smem + off_book + BOOK_BYTES);     // [group][2][GROUP * BK], 0 = no row
   LoraUnit* list = reinterpret_cast<LoraUnit*>(smem + off_book + BOOK_BYTES + ROWS_BYTES);
   const int max_units = npad * UNITS_PER_TOKEN;
 
@@ -145,7 +151,8 @@ __global__ void __launch_bounds__(THREADS, 1) lora_skinny_kernel(const __grid_co
 
   bool ok = true;
   int n_stages = 0;                        // LoRA stages of this CTA (known to the LoRA roles)
-  const int et = tid - 64;                 // filler / epilogue thread 0..127
+  const int filler = (warp - 2) >> 2;      // group of four warps
+  const int et = (tid - 64) & 127;         // thread of its group; of the first: epilogue thread
   if (warp == 0) {
     // ------------------------------------------------ TMA producer
     if (lane == 0) {
@@ -174,7 +181,7 @@ __global__ void __launch_bounds__(THREADS, 1) lora_skinny_kernel(const __grid_co
       if (++s == ns) { s = 0; ph ^= 1u; }
     }
     if (ok) umma_commit_elect(bar(B_ACC));
-  } else if (warp == 6) {
+  } else if (warp == 2 + 4 * ne) {
     // ------------------------------------------------ MMA issuer of the LoRA term
     ok = wait_all(bar(B_LIST), 0);
     if (ok) n_stages = *n_stage_slot;
@@ -189,86 +196,111 @@ __global__ void __launch_bounds__(THREADS, 1) lora_skinny_kernel(const __grid_co
     }
     if (ok) umma_commit_elect(bar(B_ACC));
   } else {
-    // ------------------------------------------------ list of the LoRA units, in segment order
-    int n_units = 0;
     uint32_t rpb = 1;
-    for (int s0 = 0; s0 < a.n_seg; s0 += 128) {
-      const int s = s0 + et;
-      int lo = 0, hi = 0, rank = 0;
-      uint32_t tab = 0, row0 = 0;
-      if (s < a.n_seg) {
-        lo = max(a.seg_indptr[s], 0);
-        hi = min(a.seg_indptr[s + 1], a.n_tokens);
-        const int lid = a.lora_ids[s];
-        if (lid >= 0 && hi > lo) {
-          if ((uint32_t)lid >= a.pv.dir_cap || a.pv.dir[lid].rank <= 0 || a.mat_index[j] >= a.pv.dir[lid].n_mats) {
-            atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_LORA);
-          } else {
-            const LoraEntry* en = a.pv.dir + lid;
-            rank = min(en->rank, a.rmax);
-            const LoraMat lm = en->mats[a.mat_index[j]];
-            tab = en->table_off + lm.b_tab;
-            row0 = lm.b_row0;
-            rpb = lm.b_rpb;          // the same for every adapter: they share the projection's shape
+    if (filler == 0) {
+      // ------------------------------------------------ list of the LoRA units, in segment order
+      int n_units = 0;
+      for (int s0 = 0; s0 < a.n_seg; s0 += 128) {
+        const int s = s0 + et;
+        int lo = 0, hi = 0, rank = 0;
+        uint32_t tab = 0, row0 = 0;
+        if (s < a.n_seg) {
+          lo = max(a.seg_indptr[s], 0);
+          hi = min(a.seg_indptr[s + 1], a.n_tokens);
+          const int lid = a.lora_ids[s];
+          if (lid >= 0 && hi > lo) {
+            if ((uint32_t)lid >= a.pv.dir_cap || a.pv.dir[lid].rank <= 0 || a.mat_index[j] >= a.pv.dir[lid].n_mats) {
+              atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_LORA);
+            } else {
+              const LoraEntry* en = a.pv.dir + lid;
+              rank = min(en->rank, a.rmax);
+              const LoraMat lm = en->mats[a.mat_index[j]];
+              tab = en->table_off + lm.b_tab;
+              row0 = lm.b_row0;
+              rpb = lm.b_rpb;          // the same for every adapter: they share the projection's shape
+            }
           }
         }
-      }
-      const int cnt = (rank + UNIT - 1) / UNIT;
-      int incl = cnt;
+        const int cnt = (rank + UNIT - 1) / UNIT;
+        int incl = cnt;
 #pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const int o = __shfl_up_sync(0xffffffffu, incl, d);
-        if (lane >= d) incl += o;
-      }
-      if (lane == 31) scan[warp - 2] = incl;
-      asm volatile("bar.sync 1, 128;" ::: "memory");
-      int at = n_units + incl - cnt;
-      for (int w = 0; w < 4; ++w) {
-        const int t = scan[w];
-        if (w < warp - 2) at += t;
-        n_units += t;
-      }
-      asm volatile("bar.sync 1, 128;" ::: "memory");
-      for (int r0 = 0; r0 < rank; r0 += UNIT, ++at)
-        if (at < max_units) {
-          LoraUnit u;
-          u.lo = (uint16_t)lo;
-          u.hi = (uint16_t)hi;
-          u.r0 = (uint16_t)r0;
-          u.nr = (uint16_t)min(UNIT, rank - r0);
-          u.tab = tab;
-          u.row0 = row0 + r0;
-          list[at] = u;
+        for (int d = 1; d < 32; d <<= 1) {
+          const int o = __shfl_up_sync(0xffffffffu, incl, d);
+          if (lane >= d) incl += o;
         }
-    }
-    n_units = min(n_units, max_units);           // (overlapping segments, which the interface rules out, could exceed it)
-    const int all_stages = (n_units + 3) / 4;
-    if (et < all_stages * 4 - n_units) {
-      LoraUnit none = {};
-      list[n_units + et] = none;
-    }
-    {
-      const uint32_t m = __reduce_max_sync(0xffffffffu, rpb);
-      if (lane == 0) scan[warp - 2] = (int)m;
+        if (lane == 31) scan[warp - 2] = incl;
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        int at = n_units + incl - cnt;
+        for (int w = 0; w < 4; ++w) {
+          const int t = scan[w];
+          if (w < warp - 2) at += t;
+          n_units += t;
+        }
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        for (int r0 = 0; r0 < rank; r0 += UNIT, ++at)
+          if (at < max_units) {
+            LoraUnit u;
+            u.lo = (uint16_t)lo;
+            u.hi = (uint16_t)hi;
+            u.r0 = (uint16_t)r0;
+            u.nr = (uint16_t)min(UNIT, rank - r0);
+            u.tab = tab;
+            u.row0 = row0 + r0;
+            list[at] = u;
+          }
+      }
+      n_units = min(n_units, max_units);           // (overlapping segments, which the interface rules out, could exceed it)
+      const int all_stages = (n_units + 3) / 4;
+      if (et < all_stages * 4 - n_units) {
+        LoraUnit none = {};
+        list[n_units + et] = none;
+      }
+      {
+        const uint32_t m = __reduce_max_sync(0xffffffffu, rpb);
+        if (lane == 0) scan[warp - 2] = (int)m;
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        for (int w = 0; w < 4; ++w) rpb = max(rpb, (uint32_t)scan[w]);
+      }
+      // stages are dealt round robin over the cluster
+      n_stages = all_stages > crank ? (all_stages - crank + split - 1) / split : 0;
+      // the v rows of the ring start at zero
+      if (n_stages > 0)
+        for (int e = 0; e < ne; ++e)
+          for (int c = et; c < npad * 8; c += 128)
+            *reinterpret_cast<uint4*>(smem + off_ext + e * stage_bytes + c * 16) = make_uint4(0u, 0u, 0u, 0u);
+      fence_async_smem();
       asm volatile("bar.sync 1, 128;" ::: "memory");
-      for (int w = 0; w < 4; ++w) rpb = max(rpb, (uint32_t)scan[w]);
-    }
-    // stages are dealt round robin over the cluster
-    n_stages = all_stages > crank ? (all_stages - crank + split - 1) / split : 0;
-    if (et == 0) {
-      *n_stage_slot = n_stages;
-      mbar_arrive(bar(B_LIST));
+      if (et == 0) {
+        *n_stage_slot = n_stages;
+        *rpb_slot = (int)rpb;
+        mbar_arrive(bar(B_LIST));
+      }
+    } else {
+      ok = mbar_wait(bar(B_LIST), 0, abort_flag);
+      if (ok) {
+        n_stages = *n_stage_slot;
+        rpb = (uint32_t)*rpb_slot;
+      }
+      ok = group_and(ok, 1 + filler, 128);
+      if (!ok) n_stages = 0;
     }
     // ------------------------------------------------ fill the LoRA stages
-    // Addresses of a group's B rows, looked up side by side a group ahead of their use, and their 256 bytes asked into L2:
-    // under the stream of W a load takes 2 us, and a stage that had to wait for its table entry and then for its rows took
-    // 3.5 us (decode step of 48 tokens and 35 adapters of rank 32, d_out 15360).
+    // Addresses of the B rows of this group's next stages, looked up side by side ahead of their use, and their 256 bytes asked
+    // into L2: under the stream of W a load takes 2 us, and a stage that had to wait for its table entry and then for its rows
+    // took 3.5 us (decode step of 48 tokens and 35 adapters of rank 32, d_out 15360).  Issuing a stage's copies takes four
+    // warps about 3000 cycles, most of them in the load/store unit's queue, hence three groups.
+    unsigned long long* const my_rows = row_ptr + filler * (2 * GROUP * BK);
+    // One group per slot of the ring: a group then knows, from the stage it filled before, that the slot's use before last is
+    // over, and a parity wait tells the last one from it.
+    const int n_mine = n_stages > filler ? (n_stages - filler + ne - 1) / ne : 0;     // stages filler, filler + ne, ..
+    auto units_of = [&](int k) { return list + 4 * (crank + (filler + k * ne) * split); };
     auto find_rows = [&](int g) {
-      for (int i = et; i < GROUP * BK; i += 128) {
-        const int st = g * GROUP + i / BK, r = i % BK;
+#pragma unroll
+      for (int i = 0; i < GROUP * BK / 128; ++i) {
+        const int c = et + 128 * i, k = g * GROUP + c / BK, r = c % BK;
         unsigned long long at = 0;
-        if (st < n_stages) {
-          const LoraUnit x = list[4 * (crank + st * split) + r / UNIT];
+        if (k < n_mine) {
+          const LoraUnit x = units_of(k)[r / UNIT];
           if (r % UNIT < x.nr) {
             const uint32_t gr = x.row0 + r % UNIT;
             const uint32_t blk = a.pv.tables[x.tab + gr / rpb];
@@ -282,31 +314,27 @@ __global__ void __launch_bounds__(THREADS, 1) lora_skinny_kernel(const __grid_co
             }
           }
         }
-        row_ptr[(g & 1) * GROUP * BK + i] = at;
+        my_rows[(g & 1) * GROUP * BK + c] = at;
       }
     };
     const int row = et >> 4, ch = et & 15;               // B rows row + 8 i, 16-byte chunk ch of the 128 columns
     const int vrow = et >> 3, vch = et & 7;              // v rows vrow + 16 i, ranks 8 vch .. of the stage's 64
     const bool col_ok = n0 + ch * 8 < d_out;
-    auto landed = [&](int pending) {                     // all but this thread's newest `pending` stages have landed
-      if (pending == 0) cp_async_wait<0>();
-      else if (pending == 1) cp_async_wait<1>();
-      else cp_async_wait<2>();
-      fence_async_smem();
+    auto range_of = [](const LoraUnit* u, int& lo, int& hi) {      // tokens of a stage: segments come in token order
+      lo = u[0].lo;
+      hi = u[0].hi;
+#pragma unroll
+      for (int q = 1; q < 4; ++q)
+        if (u[q].nr) hi = max(hi, (int)u[q].hi);
     };
-    if (n_stages > 0) {
-      find_rows(0);
-      asm volatile("bar.sync 1, 128;" ::: "memory");
-    }
-    int s = 0, done = 0, ds = 0;
-    uint32_t ph = 1;
-    for (int i = 0; i < n_stages; ++i) {
-      // (the barrier also makes the addresses of a group visible that were looked up some stages ago)
-      if (i >= ne) ok = group_and(mbar_wait(bar(B_EEMPTY + s), ph, abort_flag), 1, 128);
+    if (n_mine > 0) find_rows(0);
+    for (int k = 0; k < n_mine; ++k) {
+      if (k > 0) ok = mbar_wait(bar(B_EEMPTY + filler), (uint32_t)((k - 1) & 1), abort_flag);
+      ok = group_and(ok, 1 + filler, 128);               // (also makes the addresses visible that were looked up before)
       if (!ok) break;
-      const LoraUnit* u = list + 4 * (crank + i * split);
-      const unsigned long long* rp = row_ptr + (i % (2 * GROUP)) * BK;
-      const uint32_t vb = sbase + off_ext + s * stage_bytes, bb = vb + x_bytes;
+      const LoraUnit* u = units_of(k);
+      const unsigned long long* rp = my_rows + (k % (2 * GROUP)) * BK;
+      const uint32_t vb = sbase + off_ext + filler * stage_bytes, bb = vb + x_bytes;
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
         const int r = row + 8 * q;
@@ -314,43 +342,42 @@ __global__ void __launch_bounds__(THREADS, 1) lora_skinny_kernel(const __grid_co
         cp_async16(bb + (ch >> 3) * W_GROUP + r * 128 + (((ch & 7) ^ (r & 7)) << 4),
                    at ? reinterpret_cast<const unsigned char*>(at) + ch * 16 : a.pv.slab, at && col_ok);
       }
-      if (i == 0) pdl_wait();                            // v is the shrink's output
+      if (k == 0) pdl_wait();                            // v is the shrink's output
       {
         const LoraUnit x = u[vch >> 1];
         const int r = x.r0 + 8 * (vch & 1);
         const bool live = 8 * (vch & 1) < x.nr;
         const __nv_bfloat16* src = a.v + ((size_t)j * a.n_tokens) * a.rmax + r;
-        for (int t = vrow; t < npad; t += 16) {
+        // Only the rows of the stage's own tokens are written, and zeros over those of the stage before it in this slot (a
+        // decode step: four rows each instead of all).
+        int lo, hi;
+        range_of(u, lo, hi);
+        for (int t = lo + vrow; t < hi; t += 16) {
           const bool mine = live && t >= x.lo && t < x.hi;
           cp_async16(vb + t * 128 + ((vch ^ (t & 7)) << 4), mine ? src + (size_t)t * a.rmax : a.v, mine);
         }
+        if (k > 0) {
+          int lo0, hi0;
+          range_of(units_of(k - 1), lo0, hi0);
+          for (int t = lo0 + vrow; t < hi0; t += 16)
+            if (t < lo || t >= hi) cp_async16(vb + t * 128 + ((vch ^ (t & 7)) << 4), a.v, false);
+        }
       }
       cp_async_commit();
-      if (++s == ne) { s = 0; ph ^= 1u; }
-      if (i % GROUP == 0 && i + GROUP < n_stages) find_rows(i / GROUP + 1);
-      if (i + 1 >= ne) {
-        landed(ne - 1);
-        mbar_arrive(bar(B_EFULL + ds));
-        if (++ds == ne) ds = 0;
-        ++done;
-      }
-    }
-    if (ok && done < n_stages) {
-      landed(0);
-      for (; done < n_stages; ++done) {
-        mbar_arrive(bar(B_EFULL + ds));
-        if (++ds == ne) ds = 0;
-      }
+      if (k % GROUP == 0 && k + GROUP < n_mine) find_rows(k / GROUP + 1);
+      cp_async_wait<0>();
+      fence_async_smem();
+      mbar_arrive(bar(B_EFULL + filler));
     }
     cp_async_wait<0>();
-    if (n_stages == 0) pdl_wait();
+    if (n_mine == 0) pdl_wait();
   }
 
   // ------------------------------------------------ epilogue: this thread's token row(s)
   const int quarter = warp & 3;
   const int lrow = quarter * 32 + lane;                       // row of the tile = TMEM lane
   const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
-  const bool epi = warp >= 2 && warp < 6;
+  const bool epi = filler == 0;
   const int side = a.kv_side[j];
   uint32_t kv_blk[2] = {0, 0};
   int kv_slot[2] = {-1, -1};
@@ -426,6 +453,11 @@ __global__ void __launch_bounds__(THREADS, 1) lora_skinny_kernel(const __grid_co
     cluster_sync();
   }
   if (epi && ok) {
+    // The finished rows as bf16 through shared memory (behind the partial sums; pitch an odd number of 16-byte chunks), so that
+    // they go out a whole row piece at a time: stored by the thread that owns the row, 16 bytes of 32 rows per instruction,
+    // the rows and the cleared V slots of a decode batch of 128 took up to 18 us.
+    const int nch = (c1 - c0) / 8, row_bytes = share * 2 + 16;
+    unsigned char* out = smem + (size_t)(split - 1) * npad * pitch * 4;
     for (int m = 0; m < mt; ++m) {
       const int t = m * 128 + lrow;
       for (int c = c0; c < c1; c += 16) {
@@ -446,23 +478,42 @@ __global__ void __launch_bounds__(THREADS, 1) lora_skinny_kernel(const __grid_co
             f[4 * q] += v.x; f[4 * q + 1] += v.y; f[4 * q + 2] += v.z; f[4 * q + 3] += v.w;
           }
         }
+        uint4* dst = reinterpret_cast<uint4*>(out + t * row_bytes + (c - c0) * 2);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int col = n0 + c + 8 * h;
-          if (col >= d_out) continue;
-          const uint4 q = make_uint4(pack_bf16(f[8 * h], f[8 * h + 1]), pack_bf16(f[8 * h + 2], f[8 * h + 3]),
-                                     pack_bf16(f[8 * h + 4], f[8 * h + 5]), pack_bf16(f[8 * h + 6], f[8 * h + 7]));
-          if (side < 0) {
-            *reinterpret_cast<uint4*>(a.y[j] + (size_t)t * d_out + col) = q;
-          } else if (kv_slot[m] >= 0) {
-            // [K|V][kv head][slot][128] inside the block
-            unsigned char* dst = a.pv.slab + (size_t)kv_blk[m] * a.pv.block_bytes +
-                                 ((size_t)(side * a.n_kv + col / FL_HEAD_DIM) * a.bt + kv_slot[m]) * (FL_HEAD_DIM * 2) + (col % FL_HEAD_DIM) * 2;
-            *reinterpret_cast<uint4*>(dst) = q;
-            if (side == 1 && kv_last[m])       // V of a request's last token: clear the slots behind it
-              for (int z = kv_slot[m] + 1; z < a.bt; ++z)
-                *reinterpret_cast<uint4*>(dst + (size_t)(z - kv_slot[m]) * (FL_HEAD_DIM * 2)) = make_uint4(0u, 0u, 0u, 0u);
-          }
+        for (int h = 0; h < 2; ++h)
+          dst[h] = make_uint4(pack_bf16(f[8 * h], f[8 * h + 1]), pack_bf16(f[8 * h + 2], f[8 * h + 3]),
+                              pack_bf16(f[8 * h + 4], f[8 * h + 5]), pack_bf16(f[8 * h + 6], f[8 * h + 7]));
+      }
+      if (side >= 0 && t < a.n_tokens) {
+        // a column tile is one KV head: [K|V][kv head][slot][128] inside the block; in the top bits the V slots to clear
+        unsigned long long at = 0;
+        if (kv_slot[m] >= 0)
+          at = reinterpret_cast<unsigned long long>(a.pv.slab + (size_t)kv_blk[m] * a.pv.block_bytes +
+                                                    ((size_t)(side * a.n_kv + n0 / FL_HEAD_DIM) * a.bt + kv_slot[m]) * (FL_HEAD_DIM * 2)) |
+               (unsigned long long)(side == 1 && kv_last[m] ? a.bt - 1 - kv_slot[m] : 0) << 48;
+        row_ptr[t] = at;
+      }
+    }
+    static_assert(BN == FL_HEAD_DIM && skinny::MAX_TOKENS * 8 <= ROWS_BYTES, "rows of one head, their addresses where the B rows' were");
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    for (int i = et; i < a.n_tokens * nch; i += 128) {
+      const int t = i / nch, ch = i - t * nch;
+      const uint4 q = *reinterpret_cast<const uint4*>(out + t * row_bytes + ch * 16);
+      const int col = n0 + c0 + 8 * ch;
+      if (side < 0) {
+        if (col < d_out) *reinterpret_cast<uint4*>(a.y[j] + (size_t)t * d_out + col) = q;
+      } else if (const unsigned long long at = row_ptr[t] << 16 >> 16) {
+        *reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(at) + (c0 + 8 * ch) * 2) = q;
+      }
+    }
+    if (side == 1) {             // V behind a request's last token
+      for (int t = warp - 2; t < a.n_tokens; t += 4) {
+        const unsigned long long w = row_ptr[t];
+        unsigned char* at = reinterpret_cast<unsigned char*>(w << 16 >> 16) + c0 * 2;
+        const int n = (int)(w >> 48) * nch;
+        for (int i = lane; i < n; i += 32) {
+          const int z = i / nch;
+          *reinterpret_cast<uint4*>(at + (size_t)(z + 1) * (FL_HEAD_DIM * 2) + (i - z * nch) * 16) = make_uint4(0u, 0u, 0u, 0u);
         }
       }
     }
@@ -501,18 +552,24 @@ void layout(const fl_pool* p, const skinny::Args& a, KArgs* out, uint32_t* smem)
   ka.tmem_cols = ka.npad > 128 ? 512 : 256;
   const uint32_t fixed = BOOK_BYTES + ROWS_BYTES + ka.npad * UNITS_PER_TOKEN * sizeof(LoraUnit) + 1024;
   const uint32_t stage = W_BYTES + (uint32_t)ka.npad * 128;
-  const int fit = (int)((SMEM_LIMIT - fixed) / stage);
-  ka.ne = fit >= 9 ? 3 : fit >= 6 ? 2 : 1;
-  ka.ns = std::min(MAX_NS, fit - ka.ne);
   // As many CTAs per column tile as the SMs hold at once (clusters above two do not fill every SM), every one with at least
-  // four stages of d_in, as long as the partial sums fit in the ring that they reuse.
+  // four stages of d_in.
   const int nk = (a.d_in + BK - 1) / BK;
   ka.split = 1;
-  for (int s = 2; s <= MAX_SPLIT; ++s) {
-    const int share = (BN / 16 + s - 1) / s * 16;
-    if (tiles * s <= (s == 2 ? p->sm_count : p->sm_count * 9 / 10) && nk / s >= 4 &&
-        (uint32_t)((s - 1) * ka.npad * (share + 4) * 4) <= ka.ns * stage)
-      ka.split = s;
+  for (int s = 2; s <= MAX_SPLIT; ++s)
+    if (tiles * s <= (s == 2 ? p->sm_count : p->sm_count * 9 / 10) && nk / s >= 4) ka.split = s;
+  // The two rings share the memory as a CTA's main stages and LoRA stages (at most; ranks may be lower) share its work: both
+  // are bound by the bytes they have in flight.
+  const int lora = (a.n_seg * ((a.rmax + UNIT - 1) / UNIT) + 3) / 4;
+  const int lora_cta = (lora + ka.split - 1) / ka.split, main_cta = nk / ka.split;
+  const int fit = (int)(((ka.npad > 32 || lora_cta >= 8 ? SMEM_MAX : SMEM_LIMIT) - fixed) / stage);
+  const int by_work = (fit * lora_cta + (lora_cta + main_cta) / 2) / (lora_cta + main_cta);
+  ka.ne = std::max(1, std::min({FILLERS, fit - 4, by_work}));
+  ka.ns = std::min(MAX_NS, fit - ka.ne);
+  // the partial sums and the finished rows have to fit in the ring that they reuse
+  for (; ka.split > 1; --ka.split) {
+    const int share = (BN / 16 + ka.split - 1) / ka.split * 16;
+    if ((uint32_t)(ka.npad * ((ka.split - 1) * (share + 4) * 4 + share * 2 + 16)) <= ka.ns * stage) break;
   }
   *smem = fixed + (ka.ns + ka.ne) * stage;
 }
@@ -544,10 +601,10 @@ int launch(fl_pool* p, const Args& a, const void* x, const void* const* w, cudaS
   }
   static bool configured[16] = {};
   if (!configured[p->device & 15]) {
-    FL_CUDA(p, cudaFuncSetAttribute(lora_skinny_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT));
+    FL_CUDA(p, cudaFuncSetAttribute(lora_skinny_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX));
     configured[p->device & 15] = true;
   }
-  FL_CUDA(p, launch_pdl_cluster(lora_skinny_kernel, dim3(ctas), dim3((unsigned)ka.split), dim3(THREADS), smem, st, ka, maps));
+  FL_CUDA(p, launch_pdl_cluster(lora_skinny_kernel, dim3(ctas), dim3((unsigned)ka.split), dim3((unsigned)(96 + 128 * ka.ne)), smem, st, ka, maps));
   FL_CUDA(p, cudaGetLastError());
   return FL_OK;
 }

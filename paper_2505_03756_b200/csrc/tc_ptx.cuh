@@ -6,7 +6,7 @@
 
 namespace tc {
 
-constexpr uint32_t WAIT_LIMIT = 1u << 22;   // polls of one bounded mbarrier wait
+constexpr uint32_t WAIT_LIMIT = 1u << 20;   // polls of one bounded mbarrier wait
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
