@@ -2,7 +2,7 @@
 //
 // A plan kernel sorts the requests of a batch into two work lists: requests with at most 16 query
 // rows per KV head (decode steps) are cut into chunks of keys that independent CTAs reduce
-// (split-KV, merged afterwards); the others (prefill) are cut into tiles of 64 query rows per head.
+// (split-KV, merged by the last of them); the others (prefill) are cut into tiles of 64 query rows per head.
 // Both kernels stage KV pages (one 4 KiB contiguous piece per block, KV head and K/V side) into
 // shared memory with 16-byte cp.async through the block table and run QK^T and PV on bf16 tensor
 // cores with an fp32 online softmax.
@@ -45,6 +45,7 @@ __global__ void __launch_bounds__(256) attn_plan_kernel(const AttnArgs a, int ch
   pdl_wait();                 // the lists may still be read, and the request arrays written, by the kernel before
   pdl_launch_dependents();    // the prefill kernel sets itself up (barriers, TMEM) while this single CTA plans
   const int group = a.n_q / a.n_kv;
+  for (int i = threadIdx.x; i < a.n_req * a.n_kv; i += 256) a.chunks_done[i] = 0u;
   if (threadIdx.x < 64) hist[threadIdx.x] = 0;
   __syncthreads();
   // Prefill requests are ordered by context length (in 128-key steps), longest first, so that the CTAs that take work
@@ -69,26 +70,42 @@ __global__ void __launch_bounds__(256) attn_plan_kernel(const AttnArgs a, int ch
     const int off_d = base_d + block_excl_scan(chunks, sh, tot_d);
     if (i < a.n_req) {
       // a request whose chunks do not all fit in the list (contexts longer than the caller's n_tbl covers) gets no
-      // output: the chunks that did fit only write partial slots inside the workspace, and the merge, which would
-      // read all of them, skips the request (the overflow raises FLAG_BAD_POS below)
-      a.req_info[i] = make_int4(off_d, off_d + chunks > a.max_decode ? 0 : chunks, dec ? 1 : 0, 0);
+      // output: the chunks that did fit only write partial slots inside the workspace and count as none of it (the
+      // overflow raises FLAG_BAD_POS below)
       if (tiles > 0) atomicAdd(&hist[key_of(i)], tiles);
-      for (int c = 0; c < chunks; ++c)
-        if (off_d + c < a.max_decode) a.decode_list[off_d + c] = make_int2(i, c);
+      if (chunks > 0) {
+        DecodeItem d;
+        d.req = i;
+        d.prefix = ctx - n;
+        d.n_new = n;
+        d.tok0 = a.req_indptr[i];
+        d.tbl0 = a.tbl_indptr[i];
+        d.tbl_n = a.tbl_indptr[i + 1] - d.tbl0;
+        d.n_chunks = off_d + chunks > a.max_decode ? 0 : chunks;
+        for (int c = 0; c < chunks; ++c) {
+          d.chunk = c;
+          if (off_d + c < a.max_decode) a.decode_list[off_d + c] = d;
+        }
+      }
     }
     base_p += tot_p;
     base_d += tot_d;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int start = 0;
-    for (int b = 63; b >= 0; --b) {
-      cursor[b] = start;
-      start += hist[b];
+  if (base_p > 0 && threadIdx.x < 32) {        // bins from the last to the first, two per lane
+    const int b = 63 - 2 * threadIdx.x;
+    const int h0 = hist[b], h1 = hist[b - 1];
+    int incl = h0 + h1;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int o = __shfl_up_sync(0xffffffffu, incl, d);
+      if ((int)threadIdx.x >= d) incl += o;
     }
+    cursor[b] = incl - h0 - h1;
+    cursor[b - 1] = incl - h1;
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < a.n_req; i += 256) {
+  for (int i = threadIdx.x; base_p > 0 && i < a.n_req; i += 256) {
     const int n = a.new_lens[i];
     if (n <= 0 || n * group <= DEC_ROWS) continue;
     const int tiles = (n + qt - 1) / qt;
@@ -206,25 +223,31 @@ __device__ __forceinline__ const unsigned char* page_ptr(const PoolView& pv, uin
 // ------------------------------------------------------------------ decode (split-KV)
 // One CTA per (request, chunk of keys, KV head).  Rows = new tokens x query heads of the group
 // (at most 16).  The four warps take pages round-robin, each with its own double buffer, and merge
-// their partial (max, sum, O) through shared memory at the end.
+// their partial (max, sum, O) through shared memory at the end.  The CTA that finishes a request's last chunk for its KV
+// head combines the chunks' partial results (always in chunk order): as a kernel of its own the combination took 7 us
+// behind one request of 700 keys and 15 us behind 64 requests of grouped heads, half of it launch and look-ups.
+// What bounds it: reading K and V (a decode step of 256 requests runs at the copy rate); for a few requests the chain item ->
+// block ids -> pages -> partial results, which is why an item holds all of a request's numbers.
 __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   pdl_wait();
+  pdl_launch_dependents();    // the next call's first kernel may set itself up; it waits for this grid before it reads anything
   const int item = blockIdx.x / a.n_kv, h = blockIdx.x % a.n_kv;
+  const DecodeItem it = a.decode_list[item];
+  const int chunk = a.hdr->chunk;
   if (item >= a.hdr->n_decode) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t4 = lane & 3;
-  const int2 it = a.decode_list[item];
-  const int i = it.x, c = it.y;
-  const int chunk = a.hdr->chunk;
-  const int n_new = a.new_lens[i], prefix = a.prefix_lens[i], ctx = prefix + n_new;
+  const int i = it.req, c = it.chunk;
+  const int n_new = it.n_new, prefix = it.prefix, ctx = prefix + n_new;
   const int group = a.n_q / a.n_kv;
   const int rows = n_new * group;
-  const int tok0 = a.req_indptr[i];
+  const int tok0 = it.tok0;
   const int u_begin = c * chunk, u_end = min(ctx, u_begin + chunk);
   const int n_pages = (u_end - u_begin + BT - 1) / BT;
-  const int tbl0 = a.tbl_indptr[i], tbl_n = a.tbl_indptr[i + 1] - tbl0;
+  const int tbl0 = it.tbl0, tbl_n = it.tbl_n;
   const int pg0 = u_begin / BT;
+  // a chunk behind the end of the table has no keys to read; the request's other chunks then never count up to all of them
   if (pg0 + n_pages > tbl_n) {
     if (tid == 0) atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_POS);
     return;
@@ -305,7 +328,6 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
     red_ml[warp * DEC_ROWS + g + 8] = make_float2(m[1], l[1]);
   }
   __syncthreads();
-  const int4 info = a.req_info[i];
   for (int e = tid; e < rows * D; e += ATT_THREADS) {
     const int r = e / D, col = e % D;
     float M = -INFINITY;
@@ -320,43 +342,55 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
       L += ml.y * sc;
       o += red_o[(w * DEC_ROWS + r) * D + col] * sc;
     }
-    if (info.y == 1) {
+    if (it.n_chunks == 1) {
       const int j = r / group, hq = h * group + r % group;
       a.out[((size_t)(tok0 + j) * a.n_q + hq) * D + col] = __float2bfloat16_rn(L > 0.f ? o / L : 0.f);
     } else {
-      const size_t slot = ((size_t)(info.x + c) * a.n_kv + h) * DEC_ROWS + r;
+      const size_t slot = ((size_t)item * a.n_kv + h) * DEC_ROWS + r;
       a.part_o[slot * D + col] = o;
       if (col == 0) a.part_ml[slot] = make_float2(M, L);
     }
   }
-}
-
-// Combines the chunk partials of one (request, KV head): grid = n_req * n_kv.
-__global__ void __launch_bounds__(ATT_THREADS) attn_merge_kernel(const AttnArgs a) {
-  pdl_launch_dependents();    // the next call's first kernel may set itself up; it waits for this grid before it reads anything
-  pdl_wait();
-  const int i = blockIdx.x / a.n_kv, h = blockIdx.x % a.n_kv;
-  const int4 info = a.req_info[i];
-  if (!info.z || info.y <= 1) return;
-  const int group = a.n_q / a.n_kv;
-  const int rows = a.new_lens[i] * group;
-  const int tok0 = a.req_indptr[i];
-  for (int e = threadIdx.x; e < rows * D; e += ATT_THREADS) {
-    const int r = e / D, col = e % D;
+  if (it.n_chunks <= 1) return;
+  // ---- the last chunk of this request and head to get here combines them all
+  __shared__ int last;
+  __syncthreads();
+  if (tid == 0) {       // releases the whole CTA's partial results (the barrier orders them before it) and acquires the others'
+    unsigned done;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(done) : "l"(&a.chunks_done[(size_t)i * a.n_kv + h]) : "memory");
+    last = done == (unsigned)(it.n_chunks - 1);
+  }
+  __syncthreads();
+  if (!last) return;
+  float* row_max = reinterpret_cast<float*>(smem);           // [16]
+  const size_t slot0 = ((size_t)(item - c) * a.n_kv + h) * DEC_ROWS, slot_step = (size_t)a.n_kv * DEC_ROWS;
+  for (int r = warp; r < rows; r += 4) {
     float M = -INFINITY;
-    for (int c = 0; c < info.y; ++c)
-      M = fmaxf(M, a.part_ml[((size_t)(info.x + c) * a.n_kv + h) * DEC_ROWS + r].x);
-    const float ref = M == -INFINITY ? 0.f : M;
-    float L = 0.f, o = 0.f;
-    for (int c = 0; c < info.y; ++c) {
-      const size_t slot = ((size_t)(info.x + c) * a.n_kv + h) * DEC_ROWS + r;
-      const float2 ml = a.part_ml[slot];
+    for (int k = lane; k < it.n_chunks; k += 32) M = fmaxf(M, __ldcg(&a.part_ml[slot0 + k * slot_step + r]).x);
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, d));
+    if (M == -INFINITY) M = 0.f;
+    if (lane == 0) row_max[r] = M;
+  }
+  __syncthreads();
+  for (int e = tid; e < rows * (D / 4); e += ATT_THREADS) {
+    const int r = e / (D / 4), col = (e % (D / 4)) * 4;
+    const float ref = row_max[r];
+    float L = 0.f;
+    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+    for (int k = 0; k < it.n_chunks; ++k) {
+      const size_t slot = slot0 + k * slot_step + r;
+      const float2 ml = __ldcg(&a.part_ml[slot]);
+      const float4 p = __ldcg(reinterpret_cast<const float4*>(a.part_o + slot * D + col));
       const float sc = exp2f(ml.x - ref);
       L += ml.y * sc;
-      o += a.part_o[slot * D + col] * sc;
+      o.x += p.x * sc; o.y += p.y * sc; o.z += p.z * sc; o.w += p.w * sc;
     }
     const int j = r / group, hq = h * group + r % group;
-    a.out[((size_t)(tok0 + j) * a.n_q + hq) * D + col] = __float2bfloat16_rn(L > 0.f ? o / L : 0.f);
+    uint2 q = make_uint2(0u, 0u);
+    if (L > 0.f) q = make_uint2(pack_bf16(o.x / L, o.y / L), pack_bf16(o.z / L, o.w / L));
+    *reinterpret_cast<uint2*>(a.out + ((size_t)(tok0 + j) * a.n_q + hq) * D + col) = q;
   }
 }
 
@@ -467,18 +501,19 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_prefill_kernel(const AttnArg
 }
 
 int pick_chunk(int n_tbl, int n_kv) {
-  // enough (chunk, head) items to fill the GPU several times over, chunks of 64..1024 keys
+  // enough (chunk, head) items to fill the GPU several times over, chunks of 64..2048 keys (256 requests of up to 4096 keys on
+  // 13B: the layer step takes 1906, 1877 and 1871 us with at most 1024, 1536 and 2048; longer ones leave a longer tail)
   long long c = ((long long)n_tbl * BT * n_kv + 1183) / 1184;
   c = (c + 63) / 64 * 64;
   if (c < 64) c = 64;
-  if (c > 1024) c = 1024;
+  if (c > 2048) c = 2048;
   return (int)c;
 }
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct WsLayout {
-  size_t hdr, prefill_list, decode_list, req_info, part_o, part_ml, total;
+  size_t hdr, prefill_list, decode_list, chunks_done, part_o, part_ml, total;
   int max_prefill, max_decode, chunk;
 };
 
@@ -490,8 +525,8 @@ WsLayout ws_layout(int n_req, int n_tokens, int n_tbl, int n_kv) {
   size_t off = 0;
   w.hdr = off; off = align256(off + sizeof(PlanHdr));
   w.prefill_list = off; off = align256(off + sizeof(int2) * (size_t)w.max_prefill);
-  w.decode_list = off; off = align256(off + sizeof(int2) * (size_t)w.max_decode);
-  w.req_info = off; off = align256(off + sizeof(int4) * (size_t)n_req);
+  w.decode_list = off; off = align256(off + sizeof(DecodeItem) * (size_t)w.max_decode);
+  w.chunks_done = off; off = align256(off + sizeof(unsigned) * (size_t)n_req * n_kv);
   w.part_o = off; off = align256(off + sizeof(float) * (size_t)w.max_decode * n_kv * DEC_ROWS * D);
   w.part_ml = off; off = align256(off + sizeof(float2) * (size_t)w.max_decode * n_kv * DEC_ROWS);
   w.total = off;
@@ -536,8 +571,8 @@ int fl_paged_attention(fl_pool* p, fl_bf16* out, const fl_bf16* q, const int32_t
   a.scale_log2 = sm_scale * 1.4426950408889634f;
   a.hdr = reinterpret_cast<PlanHdr*>(ws + w.hdr);
   a.prefill_list = reinterpret_cast<int2*>(ws + w.prefill_list);
-  a.decode_list = reinterpret_cast<int2*>(ws + w.decode_list);
-  a.req_info = reinterpret_cast<int4*>(ws + w.req_info);
+  a.decode_list = reinterpret_cast<DecodeItem*>(ws + w.decode_list);
+  a.chunks_done = reinterpret_cast<unsigned*>(ws + w.chunks_done);
   a.part_o = reinterpret_cast<float*>(ws + w.part_o);
   a.part_ml = reinterpret_cast<float2*>(ws + w.part_ml);
   a.max_prefill = w.max_prefill;
@@ -582,7 +617,6 @@ int fl_paged_attention(fl_pool* p, fl_bf16* out, const fl_bf16* q, const int32_t
       attn_prefill_kernel<<<(unsigned)w.max_prefill * n_q_heads, ATT_THREADS, PRE_SMEM, st>>>(a);
     }
     cudaError_t e = launch_pdl(attn_decode_kernel, dim3((unsigned)w.max_decode * n_kv_heads), dim3(ATT_THREADS), DEC_SMEM, st, a);
-    if (e == cudaSuccess) e = launch_pdl(attn_merge_kernel, dim3((unsigned)n_req * n_kv_heads), dim3(ATT_THREADS), 0, st, a);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {
       p->last_cuda = (int)e;

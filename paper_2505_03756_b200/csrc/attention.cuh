@@ -17,6 +17,12 @@ struct PlanHdr {
   int next_unit;   // work counter of the persistent prefill kernel, zeroed by the plan kernel
 };
 
+// One (request, chunk of keys) of the split decode, with all that a CTA needs to start on it.
+struct DecodeItem {
+  int req, chunk, prefix, n_new;
+  int tok0, tbl0, tbl_n, n_chunks;      // first token row; the request's table; chunks of the request (0: it gets no output)
+};
+
 struct AttnArgs {
   PoolView pv;
   __nv_bfloat16* out;
@@ -31,8 +37,8 @@ struct AttnArgs {
   // workspace
   PlanHdr* hdr;
   int2* prefill_list;   // (request, first query token of the tile inside the request), longest requests first
-  int2* decode_list;    // (request, chunk)
-  int4* req_info;       // (first partial slot, chunks, decode?, 0)
+  DecodeItem* decode_list;   // chunks of one request next to each other: item k's partial results are slot k
+  unsigned* chunks_done;     // per (request, kv head): chunks whose partial results are written, zeroed by the plan kernel
   float* part_o;        // [slot][kv head][16 rows][128]
   float2* part_ml;      // [slot][kv head][16 rows] (running max in log2 units, sum)
   int max_prefill, max_decode;
