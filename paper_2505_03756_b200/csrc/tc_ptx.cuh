@@ -209,8 +209,8 @@ __device__ __forceinline__ void umma_s_tile_elect(uint32_t d_tmem, uint32_t q_lo
       "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%6];\n\t}"
       ::"r"(d_tmem), "r"(q_lo), "r"(k_lo), "r"(q_hi), "r"(k_hi), "r"(idesc), "r"(commit_bar) : "memory");
 }
-// O (+)= P V for one 128-key tile: P as bf16 pairs in TMEM (8 columns per k-step), V as eight 4 KiB pages, one per k-step.
-__device__ __forceinline__ void umma_pv_tile_elect(uint32_t o_tmem, uint32_t p_tmem, uint32_t v_lo, uint32_t v_hi, uint32_t idesc,
+// O (+)= P V for 64 keys: P as bf16 pairs in TMEM (8 columns per k-step), V as four 4 KiB pages, one per k-step.
+__device__ __forceinline__ void umma_pv_half_elect(uint32_t o_tmem, uint32_t p_tmem, uint32_t v_lo, uint32_t v_hi, uint32_t idesc,
                                                    uint32_t accumulate_first) {
   asm volatile(
       "{\n\t.reg .pred e, pt, p0;\n\t.reg .b64 db;\n\t.reg .b32 a, b;\n\t"
@@ -223,14 +223,6 @@ __device__ __forceinline__ void umma_pv_tile_elect(uint32_t o_tmem, uint32_t p_t
       "add.u32 a, %1, 16;\n\tadd.u32 b, %2, 512;\n\tmov.b64 db, {b, %3};\n\t"
       "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], db, %4, pt;\n\t"
       "add.u32 a, %1, 24;\n\tadd.u32 b, %2, 768;\n\tmov.b64 db, {b, %3};\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], db, %4, pt;\n\t"
-      "add.u32 a, %1, 32;\n\tadd.u32 b, %2, 1024;\n\tmov.b64 db, {b, %3};\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], db, %4, pt;\n\t"
-      "add.u32 a, %1, 40;\n\tadd.u32 b, %2, 1280;\n\tmov.b64 db, {b, %3};\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], db, %4, pt;\n\t"
-      "add.u32 a, %1, 48;\n\tadd.u32 b, %2, 1536;\n\tmov.b64 db, {b, %3};\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], db, %4, pt;\n\t"
-      "add.u32 a, %1, 56;\n\tadd.u32 b, %2, 1792;\n\tmov.b64 db, {b, %3};\n\t"
       "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a], db, %4, pt;\n\t"
       "}"
       ::"r"(o_tmem), "r"(p_tmem), "r"(v_lo), "r"(v_hi), "r"(idesc), "r"(accumulate_first) : "memory");
