@@ -66,7 +66,8 @@ struct Cfg {
 
 struct LinArgs {
   PoolView pv;
-  const float* v;              // shrink partial sums [projection][slice][token][rmax]
+  const float* v;              // shrink partial sums [projection][slice][token][rmax] ..
+  const __nv_bfloat16* v16;    // .. or, where not null, the scaled result in bf16, [projection][token][rmax]
   int ksplit, rmax;
   float scale;
   const int32_t* seg_indptr;
@@ -453,38 +454,48 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
           cp_async16(bs + (ch >> 3) * B_GROUP + (ER * slot + r) * 128 + (((ch & 7) ^ (r & 7)) << 4),
                      have ? reinterpret_cast<const unsigned char*>(at) + ch * 16 : a.pv.slab, have);
         }
-        cp_async_commit();
         // shrink results of this CTA's 128 rows at the stage's ranks
         const int u = 2 * e + (vch >> 1);
         const unsigned long long x = u < n_units ? list[u] : 0ull;
         const int lo = (int)(x >> 9 & 511), hi = (int)(x & 511), r0 = (int)(x >> 23 & 3) * UNIT + 8 * (vch & 1);
         const bool live = 8 * (vch & 1) < (int)(x >> 18 & 31);
-        float4 f[4][2];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) f[i][0] = f[i][1] = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int sp = 0; sp < a.ksplit; ++sp) {
+        if (a.v16) {
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            const int rt = crank * BM + vrow + 32 * i;
-            if (live && rt >= lo && rt < hi) {
-              const float4* src = reinterpret_cast<const float4*>(
-                  a.v + ((size_t)(t.j * a.ksplit + sp) * a.n_tokens + tok0 + rt) * RMAX + r0);
-              const float4 p = src[0], q = src[1];
-              f[i][0].x += p.x; f[i][0].y += p.y; f[i][0].z += p.z; f[i][0].w += p.w;
-              f[i][1].x += q.x; f[i][1].y += q.y; f[i][1].z += q.z; f[i][1].w += q.w;
+            const int row = vrow + 32 * i, rt = crank * BM + row;
+            const bool mine = live && rt >= lo && rt < hi;
+            cp_async16(sbase + C::OFF_EXT + row * 128 + (((4 * slot + vch) ^ (row & 7)) << 4),
+                       mine ? a.v16 + ((size_t)t.j * a.n_tokens + tok0 + rt) * RMAX + r0 : a.v16, mine);
+          }
+        } else {
+          float4 f[4][2];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) f[i][0] = f[i][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+          for (int sp = 0; sp < a.ksplit; ++sp) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const int rt = crank * BM + vrow + 32 * i;
+              if (live && rt >= lo && rt < hi) {
+                const float4* src = reinterpret_cast<const float4*>(
+                    a.v + ((size_t)(t.j * a.ksplit + sp) * a.n_tokens + tok0 + rt) * RMAX + r0);
+                const float4 p = src[0], q = src[1];
+                f[i][0].x += p.x; f[i][0].y += p.y; f[i][0].z += p.z; f[i][0].w += p.w;
+                f[i][1].x += q.x; f[i][1].y += q.y; f[i][1].z += q.z; f[i][1].w += q.w;
+              }
             }
           }
-        }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int row = vrow + 32 * i;
-          uint4 q;
-          q.x = pack_bf16(f[i][0].x * a.scale, f[i][0].y * a.scale);
-          q.y = pack_bf16(f[i][0].z * a.scale, f[i][0].w * a.scale);
-          q.z = pack_bf16(f[i][1].x * a.scale, f[i][1].y * a.scale);
-          q.w = pack_bf16(f[i][1].z * a.scale, f[i][1].w * a.scale);
-          *reinterpret_cast<uint4*>(as + row * 128 + (((4 * slot + vch) ^ (row & 7)) << 4)) = q;
+          for (int i = 0; i < 4; ++i) {
+            const int row = vrow + 32 * i;
+            uint4 q;
+            q.x = pack_bf16(f[i][0].x * a.scale, f[i][0].y * a.scale);
+            q.y = pack_bf16(f[i][0].z * a.scale, f[i][0].w * a.scale);
+            q.z = pack_bf16(f[i][1].x * a.scale, f[i][1].y * a.scale);
+            q.w = pack_bf16(f[i][1].z * a.scale, f[i][1].w * a.scale);
+            *reinterpret_cast<uint4*>(as + row * 128 + (((4 * slot + vch) ^ (row & 7)) << 4)) = q;
+          }
         }
+        cp_async_commit();
         cp_async_wait<0>();
         fence_async_smem();                              // the tensor core reads shared memory through the async proxy
         asm volatile("bar.sync %0, 128;" ::"r"(3 + slot) : "memory");
@@ -629,15 +640,16 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
     a.n_kv = kv->n_kv;
     a.bt = (int)(p->block_bytes / per_tok);
   }
-  // Columns per tile, 256 or 128: the width whose rounds over the pairs of SMs cost less.  A tile of 128 columns costs more
-  // than half of one of 256 (three quarters of the shared-memory fill for half the product).
+  // Columns per tile, 256 or 128: the width whose rounds over the pairs of SMs cost less.  A round of 128 columns takes about
+  // 16.5 us where one of 256 takes 20 (d_in 4096): both are bound by the 64 bytes per clock that an SM gets from L2, 32 KB per
+  // k-step at 256 columns and 24 KB at 128.
   int bn = 256;
   {
     auto cost = [&](int w) {
       long t = 0;
       for (int j = 0; j < n_mats; ++j) t += (long)a.m_tiles * ((a.d_out[j] + w - 1) / w);
       const long pairs = std::max(1, p->sm_count / 2);
-      return (t + pairs - 1) / pairs * (w + 48);
+      return (t + pairs - 1) / pairs * (w == 256 ? 100 : 82);
     };
     if (cost(128) < cost(256)) bn = 128;
   }
@@ -723,9 +735,16 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
       break;
     }
     if (n_seg > 0) {
-      rc = sgmv::shrink(p, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, workspace,
-                        v_bytes, stream, &info);
+      // Where segments are short (128 tokens on average) tiles need many LoRA stages, and the shrink in tiles of 16 tokens, which
+      // leaves its result final, is the better one: the others split d_in to fill the SMs, and a stage that sums fp32 slices
+      // takes 5600 cycles instead of 1500 (q, k, v of 28 one-token segments and 4 prompts on 7B, ranks 8 to 64: 149 -> 131 us; of
+      // one prompt of 1024 tokens on 34B, rank 64, the other way round 199 and 216 us).
+      const bool final = n_tokens <= 128 * n_seg;
+      rc = final ? sgmv::shrink_scaled(p, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace, v_bytes,
+                                       stream, &info)
+                 : sgmv::shrink(p, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, workspace, v_bytes, stream, &info);
       if (rc != FL_OK) break;
+      if (final) a.v16 = reinterpret_cast<const __nv_bfloat16*>(workspace);
     }
     a.ksplit = info.ksplit;
     a.rmax = info.rmax;
