@@ -1,4 +1,5 @@
-"""ctypes binding of libfastpool.so: argument marshalling only, one Python function per C call,
+"""Binding of libfastpool.so: argument marshalling only (ctypes, and csrc/native.cpp for the calls of a
+layer step), one Python function per C call,
 same names.  Device arguments are torch CUDA tensors (or raw integer addresses), host id lists are
 numpy arrays.  Every step of the path runs inside the library; there is no Python or CPU fallback:
 if the library has not been built, importing this module raises.
@@ -17,6 +18,10 @@ if not os.path.exists(LIB_PATH):
     raise ImportError(f"{LIB_PATH} is missing: build it with `python -m paper_2505_03756_b200.build` "
                       "(there is no fallback path)")
 lib = C.CDLL(LIB_PATH)
+
+import torch  # noqa: E402,F401  (its libraries are what _native links against)
+
+from . import _native  # noqa: E402  marshals the calls of a layer step: same arguments, tensors or integer addresses
 
 FL_OK, FL_EINVAL, FL_ENOMEM, FL_EBADID, FL_EBUSY, FL_ECUDA, FL_ETIMEOUT = 0, -1, -2, -3, -4, -5, -6
 _NAMES = {0: "FL_OK", -1: "FL_EINVAL", -2: "FL_ENOMEM", -3: "FL_EBADID", -4: "FL_EBUSY", -5: "FL_ECUDA",
@@ -303,9 +308,9 @@ def fl_lora_sgmv_workspace(n_tokens, n_mats=1):
 
 
 def fl_lora_sgmv(pool, y, x, mat_index, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace, stream=None):
-    _check(lib.fl_lora_sgmv(pool, _dev(y), _dev(x), mat_index, _dev(seg_indptr), _dev(lora_ids), n_seg, n_tokens,
-                            scale, _dev(workspace), workspace.numel() * workspace.element_size(), _stream(stream)),
-           "fl_lora_sgmv")
+    rc = _native.lora_sgmv(pool, y, x, mat_index, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace, stream)
+    if rc:
+        raise FlError(rc, "fl_lora_sgmv")
 
 
 FL_SGMV_STATIC_BYTES = 8 << 20
@@ -313,25 +318,23 @@ FL_SGMV_STATIC_BYTES = 8 << 20
 
 def fl_lora_sgmv_static(pool, y, x, mat_index, seg_indptr, lora_ids, n_seg, n_tokens, scale, stream=None):
     """fl_lora_sgmv on the library's built-in scratch: the caller passes no workspace and nothing is allocated."""
-    _check(lib.fl_lora_sgmv_static(pool, _dev(y), _dev(x), mat_index, _dev(seg_indptr), _dev(lora_ids), n_seg,
-                                   n_tokens, scale, _stream(stream)), "fl_lora_sgmv_static")
+    rc = _native.lora_sgmv_static(pool, y, x, mat_index, seg_indptr, lora_ids, n_seg, n_tokens, scale, stream)
+    if rc:
+        raise FlError(rc, "fl_lora_sgmv_static")
 
 
 def fl_lora_sgmv_multi(pool, ys, x, mat_indices, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace, stream=None):
-    py = (_vp * len(ys))(*[_dev(y) for y in ys])
-    mi = (C.c_int32 * len(ys))(*[int(m) for m in mat_indices])
-    _check(lib.fl_lora_sgmv_multi(pool, py, _dev(x), mi, len(ys), _dev(seg_indptr), _dev(lora_ids), n_seg, n_tokens,
-                                  scale, _dev(workspace), workspace.numel() * workspace.element_size(),
-                                  _stream(stream)), "fl_lora_sgmv_multi")
+    rc = _native.lora_sgmv_multi(pool, ys, x, mat_indices, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace, stream)
+    if rc:
+        raise FlError(rc, "fl_lora_sgmv_multi")
 
 
 def fl_lora_sgmv_qkv_append(pool, y_q, y_k, y_v, x, mat_q, mat_k, mat_v, seg_indptr, lora_ids, n_seg, n_tokens, scale,
                             req_indptr, kv_tbl_indptr, kv_tbl, prefix_lens, n_req, n_kv_heads, workspace, stream=None):
-    _check(lib.fl_lora_sgmv_qkv_append(pool, _dev(y_q), _dev(y_k), _dev(y_v), _dev(x), mat_q, mat_k, mat_v,
-                                       _dev(seg_indptr), _dev(lora_ids), n_seg, n_tokens, scale, _dev(req_indptr),
-                                       _dev(kv_tbl_indptr), _dev(kv_tbl), _dev(prefix_lens), n_req, n_kv_heads,
-                                       _dev(workspace), workspace.numel() * workspace.element_size(), _stream(stream)),
-           "fl_lora_sgmv_qkv_append")
+    rc = _native.lora_sgmv_qkv_append(pool, y_q, y_k, y_v, x, mat_q, mat_k, mat_v, seg_indptr, lora_ids, n_seg, n_tokens, scale, req_indptr,
+                                      kv_tbl_indptr, kv_tbl, prefix_lens, n_req, n_kv_heads, workspace, stream)
+    if rc:
+        raise FlError(rc, "fl_lora_sgmv_qkv_append")
 
 
 def fl_lora_linear_workspace(n_tokens, n_mats=1):
@@ -339,36 +342,33 @@ def fl_lora_linear_workspace(n_tokens, n_mats=1):
 
 
 def fl_lora_linear(pool, y, x, w, mat_index, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace, stream=None):
-    _check(lib.fl_lora_linear(pool, _dev(y), _dev(x), _dev(w), mat_index, _dev(seg_indptr), _dev(lora_ids), n_seg,
-                              n_tokens, scale, _dev(workspace), workspace.numel() * workspace.element_size(),
-                              _stream(stream)), "fl_lora_linear")
+    rc = _native.lora_linear(pool, y, x, w, mat_index, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace, stream)
+    if rc:
+        raise FlError(rc, "fl_lora_linear")
 
 
 def fl_lora_linear_multi(pool, ys, x, ws, mat_indices, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace,
                          stream=None):
-    py = (_vp * len(ys))(*[_dev(y) for y in ys])
-    pw = (_vp * len(ws))(*[_dev(w) for w in ws])
-    mi = (C.c_int32 * len(ys))(*[int(m) for m in mat_indices])
-    _check(lib.fl_lora_linear_multi(pool, py, _dev(x), pw, mi, len(ys), _dev(seg_indptr), _dev(lora_ids), n_seg,
-                                    n_tokens, scale, _dev(workspace), workspace.numel() * workspace.element_size(),
-                                    _stream(stream)), "fl_lora_linear_multi")
+    rc = _native.lora_linear_multi(pool, ys, x, ws, mat_indices, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace, stream)
+    if rc:
+        raise FlError(rc, "fl_lora_linear_multi")
 
 
 def fl_lora_linear_qkv_append(pool, y_q, x, w_q, w_k, w_v, mat_q, mat_k, mat_v, seg_indptr, lora_ids, n_seg, n_tokens,
                               scale, req_indptr, kv_tbl_indptr, kv_tbl, prefix_lens, n_req, n_kv_heads, scratch_k,
                               scratch_v, workspace, stream=None):
-    _check(lib.fl_lora_linear_qkv_append(pool, _dev(y_q), _dev(x), _dev(w_q), _dev(w_k), _dev(w_v), mat_q, mat_k, mat_v,
-                                         _dev(seg_indptr), _dev(lora_ids), n_seg, n_tokens, scale, _dev(req_indptr),
-                                         _dev(kv_tbl_indptr), _dev(kv_tbl), _dev(prefix_lens), n_req, n_kv_heads,
-                                         _dev(scratch_k), _dev(scratch_v), _dev(workspace),
-                                         workspace.numel() * workspace.element_size(), _stream(stream)),
-           "fl_lora_linear_qkv_append")
+    rc = _native.lora_linear_qkv_append(pool, y_q, x, w_q, w_k, w_v, mat_q, mat_k, mat_v, seg_indptr, lora_ids, n_seg, n_tokens, scale,
+                                        req_indptr, kv_tbl_indptr, kv_tbl, prefix_lens, n_req, n_kv_heads, scratch_k, scratch_v, workspace,
+                                        stream)
+    if rc:
+        raise FlError(rc, "fl_lora_linear_qkv_append")
 
 
 def fl_kv_append(pool, k_new, v_new, req_indptr, kv_tbl_indptr, kv_tbl, prefix_lens, n_req, n_tokens, n_kv_heads,
                  stream=None):
-    _check(lib.fl_kv_append(pool, _dev(k_new), _dev(v_new), _dev(req_indptr), _dev(kv_tbl_indptr), _dev(kv_tbl),
-                            _dev(prefix_lens), n_req, n_tokens, n_kv_heads, _stream(stream)), "fl_kv_append")
+    rc = _native.kv_append(pool, k_new, v_new, req_indptr, kv_tbl_indptr, kv_tbl, prefix_lens, n_req, n_tokens, n_kv_heads, stream)
+    if rc:
+        raise FlError(rc, "fl_kv_append")
 
 
 def fl_paged_attention_workspace(n_req, n_tokens, n_tbl, n_q_heads, n_kv_heads):
@@ -377,10 +377,10 @@ def fl_paged_attention_workspace(n_req, n_tokens, n_tbl, n_q_heads, n_kv_heads):
 
 def fl_paged_attention(pool, out, q, req_indptr, kv_tbl_indptr, kv_tbl, prefix_lens, new_lens, n_req, n_tokens, n_tbl,
                        n_q_heads, n_kv_heads, sm_scale, workspace, stream=None):
-    _check(lib.fl_paged_attention(pool, _dev(out), _dev(q), _dev(req_indptr), _dev(kv_tbl_indptr), _dev(kv_tbl),
-                                  _dev(prefix_lens), _dev(new_lens), n_req, n_tokens, n_tbl, n_q_heads, n_kv_heads,
-                                  sm_scale, _dev(workspace), workspace.numel() * workspace.element_size(),
-                                  _stream(stream)), "fl_paged_attention")
+    rc = _native.paged_attention(pool, out, q, req_indptr, kv_tbl_indptr, kv_tbl, prefix_lens, new_lens, n_req, n_tokens, n_tbl, n_q_heads,
+                                 n_kv_heads, sm_scale, workspace, stream)
+    if rc:
+        raise FlError(rc, "fl_paged_attention")
 
 
 def fl_swap_out(pool, dev_ids, host_ids, side_stream):

@@ -7,6 +7,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libfastpool.so")
+NATIVE = os.path.join(HERE, "_native.so")          # Python module: argument marshalling of the calls of a layer step
 SOURCES = ["pool.cu", "swap.cu", "sgmv.cu", "sgmv_tc.cu", "attention.cu", "attention_tc2.cu", "tmap.cu", "lora_linear.cu", "lora_skinny.cu", "swapper.cu", "tree.cu", "cache_sim.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "--use_fast_math", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", CSRC]
@@ -44,7 +45,23 @@ def build(verbose=False, force=False):
         raise RuntimeError("nvcc failed")
     if procs or not os.path.exists(LIB):
         subprocess.check_call([nvcc, "-shared", "-o", LIB] + objs + ["-lcudart"])
+    src = os.path.join(CSRC, "native.cpp")
+    if force or _stale(NATIVE, [src, os.path.join(ROOT, "include", "fastpool.h")]):
+        _build_native(src)
     return LIB
+
+
+def _build_native(src):
+    import sysconfig
+    import torch
+    tdir = os.path.dirname(torch.__file__)
+    inc = [os.path.join(ROOT, "include"), sysconfig.get_paths()["include"], os.path.join(tdir, "include"),
+           os.path.join(tdir, "include", "torch", "csrc", "api", "include"), "/usr/local/cuda/include"]
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", src, "-o", NATIVE]
+    cmd += [f for i in inc for f in ("-isystem" if "torch" in i else "-I", i)]
+    cmd += ["-L", HERE, "-l:libfastpool.so", "-L", os.path.join(tdir, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda",
+            "-Wl,-rpath,$ORIGIN", "-Wl,-rpath," + os.path.join(tdir, "lib")]
+    subprocess.check_call(cmd)
 
 
 if __name__ == "__main__":
