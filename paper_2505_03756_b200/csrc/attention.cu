@@ -17,6 +17,7 @@ using namespace attn;
 namespace {
 
 constexpr int QT = QT_MMA;
+constexpr int MAX_CHUNK = 2048;       // keys per work item of the split decode at most
 
 __device__ __forceinline__ int block_excl_scan(int val, int* sh, int& total) {
   // exclusive scan over the 256 threads of the plan CTA
@@ -39,7 +40,21 @@ __device__ __forceinline__ int block_excl_scan(int val, int* sh, int& total) {
   return wbase + incl - val;
 }
 
-__global__ void __launch_bounds__(256) attn_plan_kernel(const AttnArgs a, int chunk, int qt) {
+// What a batch with both kinds of work takes, in us, when the persistent prefill kernel has p of the SMs and the decode kernel
+// the others, and all of them behind the prefill kernel's end.  The decode kernel is bound by the copy rate from DECODE_SMS SMs
+// on; a prefill unit's step takes STEP_US, one fifth longer beside it.  (7B, 16 x 512 new tokens behind 512 and 48 decode requests
+// of about 1400 keys: 299 us one after the other, 279, 270, 264 and 351 us with 100, 82, 70 and 50 SMs for the prefill kernel;
+// 1000 prefill tokens beside 1.2 GB of decode pages: 198 us, 194, 191 and 228 us with 90, 50 and 8.)
+constexpr float STEP_US = 1.7f, KEY_US = 8e-5f, DECODE_SMS = 112.f;
+__device__ __forceinline__ float shared_time(int p, int sms, float unit_us, int n_units, float decode_us) {
+  const float pre = unit_us * (p < sms ? 1.2f : 1.f) * ((n_units + p - 1) / p);
+  const float done = pre * fminf(1.f, (sms - p) / DECODE_SMS);
+  return pre + fmaxf(0.f, decode_us - done);
+}
+
+__global__ void __launch_bounds__(256) attn_plan_kernel(const AttnArgs a, int chunk, int qt, int sms) {
+  __shared__ unsigned steps, keys;           // 128-key steps of all prefill tiles; keys of the decode requests
+  __shared__ unsigned long long best;
   __shared__ int sh[8];
   __shared__ int hist[64], cursor[64];
   pdl_wait();                 // the lists may still be read, and the request arrays written, by the kernel before
@@ -47,6 +62,7 @@ __global__ void __launch_bounds__(256) attn_plan_kernel(const AttnArgs a, int ch
   const int group = a.n_q / a.n_kv;
   for (int i = threadIdx.x; i < a.n_req * a.n_kv; i += 256) a.chunks_done[i] = 0u;
   if (threadIdx.x < 64) hist[threadIdx.x] = 0;
+  if (threadIdx.x == 0) { steps = keys = 0; best = ~0ull; }
   __syncthreads();
   // Prefill requests are ordered by context length (in 128-key steps), longest first, so that the CTAs that take work
   // from the list finish together; the tiles of one request stay next to each other (its later tiles first), so the
@@ -72,7 +88,12 @@ __global__ void __launch_bounds__(256) attn_plan_kernel(const AttnArgs a, int ch
       // a request whose chunks do not all fit in the list (contexts longer than the caller's n_tbl covers) gets no
       // output: the chunks that did fit only write partial slots inside the workspace and count as none of it (the
       // overflow raises FLAG_BAD_POS below)
-      if (tiles > 0) atomicAdd(&hist[key_of(i)], tiles);
+      if (tiles > 0) {
+        atomicAdd(&hist[key_of(i)], tiles);
+        // a tile reads the keys up to its last row; one and a half steps more are a unit's start and end
+        atomicAdd(&steps, (unsigned)((long long)tiles * (2 * (ctx - n) + n + qt + 3 * 128) / 256));
+      }
+      if (chunks > 0) atomicAdd(&keys, (unsigned)ctx);
       if (chunks > 0) {
         DecodeItem d;
         d.req = i;
@@ -120,12 +141,18 @@ __global__ void __launch_bounds__(256) attn_plan_kernel(const AttnArgs a, int ch
       if (first + t < a.max_prefill) a.prefill_list[first + t] = make_int2(i, q0);
     }
   }
+  if (base_p > 0 && base_d > 0) {        // the share that takes the least time, the largest of several
+    const int n_units = base_p * tc2_heads_per_item(a.n_q, a.n_kv);
+    for (int p = threadIdx.x + 1; p <= sms; p += 256)
+      atomicMin(&best, (unsigned long long)__float_as_uint(shared_time(p, sms, STEP_US * steps / base_p, n_units, KEY_US * keys * a.n_kv)) << 32 | (unsigned)(sms - p));
+    __syncthreads();
+  }
   if (threadIdx.x == 0) {
     if (base_p > a.max_prefill || base_d > a.max_decode) atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_POS);
     a.hdr->n_prefill = min(base_p, a.max_prefill);
     a.hdr->n_decode = min(base_d, a.max_decode);
-    a.hdr->chunk = chunk;
     a.hdr->next_unit = 0;
+    a.hdr->prefill_ctas = base_p > 0 && base_d > 0 ? sms - (int)(unsigned)best : sms;
   }
 }
 
@@ -221,6 +248,11 @@ __device__ __forceinline__ const unsigned char* page_ptr(const PoolView& pv, uin
 }
 
 // ------------------------------------------------------------------ decode (split-KV)
+template <bool PAST_L1>
+__device__ __forceinline__ uint32_t load_word(const __nv_bfloat16* p) {
+  return PAST_L1 ? __ldcg(reinterpret_cast<const uint32_t*>(p)) : *reinterpret_cast<const uint32_t*>(p);
+}
+
 // One CTA per (request, chunk of keys, KV head).  Rows = new tokens x query heads of the group
 // (at most 16).  The four warps take pages round-robin, each with its own double buffer, and merge
 // their partial (max, sum, O) through shared memory at the end.  The CTA that finishes a request's last chunk for its KV
@@ -228,14 +260,27 @@ __device__ __forceinline__ const unsigned char* page_ptr(const PoolView& pv, uin
 // behind one request of 700 keys and 15 us behind 64 requests of grouped heads, half of it launch and look-ups.
 // What bounds it: reading K and V (a decode step of 256 requests runs at the copy rate); for a few requests the chain item ->
 // block ids -> pages -> partial results, which is why an item holds all of a request's numbers.
-__global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs a) {
+// BESIDE: behind the persistent prefill kernel this one starts while that one runs.  The kernels before the prefill kernel are
+// complete then (it lets this one start after its own wait) and nothing of what it writes is read here; what they wrote is
+// read past L1.  One CTA more than the work needs waits for the prefill kernel's end, so that this grid does not end, and
+// the kernel behind it does not start, before it.
+template <bool BESIDE>
+__global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs a, int chunk) {
   extern __shared__ __align__(128) unsigned char smem[];
-  pdl_wait();
+  if (!BESIDE || blockIdx.x == gridDim.x - 1) pdl_wait();
   pdl_launch_dependents();    // the next call's first kernel may set itself up; it waits for this grid before it reads anything
   const int item = blockIdx.x / a.n_kv, h = blockIdx.x % a.n_kv;
-  const DecodeItem it = a.decode_list[item];
-  const int chunk = a.hdr->chunk;
-  if (item >= a.hdr->n_decode) return;
+  if (BESIDE && item >= a.max_decode) return;
+  DecodeItem it;
+  if (BESIDE) {
+    const int4* src = reinterpret_cast<const int4*>(a.decode_list + item);
+    const int4 lo = __ldcg(src), hi = __ldcg(src + 1);
+    it.req = lo.x; it.chunk = lo.y; it.prefix = lo.z; it.n_new = lo.w;
+    it.tok0 = hi.x; it.tbl0 = hi.y; it.tbl_n = hi.z; it.n_chunks = hi.w;
+  } else {
+    it = a.decode_list[item];
+  }
+  if (item >= (BESIDE ? __ldcg(&a.hdr->n_decode) : a.hdr->n_decode)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t4 = lane & 3;
   const int i = it.req, c = it.chunk;
@@ -252,6 +297,9 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
     if (tid == 0) atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_POS);
     return;
   }
+  // lane k holds the block of this warp's k-th page
+  static_assert(MAX_CHUNK / BT <= 4 * 32, "one page per lane");
+  const uint32_t my_blk = BESIDE && warp + 4 * lane < n_pages ? __ldcg(a.tbl + tbl0 + pg0 + warp + 4 * lane) : 0u;
   // query fragments: row r -> (new token r / group, query head h*group + r % group)
   uint32_t qf[8][4];
   int lim[2];
@@ -264,8 +312,8 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
     const __nv_bfloat16* qp = a.q + ((size_t)(tok0 + j) * a.n_q + (h * group + (ok ? r % group : 0))) * D;
 #pragma unroll
     for (int ks = 0; ks < 8; ++ks) {
-      qf[ks][hh] = ok ? *reinterpret_cast<const uint32_t*>(qp + 16 * ks + 2 * t4) : 0u;
-      qf[ks][hh + 2] = ok ? *reinterpret_cast<const uint32_t*>(qp + 16 * ks + 2 * t4 + 8) : 0u;
+      qf[ks][hh] = ok ? load_word<BESIDE>(qp + 16 * ks + 2 * t4) : 0u;
+      qf[ks][hh + 2] = ok ? load_word<BESIDE>(qp + 16 * ks + 2 * t4 + 8) : 0u;
     }
   }
   float O[16][4];
@@ -275,7 +323,7 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
 
   const uint32_t wbase = smem_u32(smem) + warp * (4 * PAGE_BYTES);   // per warp: 2 stages x (K page, V page)
   auto load_page = [&](int pg, int st) {
-    const uint32_t blk = a.tbl[tbl0 + pg0 + pg];
+    const uint32_t blk = BESIDE ? __shfl_sync(0xffffffffu, my_blk, pg >> 2) : a.tbl[tbl0 + pg0 + pg];
     bool ok;
     const unsigned char* kp = page_ptr(a.pv, blk, h, ok);
     const unsigned char* vp = kp + (size_t)a.n_kv * PAGE_BYTES;
@@ -506,7 +554,7 @@ int pick_chunk(int n_tbl, int n_kv) {
   long long c = ((long long)n_tbl * BT * n_kv + 1183) / 1184;
   c = (c + 63) / 64 * 64;
   if (c < 64) c = 64;
-  if (c > 2048) c = 2048;
+  if (c > MAX_CHUNK) c = MAX_CHUNK;
   return (int)c;
 }
 
@@ -587,7 +635,8 @@ int fl_paged_attention(fl_pool* p, fl_bf16* out, const fl_bf16* q, const int32_t
   int rc = FL_OK;
   do {
     if (!configured[p->device & 15]) {
-      if (cudaFuncSetAttribute(attn_decode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DEC_SMEM) != cudaSuccess ||
+      if (cudaFuncSetAttribute(attn_decode_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, DEC_SMEM) != cudaSuccess ||
+          cudaFuncSetAttribute(attn_decode_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, DEC_SMEM) != cudaSuccess ||
           cudaFuncSetAttribute(attn_prefill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PRE_SMEM) != cudaSuccess) {
         p->last_cuda = (int)cudaGetLastError();
         rc = FL_ECUDA;
@@ -600,11 +649,12 @@ int fl_paged_attention(fl_pool* p, fl_bf16* out, const fl_bf16* q, const int32_t
     // every kernel of the call is a programmatic dependent launch: it may start while the one before it drains
     // and waits inside for that kernel's results
     if (launch_pdl(attn_plan_kernel, dim3(1), dim3(256), 0, st, a, w.chunk,
-                   kind == 0 ? tc2_tile_tokens(n_q_heads, n_kv_heads) : QT_MMA) != cudaSuccess) {
+                   kind == 0 ? tc2_tile_tokens(n_q_heads, n_kv_heads) : QT_MMA, p->sm_count) != cudaSuccess) {
       p->last_cuda = (int)cudaGetLastError();
       rc = FL_ECUDA;
       break;
     }
+    bool beside = false;       // a prefill kernel that the decode kernel works beside
     if (kind == 0) {
       // upper bound of the plan's tile count: full tiles plus one ragged tile per prefill request, and a
       // request is a prefill only with more than DEC_ROWS / group new tokens
@@ -613,10 +663,12 @@ int fl_paged_attention(fl_pool* p, fl_bf16* out, const fl_bf16* q, const int32_t
       const int max_items = std::min(w.max_prefill, n_tokens / tc2_tile_tokens(n_q_heads, n_kv_heads) + max_req);
       rc = launch_prefill_tc2(p, a, n_tokens, max_items, st);
       if (rc != FL_OK) break;
+      beside = max_items > 0;
     } else {
       attn_prefill_kernel<<<(unsigned)w.max_prefill * n_q_heads, ATT_THREADS, PRE_SMEM, st>>>(a);
     }
-    cudaError_t e = launch_pdl(attn_decode_kernel, dim3((unsigned)w.max_decode * n_kv_heads), dim3(ATT_THREADS), DEC_SMEM, st, a);
+    cudaError_t e = launch_pdl(beside ? attn_decode_kernel<true> : attn_decode_kernel<false>, dim3((unsigned)w.max_decode * n_kv_heads + (beside ? 1u : 0u)),
+                               dim3(ATT_THREADS), DEC_SMEM, st, a, w.chunk);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {
       p->last_cuda = (int)e;

@@ -13,8 +13,9 @@ constexpr int ATT_THREADS = 128;
 constexpr int DEC_ROWS = 16;
 
 struct PlanHdr {
-  int n_prefill, n_decode, chunk;
+  int n_prefill, n_decode;
   int next_unit;   // work counter of the persistent prefill kernel, zeroed by the plan kernel
+  int prefill_ctas;   // how many CTAs of the persistent prefill kernel take part
 };
 
 // One (request, chunk of keys) of the split decode, with all that a CTA needs to start on it.
@@ -47,6 +48,7 @@ struct AttnArgs {
 
 // Launches the two-tiles-per-CTA kernel; the plan's tiles are tc2_tile_tokens(n_q, n_kv) tokens long.
 int launch_prefill_tc2(fl_pool* p, const AttnArgs& a, int n_tokens, int max_items, cudaStream_t st);
+__host__ __device__ inline int tc2_heads_per_item(int n_q, int n_kv) { return (n_q / n_kv) % 2 == 0 ? n_q / 2 : n_q; }
 inline int tc2_tile_tokens(int n_q, int n_kv) { return (n_q / n_kv) % 2 == 0 ? 128 : 256; }
 
 }  // namespace attn

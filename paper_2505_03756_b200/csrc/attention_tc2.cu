@@ -148,7 +148,9 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
   // everything above touched only this CTA's shared memory and TMEM; the plan (and q, K, V) are the work of the
   // kernels before this one
   pdl_wait();
+  pdl_launch_dependents();    // the decode kernel works beside this one, on the SMs whose CTAs have no unit (any more)
   const int n_units = a.hdr->n_prefill * heads_per_item;   // a CTA beyond the last unit finds no work and tears down
+  const int n_ctas = min((int)gridDim.x, a.hdr->prefill_ctas);
 
   // Readers take the k-th unit of this CTA from slot k & 1 (index -1 = no more work) and release the slot.
 
@@ -169,7 +171,7 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
           t.index = -1;
           t.valid = 0;
           if (k < 2 || mbar_wait(bar(C_UEMPTY + (k & 1)), ((k >> 1) - 1) & 1, abort_flag)) {
-            const int u = k == 0 ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(&a.hdr->next_unit, 1);
+            const int u = (int)blockIdx.x >= n_ctas ? n_units : k == 0 ? (int)blockIdx.x : n_ctas + atomicAdd(&a.hdr->next_unit, 1);
             if (u < n_units) t = decode_unit(a, u, heads_per_item);
           }
           unit_slot[k & 1] = t;
@@ -472,8 +474,7 @@ int launch_prefill_tc2(fl_pool* p, const AttnArgs& a, int n_tokens, int max_item
     FL_CUDA(p, cudaFuncSetAttribute(attn_prefill_tc2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T2_SMEM));
     configured[p->device & 15] = true;
   }
-  const int group = a.n_q / a.n_kv;
-  const int heads_per_item = group % 2 == 0 ? a.n_q / 2 : a.n_q;
+  const int heads_per_item = tc2_heads_per_item(a.n_q, a.n_kv);
   // one CTA per SM (shared memory and TMEM allow no more); a CTA beyond the plan's unit count finds no work and tears down
   const long long units = (long long)max_items * heads_per_item;
   const unsigned grid = (unsigned)std::min<long long>(units, p->sm_count);
