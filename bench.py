@@ -293,8 +293,8 @@ def bench_workload(args, name, world, rank, local, oracle_budget_s):
     ev_side, ev_side_in = torch.cuda.Event(), torch.cuda.Event()
     calls = (["sgmv_qkv", "kv_append"] if args.separate_append else ["sgmv_qkv_append"]) + ["attention", "sgmv_o"] + \
         (["sgmv_up", "sgmv_down"] if s.inter else [])
-    # shrink + expand per SGMV call, KV append, plan + prefill + decode + merge, swap gather + scatter
-    launches_per_step = 2 + (1 if args.separate_append else 0) + 4 + 2 + (4 if s.inter else 0) + \
+    # shrink + expand per SGMV call, KV append, plan + prefill + decode, swap gather + scatter
+    launches_per_step = 2 + (1 if args.separate_append else 0) + 3 + 2 + (4 if s.inter else 0) + \
         (2 * -(-n_swap // 256) if n_swap > 1 else 0)
 
     def compute(k, evs=None):
