@@ -248,6 +248,7 @@ __device__ __forceinline__ const unsigned char* page_ptr(const PoolView& pv, uin
 }
 
 // ------------------------------------------------------------------ decode (split-KV)
+constexpr int CL_OFF = 4 * DEC_ROWS * D * 4 + 4 * DEC_ROWS * 8;        // a CTA's own result, behind those of its four warps
 template <bool PAST_L1>
 __device__ __forceinline__ uint32_t load_word(const __nv_bfloat16* p) {
   return PAST_L1 ? __ldcg(reinterpret_cast<const uint32_t*>(p)) : *reinterpret_cast<const uint32_t*>(p);
@@ -264,15 +265,35 @@ __device__ __forceinline__ uint32_t load_word(const __nv_bfloat16* p) {
 // complete then (it lets this one start after its own wait) and nothing of what it writes is read here; what they wrote is
 // read past L1.  One CTA more than the work needs waits for the prefill kernel's end, so that this grid does not end, and
 // the kernel behind it does not start, before it.
-template <bool BESIDE>
-__global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs a, int chunk) {
+// CLUSTER: a few decode requests and nothing else.  No plan: the CTAs of a cluster share the pages of one (request, KV head) and
+// the first of them fetches the others' partial results from their shared memory.
+enum { PLAIN = 0, BESIDE = 1, CLUSTER = 2 };
+template <int MODE>
+__global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs a, int chunk, int n_tbl) {
   extern __shared__ __align__(128) unsigned char smem[];
-  if (!BESIDE || blockIdx.x == gridDim.x - 1) pdl_wait();
+  if (MODE != BESIDE || blockIdx.x == gridDim.x - 1) pdl_wait();
   pdl_launch_dependents();    // the next call's first kernel may set itself up; it waits for this grid before it reads anything
-  const int item = blockIdx.x / a.n_kv, h = blockIdx.x % a.n_kv;
-  if (BESIDE && item >= a.max_decode) return;
+  const int csize = MODE == CLUSTER ? chunk : 1;            // CTAs per cluster
+  const int item = blockIdx.x / csize / a.n_kv, h = blockIdx.x / csize % a.n_kv;
+  if (MODE == BESIDE && item >= a.max_decode) return;
   DecodeItem it;
-  if (BESIDE) {
+  if (MODE == CLUSTER) {
+    it.req = item;
+    it.chunk = blockIdx.x % csize;
+    it.n_chunks = csize;
+    it.n_new = a.new_lens[item];
+    it.prefix = a.prefix_lens[item];
+    it.tok0 = a.req_indptr[item];
+    it.tbl0 = a.tbl_indptr[item];
+    it.tbl_n = a.tbl_indptr[item + 1] - it.tbl0;
+    if (it.n_new <= 0) return;                              // (the same answer in the whole cluster)
+    const int pages = (it.prefix + it.n_new + BT - 1) / BT;
+    if (pages > it.tbl_n || it.tbl0 + it.tbl_n > n_tbl || it.n_new * (a.n_q / a.n_kv) > DEC_ROWS) {
+      if (threadIdx.x == 0) atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_POS);
+      return;
+    }
+    chunk = max(4, (pages + csize - 1) / csize) * BT;       // a page for every warp at least
+  } else if (MODE == BESIDE) {
     const int4* src = reinterpret_cast<const int4*>(a.decode_list + item);
     const int4 lo = __ldcg(src), hi = __ldcg(src + 1);
     it.req = lo.x; it.chunk = lo.y; it.prefix = lo.z; it.n_new = lo.w;
@@ -280,7 +301,7 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
   } else {
     it = a.decode_list[item];
   }
-  if (item >= (BESIDE ? __ldcg(&a.hdr->n_decode) : a.hdr->n_decode)) return;
+  if (MODE != CLUSTER && item >= (MODE == BESIDE ? __ldcg(&a.hdr->n_decode) : a.hdr->n_decode)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t4 = lane & 3;
   const int i = it.req, c = it.chunk;
@@ -289,17 +310,17 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
   const int rows = n_new * group;
   const int tok0 = it.tok0;
   const int u_begin = c * chunk, u_end = min(ctx, u_begin + chunk);
-  const int n_pages = (u_end - u_begin + BT - 1) / BT;
+  const int n_pages = max(0, (u_end - u_begin + BT - 1) / BT);       // (none for the last CTAs of a cluster with few pages)
   const int tbl0 = it.tbl0, tbl_n = it.tbl_n;
   const int pg0 = u_begin / BT;
   // a chunk behind the end of the table has no keys to read; the request's other chunks then never count up to all of them
-  if (pg0 + n_pages > tbl_n) {
+  if (MODE != CLUSTER && pg0 + n_pages > tbl_n) {
     if (tid == 0) atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_POS);
     return;
   }
   // lane k holds the block of this warp's k-th page
   static_assert(MAX_CHUNK / BT <= 4 * 32, "one page per lane");
-  const uint32_t my_blk = BESIDE && warp + 4 * lane < n_pages ? __ldcg(a.tbl + tbl0 + pg0 + warp + 4 * lane) : 0u;
+  const uint32_t my_blk = MODE == BESIDE && warp + 4 * lane < n_pages ? __ldcg(a.tbl + tbl0 + pg0 + warp + 4 * lane) : 0u;
   // query fragments: row r -> (new token r / group, query head h*group + r % group)
   uint32_t qf[8][4];
   int lim[2];
@@ -312,8 +333,8 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
     const __nv_bfloat16* qp = a.q + ((size_t)(tok0 + j) * a.n_q + (h * group + (ok ? r % group : 0))) * D;
 #pragma unroll
     for (int ks = 0; ks < 8; ++ks) {
-      qf[ks][hh] = ok ? load_word<BESIDE>(qp + 16 * ks + 2 * t4) : 0u;
-      qf[ks][hh + 2] = ok ? load_word<BESIDE>(qp + 16 * ks + 2 * t4 + 8) : 0u;
+      qf[ks][hh] = ok ? load_word<MODE == BESIDE>(qp + 16 * ks + 2 * t4) : 0u;
+      qf[ks][hh + 2] = ok ? load_word<MODE == BESIDE>(qp + 16 * ks + 2 * t4 + 8) : 0u;
     }
   }
   float O[16][4];
@@ -323,7 +344,7 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
 
   const uint32_t wbase = smem_u32(smem) + warp * (4 * PAGE_BYTES);   // per warp: 2 stages x (K page, V page)
   auto load_page = [&](int pg, int st) {
-    const uint32_t blk = BESIDE ? __shfl_sync(0xffffffffu, my_blk, pg >> 2) : a.tbl[tbl0 + pg0 + pg];
+    const uint32_t blk = MODE == BESIDE ? __shfl_sync(0xffffffffu, my_blk, pg >> 2) : a.tbl[tbl0 + pg0 + pg];
     bool ok;
     const unsigned char* kp = page_ptr(a.pv, blk, h, ok);
     const unsigned char* vp = kp + (size_t)a.n_kv * PAGE_BYTES;
@@ -390,7 +411,11 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
       L += ml.y * sc;
       o += red_o[(w * DEC_ROWS + r) * D + col] * sc;
     }
-    if (it.n_chunks == 1) {
+    if (MODE == CLUSTER && csize > 1) {
+      float* const mine = reinterpret_cast<float*>(smem + CL_OFF);
+      mine[e] = o;
+      if (col == 0) reinterpret_cast<float2*>(smem + CL_OFF + DEC_ROWS * D * 4)[r] = make_float2(M, L);
+    } else if (it.n_chunks == 1) {
       const int j = r / group, hq = h * group + r % group;
       a.out[((size_t)(tok0 + j) * a.n_q + hq) * D + col] = __float2bfloat16_rn(L > 0.f ? o / L : 0.f);
     } else {
@@ -400,6 +425,42 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
     }
   }
   if (it.n_chunks <= 1) return;
+  if (MODE == CLUSTER) {
+    __syncwarp();
+    cluster_sync();
+    if (c == 0)
+      for (int e = tid; e < rows * (D / 4); e += ATT_THREADS) {
+        const int r = e / (D / 4);
+        const uint32_t po = smem_u32(smem) + CL_OFF + e * 16, pm = smem_u32(smem) + CL_OFF + DEC_ROWS * D * 4 + r * 8;
+        float4 p[8];
+        float2 ml[8];
+        float ref = -INFINITY;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          if (k < csize) {
+            p[k] = ld_cluster_f32x4(map_cluster_rank(po, k));
+            ml[k] = ld_cluster_f32x2(map_cluster_rank(pm, k));
+            ref = fmaxf(ref, ml[k].x);
+          }
+        if (ref == -INFINITY) ref = 0.f;
+        float L = 0.f;
+        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          if (k < csize) {
+            const float sc = exp2f(ml[k].x - ref);
+            L += ml[k].y * sc;
+            o.x += p[k].x * sc; o.y += p[k].y * sc; o.z += p[k].z * sc; o.w += p[k].w * sc;
+          }
+        const int j = r / group, hq = h * group + r % group;
+        uint2 q = make_uint2(0u, 0u);
+        if (L > 0.f) q = make_uint2(pack_bf16(o.x / L, o.y / L), pack_bf16(o.z / L, o.w / L));
+        *reinterpret_cast<uint2*>(a.out + ((size_t)(tok0 + j) * a.n_q + hq) * D + (e % (D / 4)) * 4) = q;
+      }
+    __syncwarp();
+    cluster_sync();              // nobody leaves while its results are still being read
+    return;
+  }
   // ---- the last chunk of this request and head to get here combines them all
   __shared__ int last;
   __syncthreads();
@@ -558,6 +619,20 @@ int pick_chunk(int n_tbl, int n_kv) {
   return (int)c;
 }
 
+// CTAs that share the pages of a (request, KV head) where a few decode requests are served without a plan, 0 = with one.  Without it
+// the contexts' lengths are not known when the grid is chosen: enough CTAs that a warp has no more than 40 pages (30 us) even if one
+// request had them all, more where SMs are idle and a CTA keeps eight pages, and a plan where that needs more than 600 CTAs.
+// KV append and attention of a 7B layer, with the plan and without: 1 request of 134 keys 12.5 and 9.4 us, of 3000 28.8 and
+// 19.8; 3 of 140 14.6 and 10.5; 8 of 550 34.3 and 27.9; 16 of 130 32.5 and 20.2; but 8 of 1500 50 and 61, 9 of 1200 (13B) 55 and 77 us.
+int cluster_size(int n_req, int n_tbl, int n_kv, int sms) {
+  const long long units = (long long)n_req * n_kv;
+  int cs = 1;
+  while (cs <= 8 && n_tbl > 160 * cs) cs *= 2;
+  if (cs > 8 || units * cs > 600) return 0;
+  while (cs < 8 && units * cs * 2 <= 2 * sms && n_tbl >= 16ll * cs * n_req) cs *= 2;
+  return cs;
+}
+
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct WsLayout {
@@ -635,8 +710,9 @@ int fl_paged_attention(fl_pool* p, fl_bf16* out, const fl_bf16* q, const int32_t
   int rc = FL_OK;
   do {
     if (!configured[p->device & 15]) {
-      if (cudaFuncSetAttribute(attn_decode_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, DEC_SMEM) != cudaSuccess ||
-          cudaFuncSetAttribute(attn_decode_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, DEC_SMEM) != cudaSuccess ||
+      if (cudaFuncSetAttribute(attn_decode_kernel<PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, DEC_SMEM) != cudaSuccess ||
+          cudaFuncSetAttribute(attn_decode_kernel<BESIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, DEC_SMEM) != cudaSuccess ||
+          cudaFuncSetAttribute(attn_decode_kernel<CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize, DEC_SMEM) != cudaSuccess ||
           cudaFuncSetAttribute(attn_prefill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PRE_SMEM) != cudaSuccess) {
         p->last_cuda = (int)cudaGetLastError();
         rc = FL_ECUDA;
@@ -646,6 +722,21 @@ int fl_paged_attention(fl_pool* p, fl_bf16* out, const fl_bf16* q, const int32_t
     }
     // the tensor-core kernels fold sm_scale into the exponent and take row maxima of raw scores: they need sm_scale > 0
     const int kind = sm_scale > 0.f ? p->prefill_kernel : 1;
+    // upper bound of the plan's tile count: full tiles plus one ragged tile per prefill request, and a
+    // request is a prefill only with more than DEC_ROWS / group new tokens
+    const int group = n_q_heads / n_kv_heads;
+    const int max_req = std::min(n_req, n_tokens / (DEC_ROWS / group + 1));
+    const int max_items = std::min(w.max_prefill, n_tokens / tc2_tile_tokens(n_q_heads, n_kv_heads) + max_req);
+    const int csize = kind == 0 && max_items == 0 ? cluster_size(n_req, n_tbl, n_kv_heads, p->sm_count) : 0;
+    if (csize > 0) {
+      const cudaError_t e = launch_pdl_cluster(attn_decode_kernel<CLUSTER>, dim3((unsigned)(n_req * n_kv_heads * csize)), dim3((unsigned)csize),
+                                               dim3(ATT_THREADS), DEC_SMEM, st, a, csize, n_tbl);
+      if (e != cudaSuccess) {
+        p->last_cuda = (int)e;
+        rc = FL_ECUDA;
+      }
+      break;
+    }
     // every kernel of the call is a programmatic dependent launch: it may start while the one before it drains
     // and waits inside for that kernel's results
     if (launch_pdl(attn_plan_kernel, dim3(1), dim3(256), 0, st, a, w.chunk,
@@ -656,19 +747,14 @@ int fl_paged_attention(fl_pool* p, fl_bf16* out, const fl_bf16* q, const int32_t
     }
     bool beside = false;       // a prefill kernel that the decode kernel works beside
     if (kind == 0) {
-      // upper bound of the plan's tile count: full tiles plus one ragged tile per prefill request, and a
-      // request is a prefill only with more than DEC_ROWS / group new tokens
-      const int group = n_q_heads / n_kv_heads;
-      const int max_req = std::min(n_req, n_tokens / (DEC_ROWS / group + 1));
-      const int max_items = std::min(w.max_prefill, n_tokens / tc2_tile_tokens(n_q_heads, n_kv_heads) + max_req);
       rc = launch_prefill_tc2(p, a, n_tokens, max_items, st);
       if (rc != FL_OK) break;
       beside = max_items > 0;
     } else {
       attn_prefill_kernel<<<(unsigned)w.max_prefill * n_q_heads, ATT_THREADS, PRE_SMEM, st>>>(a);
     }
-    cudaError_t e = launch_pdl(beside ? attn_decode_kernel<true> : attn_decode_kernel<false>, dim3((unsigned)w.max_decode * n_kv_heads + (beside ? 1u : 0u)),
-                               dim3(ATT_THREADS), DEC_SMEM, st, a, w.chunk);
+    cudaError_t e = launch_pdl(beside ? attn_decode_kernel<BESIDE> : attn_decode_kernel<PLAIN>, dim3((unsigned)w.max_decode * n_kv_heads + (beside ? 1u : 0u)),
+                               dim3(ATT_THREADS), DEC_SMEM, st, a, w.chunk, n_tbl);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {
       p->last_cuda = (int)e;
