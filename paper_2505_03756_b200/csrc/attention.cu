@@ -267,6 +267,7 @@ __device__ __forceinline__ uint32_t load_word(const __nv_bfloat16* p) {
 // the kernel behind it does not start, before it.
 // CLUSTER: a few decode requests and nothing else.  No plan: the CTAs of a cluster share the pages of one (request, KV head) and
 // the first of them fetches the others' partial results from their shared memory.
+constexpr int MAX_FEW_ROWS = 64;      // query rows per KV head, in all, of a batch served without a plan
 enum { PLAIN = 0, BESIDE = 1, CLUSTER = 2 };
 template <int MODE>
 __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs a, int chunk, int n_tbl) {
@@ -286,9 +287,9 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
     it.tok0 = a.req_indptr[item];
     it.tbl0 = a.tbl_indptr[item];
     it.tbl_n = a.tbl_indptr[item + 1] - it.tbl0;
-    if (it.n_new <= 0) return;                              // (the same answer in the whole cluster)
+    if (it.n_new * (a.n_q / a.n_kv) <= (int)blockIdx.y * DEC_ROWS) return;       // (the same answer in the whole cluster)
     const int pages = (it.prefix + it.n_new + BT - 1) / BT;
-    if (pages > it.tbl_n || it.tbl0 + it.tbl_n > n_tbl || it.n_new * (a.n_q / a.n_kv) > DEC_ROWS) {
+    if (pages > it.tbl_n || it.tbl0 + it.tbl_n > n_tbl || it.n_new * (a.n_q / a.n_kv) > MAX_FEW_ROWS) {
       if (threadIdx.x == 0) atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_POS);
       return;
     }
@@ -307,7 +308,9 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
   const int i = it.req, c = it.chunk;
   const int n_new = it.n_new, prefix = it.prefix, ctx = prefix + n_new;
   const int group = a.n_q / a.n_kv;
-  const int rows = n_new * group;
+  // a plan's items have at most 16 rows; where there is none, clusters further back in the grid take a request's rows from 16 on
+  const int r0 = MODE == CLUSTER ? (int)blockIdx.y * DEC_ROWS : 0;
+  const int rows = min(DEC_ROWS, n_new * group - r0);
   const int tok0 = it.tok0;
   const int u_begin = c * chunk, u_end = min(ctx, u_begin + chunk);
   const int n_pages = max(0, (u_end - u_begin + BT - 1) / BT);       // (none for the last CTAs of a cluster with few pages)
@@ -321,16 +324,16 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
   // lane k holds the block of this warp's k-th page
   static_assert(MAX_CHUNK / BT <= 4 * 32, "one page per lane");
   const uint32_t my_blk = MODE == BESIDE && warp + 4 * lane < n_pages ? __ldcg(a.tbl + tbl0 + pg0 + warp + 4 * lane) : 0u;
-  // query fragments: row r -> (new token r / group, query head h*group + r % group)
+  // query fragments: row r -> (new token (r0 + r) / group, query head h*group + (r0 + r) % group)
   uint32_t qf[8][4];
   int lim[2];
 #pragma unroll
   for (int hh = 0; hh < 2; ++hh) {
     const int r = g + 8 * hh;
     const bool ok = r < rows;
-    const int j = ok ? r / group : 0;
+    const int j = ok ? (r0 + r) / group : 0;
     lim[hh] = ok ? prefix + j : -1;
-    const __nv_bfloat16* qp = a.q + ((size_t)(tok0 + j) * a.n_q + (h * group + (ok ? r % group : 0))) * D;
+    const __nv_bfloat16* qp = a.q + ((size_t)(tok0 + j) * a.n_q + (h * group + (ok ? (r0 + r) % group : 0))) * D;
 #pragma unroll
     for (int ks = 0; ks < 8; ++ks) {
       qf[ks][hh] = ok ? load_word<MODE == BESIDE>(qp + 16 * ks + 2 * t4) : 0u;
@@ -416,7 +419,7 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
       mine[e] = o;
       if (col == 0) reinterpret_cast<float2*>(smem + CL_OFF + DEC_ROWS * D * 4)[r] = make_float2(M, L);
     } else if (it.n_chunks == 1) {
-      const int j = r / group, hq = h * group + r % group;
+      const int j = (r0 + r) / group, hq = h * group + (r0 + r) % group;
       a.out[((size_t)(tok0 + j) * a.n_q + hq) * D + col] = __float2bfloat16_rn(L > 0.f ? o / L : 0.f);
     } else {
       const size_t slot = ((size_t)item * a.n_kv + h) * DEC_ROWS + r;
@@ -452,7 +455,7 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
             L += ml[k].y * sc;
             o.x += p[k].x * sc; o.y += p[k].y * sc; o.z += p[k].z * sc; o.w += p[k].w * sc;
           }
-        const int j = r / group, hq = h * group + r % group;
+        const int j = (r0 + r) / group, hq = h * group + (r0 + r) % group;
         uint2 q = make_uint2(0u, 0u);
         if (L > 0.f) q = make_uint2(pack_bf16(o.x / L, o.y / L), pack_bf16(o.z / L, o.w / L));
         *reinterpret_cast<uint2*>(a.out + ((size_t)(tok0 + j) * a.n_q + hq) * D + (e % (D / 4)) * 4) = q;
@@ -496,7 +499,7 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
       L += ml.y * sc;
       o.x += p.x * sc; o.y += p.y * sc; o.z += p.z * sc; o.w += p.w * sc;
     }
-    const int j = r / group, hq = h * group + r % group;
+    const int j = (r0 + r) / group, hq = h * group + (r0 + r) % group;
     uint2 q = make_uint2(0u, 0u);
     if (L > 0.f) q = make_uint2(pack_bf16(o.x / L, o.y / L), pack_bf16(o.z / L, o.w / L));
     *reinterpret_cast<uint2*>(a.out + ((size_t)(tok0 + j) * a.n_q + hq) * D + col) = q;
@@ -620,15 +623,17 @@ int pick_chunk(int n_tbl, int n_kv) {
 }
 
 // CTAs that share the pages of a (request, KV head) where a few decode requests are served without a plan, 0 = with one.  Without it
-// the contexts' lengths are not known when the grid is chosen: enough CTAs that a warp has no more than 40 pages (30 us) even if one
-// request had them all, more where SMs are idle and a CTA keeps eight pages, and a plan where that needs more than 600 CTAs.
-// KV append and attention of a 7B layer, with the plan and without: 1 request of 134 keys 12.5 and 9.4 us, of 3000 28.8 and
-// 19.8; 3 of 140 14.6 and 10.5; 8 of 550 34.3 and 27.9; 16 of 130 32.5 and 20.2; but 8 of 1500 50 and 61, 9 of 1200 (13B) 55 and 77 us.
+// the contexts' lengths are not known when the grid is chosen: enough CTAs that a warp has no more than about 40 pages (30 us) even
+// if one request had them all, more where SMs are idle and a CTA keeps eight pages, and a plan where that needs more than 600 CTAs.
+// KV append and attention of a layer, with the plan and without.  7B: 1 request of 134 keys 12.5 and 9.4 us, of 3000 28.8 and 19.8;
+// 3 of 140 14.6 and 10.5; 8 of 550 34.3 and 27.9; 16 of 130 32.5 and 20.2; 26 of 95 29.6 and 22.8; 40 of 60 29.2 and 26.5; but 8 of
+// 1500 50 and 61.  34B: 3 of 2000 40.3 and 17.2, 8 of 550 21.3 and 12.2 us.  13B: 30 of 95 34.5 and 28.2; but 9 of 1200 55 and 77 us.
 int cluster_size(int n_req, int n_tbl, int n_kv, int sms) {
   const long long units = (long long)n_req * n_kv;
+  const int worst = 160 + 4 * n_req;
   int cs = 1;
-  while (cs <= 8 && n_tbl > 160 * cs) cs *= 2;
-  if (cs > 8 || units * cs > 600) return 0;
+  while (cs <= 8 && n_tbl > worst * cs) cs *= 2;
+  if (cs > 8 || (cs > 1 && units * cs > 600)) return 0;
   while (cs < 8 && units * cs * 2 <= 2 * sms && n_tbl >= 16ll * cs * n_req) cs *= 2;
   return cs;
 }
@@ -727,9 +732,13 @@ int fl_paged_attention(fl_pool* p, fl_bf16* out, const fl_bf16* q, const int32_t
     const int group = n_q_heads / n_kv_heads;
     const int max_req = std::min(n_req, n_tokens / (DEC_ROWS / group + 1));
     const int max_items = std::min(w.max_prefill, n_tokens / tc2_tile_tokens(n_q_heads, n_kv_heads) + max_req);
-    const int csize = kind == 0 && max_items == 0 ? cluster_size(n_req, n_tbl, n_kv_heads, p->sm_count) : 0;
+    // No prefill request is possible, or decode steps are meant (a request with more than 16 rows, next to some without any, takes
+    // several clusters; in the grid they cost the 64 requests of 40 keys of a 7B layer what the plan does: 37 against 36 us).
+    const int passes = max_items == 0 ? 1 : (n_tokens * group + DEC_ROWS - 1) / DEC_ROWS;
+    const bool few = max_items == 0 || (n_tokens <= n_req && n_tokens * group <= MAX_FEW_ROWS && (long long)n_req * n_kv_heads * passes <= 6000);
+    const int csize = kind == 0 && few ? cluster_size(n_req, n_tbl, n_kv_heads, p->sm_count) : 0;
     if (csize > 0) {
-      const cudaError_t e = launch_pdl_cluster(attn_decode_kernel<CLUSTER>, dim3((unsigned)(n_req * n_kv_heads * csize)), dim3((unsigned)csize),
+      const cudaError_t e = launch_pdl_cluster(attn_decode_kernel<CLUSTER>, dim3((unsigned)(n_req * n_kv_heads * csize), (unsigned)passes), dim3((unsigned)csize),
                                                dim3(ATT_THREADS), DEC_SMEM, st, a, csize, n_tbl);
       if (e != cudaSuccess) {
         p->last_cuda = (int)e;

@@ -18,7 +18,8 @@ from _util import assert_close, oracle_context
 @pytest.mark.parametrize("heads,prefix,new", [
     ((4, 4), [0], [1]), ((4, 4), [15], [1]), ((4, 4), [16, 600], [1, 0]), ((2, 2), [63, 64, 65], [1, 1, 1]), ((4, 4), [40, 0], [9, 7]),
     ((8, 8), [2600], [1]), ((8, 2), [1000, 17], [1, 3]), ((8, 1), [130, 131], [1, 1]), ((16, 16), [100 + 7 * i for i in range(16)], [1] * 16),
-    ((1, 1), [511, 0, 5], [3, 12, 1])])
+    ((1, 1), [511, 0, 5], [3, 12, 1]), ((4, 4), [5 * i for i in range(40)], [1] * 40), ((8, 1), [700, 3, 0, 90, 16], [1, 1, 1, 2, 0]),
+    ((2, 2), [30, 9] + [7] * 30, [25, 6] + [0] * 30), ((16, 2), [2000, 31, 600], [1, 1, 1])])
 def test_few_decode_requests(heads, prefix, new):
     from paper_2505_03756_b200 import harness as H
     wl = synth.make_workload("tiny", n_req=len(new), len_range=(0, 0), n_adapters=1, shape=synth.LayerShape(heads[0] * 128, *heads))
