@@ -101,11 +101,19 @@ struct Ptrs {
 };
 struct Ints {
   int p[FL_MAX_MATS] = {};
+  Py_ssize_t n;
   explicit Ints(PyObject* o) {
     Items v(o);
-    for (Py_ssize_t i = 0; i < v.n && i < FL_MAX_MATS; ++i) p[i] = integer(v[i]);
+    n = v.n;
+    for (Py_ssize_t i = 0; i < n && i < FL_MAX_MATS; ++i) p[i] = integer(v[i]);
   }
 };
+// The library takes one count for all of them: an entry too few would be read as null or as projection 0.
+void same_length(Py_ssize_t ys, Py_ssize_t others) {
+  if (ys == others) return;
+  PyErr_Format(PyExc_ValueError, "%zd outputs, but %zd entries in a list that goes with them", ys, others);
+  throw Bad();
+}
 
 template <typename F>
 PyObject* guarded(Py_ssize_t n, Py_ssize_t want, F f) {
@@ -147,6 +155,7 @@ CALL(lora_sgmv_multi) {
   return guarded(n, 11, [&] {
     const Ptrs ys(a[1]);
     const Ints mats(a[3]);
+    same_length(ys.n, mats.n);
     size_t wb = 0;
     void* ws = address(a[9], &wb);
     return fl_lora_sgmv_multi(handle<fl_pool>(a[0]), ys.p, bf16(a[2]), mats.p, (int)ys.n, i32(a[4]), i32(a[5]), integer(a[6]), integer(a[7]),
@@ -178,6 +187,8 @@ CALL(lora_linear_multi) {
   return guarded(n, 12, [&] {
     const Ptrs ys(a[1]), w(a[3]);
     const Ints mats(a[4]);
+    same_length(ys.n, w.n);
+    same_length(ys.n, mats.n);
     size_t wb = 0;
     void* ws = address(a[10], &wb);
     return fl_lora_linear_multi(handle<fl_pool>(a[0]), ys.p, bf16(a[2]), w.p, mats.p, (int)ys.n, i32(a[5]), i32(a[6]), integer(a[7]),
