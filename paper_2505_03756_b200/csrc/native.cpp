@@ -115,6 +115,18 @@ void same_length(Py_ssize_t ys, Py_ssize_t others) {
   throw Bad();
 }
 
+// Runs a library call, whose arguments have been read, without the interpreter's lock, as ctypes does: a launch may block (a full
+// launch queue, a module that is loaded on its first use), and other threads go on meanwhile.
+struct Unlocked {
+  PyThreadState* state = PyEval_SaveThread();
+  ~Unlocked() { PyEval_RestoreThread(state); }
+};
+template <typename F, typename... A>
+int unlocked(F* call, A... args) {
+  Unlocked u;
+  return call(args...);
+}
+
 template <typename F>
 PyObject* guarded(Py_ssize_t n, Py_ssize_t want, F f) {
   if (n != want) {
@@ -139,14 +151,14 @@ CALL(lora_sgmv) {
   return guarded(n, 11, [&] {
     size_t wb = 0;
     void* ws = address(a[9], &wb);
-    return fl_lora_sgmv(handle<fl_pool>(a[0]), bf16_out(a[1]), bf16(a[2]), integer(a[3]), i32(a[4]), i32(a[5]), integer(a[6]), integer(a[7]),
+    return unlocked(fl_lora_sgmv, handle<fl_pool>(a[0]), bf16_out(a[1]), bf16(a[2]), integer(a[3]), i32(a[4]), i32(a[5]), integer(a[6]), integer(a[7]),
                         real(a[8]), ws, wb, stream(a[10]));
   });
 }
 // pool, y, x, mat_index, seg_indptr, lora_ids, n_seg, n_tokens, scale, stream
 CALL(lora_sgmv_static) {
   return guarded(n, 10, [&] {
-    return fl_lora_sgmv_static(handle<fl_pool>(a[0]), bf16_out(a[1]), bf16(a[2]), integer(a[3]), i32(a[4]), i32(a[5]), integer(a[6]),
+    return unlocked(fl_lora_sgmv_static, handle<fl_pool>(a[0]), bf16_out(a[1]), bf16(a[2]), integer(a[3]), i32(a[4]), i32(a[5]), integer(a[6]),
                                integer(a[7]), real(a[8]), stream(a[9]));
   });
 }
@@ -158,7 +170,7 @@ CALL(lora_sgmv_multi) {
     same_length(ys.n, mats.n);
     size_t wb = 0;
     void* ws = address(a[9], &wb);
-    return fl_lora_sgmv_multi(handle<fl_pool>(a[0]), ys.p, bf16(a[2]), mats.p, (int)ys.n, i32(a[4]), i32(a[5]), integer(a[6]), integer(a[7]),
+    return unlocked(fl_lora_sgmv_multi, handle<fl_pool>(a[0]), ys.p, bf16(a[2]), mats.p, (int)ys.n, i32(a[4]), i32(a[5]), integer(a[6]), integer(a[7]),
                               real(a[8]), ws, wb, stream(a[10]));
   });
 }
@@ -168,7 +180,7 @@ CALL(lora_sgmv_qkv_append) {
   return guarded(n, 21, [&] {
     size_t wb = 0;
     void* ws = address(a[19], &wb);
-    return fl_lora_sgmv_qkv_append(handle<fl_pool>(a[0]), bf16_out(a[1]), bf16(a[2]), bf16(a[3]), bf16(a[4]), integer(a[5]), integer(a[6]),
+    return unlocked(fl_lora_sgmv_qkv_append, handle<fl_pool>(a[0]), bf16_out(a[1]), bf16(a[2]), bf16(a[3]), bf16(a[4]), integer(a[5]), integer(a[6]),
                                    integer(a[7]), i32(a[8]), i32(a[9]), integer(a[10]), integer(a[11]), real(a[12]), i32(a[13]), i32(a[14]),
                                    u32(a[15]), i32(a[16]), integer(a[17]), integer(a[18]), ws, wb, stream(a[20]));
   });
@@ -178,7 +190,7 @@ CALL(lora_linear) {
   return guarded(n, 12, [&] {
     size_t wb = 0;
     void* ws = address(a[10], &wb);
-    return fl_lora_linear(handle<fl_pool>(a[0]), bf16_out(a[1]), bf16(a[2]), bf16(a[3]), integer(a[4]), i32(a[5]), i32(a[6]), integer(a[7]),
+    return unlocked(fl_lora_linear, handle<fl_pool>(a[0]), bf16_out(a[1]), bf16(a[2]), bf16(a[3]), integer(a[4]), i32(a[5]), i32(a[6]), integer(a[7]),
                           integer(a[8]), real(a[9]), ws, wb, stream(a[11]));
   });
 }
@@ -191,7 +203,7 @@ CALL(lora_linear_multi) {
     same_length(ys.n, mats.n);
     size_t wb = 0;
     void* ws = address(a[10], &wb);
-    return fl_lora_linear_multi(handle<fl_pool>(a[0]), ys.p, bf16(a[2]), w.p, mats.p, (int)ys.n, i32(a[5]), i32(a[6]), integer(a[7]),
+    return unlocked(fl_lora_linear_multi, handle<fl_pool>(a[0]), ys.p, bf16(a[2]), w.p, mats.p, (int)ys.n, i32(a[5]), i32(a[6]), integer(a[7]),
                                 integer(a[8]), real(a[9]), ws, wb, stream(a[11]));
   });
 }
@@ -201,7 +213,7 @@ CALL(lora_linear_qkv_append) {
   return guarded(n, 24, [&] {
     size_t wb = 0;
     void* ws = address(a[22], &wb);
-    return fl_lora_linear_qkv_append(handle<fl_pool>(a[0]), bf16_out(a[1]), bf16(a[2]), bf16(a[3]), bf16(a[4]), bf16(a[5]), integer(a[6]),
+    return unlocked(fl_lora_linear_qkv_append, handle<fl_pool>(a[0]), bf16_out(a[1]), bf16(a[2]), bf16(a[3]), bf16(a[4]), bf16(a[5]), integer(a[6]),
                                      integer(a[7]), integer(a[8]), i32(a[9]), i32(a[10]), integer(a[11]), integer(a[12]), real(a[13]),
                                      i32(a[14]), i32(a[15]), u32(a[16]), i32(a[17]), integer(a[18]), integer(a[19]), bf16_out(a[20]),
                                      bf16_out(a[21]), ws, wb, stream(a[23]));
@@ -210,7 +222,7 @@ CALL(lora_linear_qkv_append) {
 // pool, k_new, v_new, req_indptr, kv_tbl_indptr, kv_tbl, prefix_lens, n_req, n_tokens, n_kv_heads, stream
 CALL(kv_append) {
   return guarded(n, 11, [&] {
-    return fl_kv_append(handle<fl_pool>(a[0]), bf16(a[1]), bf16(a[2]), i32(a[3]), i32(a[4]), u32(a[5]), i32(a[6]), integer(a[7]), integer(a[8]),
+    return unlocked(fl_kv_append, handle<fl_pool>(a[0]), bf16(a[1]), bf16(a[2]), i32(a[3]), i32(a[4]), u32(a[5]), i32(a[6]), integer(a[7]), integer(a[8]),
                         integer(a[9]), stream(a[10]));
   });
 }
@@ -220,7 +232,7 @@ CALL(paged_attention) {
   return guarded(n, 16, [&] {
     size_t wb = 0;
     void* ws = address(a[14], &wb);
-    return fl_paged_attention(handle<fl_pool>(a[0]), bf16_out(a[1]), bf16(a[2]), i32(a[3]), i32(a[4]), u32(a[5]), i32(a[6]), i32(a[7]),
+    return unlocked(fl_paged_attention, handle<fl_pool>(a[0]), bf16_out(a[1]), bf16(a[2]), i32(a[3]), i32(a[4]), u32(a[5]), i32(a[6]), i32(a[7]),
                               integer(a[8]), integer(a[9]), integer(a[10]), integer(a[11]), integer(a[12]), real(a[13]), ws, wb, stream(a[15]));
   });
 }
