@@ -19,9 +19,20 @@ if not os.path.exists(LIB_PATH):
                       "(there is no fallback path)")
 lib = C.CDLL(LIB_PATH)
 
-import torch  # noqa: E402,F401  (its libraries are what _native links against)
 
-from . import _native  # noqa: E402  marshals the calls of a layer step: same arguments, tensors or integer addresses
+class _Native:
+    """Stands for the module that marshals the calls of a layer step (csrc/native.cpp), loaded with torch, whose libraries it links
+    against, on the first of them: the functions that work on host data alone need neither."""
+
+    def __getattr__(self, name):
+        global _native
+        import torch  # noqa: F401
+        from . import _native as module
+        _native = module
+        return getattr(module, name)
+
+
+_native = _Native()
 
 FL_OK, FL_EINVAL, FL_ENOMEM, FL_EBADID, FL_EBUSY, FL_ECUDA, FL_ETIMEOUT = 0, -1, -2, -3, -4, -5, -6
 _NAMES = {0: "FL_OK", -1: "FL_EINVAL", -2: "FL_ENOMEM", -3: "FL_EBADID", -4: "FL_EBUSY", -5: "FL_ECUDA",
