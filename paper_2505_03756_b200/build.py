@@ -46,9 +46,22 @@ def build(verbose=False, force=False):
     if procs or not os.path.exists(LIB):
         subprocess.check_call([nvcc, "-shared", "-o", LIB] + objs + ["-lcudart"])
     src = os.path.join(CSRC, "native.cpp")
-    if force or _stale(NATIVE, [src, os.path.join(ROOT, "include", "fastpool.h")]):
+    if force or _native_stale(src):
         _build_native(src)
     return LIB
+
+
+def _native_tag():
+    """What the module is built against: it links torch's C++ libraries and Python's."""
+    from importlib.metadata import version
+    return f"fastpool-native python {sys.version_info[0]}.{sys.version_info[1]} torch {version('torch')}"
+
+
+def _native_stale(src):
+    if _stale(NATIVE, [src, os.path.join(ROOT, "include", "fastpool.h")]):
+        return True
+    with open(NATIVE, "rb") as f:
+        return _native_tag().encode() + b"\0" not in f.read()
 
 
 def _build_native(src):
@@ -57,7 +70,7 @@ def _build_native(src):
     tdir = os.path.dirname(torch.__file__)
     inc = [os.path.join(ROOT, "include"), sysconfig.get_paths()["include"], os.path.join(tdir, "include"),
            os.path.join(tdir, "include", "torch", "csrc", "api", "include"), "/usr/local/cuda/include"]
-    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", src, "-o", NATIVE]
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f'-DFL_NATIVE_TAG="{_native_tag()}"', f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", src, "-o", NATIVE]
     cmd += [f for i in inc for f in ("-isystem" if "torch" in i else "-I", i)]
     cmd += ["-L", HERE, "-l:libfastpool.so", "-L", os.path.join(tdir, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda",
             "-Wl,-rpath,$ORIGIN", "-Wl,-rpath," + os.path.join(tdir, "lib")]

@@ -245,4 +245,12 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, methods, nu
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__native() { return PyModule_Create(&module); }
+// What the module was built against, for build.py, which finds it in the file.
+PyMODINIT_FUNC PyInit__native() {
+  PyObject* m = PyModule_Create(&module);
+  if (m && PyModule_AddStringConstant(m, "built_against", FL_NATIVE_TAG) < 0) {
+    Py_DECREF(m);
+    return nullptr;
+  }
+  return m;
+}
