@@ -23,10 +23,12 @@
 // is computed, the calls take 25 and 17 us; before, with the GEMM for long batches followed by the segmented projection,
 // they took 44 and 32 us.  The rest is the shrink's chain of look-ups in front and the sum over the cluster behind.
 // Every mbarrier wait is bounded; a wait that gives up raises a sticky flag and the CTA still meets its cluster's
-// barriers, drains its copies and frees its TMEM.  No multicast.
+// barriers, where it tells the others that its part of the sum is missing (none of them stores anything then), drains its copies
+// and frees its TMEM.  No multicast.
 #include <cuda.h>
 #include <string.h>
 #include <algorithm>
+#include "giveup.cuh"
 #include "lora_skinny.cuh"
 #include "mma_utils.cuh"
 #include "tc_ptx.cuh"
@@ -92,6 +94,7 @@ __global__ void __launch_bounds__(MAX_THREADS, 1) lora_skinny_kernel(const __gri
   volatile int* n_stage_slot = reinterpret_cast<volatile int*>(smem + off_book + 8 * B_COUNT + 8);
   int* scan = reinterpret_cast<int*>(smem + off_book + 8 * B_COUNT + 16);      // [4], one per filler warp
   volatile int* rpb_slot = reinterpret_cast<volatile int*>(smem + off_book + 8 * B_COUNT + 12);
+  volatile int* told_slot = reinterpret_cast<volatile int*>(smem + off_book + 8 * B_COUNT + 32);       // a CTA of the cluster has no part of the sum
   unsigned long long* row_ptr = reinterpret_cast<unsigned long long*>(smem + off_book + BOOK_BYTES);     // [group][2][GROUP * BK], 0 = no row
   LoraUnit* list = reinterpret_cast<LoraUnit*>(smem + off_book + BOOK_BYTES + ROWS_BYTES);
   const int max_units = npad * UNITS_PER_TOKEN;
@@ -117,6 +120,7 @@ __global__ void __launch_bounds__(MAX_THREADS, 1) lora_skinny_kernel(const __gri
     mbar_init(bar(B_LIST), 1);
     mbar_init(bar(B_ACC), 2);            // both issuers
     *abort_flag = 0;
+    *told_slot = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -420,6 +424,8 @@ __global__ void __launch_bounds__(MAX_THREADS, 1) lora_skinny_kernel(const __gri
   const int c0 = min(crank * share, BN), c1 = min(c0 + share, BN);
   if (split > 1) {
     cluster_sync();                                           // every CTA of the cluster is done with its rings
+    if (tid == 64)
+      giveup::tell_cluster(ok, crank, split, [&](int p) { st_cluster_u32(map_cluster_rank(smem_u32(const_cast<int*>(told_slot)), (uint32_t)p), 1u); });
     if (epi && ok) {
       for (int p = 0; p < split; ++p) {
         if (p == crank) continue;
@@ -451,6 +457,7 @@ __global__ void __launch_bounds__(MAX_THREADS, 1) lora_skinny_kernel(const __gri
     }
     __syncwarp();
     cluster_sync();
+    ok = giveup::may_store(ok, *told_slot);
   }
   if (epi && ok) {
     // The finished rows as bf16 through shared memory (behind the partial sums; pitch an odd number of 16-byte chunks), so that
