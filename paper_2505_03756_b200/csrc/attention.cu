@@ -270,7 +270,7 @@ __device__ __forceinline__ uint32_t load_word(const __nv_bfloat16* p) {
 constexpr int MAX_FEW_ROWS = 64;      // query rows per KV head, in all, of a batch served without a plan
 enum { PLAIN = 0, BESIDE = 1, CLUSTER = 2 };
 template <int MODE>
-__global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs a, int chunk, int n_tbl) {
+__global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs a, int chunk) {
   extern __shared__ __align__(128) unsigned char smem[];
   if (MODE != BESIDE || blockIdx.x == gridDim.x - 1) pdl_wait();
   pdl_launch_dependents();    // the next call's first kernel may set itself up; it waits for this grid before it reads anything
@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
     it.tbl_n = a.tbl_indptr[item + 1] - it.tbl0;
     if (it.n_new * (a.n_q / a.n_kv) <= (int)blockIdx.y * DEC_ROWS) return;       // (the same answer in the whole cluster)
     const int pages = (it.prefix + it.n_new + BT - 1) / BT;
-    if (pages > it.tbl_n || it.tbl0 + it.tbl_n > n_tbl || it.n_new * (a.n_q / a.n_kv) > MAX_FEW_ROWS) {
+    if (pages > it.tbl_n || it.n_new * (a.n_q / a.n_kv) > MAX_FEW_ROWS) {
       if (threadIdx.x == 0) atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_POS);
       return;
     }
@@ -739,7 +739,7 @@ int fl_paged_attention(fl_pool* p, fl_bf16* out, const fl_bf16* q, const int32_t
     const int csize = kind == 0 && few ? cluster_size(n_req, n_tbl, n_kv_heads, p->sm_count) : 0;
     if (csize > 0) {
       const cudaError_t e = launch_pdl_cluster(attn_decode_kernel<CLUSTER>, dim3((unsigned)(n_req * n_kv_heads * csize), (unsigned)passes), dim3((unsigned)csize),
-                                               dim3(ATT_THREADS), DEC_SMEM, st, a, csize, n_tbl);
+                                               dim3(ATT_THREADS), DEC_SMEM, st, a, csize);
       if (e != cudaSuccess) {
         p->last_cuda = (int)e;
         rc = FL_ECUDA;
@@ -763,7 +763,7 @@ int fl_paged_attention(fl_pool* p, fl_bf16* out, const fl_bf16* q, const int32_t
       attn_prefill_kernel<<<(unsigned)w.max_prefill * n_q_heads, ATT_THREADS, PRE_SMEM, st>>>(a);
     }
     cudaError_t e = launch_pdl(beside ? attn_decode_kernel<BESIDE> : attn_decode_kernel<PLAIN>, dim3((unsigned)w.max_decode * n_kv_heads + (beside ? 1u : 0u)),
-                               dim3(ATT_THREADS), DEC_SMEM, st, a, w.chunk, n_tbl);
+                               dim3(ATT_THREADS), DEC_SMEM, st, a, w.chunk);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {
       p->last_cuda = (int)e;

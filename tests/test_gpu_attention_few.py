@@ -55,3 +55,31 @@ def test_few_decode_requests(heads, prefix, new):
             assert s.status(clear=True)["device_flags"] != 0
     finally:
         s.close()
+
+
+def test_tables_longer_than_the_contexts():
+    """Blocks allocated ahead: the tables have more entries than the batch's contexts need, and n_tbl counts those in use."""
+    from paper_2505_03756_b200 import harness as H
+    wl = synth.make_workload("tiny", n_req=5, len_range=(0, 0), n_adapters=1, shape=synth.LayerShape(512, 4, 4))
+    wl.prefix_lens[:], wl.new_lens[:] = [100, 17, 300, 40, 15], [1, 1, 1, 1, 1]
+    used = int(np.sum((wl.prefix_lens + wl.new_lens + 15) // 16))
+    wl.pool_blocks = used + 64
+    s = H.Session(wl, adapters=[])
+    try:
+        s.build_batch()
+        s.fill_prefix_kv()
+        k_new, v_new = wl.kv_new()
+        s.kv_append(H.f32_to_dev(k_new, s.dev), H.f32_to_dev(v_new, s.dev))
+        q = H.f32_to_dev(wl.q(), s.dev)
+        want = torch.empty(q.shape, dtype=torch.bfloat16, device=s.dev)
+        s.attention(want, q)
+        long_tables = [np.concatenate([t, s.alloc(7)]) for t in s.kv_tables]
+        s.t_tbl_indptr = torch.from_numpy(np.cumsum([0] + [len(t) for t in long_tables]).astype(np.int32)).to(s.dev)
+        s.t_tbl = torch.from_numpy(np.concatenate(long_tables).astype(np.uint32).view(np.int32)).to(s.dev)
+        assert s.n_tbl == used
+        out = torch.full_like(want, float("nan"))
+        s.attention(out, q)
+        assert torch.equal(out, want)
+        assert s.status()["device_flags"] == 0
+    finally:
+        s.close()
