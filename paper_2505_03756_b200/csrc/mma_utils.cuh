@@ -41,9 +41,20 @@ __device__ __forceinline__ float2 unpack_bf16(uint32_t u) {
   return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xFFFF0000u));
 }
 
+// Bits 15 and 31: whether the lower and the upper bf16 of a pair is an infinity or NaN (its exponent is all ones).
+__device__ __forceinline__ uint32_t nonfinite_pair(uint32_t u) { return ((u & 0x7f807f80u) + 0x00800080u) & 0x80008000u; }
+__device__ __forceinline__ uint32_t nonfinite_chunk(uint4 q) {
+  return nonfinite_pair(q.x) | nonfinite_pair(q.y) | nonfinite_pair(q.z) | nonfinite_pair(q.w);
+}
+// The pair with zeros in the place of infinities and NaNs.
+__device__ __forceinline__ uint32_t finite_part(uint32_t u) { return u & ~((nonfinite_pair(u) >> 15) * 0xffffu); }
+
 // Four 8 x 8 bf16 matrices in accumulator layout -> shared memory rows of 16 bytes (lane l gives the address of row l % 8 of matrix l / 8).
 __device__ __forceinline__ void stmatrix_x4(uint32_t addr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
   asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1,%2,%3,%4};\n" ::"r"(addr), "r"(r0), "r"(r1), "r"(r2), "r"(r3) : "memory");
+}
+__device__ __forceinline__ void st_shared_v4(uint32_t addr, uint4 v) {
+  asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 __device__ __forceinline__ uint4 ld_shared_v4(uint32_t addr) {
   uint4 v;
