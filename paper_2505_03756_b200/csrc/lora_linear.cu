@@ -115,6 +115,47 @@ __device__ __forceinline__ unsigned long long pack_unit(int lid, int q, int nr, 
 }
 static_assert(FL_MAX_LORA_ID <= 1 << 20 && FL_MAX_RANK / UNIT <= 4 && 2 * BM < 512, "fields of a LoRA unit");
 
+// Infinities and NaNs in an adapter's B rows stay out of a LoRA stage: times the zeros of the tile's other tokens they would make
+// NaNs of these tokens' rows.  What they give their own token's 32 columns from col on is added here, to the values of its row.
+template <int RMAX>
+__device__ __noinline__ void add_nonfinite_terms(const LinArgs& a, int j, int tok, int col, uint32_t (&o)[32]) {
+  int lo = 0, hi = a.n_seg;                // first segment that ends behind tok
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (a.seg_indptr[mid + 1] > tok) hi = mid; else lo = mid + 1;
+  }
+  if (lo >= a.n_seg || a.seg_indptr[lo] > tok) return;
+  const int lid = a.lora_ids[lo], mat = a.mat_index[j];
+  if (lid < 0 || (uint32_t)lid >= a.pv.dir_cap || a.pv.dir[lid].rank <= 0 || mat >= a.pv.dir[lid].n_mats) return;
+  const LoraEntry* en = a.pv.dir + lid;
+  const LoraMat lm = en->mats[mat];
+  const int rank = min(en->rank, RMAX);
+  for (int r = 0; r < rank; ++r) {
+    const uint32_t gr = lm.b_row0 + r, blk = a.pv.tables[en->table_off + lm.b_tab + gr / lm.b_rpb];
+    if (blk >= a.pv.n_blocks) continue;
+    const uint4* b = reinterpret_cast<const uint4*>(a.pv.slab + (size_t)blk * a.pv.block_bytes + ((size_t)(gr % lm.b_rpb) * a.d_out[j] + col) * 2);
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      if (col + 8 * h >= a.d_out[j]) break;
+      const uint4 q = b[h];
+      if (nonfinite_chunk(q) == 0u) continue;
+      float v = 0.f;
+      if (a.v16) {
+        v = __bfloat162float(a.v16[((size_t)j * a.n_tokens + tok) * RMAX + r]);
+      } else {
+        for (int sp = 0; sp < a.ksplit; ++sp) v += a.v[((size_t)(j * a.ksplit + sp) * a.n_tokens + tok) * RMAX + r];
+        v = __bfloat162float(__float2bfloat16_rn(v * a.scale));
+      }
+      const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        const float bv = __uint_as_float(c & 1 ? w[c >> 1] & 0xffff0000u : w[c >> 1] << 16);
+        if ((__float_as_uint(bv) & 0x7f800000u) == 0x7f800000u) o[8 * h + c] = __float_as_uint(fmaf(v, bv, __uint_as_float(o[8 * h + c])));
+      }
+    }
+  }
+}
+
 template <int BN, int RMAX>
 __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid_constant__ LinArgs a, const __grid_constant__ LinMaps maps) {
   using C = Cfg<BN>;
@@ -134,7 +175,8 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_BAR + 8 * B_COUNT + 4);
   volatile int* n_ext_slot = reinterpret_cast<volatile int*>(smem + C::OFF_BAR + 8 * B_COUNT + 8);   // [2] LoRA stages of a tile
   int* scan = reinterpret_cast<int*>(smem + C::OFF_BAR + 8 * B_COUNT + 16);                          // [8] per filler warp
-  static_assert(8 * B_COUNT + 16 + 32 <= 512, "bookkeeping area too small");
+  volatile int* nonfinite_slot = reinterpret_cast<volatile int*>(smem + C::OFF_BAR + 8 * B_COUNT + 48);   // a B row held an infinity or NaN
+  static_assert(8 * B_COUNT + 16 + 32 + 16 <= 512, "bookkeeping area too small");
 
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) {
@@ -150,6 +192,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
       mbar_init(bar(B_LEMPTY + b), 1);
     }
     *abort_flag = 0;
+    *nonfinite_slot = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -298,6 +341,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
       tc_fence_after();
       __nv_bfloat16* yrow = side < 0 ? a.y[t.j] + (size_t)tok * d_out + n0 : nullptr;
       const bool wide = side < 0 && a.wide[t.j];
+      const bool nonfinite = *nonfinite_slot != 0;       // (of this tile or one before or behind it: then a look at the token's own rows)
 #pragma unroll 2
       for (int cb = 0; cb < BN; cb += 32) {
         uint32_t o[32];
@@ -305,6 +349,14 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
         tmem_ld32(lane_addr + buf * BN + cb, o);
         tmem_wait_ld();
         if (tok < a.n_tokens) {
+          if (nonfinite) {
+            uint32_t f[32];
+#pragma unroll
+            for (int c = 0; c < 32; ++c) f[c] = o[c];
+            add_nonfinite_terms<RMAX>(a, t.j, tok, n0 + cb, f);
+#pragma unroll
+            for (int c = 0; c < 32; ++c) o[c] = f[c];
+          }
           uint32_t pk[16];
 #pragma unroll
           for (int c = 0; c < 16; ++c) pk[c] = pack_bf16(__uint_as_float(o[2 * c]), __uint_as_float(o[2 * c + 1]));
@@ -497,6 +549,24 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
         }
         cp_async_commit();
         cp_async_wait<0>();
+        // infinities and NaNs out of the B rows (this thread's own pieces; add_nonfinite_terms has the reason)
+        uint32_t found = 0;
+#pragma unroll
+        for (int i = 0; i < ER * CPR / 128; ++i) {
+          const int c = et + 128 * i, r = c / CPR, ch = c % CPR;
+          found |= nonfinite_chunk(ld_shared_v4(bs + (ch >> 3) * B_GROUP + (ER * slot + r) * 128 + (((ch & 7) ^ (r & 7)) << 4)));
+        }
+        if (found) {
+          for (int i = 0; i < ER * CPR / 128; ++i) {
+            const int c = et + 128 * i, r = c / CPR, ch = c % CPR;
+            const uint32_t at = bs + (ch >> 3) * B_GROUP + (ER * slot + r) * 128 + (((ch & 7) ^ (r & 7)) << 4);
+            const uint4 q = ld_shared_v4(at);
+            st_shared_v4(at, make_uint4(finite_part(q.x), finite_part(q.y), finite_part(q.z), finite_part(q.w)));
+          }
+          // both CTAs' rows meet these columns
+          *nonfinite_slot = 1;
+          st_cluster_u32(map_cluster_rank(smem_u32(const_cast<int*>(nonfinite_slot)), (uint32_t)(crank ^ 1)), 1u);
+        }
         fence_async_smem();                              // the tensor core reads shared memory through the async proxy
         asm volatile("bar.sync %0, 128;" ::"r"(3 + slot) : "memory");
         if (et == 0 && ok) mbar_arrive_cluster(efull0 + 8u * slot);
