@@ -29,6 +29,7 @@
 #include <string.h>
 #include <algorithm>
 #include "attention.cuh"
+#include "giveup.cuh"
 #include "mma_utils.cuh"
 #include "tc_ptx.cuh"
 #include "tmap.cuh"
@@ -53,7 +54,7 @@ constexpr uint32_t T2_TMEM_COLS = 512;                 // S_A | S_B | O_A | O_B,
 constexpr float RESCALE_LOG2 = 8.f;
 
 enum { C_QFULL = 0, C_QEMPTY = 1, C_FULL = 2, C_EMPTY = C_FULL + NSLOT, C_SFULL = C_EMPTY + NSLOT, C_PFULL = C_SFULL + 2,
-       C_PHALF = C_PFULL + 2, C_ODONE = C_PHALF + 2, C_UFULL = C_ODONE + 2, C_UEMPTY = C_UFULL + 2, C_COUNT = C_UEMPTY + 2 };
+       C_PHALF = C_PFULL + 2, C_ODONE = C_PHALF + 2, C_UFULL = C_ODONE + 2, C_UEMPTY = C_UFULL + 2, C_IDLE = C_UEMPTY + 2, C_COUNT };
 constexpr int UNIT_READERS = 9;                        // MMA issuer + 8 softmax warps
 
 struct Unit {           // what a CTA works on at one time
@@ -134,6 +135,7 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
       mbar_init(bar(C_UFULL + x), 1);
       mbar_init(bar(C_UEMPTY + x), UNIT_READERS);
     }
+    mbar_init(bar(C_IDLE), 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -153,6 +155,8 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
   const int n_ctas = min((int)gridDim.x, a.hdr->prefill_ctas);
 
   // Readers take the k-th unit of this CTA from slot k & 1 (index -1 = no more work) and release the slot.
+
+  int kv_fills = 0, q_fills = 0;       // ring slots and Q buffers that the producer has armed
 
   // the softmax warpgroups keep 128 scores per thread in registers: they take the registers the third
   // warpgroup does not need
@@ -189,7 +193,10 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
         // Q buffers are free once the previous unit's last S MMA has completed
         if (lane == 0) {
           if (n_valid > 0) ok = mbar_wait(bar(C_QEMPTY), (n_valid - 1) & 1, abort_flag);
-          if (ok) mbar_expect_tx(bar(C_QFULL), rows_b > 0 ? 2 * TILE_BYTES : TILE_BYTES);
+          if (ok) {
+            mbar_expect_tx(bar(C_QFULL), rows_b > 0 ? 2 * TILE_BYTES : TILE_BYTES);
+            ++q_fills;
+          }
         }
         ++n_valid;
         ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
@@ -215,7 +222,10 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
             const int s = fill % NSLOT, use = fill / NSLOT;
             if (lane == 0) {
               if (use > 0) ok = mbar_wait(bar(C_EMPTY + s), (use - 1) & 1, abort_flag);
-              if (ok) mbar_expect_tx(bar(C_FULL + s), TILE_BYTES);
+              if (ok) {
+                mbar_expect_tx(bar(C_FULL + s), TILE_BYTES);
+                ++kv_fills;
+              }
             }
             ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;     // the transaction count is armed before any copy is issued
             if (!ok) break;
@@ -438,14 +448,12 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
   __syncthreads();
   if (*abort_flag) {
     if (tid == 0) atomicOr(a.pv.flags, (uint32_t)FLAG_WAIT_GAVE_UP);
-    // copies still in flight target this CTA's shared memory: give every armed barrier a bounded
-    // chance to complete before the CTA exits
+    // copies and MMAs still in flight use this CTA's shared memory and TMEM
+    if (warp == 9) umma_commit_elect(bar(C_IDLE));
     if (warp == 8 && lane == 0) {
-      for (int s = 0; s < NSLOT; ++s)
-        for (uint32_t k = 0; k < (1u << 16); ++k)
-          if (mbar_try(bar(C_FULL + s), 0) || mbar_try(bar(C_FULL + s), 1)) break;
-      for (uint32_t k = 0; k < (1u << 16); ++k)
-        if (mbar_try(bar(C_QFULL), 0) || mbar_try(bar(C_QFULL), 1)) break;
+      giveup::drain(kv_fills, NSLOT, [&](int s, uint32_t parity) { return mbar_try(bar(C_FULL + s), parity); });
+      giveup::drain(q_fills, 1, [&](int, uint32_t parity) { return mbar_try(bar(C_QFULL), parity); });
+      giveup::drain(1, 1, [&](int, uint32_t parity) { return mbar_try(bar(C_IDLE), parity); });
     }
     __syncthreads();
   }

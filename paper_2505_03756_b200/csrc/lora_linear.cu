@@ -23,6 +23,7 @@
 #include <cuda.h>
 #include <string.h>
 #include <algorithm>
+#include "giveup.cuh"
 #include "lora_skinny.cuh"
 #include "mma_utils.cuh"
 #include "pool.cuh"
@@ -168,7 +169,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
   const int crank = (int)cluster_ctarank();
   const bool leader = crank == 0;
   enum { B_FULL = 0, B_EMPTY = NS, B_ACC_FULL = 2 * NS, B_ACC_EMPTY = B_ACC_FULL + 2, B_EFULL = B_ACC_EMPTY + 2, B_EEMPTY = B_EFULL + 2,
-         B_LFULL = B_EEMPTY + 2, B_LEMPTY = B_LFULL + 2, B_COUNT = B_LEMPTY + 2 };
+         B_LFULL = B_EEMPTY + 2, B_LEMPTY = B_LFULL + 2, B_IDLE = B_LEMPTY + 2, B_COUNT };
   const uint32_t bar0 = sbase + C::OFF_BAR;
   auto bar = [&](int k) { return bar0 + 8u * k; };
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + C::OFF_BAR + 8 * B_COUNT);
@@ -176,6 +177,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
   volatile int* n_ext_slot = reinterpret_cast<volatile int*>(smem + C::OFF_BAR + 8 * B_COUNT + 8);   // [2] LoRA stages of a tile
   int* scan = reinterpret_cast<int*>(smem + C::OFF_BAR + 8 * B_COUNT + 16);                          // [8] per filler warp
   volatile int* nonfinite_slot = reinterpret_cast<volatile int*>(smem + C::OFF_BAR + 8 * B_COUNT + 48);   // a B row held an infinity or NaN
+  volatile int* partner_slot = reinterpret_cast<volatile int*>(smem + C::OFF_BAR + 8 * B_COUNT + 52);     // [2] its abort flag, its producer's stages
   static_assert(8 * B_COUNT + 16 + 32 + 16 <= 512, "bookkeeping area too small");
 
   if (tid == 0) {
@@ -191,6 +193,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
       mbar_init(bar(B_LFULL + b), 1);
       mbar_init(bar(B_LEMPTY + b), 1);
     }
+    mbar_init(bar(B_IDLE), 1);
     *abort_flag = 0;
     *nonfinite_slot = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -211,6 +214,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
   const int total = a.tile_base[a.n_mats];
   const int nk = (a.d_in + BK - 1) / BK;
   const int first = blockIdx.x >> 1, step = gridDim.x >> 1;      // pairs
+  int fills = 0;                                                 // stages that this CTA's producer has issued
 
   if (warp == 0) {
     // ------------------------------------------------ TMA producer (one lane): this CTA's halves; both CTAs' bytes are counted
@@ -232,6 +236,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
           tma_load_2d_pair(dst, &maps.x, fb, ks * BK, row0);
 #pragma unroll
           for (int g = 0; g < BH / 64; ++g) tma_load_2d_pair(dst + A_BYTES + g * B_GROUP, wm, fb, col0 + g * 64, ks * BK);
+          ++fills;
           if (++s == NS) { s = 0; ph ^= 1u; wrapped = true; }
         }
       }
@@ -579,17 +584,26 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
   // ------------------------------------------------ teardown: neither CTA leaves while the other's MMAs or arrivals need it
   tc_fence_before();
   __syncthreads();
-  if (*abort_flag) {
+  if (tid == 0) {
+    const uint32_t to = map_cluster_rank(smem_u32(const_cast<int*>(partner_slot)), (uint32_t)(crank ^ 1));
+    st_cluster_u32(to, (uint32_t)*abort_flag);
+    st_cluster_u32(to + 4, (uint32_t)fills);
+  }
+  __syncwarp();
+  cluster_sync();
+  if (*abort_flag || partner_slot[0]) {      // the same answer in both CTAs
     if (tid == 0) atomicOr(a.pv.flags, (uint32_t)FLAG_WAIT_GAVE_UP);
-    // copies still in flight target this CTA's shared memory: give every armed barrier a bounded chance to complete
-    if (warp == 0 && lane == 0) {
-      for (int s = 0; s < NS; ++s)
-        for (uint32_t i = 0; i < (1u << 16); ++i)
-          if (mbar_try(bar(B_FULL + s), 0) || mbar_try(bar(B_FULL + s), 1)) break;   // (an idle barrier answers at once)
+    // Copies and MMAs still in flight use both CTAs' shared memory and TMEM; the first CTA's barriers count them all.
+    if (leader && warp == 1) umma_commit_pair_elect(bar(B_IDLE));
+    if (leader && tid == 0) {
+      const long long armed = giveup::settle_pair(fills, partner_slot[1], NS, [&](int s) { mbar_expect_tx(bar(B_FULL + s), C::STAGE); },
+                                                  [&](int s) { mbar_complete_tx(bar(B_FULL + s), C::STAGE); });
+      giveup::drain(armed, NS, [&](int s, uint32_t parity) { return mbar_try_cluster(bar(B_FULL + s), parity); });
+      giveup::drain(1, 1, [&](int, uint32_t parity) { return mbar_try_cluster(bar(B_IDLE), parity); });
     }
     __syncthreads();
+    cluster_sync();
   }
-  cluster_sync();
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::TMEM_COLS) : "memory");

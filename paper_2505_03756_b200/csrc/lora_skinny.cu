@@ -71,7 +71,7 @@ struct Maps {
   CUtensorMap w[skinny::MAX_LIN];
 };
 
-enum { B_FULL = 0, B_EMPTY = MAX_NS, B_EFULL = 2 * MAX_NS, B_EEMPTY = B_EFULL + MAX_NE, B_LIST = B_EEMPTY + MAX_NE, B_ACC, B_COUNT };
+enum { B_FULL = 0, B_EMPTY = MAX_NS, B_EFULL = 2 * MAX_NS, B_EEMPTY = B_EFULL + MAX_NE, B_LIST = B_EEMPTY + MAX_NE, B_ACC, B_IDLE, B_COUNT };
 // behind the two rings: barriers and bookkeeping | B row addresses, two sets of stages per group of warps | list of LoRA units
 constexpr uint32_t BOOK_BYTES = 512, ROWS_BYTES = FILLERS * 2 * GROUP * BK * 8;
 static_assert(8 * B_COUNT + 48 <= BOOK_BYTES, "bookkeeping area too small");
@@ -169,6 +169,7 @@ __global__ void __launch_bounds__(MAX_THREADS, 1) lora_skinny_kernel(const __gri
     }
     mbar_init(bar(B_LIST), 1);
     mbar_init(bar(B_ACC), 2);            // both issuers
+    mbar_init(bar(B_IDLE), 2);
     *abort_flag = 0;
     *told_slot = 0;
     *nonfinite_slot = 0;
@@ -205,6 +206,7 @@ __global__ void __launch_bounds__(MAX_THREADS, 1) lora_skinny_kernel(const __gri
   };
 
   bool ok = true;
+  int fills = 0;                           // stages that the producer has armed
   int n_stages = 0;                        // LoRA stages of this CTA (known to the LoRA roles)
   const int filler = (warp - 2) >> 2;      // group of four warps
   const int et = (tid - 64) & 127;         // thread of its group; of the first: epilogue thread
@@ -221,6 +223,7 @@ __global__ void __launch_bounds__(MAX_THREADS, 1) lora_skinny_kernel(const __gri
         tma_load_2d(dst + x_bytes, wm, bar(B_FULL + s), n0, ks * BK);
         tma_load_2d(dst + x_bytes + W_GROUP, wm, bar(B_FULL + s), n0 + 64, ks * BK);
         tma_load_2d(dst, &maps.x, bar(B_FULL + s), ks * BK, 0);
+        ++fills;
         if (++s == ns) { s = 0; ph ^= 1u; }
       }
     }
@@ -592,11 +595,11 @@ __global__ void __launch_bounds__(MAX_THREADS, 1) lora_skinny_kernel(const __gri
   __syncthreads();
   if (*abort_flag) {
     if (tid == 0) atomicOr(a.pv.flags, (uint32_t)FLAG_WAIT_GAVE_UP);
-    // copies still in flight target this CTA's shared memory: give every armed barrier a bounded chance to complete
-    if (warp == 0 && lane == 0) {
-      for (int s = 0; s < ns; ++s)
-        for (uint32_t i = 0; i < (1u << 16); ++i)
-          if (mbar_try(bar(B_FULL + s), 0) || mbar_try(bar(B_FULL + s), 1)) break;
+    // copies and MMAs still in flight use this CTA's shared memory and TMEM
+    if (warp == 1 || warp == 2 + 4 * ne) umma_commit_elect(bar(B_IDLE));
+    if (tid == 0) {
+      giveup::drain(fills, ns, [&](int s, uint32_t parity) { return mbar_try(bar(B_FULL + s), parity); });
+      giveup::drain(1, 1, [&](int, uint32_t parity) { return mbar_try(bar(B_IDLE), parity); });
     }
     __syncthreads();
   }

@@ -13,6 +13,7 @@
 // tears down (its copies drained, its TMEM freed).  No cluster launch, no multicast.
 #include <cuda.h>
 #include <algorithm>
+#include "giveup.cuh"
 #include "mma_utils.cuh"
 #include "pool.cuh"
 #include "sgmv.cuh"
@@ -80,12 +81,13 @@ __global__ void __launch_bounds__(ST_THREADS, 1) sgmv_shrink_tc_kernel(const sgm
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const uint32_t sbase = smem_u32(smem);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  enum { B_FULL = 0, B_EMPTY = NS, B_ACC_FULL = 2 * NS, B_ACC_EMPTY = 2 * NS + 2, B_COUNT = 2 * NS + 4 };
+  enum { B_FULL = 0, B_EMPTY = NS, B_ACC_FULL = 2 * NS, B_ACC_EMPTY = 2 * NS + 2, B_IDLE = 2 * NS + 4, B_COUNT };
   const uint32_t bar0 = sbase + C::OFF_BAR;
   auto bar = [&](int k) { return bar0 + 8u * k; };
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + C::OFF_BAR + 8 * B_COUNT);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_BAR + 8 * B_COUNT + 4);
-  static_assert(8 * B_COUNT + 8 <= 256, "bookkeeping area too small");
+  volatile int* fills_slot = reinterpret_cast<volatile int*>(smem + C::OFF_BAR + 8 * B_COUNT + 8);
+  static_assert(8 * B_COUNT + 12 <= 256, "bookkeeping area too small");
 
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) {
@@ -96,6 +98,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) sgmv_shrink_tc_kernel(const sgm
       mbar_init(bar(B_ACC_FULL + b), 1);
       mbar_init(bar(B_ACC_EMPTY + b), 4);
     }
+    mbar_init(bar(B_IDLE), 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -110,6 +113,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) sgmv_shrink_tc_kernel(const sgm
   pdl_wait();                 // x may come from the kernel right before this one
   pdl_launch_dependents();    // the kernel that consumes the partial sums may set itself up while this grid runs
 
+  long long fills = 0, arrived = 0;    // x copies that the producer has issued; stages that a copy thread has signalled
   if (warp == 0) {
     // ------------------------------------------------ TMA producer (lane 0 issues; the warp decodes units together)
     long long f = 0;
@@ -125,6 +129,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) sgmv_shrink_tc_kernel(const sgm
           if (ok) {
             mbar_expect_tx(bar(B_FULL + s), X_BYTES);
             tma_load_2d(sbase + s * C::STAGE, &xmap, bar(B_FULL + s), t.kb + it * BK, t.tok0);
+            ++fills;
           }
         }
         ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
@@ -168,7 +173,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) sgmv_shrink_tc_kernel(const sgm
     const int ct = tid - 64;                      // 0..127
     constexpr int RPT = N / 16;                   // rows per thread: n = ct / 8 + 16 i
     const int cc = ct & 7;
-    long long f = 0, arrived = 0;                 // stages issued / stages this thread has signalled
+    long long f = 0;                              // stages issued
     bool ok = true;
     auto signal = [&](long long upto) {           // the copies of stages < upto have landed: make them visible, arrive
       fence_async_smem();
@@ -278,12 +283,17 @@ __global__ void __launch_bounds__(ST_THREADS, 1) sgmv_shrink_tc_kernel(const sgm
   __syncthreads();
   if (*abort_flag) {
     if (tid == 0) atomicOr(a.pv.flags, (uint32_t)FLAG_WAIT_GAVE_UP);
-    // x copies still in flight target this CTA's shared memory: give every armed barrier a bounded chance to complete
-    // (the adapter-row copies were waited for by their own threads above)
-    if (warp == 0 && lane == 0) {
-      for (int s = 0; s < NS; ++s)
-        for (uint32_t i = 0; i < (1u << 16); ++i)
-          if (mbar_try(bar(B_FULL + s), 0) || mbar_try(bar(B_FULL + s), 1)) break;
+    // x copies and MMAs still in flight use this CTA's shared memory and TMEM (the adapter-row copies were waited for by their own
+    // threads above).  A stage's phase ends with its x copy only if the copy threads signal it too; each owes at most the last
+    // phase of a slot, since the one before it was over when the producer armed it.
+    if (tid == 0) *fills_slot = (int)fills;
+    __syncthreads();
+    if (warp >= 2 && warp < 6)
+      for (; arrived < *fills_slot; ++arrived) mbar_arrive(bar(B_FULL + (int)(arrived % NS)));
+    if (warp == 1 && lane == 0) umma_commit(bar(B_IDLE));
+    if (tid == 0) {
+      giveup::drain(fills, NS, [&](int s, uint32_t parity) { return mbar_try(bar(B_FULL + s), parity); });
+      giveup::drain(1, 1, [&](int, uint32_t parity) { return mbar_try(bar(B_IDLE), parity); });
     }
     __syncthreads();
   }
