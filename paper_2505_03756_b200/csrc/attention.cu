@@ -254,6 +254,72 @@ __device__ __forceinline__ uint32_t load_word(const __nv_bfloat16* p) {
   return PAST_L1 ? __ldcg(reinterpret_cast<const uint32_t*>(p)) : *reinterpret_cast<const uint32_t*>(p);
 }
 
+// Which request's pages a CTA takes where there is no plan and a request gets as many CTAs as it has pages for: one for up to
+// `part_pages`, two or four beyond, those of four first, so that a request's CTAs lie in one cluster of four.  Every warp finds
+// it by itself from the requests' numbers, a request per lane, and has the numbers of its own at hand then.
+__device__ __forceinline__ bool find_share(const AttnArgs& a, int slot, int n_slots, int part_pages, DecodeItem& it) {
+  const int lane = threadIdx.x & 31;
+  struct Request {
+    int n_new, prefix, tok0, tbl0, tbl_n, log_parts;      // log_parts: -1 = no new token
+  };
+  auto load = [&](int i) {
+    Request r = {0, 0, 0, 0, 0, -1};
+    if (i < a.n_req) {
+      r.n_new = a.new_lens[i];
+      r.prefix = a.prefix_lens[i];
+      r.tok0 = a.req_indptr[i];
+      r.tbl0 = a.tbl_indptr[i];
+      r.tbl_n = a.tbl_indptr[i + 1] - r.tbl0;
+      const int pages = (r.prefix + r.n_new + BT - 1) / BT;
+      // (a table too short for them: no output)
+      if (r.n_new > 0) r.log_parts = pages <= part_pages || pages > r.tbl_n ? 0 : pages <= 2 * part_pages ? 1 : 2;
+    }
+    return r;
+  };
+  const Request first = load(lane);
+  int n[3] = {0, 0, 0};
+  for (int r0 = 0; r0 < a.n_req; r0 += 32) {
+    const int c = r0 == 0 ? first.log_parts : load(r0 + lane).log_parts;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) n[k] += __popc(__ballot_sync(0xffffffffu, c == k));
+  }
+  // (contexts longer than the caller's n_tbl covers: one CTA each)
+  const bool fit = n[0] + 2 * n[1] + 4 * n[2] <= n_slots;
+  if (!fit) {
+    n[0] += n[1] + n[2];
+    n[1] = n[2] = 0;
+  }
+  int behind = 0, k = 0, count = 0;
+#pragma unroll
+  for (int c = 2; c >= 0; --c) {
+    if (slot >= behind && slot < behind + (n[c] << c)) {
+      k = c;
+      count = (slot - behind) >> c;
+    }
+    behind += n[c] << c;
+  }
+  if (slot >= behind) return false;
+  for (int r0 = 0; r0 < a.n_req; r0 += 32) {
+    const Request r = r0 == 0 ? first : load(r0 + lane);
+    const uint32_t m = __ballot_sync(0xffffffffu, (!fit && r.log_parts > 0 ? 0 : r.log_parts) == k);
+    if (count < __popc(m)) {
+      const bool mine = (m >> lane & 1u) && __popc(m & ((1u << lane) - 1u)) == count;
+      const int src = __ffs(__ballot_sync(0xffffffffu, mine)) - 1;
+      it.req = r0 + src;
+      it.chunk = slot & ((1 << k) - 1);
+      it.n_chunks = 1 << k;
+      it.n_new = __shfl_sync(0xffffffffu, r.n_new, src);
+      it.prefix = __shfl_sync(0xffffffffu, r.prefix, src);
+      it.tok0 = __shfl_sync(0xffffffffu, r.tok0, src);
+      it.tbl0 = __shfl_sync(0xffffffffu, r.tbl0, src);
+      it.tbl_n = __shfl_sync(0xffffffffu, r.tbl_n, src);
+      return true;
+    }
+    count -= __popc(m);
+  }
+  return false;
+}
+
 // One CTA per (request, chunk of keys, KV head).  Rows = new tokens x query heads of the group
 // (at most 16).  The four warps take pages round-robin, each with its own double buffer, and merge
 // their partial (max, sum, O) through shared memory at the end.  The CTA that finishes a request's last chunk for its KV
@@ -267,33 +333,40 @@ __device__ __forceinline__ uint32_t load_word(const __nv_bfloat16* p) {
 // the kernel behind it does not start, before it.
 // CLUSTER: a few decode requests and nothing else.  No plan: the CTAs of a cluster share the pages of one (request, KV head) and
 // the first of them fetches the others' partial results from their shared memory.
+// PACKED: the same, with clusters of four that a long request has to itself and short ones share (find_share).
 constexpr int MAX_FEW_ROWS = 64;      // query rows per KV head, in all, of a batch served without a plan
-enum { PLAIN = 0, BESIDE = 1, CLUSTER = 2 };
+constexpr int PACK = 4;
+enum { PLAIN = 0, BESIDE = 1, CLUSTER = 2, PACKED = 3 };
 template <int MODE>
-__global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs a, int chunk) {
+__global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs a, int chunk, int n_slots) {
+  constexpr bool NO_PLAN = MODE == CLUSTER || MODE == PACKED;
   extern __shared__ __align__(128) unsigned char smem[];
   if (MODE != BESIDE || blockIdx.x == gridDim.x - 1) pdl_wait();
   pdl_launch_dependents();    // the next call's first kernel may set itself up; it waits for this grid before it reads anything
-  const int csize = MODE == CLUSTER ? chunk : 1;            // CTAs per cluster
+  const int csize = MODE == CLUSTER ? chunk : MODE == PACKED ? PACK : 1;            // CTAs per cluster
   const int item = blockIdx.x / csize / a.n_kv, h = blockIdx.x / csize % a.n_kv;
   if (MODE == BESIDE && item >= a.max_decode) return;
   DecodeItem it;
-  if (MODE == CLUSTER) {
-    it.req = item;
-    it.chunk = blockIdx.x % csize;
-    it.n_chunks = csize;
-    it.n_new = a.new_lens[item];
-    it.prefix = a.prefix_lens[item];
-    it.tok0 = a.req_indptr[item];
-    it.tbl0 = a.tbl_indptr[item];
-    it.tbl_n = a.tbl_indptr[item + 1] - it.tbl0;
-    if (it.n_new * (a.n_q / a.n_kv) <= (int)blockIdx.y * DEC_ROWS) return;       // (the same answer in the whole cluster)
+  if (NO_PLAN) {
+    if (MODE == PACKED) {
+      if (!find_share(a, item * PACK + blockIdx.x % PACK, n_slots, chunk, it)) return;       // (a cluster's barriers do without the CTAs that have left)
+    } else {
+      it.req = item;
+      it.chunk = blockIdx.x % csize;
+      it.n_chunks = csize;
+      it.n_new = a.new_lens[item];
+      it.prefix = a.prefix_lens[item];
+      it.tok0 = a.req_indptr[item];
+      it.tbl0 = a.tbl_indptr[item];
+      it.tbl_n = a.tbl_indptr[item + 1] - it.tbl0;
+    }
+    if (it.n_new * (a.n_q / a.n_kv) <= (int)blockIdx.y * DEC_ROWS) return;       // (the same answer in all of the request's CTAs)
     const int pages = (it.prefix + it.n_new + BT - 1) / BT;
     if (pages > it.tbl_n || it.n_new * (a.n_q / a.n_kv) > MAX_FEW_ROWS) {
       if (threadIdx.x == 0) atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_POS);
       return;
     }
-    chunk = max(4, (pages + csize - 1) / csize) * BT;       // a page for every warp at least
+    chunk = max(4, (pages + it.n_chunks - 1) / it.n_chunks) * BT;       // a page for every warp at least
   } else if (MODE == BESIDE) {
     const int4* src = reinterpret_cast<const int4*>(a.decode_list + item);
     const int4 lo = __ldcg(src), hi = __ldcg(src + 1);
@@ -302,14 +375,14 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
   } else {
     it = a.decode_list[item];
   }
-  if (MODE != CLUSTER && item >= (MODE == BESIDE ? __ldcg(&a.hdr->n_decode) : a.hdr->n_decode)) return;
+  if (!NO_PLAN && item >= (MODE == BESIDE ? __ldcg(&a.hdr->n_decode) : a.hdr->n_decode)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t4 = lane & 3;
   const int i = it.req, c = it.chunk;
   const int n_new = it.n_new, prefix = it.prefix, ctx = prefix + n_new;
   const int group = a.n_q / a.n_kv;
   // a plan's items have at most 16 rows; where there is none, clusters further back in the grid take a request's rows from 16 on
-  const int r0 = MODE == CLUSTER ? (int)blockIdx.y * DEC_ROWS : 0;
+  const int r0 = NO_PLAN ? (int)blockIdx.y * DEC_ROWS : 0;
   const int rows = min(DEC_ROWS, n_new * group - r0);
   const int tok0 = it.tok0;
   const int u_begin = c * chunk, u_end = min(ctx, u_begin + chunk);
@@ -317,7 +390,7 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
   const int tbl0 = it.tbl0, tbl_n = it.tbl_n;
   const int pg0 = u_begin / BT;
   // a chunk behind the end of the table has no keys to read; the request's other chunks then never count up to all of them
-  if (MODE != CLUSTER && pg0 + n_pages > tbl_n) {
+  if (!NO_PLAN && pg0 + n_pages > tbl_n) {
     if (tid == 0) atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_POS);
     return;
   }
@@ -414,7 +487,7 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
       L += ml.y * sc;
       o += red_o[(w * DEC_ROWS + r) * D + col] * sc;
     }
-    if (MODE == CLUSTER && csize > 1) {
+    if (NO_PLAN && it.n_chunks > 1) {
       float* const mine = reinterpret_cast<float*>(smem + CL_OFF);
       mine[e] = o;
       if (col == 0) reinterpret_cast<float2*>(smem + CL_OFF + DEC_ROWS * D * 4)[r] = make_float2(M, L);
@@ -428,9 +501,10 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
     }
   }
   if (it.n_chunks <= 1) return;
-  if (MODE == CLUSTER) {
+  if (NO_PLAN) {
     __syncwarp();
     cluster_sync();
+    const uint32_t first = blockIdx.x % csize;       // (read by the first of the request's CTAs)
     if (c == 0)
       for (int e = tid; e < rows * (D / 4); e += ATT_THREADS) {
         const int r = e / (D / 4);
@@ -440,9 +514,9 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
         float ref = -INFINITY;
 #pragma unroll
         for (int k = 0; k < 8; ++k)
-          if (k < csize) {
-            p[k] = ld_cluster_f32x4(map_cluster_rank(po, k));
-            ml[k] = ld_cluster_f32x2(map_cluster_rank(pm, k));
+          if (k < it.n_chunks) {
+            p[k] = ld_cluster_f32x4(map_cluster_rank(po, first + k));
+            ml[k] = ld_cluster_f32x2(map_cluster_rank(pm, first + k));
             ref = fmaxf(ref, ml[k].x);
           }
         if (ref == -INFINITY) ref = 0.f;
@@ -450,7 +524,7 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
         float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int k = 0; k < 8; ++k)
-          if (k < csize) {
+          if (k < it.n_chunks) {
             const float sc = exp2f(ml[k].x - ref);
             L += ml[k].y * sc;
             o.x += p[k].x * sc; o.y += p[k].y * sc; o.z += p[k].z * sc; o.w += p[k].w * sc;
@@ -623,8 +697,9 @@ int pick_chunk(int n_tbl, int n_kv) {
 }
 
 // CTAs that share the pages of a (request, KV head) where a few decode requests are served without a plan, 0 = with one.  Without it
-// the contexts' lengths are not known when the grid is chosen: enough CTAs that a warp has no more than about 40 pages (30 us) even
-// if one request had them all, more where SMs are idle and a CTA keeps eight pages, and a plan where that needs more than 600 CTAs.
+// the contexts' lengths are not known when the grid is chosen: enough CTAs that a CTA has no more than 160 + 4 n_req pages even if one
+// request had them all, more where SMs are idle and a CTA keeps eight pages; with more than one CTA each, a plan where that needs more than
+// 600 CTAs.  (packed_slots then looks at the batches of one long request.)
 // KV append and attention of a layer, with the plan and without.  7B: 1 request of 134 keys 12.5 and 9.4 us, of 3000 28.8 and 19.8;
 // 3 of 140 14.6 and 10.5; 8 of 550 34.3 and 27.9; 16 of 130 32.5 and 20.2; 26 of 95 29.6 and 22.8; 40 of 60 29.2 and 26.5; but 8 of
 // 1500 50 and 61.  34B: 3 of 2000 40.3 and 17.2, 8 of 550 21.3 and 12.2 us.  13B: 30 of 95 34.5 and 28.2; but 9 of 1200 55 and 77 us.
@@ -636,6 +711,31 @@ int cluster_size(int n_req, int n_tbl, int n_kv, int sms) {
   if (cs > 8 || (cs > 1 && units * cs > 600)) return 0;
   while (cs < 8 && units * cs * 2 <= 2 * sms && n_tbl >= 16ll * cs * n_req) cs *= 2;
   return cs;
+}
+
+// A batch whose n_tbl entries may be one request's nearly all: with the same number of CTAs for every request that one would keep a warp
+// busy with more than 25 to 37 pages and some more for every other request (the plan's time grows with them too).  Then a request gets
+// CTAs as it has pages: `slots` of them per KV head (a request of p pages takes at most 1 + 1.5 p / part_pages), 0 = the same number for
+// each, -1 = a plan.  Small parts as long as all CTAs run at once or nearly so; where even the large ones take twice that, the many short
+// requests are better off with a CTA each, and from 200 pages on with a plan.
+// Attention with the same number of CTAs, as here, and with the plan (of the tree that had nothing else).  One request has nearly all: 7B, 5 requests,
+// 2560 keys 37, 14 and 24 us; 8, 3200 keys 30, 15, 29; 12, 2560 keys 41, 16, 26; 13B, 8, 2560 keys 42, 17, 27.  One has four times as many as the
+// others: 13B, 4 requests of 600 keys 29, 15, 23; 7B, 6 22, 15, 23.  Lengths from one to eight times the shortest: 7B, 5 of 350 keys
+// 13.4, 13.2, 23; 8 of 370 14.4, 13.3, 19; 16 of 180 13.3, 15.2, 20; a layer of 8 KV heads, 16 of 370 11.3, 10.6, 20.
+struct Packed {
+  int slots, part_pages;
+};
+Packed packed_slots(int n_req, int n_tbl, int n_kv, int csize, int sms) {
+  const int longest = n_tbl - n_req + 1;
+  if (n_req < 2 || csize >= PACK || longest <= (csize == 1 ? 100 : 150) + n_req * csize) return {0, 0};
+  Packed p = {0, 0};
+  for (int pages : {16, 24, 32, 48}) {
+    p.part_pages = pages;
+    p.slots = (std::min(n_req + n_tbl * 3 / (2 * pages), PACK * n_req) + PACK - 1) / PACK * PACK;
+    if (p.slots * n_kv <= 4 * sms) return p;
+  }
+  if (p.slots * n_kv > 6 * sms) p.slots = longest > 200 ? -1 : 0;
+  return p;
 }
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -718,6 +818,7 @@ int fl_paged_attention(fl_pool* p, fl_bf16* out, const fl_bf16* q, const int32_t
       if (cudaFuncSetAttribute(attn_decode_kernel<PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, DEC_SMEM) != cudaSuccess ||
           cudaFuncSetAttribute(attn_decode_kernel<BESIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, DEC_SMEM) != cudaSuccess ||
           cudaFuncSetAttribute(attn_decode_kernel<CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize, DEC_SMEM) != cudaSuccess ||
+          cudaFuncSetAttribute(attn_decode_kernel<PACKED>, cudaFuncAttributeMaxDynamicSharedMemorySize, DEC_SMEM) != cudaSuccess ||
           cudaFuncSetAttribute(attn_prefill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PRE_SMEM) != cudaSuccess) {
         p->last_cuda = (int)cudaGetLastError();
         rc = FL_ECUDA;
@@ -737,9 +838,13 @@ int fl_paged_attention(fl_pool* p, fl_bf16* out, const fl_bf16* q, const int32_t
     const int passes = max_items == 0 ? 1 : (n_tokens * group + DEC_ROWS - 1) / DEC_ROWS;
     const bool few = max_items == 0 || (n_tokens <= n_req && n_tokens * group <= MAX_FEW_ROWS && (long long)n_req * n_kv_heads * passes <= 6000);
     const int csize = kind == 0 && few ? cluster_size(n_req, n_tbl, n_kv_heads, p->sm_count) : 0;
-    if (csize > 0) {
-      const cudaError_t e = launch_pdl_cluster(attn_decode_kernel<CLUSTER>, dim3((unsigned)(n_req * n_kv_heads * csize), (unsigned)passes), dim3((unsigned)csize),
-                                               dim3(ATT_THREADS), DEC_SMEM, st, a, csize);
+    const Packed packed = csize > 0 ? packed_slots(n_req, n_tbl, n_kv_heads, csize, p->sm_count) : Packed{-1, 0};
+    if (packed.slots >= 0) {
+      const cudaError_t e =
+          packed.slots > 0 ? launch_pdl_cluster(attn_decode_kernel<PACKED>, dim3((unsigned)(packed.slots * n_kv_heads), (unsigned)passes), dim3(PACK),
+                                                dim3(ATT_THREADS), DEC_SMEM, st, a, packed.part_pages, packed.slots)
+                    : launch_pdl_cluster(attn_decode_kernel<CLUSTER>, dim3((unsigned)(n_req * n_kv_heads * csize), (unsigned)passes), dim3((unsigned)csize),
+                                         dim3(ATT_THREADS), DEC_SMEM, st, a, csize, 0);
       if (e != cudaSuccess) {
         p->last_cuda = (int)e;
         rc = FL_ECUDA;
@@ -763,7 +868,7 @@ int fl_paged_attention(fl_pool* p, fl_bf16* out, const fl_bf16* q, const int32_t
       attn_prefill_kernel<<<(unsigned)w.max_prefill * n_q_heads, ATT_THREADS, PRE_SMEM, st>>>(a);
     }
     cudaError_t e = launch_pdl(beside ? attn_decode_kernel<BESIDE> : attn_decode_kernel<PLAIN>, dim3((unsigned)w.max_decode * n_kv_heads + (beside ? 1u : 0u)),
-                               dim3(ATT_THREADS), DEC_SMEM, st, a, w.chunk);
+                               dim3(ATT_THREADS), DEC_SMEM, st, a, w.chunk, 0);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {
       p->last_cuda = (int)e;

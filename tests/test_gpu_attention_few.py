@@ -19,7 +19,11 @@ from _util import assert_close, oracle_context
     ((4, 4), [0], [1]), ((4, 4), [15], [1]), ((4, 4), [16, 600], [1, 0]), ((2, 2), [63, 64, 65], [1, 1, 1]), ((4, 4), [40, 0], [9, 7]),
     ((8, 8), [2600], [1]), ((8, 2), [1000, 17], [1, 3]), ((8, 1), [130, 131], [1, 1]), ((16, 16), [100 + 7 * i for i in range(16)], [1] * 16),
     ((1, 1), [511, 0, 5], [3, 12, 1]), ((4, 4), [5 * i for i in range(40)], [1] * 40), ((8, 1), [700, 3, 0, 90, 16], [1, 1, 1, 2, 0]),
-    ((2, 2), [30, 9] + [7] * 30, [25, 6] + [0] * 30), ((16, 2), [2000, 31, 600], [1, 1, 1])])
+    ((2, 2), [30, 9] + [7] * 30, [25, 6] + [0] * 30), ((16, 2), [2000, 31, 600], [1, 1, 1]),
+    # one or a few requests hold most of the pages: a request gets one, two or four CTAs, the short ones share a cluster
+    ((4, 4), [4000] + [5] * 11, [1] * 12), ((16, 16), [1200, 10, 700, 31, 300] + [9] * 11, [1] * 16), ((4, 4), [2] * 39 + [2600], [1] * 40),
+    ((16, 16), [383, 384, 767, 768, 1200] + [1] * 11, [1] * 16), ((32, 32), [767, 768, 1535, 1536] + [1] * 4, [1] * 8), ((8, 1), [4300, 3, 40, 700] + [3] * 11 + [20], [1, 1, 2, 1] + [0] * 11 + [1]),
+    ((4, 4), [1900, 40] + [8] * 34 + [530], [2, 1] + [0, 1] * 17 + [3])])
 def test_few_decode_requests(heads, prefix, new):
     from paper_2505_03756_b200 import harness as H
     wl = synth.make_workload("tiny", n_req=len(new), len_range=(0, 0), n_adapters=1, shape=synth.LayerShape(heads[0] * 128, *heads))
