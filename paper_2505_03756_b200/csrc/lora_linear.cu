@@ -689,15 +689,13 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
   a.scale = scale;
   a.v = reinterpret_cast<const float*>(workspace);
   a.m_tiles = (n_tokens + 2 * BM - 1) / (2 * BM);
+  // Up to 256 tokens another kernel may be the faster one, which streams W once for all of them (skinny::serves).
   // Segments of a few tokens each (a large decode batch): a tile would take a LoRA stage per segment or two, each for a
   // handful of rows.  Then the GEMM computes x W alone and the segmented projection adds the LoRA term to y afterwards.
-  // Up to 256 tokens W is streamed once for all of them, by a kernel of its own.  Above 128 its stages are mostly x and its
-  // LoRA stages are filled one at a time: more than eight of them, 64 ranks each, and the two-step way is the faster one
-  // (q, k, v and o of 194 tokens on 7B, 38 adapters of rank 16: 90 against 96 us; of 160 tokens on 13B, 75 of rank 32: 141 against
-  // 173 us; of 256 tokens with one adapter 101 against 99 us; of 96 tokens on 7B, 66 of rank 64: 144 against 133 us).
+  // A batch of one tile takes up to 16 stages all the same, and is rounded once.
   const int rank_max = p->max_rank <= 16 ? 16 : (p->max_rank <= 32 ? 32 : 64);
-  const bool few = n_tokens <= skinny::MAX_TOKENS && (n_tokens <= 128 || n_seg * rank_max <= 8 * 64 || n_tokens > 16 * n_seg);
-  const bool hybrid = !few && n_seg > 0 && n_tokens <= 16 * n_seg;
+  const bool few = skinny::serves(p, a.d_out, n_mats, a.d_in, n_tokens, n_seg, rank_max);
+  const bool hybrid = !few && n_seg > 0 && n_tokens <= 16 * n_seg && (n_tokens > 2 * BM || n_seg * rank_max > 16 * ER);
   if (hybrid) a.n_seg = 0;
   for (int j = 0; j < MAX_LIN; ++j) a.kv_side[j] = -1;
   if (kv) {

@@ -609,6 +609,15 @@ __global__ void __launch_bounds__(MAX_THREADS, 1) lora_skinny_kernel(const __gri
   }
 }
 
+// As many CTAs per column tile as the SMs hold at once (clusters above two do not fill every SM), every one with at least four
+// stages of d_in.
+int cluster_split(const fl_pool* p, int tiles, int nk) {
+  int split = 1;
+  for (int s = 2; s <= MAX_SPLIT; ++s)
+    if (tiles * s <= (s == 2 ? p->sm_count : p->sm_count * 9 / 10) && nk / s >= 4) split = s;
+  return split;
+}
+
 // Tiles, split of d_in, rings and shared memory of a call.
 void layout(const fl_pool* p, const skinny::Args& a, KArgs* out, uint32_t* smem) {
   KArgs& ka = *out;
@@ -624,12 +633,8 @@ void layout(const fl_pool* p, const skinny::Args& a, KArgs* out, uint32_t* smem)
   ka.tmem_cols = ka.npad > 128 ? 512 : 256;
   const uint32_t fixed = BOOK_BYTES + ROWS_BYTES + ka.npad * UNITS_PER_TOKEN * sizeof(LoraUnit) + 1024;
   const uint32_t stage = W_BYTES + (uint32_t)ka.npad * 128;
-  // As many CTAs per column tile as the SMs hold at once (clusters above two do not fill every SM), every one with at least
-  // four stages of d_in.
   const int nk = (a.d_in + BK - 1) / BK;
-  ka.split = 1;
-  for (int s = 2; s <= MAX_SPLIT; ++s)
-    if (tiles * s <= (s == 2 ? p->sm_count : p->sm_count * 9 / 10) && nk / s >= 4) ka.split = s;
+  ka.split = cluster_split(p, tiles, nk);
   // The two rings share the memory as a CTA's main stages and LoRA stages (at most; ranks may be lower) share its work: both
   // are bound by the bytes they have in flight.
   const int lora = (a.n_seg * ((a.rmax + UNIT - 1) / UNIT) + 3) / 4;
@@ -649,6 +654,31 @@ void layout(const fl_pool* p, const skinny::Args& a, KArgs* out, uint32_t* smem)
 }  // namespace
 
 namespace skinny {
+
+// Up to 128 tokens always.  Above that a CTA brings 48 KB of x and W per stage for 128 columns where one of the GEMM for long batches
+// brings 32 KB for as many, while the GEMM takes a tile's LoRA stages (up to 32 ranks each) one after the other.
+//  - More than 16 such stages: here.  q, k, v of 200 tokens, twelve segments of rank 64, here and there: 7B 56 and 64 us, 13B 66 and 72,
+//    34B 85 and 81; o of 230 tokens on 7B 33 and 39.
+//  - d_in not split (q, k, v as a rule): here up to 176 tokens, unless one adapter serves them all (from 144 on the GEMM).  q, k, v of 176
+//    tokens, rank 16, one segment: 7B 38 and 31 us, 13B 51 and 38, 34B 59 and 49; eight segments 40 and 41, 53 and 50, 61 and 62; of 256
+//    tokens 46 and 37, 60 and 46, 72 and 58.
+//  - d_in split, at least 16 stages per CTA (o): the GEMM leaves half of the SMs idle.  Here up to 208 tokens; beyond, the sum over
+//    the cluster wants 24 stages to be small against.  o of 176 tokens, four segments: 7B 24 and 27 us, 13B 25 and 32, 34B 38 and 50; of 256
+//    29 and 28, 29 and 32, 45 and 50.
+//  - d_in split, fewer stages: here for many LoRA stages up to 176 tokens only.  A layer of 1024 hidden values, q, k, v of 144 tokens:
+//    8 segments of rank 16 23 and 19 us, 24 segments 26 and 25, o 16 and 21.
+// More than 512 ranks over short segments: the two-step way (q, k, v and o of 160 tokens on 13B, 75 adapters of rank 32: 173 us here, 141).
+bool serves(const fl_pool* p, const int* d_out, int n_mats, int d_in, int n_tokens, int n_seg, int rank_max) {
+  if (n_tokens <= 128) return true;
+  if (n_tokens > MAX_TOKENS || (n_seg * rank_max > 8 * 64 && n_tokens <= 16 * n_seg)) return false;
+  int tiles = 0;
+  for (int j = 0; j < n_mats; ++j) tiles += (d_out[j] + BN - 1) / BN;
+  const int nk = (d_in + BK - 1) / BK, split = cluster_split(p, tiles, nk);
+  if (n_seg * rank_max > 16 * 32) return true;
+  if (split == 1) return n_tokens <= 176 && (n_seg > 1 || n_tokens < 144);
+  if (nk / split < 16) return n_seg * rank_max > 8 * 32 && n_tokens <= 176;
+  return n_tokens <= 208 || nk / split >= 24;
+}
 
 int launch(fl_pool* p, const Args& a, const void* x, const void* const* w, cudaStream_t st) {
   KArgs ka;

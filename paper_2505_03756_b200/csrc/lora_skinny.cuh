@@ -24,6 +24,9 @@ struct Args {
   int n_req, n_kv, bt;
 };
 
+// Whether `launch` is the faster way for a call (n_seg = 0: no adapters).
+bool serves(const fl_pool* p, const int* d_out, int n_mats, int d_in, int n_tokens, int n_seg, int rank_max);
+
 // y = x W + (scaled x A) B for n_tokens <= MAX_TOKENS.  With n_seg > 0 the shrink that writes v must be the launch right
 // before this one on the stream.
 int launch(fl_pool* p, const Args& a, const void* x, const void* const* w, cudaStream_t st);

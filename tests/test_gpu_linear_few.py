@@ -32,7 +32,8 @@ def _workload(T, shape, per_req, n_adapters):
 @pytest.mark.parametrize("T,per_req,hidden,heads", [
     (1, 1, 1024, (8, 8)), (2, 1, 4096, (32, 32)), (15, 1, 328, (3, 1)), (16, 16, 328, (3, 1)), (17, 1, 1024, (8, 8)),
     (33, 11, 200, (2, 1)), (127, 1, 1024, (8, 8)), (129, 43, 328, (3, 1)), (200, 100, 1024, (8, 2)), (255, 1, 328, (3, 1)),
-    (256, 256, 1024, (8, 8)), (256, 1, 2048, (4, 1)), (257, 1, 328, (3, 1))])
+    (256, 256, 1024, (8, 8)), (256, 1, 2048, (4, 1)), (257, 1, 328, (3, 1)),
+    (176, 44, 4096, (8, 8)), (177, 1, 4096, (64, 8)), (209, 9, 1024, (8, 8))])
 def test_linear_of_few_tokens(T, per_req, hidden, heads):
     from paper_2505_03756_b200 import binding as fl, harness as H
     wl = _workload(T, synth.LayerShape(hidden, *heads), per_req, 12)
