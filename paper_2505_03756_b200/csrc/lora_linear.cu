@@ -797,7 +797,7 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
     }
     for (int j = n_mats; j < MAX_LIN; ++j) maps.w[j] = maps.w[0];
     if (rc != FL_OK) break;
-    sgmv::ShrinkInfo info = {1, p->max_rank <= 16 ? 16 : (p->max_rank <= 32 ? 32 : 64)};
+    sgmv::ShrinkInfo info = {1, rank_max};
     if (hybrid) {
       // y = x W from the GEMM alone, then the segmented projection adds the LoRA term to it
       a.ksplit = 1;
@@ -817,11 +817,17 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
       break;
     }
     if (n_seg > 0) {
-      // Where segments are short (128 tokens on average) tiles need many LoRA stages, and the shrink in tiles of 16 tokens, which
-      // leaves its result final, is the better one: the others split d_in to fill the SMs, and a stage that sums fp32 slices
-      // takes 5600 cycles instead of 1500 (q, k, v of 28 one-token segments and 4 prompts on 7B, ranks 8 to 64: 149 -> 131 us; of
-      // one prompt of 1024 tokens on 34B, rank 64, the other way round 199 and 216 us).
-      const bool final = n_tokens <= 128 * n_seg;
+      // Two shrinks: in tiles of 16 tokens, whose result is final, and in tiles of 64 (rank 16) or 128 tokens, which read the adapters' rows
+      // less often but split d_in where tiles are few, and a LoRA stage that sums fp32 slices takes 5600 cycles instead of 1500.  The
+      // first one is the better one as long as a segment's x and the rows that it reads again are few (at rank 64, where it reads the
+      // most, as long as the batch is small too).  q, k, v, first and second one: rank 16, 7B, 288 tokens, 20 per segment 64 and 67 us, 72
+      // per segment 59 and 54; 1000 tokens of 1024 values, 100 per segment 23 and 25.  Rank 32, 7B, 1024 tokens, 20 per segment 116 and 162, 102
+      // 95 and 92; 1024 values, 100 26 and 29.  Rank 64, 7B, 1024 tokens, 20 per segment 158 and 294, 102 99 and 112, 8192 tokens, 128 per
+      // segment 780 and 707; 34B, 16384 tokens, 128 per segment 2570 and 2096 us.  Over 960 such batches the choice is 1 % behind the
+      // better one.
+      const double per = (double)n_tokens / n_seg * a.d_in;
+      const bool final = rank_max == 16 ? per <= 1.7e5 : rank_max == 32 ? per <= 3e5
+                       : n_tokens <= 40 * n_seg || (n_tokens <= 128 * n_seg && per * n_tokens <= 4e8);
       rc = final ? sgmv::shrink_scaled(p, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace, v_bytes,
                                        stream, &info)
                  : sgmv::shrink(p, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, workspace, v_bytes, stream, &info);
