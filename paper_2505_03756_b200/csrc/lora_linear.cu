@@ -47,12 +47,12 @@ constexpr int RASTER = 8;                        // token tiles that are walked 
 constexpr uint32_t A_BYTES = BM * BK * 2;        // x tile, K-major: 128 rows of 128 bytes
 constexpr uint32_t B_GROUP = BK * 128;           // one 64-column group of a W tile: 64 k-rows of 128 bytes
 
-template <int BN>
+template <int BN, int G>
 struct Cfg {
-  static constexpr int BH = BN / 2;                           // columns of W this CTA loads
+  static constexpr int BH = BN / G;                           // columns of W this CTA loads
   static constexpr uint32_t B_BYTES = (BH / 64) * B_GROUP;
   static constexpr uint32_t STAGE = A_BYTES + B_BYTES;
-  static constexpr int NS = BN == 256 ? 5 : 7;
+  static constexpr int NS = G == 1 ? 3 : BN == 256 ? 5 : 7;
   // two LoRA stages side by side in one buffer of a main stage's layout: ranks 0-31 and 32-63 of every row
   static constexpr uint32_t OFF_EXT = NS * STAGE;
   static constexpr uint32_t OFF_ROWS = OFF_EXT + STAGE;       // B row addresses of two groups of LoRA stages
@@ -157,16 +157,17 @@ __device__ __noinline__ void add_nonfinite_terms(const LinArgs& a, int j, int to
   }
 }
 
-template <int BN, int RMAX>
+template <int BN, int RMAX, int G>
 __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid_constant__ LinArgs a, const __grid_constant__ LinMaps maps) {
-  using C = Cfg<BN>;
+  using C = Cfg<BN, G>;
+  constexpr int TM = G * BM;                 // token rows of a tile
   constexpr int NS = C::NS, BH = C::BH;
   extern __shared__ unsigned char smem_raw[];
   // the swizzled operand tiles need 1024-byte alignment
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const uint32_t sbase = smem_u32(smem);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int crank = (int)cluster_ctarank();
+  const int crank = G == 2 ? (int)cluster_ctarank() : 0;
   const bool leader = crank == 0;
   enum { B_FULL = 0, B_EMPTY = NS, B_ACC_FULL = 2 * NS, B_ACC_EMPTY = B_ACC_FULL + 2, B_EFULL = B_ACC_EMPTY + 2, B_EEMPTY = B_EFULL + 2,
          B_LFULL = B_EEMPTY + 2, B_LEMPTY = B_LFULL + 2, B_IDLE = B_LEMPTY + 2, B_COUNT };
@@ -187,8 +188,8 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(bar(B_ACC_FULL + b), 1);
-      mbar_init(bar(B_ACC_EMPTY + b), 8);      // the epilogue warps of both CTAs
-      mbar_init(bar(B_EFULL + b), 2);          // both CTAs' fillers
+      mbar_init(bar(B_ACC_EMPTY + b), 4 * G);      // the epilogue warps of both CTAs
+      mbar_init(bar(B_EFULL + b), G);              // both CTAs' fillers
       mbar_init(bar(B_EEMPTY + b), 1);
       mbar_init(bar(B_LFULL + b), 1);
       mbar_init(bar(B_LEMPTY + b), 1);
@@ -199,12 +200,17 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void*)tmem_slot)), "r"(C::TMEM_COLS) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    if constexpr (G == 2) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void*)tmem_slot)), "r"(C::TMEM_COLS) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32((const void*)tmem_slot)), "r"(C::TMEM_COLS) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
   }
   tc_fence_before();
   __syncthreads();
-  cluster_sync();          // both CTAs' barriers exist
+  if (G == 2) cluster_sync();          // both CTAs' barriers exist
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   // Behind the shrink everything but v was finished before this kernel could start (the shrink lets it start after its own
@@ -213,7 +219,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
 
   const int total = a.tile_base[a.n_mats];
   const int nk = (a.d_in + BK - 1) / BK;
-  const int first = blockIdx.x >> 1, step = gridDim.x >> 1;      // pairs
+  const int first = blockIdx.x / G, step = gridDim.x / G;        // pairs
   int fills = 0;                                                 // stages that this CTA's producer has issued
 
   if (warp == 0) {
@@ -227,15 +233,15 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
       for (int idx = first; ok && idx < total; idx += step) {
         const Tile t = decode_tile(a, idx);
         const CUtensorMap* wm = &maps.w[t.j];
-        const int row0 = t.m * (2 * BM) + crank * BM, col0 = t.n * BN + crank * BH;
+        const int row0 = t.m * TM + crank * BM, col0 = t.n * BN + crank * BH;
         for (int ks = 0; ks < nk; ++ks) {
           if (wrapped) ok = mbar_wait(bar(B_EMPTY + s), ph, abort_flag);
           if (!ok) break;
-          if (leader) mbar_expect_tx(bar(B_FULL + s), 2 * C::STAGE);
+          if (leader) mbar_expect_tx(bar(B_FULL + s), G * C::STAGE);
           const uint32_t dst = sbase + s * C::STAGE, fb = full0 + 8u * s;
-          tma_load_2d_pair(dst, &maps.x, fb, ks * BK, row0);
+          tma_load_2d_group<G>(dst, &maps.x, fb, ks * BK, row0);
 #pragma unroll
-          for (int g = 0; g < BH / 64; ++g) tma_load_2d_pair(dst + A_BYTES + g * B_GROUP, wm, fb, col0 + g * 64, ks * BK);
+          for (int g = 0; g < BH / 64; ++g) tma_load_2d_group<G>(dst + A_BYTES + g * B_GROUP, wm, fb, col0 + g * 64, ks * BK);
           ++fills;
           if (++s == NS) { s = 0; ph ^= 1u; wrapped = true; }
         }
@@ -244,7 +250,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer: the whole warp runs converged, an elected lane issues
     if (leader) {
-      constexpr uint32_t IDESC = instr_desc_pair(BN, true);     // A (x, v) K-major, B (W, adapter rows) N-contiguous
+      constexpr uint32_t IDESC = G == 2 ? instr_desc_pair(BN, true) : instr_desc(BN, true);     // A (x, v) K-major, B (W, adapter rows) N-contiguous
       constexpr uint32_t HI = desc_hi(1024);
       auto wait_all = [&](uint32_t b, uint32_t parity) {
         if (__all_sync(0xffffffffu, mbar_try_cluster(b, parity))) return true;       // the common case: one test
@@ -271,8 +277,8 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
           const uint32_t a_lo = a_lo0 + s * (C::STAGE >> 4), b_lo = b_lo0 + s * (C::STAGE >> 4);
 #pragma unroll
           for (int q = 0; q < BK / 16; ++q)
-            umma_ss_pair_elect(d, a_lo + q * 2, HI, b_lo + q * (16 * 128 / 16), HI, IDESC, st > 0 || q > 0 ? 1u : 0u);
-          umma_commit_pair_elect(bar(B_EMPTY + s));
+            umma_ss_group_elect<G>(d, a_lo + q * 2, HI, b_lo + q * (16 * 128 / 16), HI, IDESC, st > 0 || q > 0 ? 1u : 0u);
+          umma_commit_group_elect<G>(bar(B_EMPTY + s));
           if (++s == NS) { s = 0; ph ^= 1u; }
           if (st >= half) {
             if (st == half && a.n_seg > 0) {
@@ -289,15 +295,15 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
               tc_fence_after();
 #pragma unroll
               for (int q = 0; q < ER / 16; ++q)
-                umma_ss_pair_elect(d, ea_lo0 + es * (ER * 2 / 16) + q * 2, HI, eb_lo0 + es * (ER * 128 / 16) + q * (16 * 128 / 16), HI, IDESC, 1u);
-              umma_commit_pair_elect(bar(B_EEMPTY + es));
+                umma_ss_group_elect<G>(d, ea_lo0 + es * (ER * 2 / 16) + q * 2, HI, eb_lo0 + es * (ER * 128 / 16) + q * (16 * 128 / 16), HI, IDESC, 1u);
+              umma_commit_group_elect<G>(bar(B_EEMPTY + es));
               es ^= 1;
               if (es == 0) eph ^= 1u;
             }
             if (!ok) break;
           }
         }
-        if (ok) umma_commit_pair_elect(bar(B_ACC_FULL + buf));
+        if (ok) umma_commit_group_elect<G>(bar(B_ACC_FULL + buf));
       }
     }
   } else if (warp < 6) {
@@ -312,7 +318,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
     for (int idx = first; idx < total; idx += step, ++k) {
       const Tile t = decode_tile(a, idx);
       const int buf = k & 1;
-      const int tok = t.m * (2 * BM) + crank * BM + row;
+      const int tok = t.m * TM + crank * BM + row;
       const int d_out = a.d_out[t.j];
       const int n0 = t.n * BN;
       const int side = a.kv_side[t.j];
@@ -408,7 +414,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
     if (a.n_seg > 0) pdl_wait();             // v is the shrink's output
     for (int idx = first; a.n_seg > 0 && ok && idx < total; idx += step, ++k) {
       const Tile t = decode_tile(a, idx);
-      const int tok0 = t.m * (2 * BM), tok1 = min(a.n_tokens, tok0 + 2 * BM);
+      const int tok0 = t.m * TM, tok1 = min(a.n_tokens, tok0 + TM);
       // ---- the tile's units, in segment order
       int lo_s = 0, hi_s = a.n_seg;          // first segment that ends behind tok0
       while (lo_s < hi_s) {
@@ -481,7 +487,9 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
                 const unsigned char* p = a.pv.slab + (size_t)blk * a.pv.block_bytes + ((size_t)(gr % lm.b_rpb) * d_out + col0) * 2;
                 at = reinterpret_cast<unsigned long long>(p);
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-                if (BH > 64 && col0 + 64 < d_out) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + 128));
+#pragma unroll
+                for (int g = 1; g < BH / 64; ++g)
+                  if (col0 + 64 * g < d_out) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + 128 * g));
               }
             }
           }
@@ -570,7 +578,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
           }
           // both CTAs' rows meet these columns
           *nonfinite_slot = 1;
-          st_cluster_u32(map_cluster_rank(smem_u32(const_cast<int*>(nonfinite_slot)), (uint32_t)(crank ^ 1)), 1u);
+          if (G == 2) st_cluster_u32(map_cluster_rank(smem_u32(const_cast<int*>(nonfinite_slot)), (uint32_t)(crank ^ 1)), 1u);
         }
         fence_async_smem();                              // the tensor core reads shared memory through the async proxy
         asm volatile("bar.sync %0, 128;" ::"r"(3 + slot) : "memory");
@@ -584,53 +592,58 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
   // ------------------------------------------------ teardown: neither CTA leaves while the other's MMAs or arrivals need it
   tc_fence_before();
   __syncthreads();
-  if (tid == 0) {
-    const uint32_t to = map_cluster_rank(smem_u32(const_cast<int*>(partner_slot)), (uint32_t)(crank ^ 1));
-    st_cluster_u32(to, (uint32_t)*abort_flag);
-    st_cluster_u32(to + 4, (uint32_t)fills);
+  if (G == 2) {
+    if (tid == 0) {
+      const uint32_t to = map_cluster_rank(smem_u32(const_cast<int*>(partner_slot)), (uint32_t)(crank ^ 1));
+      st_cluster_u32(to, (uint32_t)*abort_flag);
+      st_cluster_u32(to + 4, (uint32_t)fills);
+    }
+    __syncwarp();
+    cluster_sync();
   }
-  __syncwarp();
-  cluster_sync();
-  if (*abort_flag || partner_slot[0]) {      // the same answer in both CTAs
+  if (*abort_flag || (G == 2 && partner_slot[0])) {      // the same answer in both CTAs
     if (tid == 0) atomicOr(a.pv.flags, (uint32_t)FLAG_WAIT_GAVE_UP);
     // Copies and MMAs still in flight use both CTAs' shared memory and TMEM; the first CTA's barriers count them all.
-    if (leader && warp == 1) umma_commit_pair_elect(bar(B_IDLE));
+    if (leader && warp == 1) umma_commit_group_elect<G>(bar(B_IDLE));
     if (leader && tid == 0) {
-      const long long armed = giveup::settle_pair(fills, partner_slot[1], NS, [&](int s) { mbar_expect_tx(bar(B_FULL + s), C::STAGE); },
+      const long long armed = giveup::settle_pair(fills, G == 2 ? partner_slot[1] : fills, NS, [&](int s) { mbar_expect_tx(bar(B_FULL + s), C::STAGE); },
                                                   [&](int s) { mbar_complete_tx(bar(B_FULL + s), C::STAGE); });
       giveup::drain(armed, NS, [&](int s, uint32_t parity) { return mbar_try_cluster(bar(B_FULL + s), parity); });
       giveup::drain(1, 1, [&](int, uint32_t parity) { return mbar_try_cluster(bar(B_IDLE), parity); });
     }
     __syncthreads();
-    cluster_sync();
+    if (G == 2) cluster_sync();
   }
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::TMEM_COLS) : "memory");
+    if constexpr (G == 2) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::TMEM_COLS) : "memory");
+    else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::TMEM_COLS) : "memory");
   }
 }
 
-template <int BN, int RMAX>
+template <int BN, int RMAX, int G>
 int launch_linear(fl_pool* p, const LinArgs& a, const LinMaps& maps, cudaStream_t st) {
-  using C = Cfg<BN>;
+  using C = Cfg<BN, G>;
   static bool configured[16] = {};
   if (!configured[p->device & 15]) {
-    FL_CUDA(p, cudaFuncSetAttribute(lora_linear_kernel<BN, RMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM));
+    FL_CUDA(p, cudaFuncSetAttribute(lora_linear_kernel<BN, RMAX, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM));
     configured[p->device & 15] = true;
   }
   const int total = a.tile_base[a.n_mats];
-  const unsigned pairs = (unsigned)std::min(total, p->sm_count / 2);
-  FL_CUDA(p, launch_pdl_cluster(lora_linear_kernel<BN, RMAX>, dim3(2 * pairs), dim3(2), dim3(LT_THREADS), C::SMEM, st, a, maps));
+  const unsigned groups = (unsigned)std::min(total, p->sm_count / G);
+  FL_CUDA(p, launch_pdl_cluster(lora_linear_kernel<BN, RMAX, G>, dim3(G * groups), dim3(G), dim3(LT_THREADS), C::SMEM, st, a, maps));
   FL_CUDA(p, cudaGetLastError());
   return FL_OK;
 }
 
-int launch_width(fl_pool* p, const LinArgs& a, const LinMaps& maps, cudaStream_t st, int bn, int rmax) {
-  if (bn == 256)
-    return rmax == 16 ? launch_linear<256, 16>(p, a, maps, st)
-         : rmax == 32 ? launch_linear<256, 32>(p, a, maps, st) : launch_linear<256, 64>(p, a, maps, st);
-  return rmax == 16 ? launch_linear<128, 16>(p, a, maps, st)
-       : rmax == 32 ? launch_linear<128, 32>(p, a, maps, st) : launch_linear<128, 64>(p, a, maps, st);
+template <int BN, int G>
+int launch_rank(fl_pool* p, const LinArgs& a, const LinMaps& maps, cudaStream_t st, int rmax) {
+  return rmax == 16 ? launch_linear<BN, 16, G>(p, a, maps, st)
+       : rmax == 32 ? launch_linear<BN, 32, G>(p, a, maps, st) : launch_linear<BN, 64, G>(p, a, maps, st);
+}
+int launch_width(fl_pool* p, const LinArgs& a, const LinMaps& maps, cudaStream_t st, int bn, int group, int rmax) {
+  return group == 1 ? launch_rank<256, 1>(p, a, maps, st, rmax)
+       : bn == 256 ? launch_rank<256, 2>(p, a, maps, st, rmax) : launch_rank<128, 2>(p, a, maps, st, rmax);
 }
 
 }  // namespace
@@ -688,7 +701,6 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
   a.n_tokens = n_tokens;
   a.scale = scale;
   a.v = reinterpret_cast<const float*>(workspace);
-  a.m_tiles = (n_tokens + 2 * BM - 1) / (2 * BM);
   // Up to 256 tokens another kernel may be the faster one, which streams W once for all of them (skinny::serves).
   // Segments of a few tokens each (a large decode batch): a tile would take a LoRA stage per segment or two, each for a
   // handful of rows.  Then the GEMM computes x W alone and the segmented projection adds the LoRA term to y afterwards.
@@ -722,19 +734,23 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
     a.n_kv = kv->n_kv;
     a.bt = (int)(p->block_bytes / per_tok);
   }
-  // Columns per tile, 256 or 128: the width whose rounds over the pairs of SMs cost less.  A round of 128 columns takes about
-  // 16.5 us where one of 256 takes 20 (d_in 4096): both are bound by the 64 bytes per clock that an SM gets from L2, 32 KB per
-  // k-step at 256 columns and 24 KB at 128.
-  int bn = 256;
+  // Tiles of 256 or 128 columns per pair of CTAs, or 128 tokens x 256 columns per CTA: the one whose rounds over the SMs cost less.  All are
+  // bound by the 64 bytes per clock that an SM gets from L2: 32 KB per k-step for a pair's 256 columns, 24 KB for its 128 (a round of
+  // d_in 4096 takes 20 and 16.5 us), 48 KB for a CTA by itself.  That one is for batches of 257 to 384 tokens, whose second tile of 256
+  // is mostly empty but costs the pairs a second round (q, k, v of 300 tokens, one adapter of rank 16: 34B 90 -> 78 us, 7B 52 -> 47).
+  int bn = 256, group = 2;
   {
-    auto cost = [&](int w) {
+    auto rounds = [&](int rows, int w, int slots) {
       long t = 0;
-      for (int j = 0; j < n_mats; ++j) t += (long)a.m_tiles * ((a.d_out[j] + w - 1) / w);
-      const long pairs = std::max(1, p->sm_count / 2);
-      return (t + pairs - 1) / pairs * (w == 256 ? 100 : 82);
+      for (int j = 0; j < n_mats; ++j) t += (long)((n_tokens + rows - 1) / rows) * ((a.d_out[j] + w - 1) / w);
+      return (t + slots - 1) / slots;
     };
-    if (cost(128) < cost(256)) bn = 128;
+    const int pairs = std::max(1, p->sm_count / 2);
+    const long wide = rounds(2 * BM, 256, pairs) * 100, narrow = rounds(2 * BM, 128, pairs) * 82, single = rounds(BM, 256, p->sm_count) * 150;
+    if (narrow < wide) bn = 128;
+    if (single < std::min(wide, narrow)) { bn = 256; group = 1; }
   }
+  a.m_tiles = (n_tokens + group * BM - 1) / (group * BM);
   for (int j = 0; j < n_mats; ++j) a.wide[j] = (reinterpret_cast<uintptr_t>(a.y[j]) & 31) == 0 && a.d_out[j] % 16 == 0;
   a.tile_base[0] = 0;
   for (int j = 0; j < n_mats; ++j) {
@@ -802,7 +818,7 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
       // y = x W from the GEMM alone, then the segmented projection adds the LoRA term to it
       a.ksplit = 1;
       a.rmax = info.rmax;
-      rc = launch_width(p, a, maps, st, bn, info.rmax);
+      rc = launch_width(p, a, maps, st, bn, group, info.rmax);
       if (rc != FL_OK) break;
       if (kv && n_mats == 3 && kv->k_slot == 1 && kv->v_slot == 2)
         rc = fl_lora_sgmv_qkv_append(p, ys[0], ys[1], ys[2], x, mat_indices[0], mat_indices[1], mat_indices[2], seg_indptr,
@@ -836,7 +852,7 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
     }
     a.ksplit = info.ksplit;
     a.rmax = info.rmax;
-    rc = launch_width(p, a, maps, st, bn, info.rmax);
+    rc = launch_width(p, a, maps, st, bn, group, info.rmax);
   } while (0);
   if (prev != p->device && prev >= 0) cudaSetDevice(prev);
   return rc;

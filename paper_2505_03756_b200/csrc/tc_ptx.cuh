@@ -284,6 +284,23 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
   *abort_flag = 1;
   return false;
 }
+// One CTA, or a pair of them.
+template <int G>
+__device__ __forceinline__ void umma_ss_group_elect(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi, uint32_t idesc,
+                                                    uint32_t accumulate) {
+  if constexpr (G == 2) umma_ss_pair_elect(d_tmem, a_lo, a_hi, b_lo, b_hi, idesc, accumulate);
+  else umma_ss_elect(d_tmem, a_lo, a_hi, b_lo, b_hi, idesc, accumulate);
+}
+template <int G>
+__device__ __forceinline__ void umma_commit_group_elect(uint32_t bar) {
+  if constexpr (G == 2) umma_commit_pair_elect(bar);
+  else umma_commit_elect(bar);
+}
+template <int G>
+__device__ __forceinline__ void tma_load_2d_group(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1) {
+  if constexpr (G == 2) tma_load_2d_pair(dst, map, bar, c0, c1);
+  else tma_load_2d(dst, map, bar, c0, c1);
+}
 // 32 bytes to a 32-byte aligned global address in one instruction.
 __device__ __forceinline__ void st_global_v8(void* dst, const uint32_t* r) {
   asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]),

@@ -33,7 +33,7 @@ def _workload(T, shape, per_req, n_adapters):
     (1, 1, 1024, (8, 8)), (2, 1, 4096, (32, 32)), (15, 1, 328, (3, 1)), (16, 16, 328, (3, 1)), (17, 1, 1024, (8, 8)),
     (33, 11, 200, (2, 1)), (127, 1, 1024, (8, 8)), (129, 43, 328, (3, 1)), (200, 100, 1024, (8, 2)), (255, 1, 328, (3, 1)),
     (256, 256, 1024, (8, 8)), (256, 1, 2048, (4, 1)), (257, 1, 328, (3, 1)),
-    (176, 44, 4096, (8, 8)), (177, 1, 4096, (64, 8)), (209, 9, 1024, (8, 8))])
+    (176, 44, 4096, (8, 8)), (177, 1, 4096, (64, 8)), (209, 9, 1024, (8, 8)), (300, 100, 328, (64, 8)), (384, 128, 328, (64, 8))])
 def test_linear_of_few_tokens(T, per_req, hidden, heads):
     from paper_2505_03756_b200 import binding as fl, harness as H
     wl = _workload(T, synth.LayerShape(hidden, *heads), per_req, 12)
@@ -79,7 +79,7 @@ def test_linear_of_few_tokens(T, per_req, hidden, heads):
 
 
 @pytest.mark.parametrize("long_tokens,n_one,hidden,heads,n_adapters", [
-    (258, 0, 328, (3, 1), 3), (382, 1, 1024, (8, 8), 3), (500, 12, 328, (3, 1), 20), (513, 0, 4096, (3, 1), 2),
+    (258, 0, 328, (3, 1), 3), (382, 1, 1024, (8, 8), 3), (258, 2, 328, (64, 8), 4), (370, 14, 200, (64, 8), 16), (500, 12, 328, (3, 1), 20), (513, 0, 4096, (3, 1), 2),
     (1024, 40, 200, (2, 1), 60), (2300, 17, 1024, (8, 2), 24)])
 def test_linear_of_long_segments_next_to_one_token_segments(long_tokens, n_one, hidden, heads, n_adapters):
     """The GEMM for longer batches: tiles of 256 tokens that end in the middle of a segment, tiles with more LoRA stages than

@@ -70,6 +70,7 @@ def test_few_tokens_of_many_adapters(T, hidden, heads):
     ([90, 1, 1, 60, 1, 1, 1, 120], [-1, 0, 1, 2, 2, 3, 4, 5], 1024, (8, 8)),      # the adapter's tokens in the middle of a tile of 256
     ([1, 200, 180, 1, 140], [1, 1, 2, 2, 3], 4096, (3, 1)),                       # in both halves of one and the start of the next
     ([300, 5, 420], [0, 2, 4], 328, (3, 1)),
-    ([700, 33, 900], [-1, 2, 3], 1024, (8, 2))])
+    ([700, 33, 900], [-1, 2, 3], 1024, (8, 2)),
+    ([120, 1, 90, 1, 101], [-1, 1, 2, 3, 4], 328, (64, 8))])                      # tiles of 128 tokens
 def test_long_batches(new_lens, lora, hidden, heads):
     check(new_lens, lora, hidden, heads, [16, 64, 33, 8, 24, 64])
