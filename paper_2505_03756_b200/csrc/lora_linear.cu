@@ -117,44 +117,51 @@ __device__ __forceinline__ unsigned long long pack_unit(int lid, int q, int nr, 
 static_assert(FL_MAX_LORA_ID <= 1 << 20 && FL_MAX_RANK / UNIT <= 4 && 2 * BM < 512, "fields of a LoRA unit");
 
 // Infinities and NaNs in an adapter's B rows stay out of a LoRA stage: times the zeros of the tile's other tokens they would make
-// NaNs of these tokens' rows.  What they give their own token's 32 columns from col on is added here, to the values of its row.
-template <int RMAX>
-__device__ __noinline__ void add_nonfinite_terms(const LinArgs& a, int j, int tok, int col, uint32_t (&o)[32]) {
+// NaNs of these tokens' rows.  What they give their own token is added here to its row of the accumulator (columns from n0 on).
+template <int BN, int RMAX>
+__device__ __noinline__ void add_nonfinite_terms(const LinArgs& a, int j, int tok, int n0, uint32_t acc) {
   int lo = 0, hi = a.n_seg;                // first segment that ends behind tok
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
     if (a.seg_indptr[mid + 1] > tok) hi = mid; else lo = mid + 1;
   }
-  if (lo >= a.n_seg || a.seg_indptr[lo] > tok) return;
-  const int lid = a.lora_ids[lo], mat = a.mat_index[j];
-  if (lid < 0 || (uint32_t)lid >= a.pv.dir_cap || a.pv.dir[lid].rank <= 0 || mat >= a.pv.dir[lid].n_mats) return;
-  const LoraEntry* en = a.pv.dir + lid;
-  const LoraMat lm = en->mats[mat];
-  const int rank = min(en->rank, RMAX);
-  for (int r = 0; r < rank; ++r) {
-    const uint32_t gr = lm.b_row0 + r, blk = a.pv.tables[en->table_off + lm.b_tab + gr / lm.b_rpb];
-    if (blk >= a.pv.n_blocks) continue;
-    const uint4* b = reinterpret_cast<const uint4*>(a.pv.slab + (size_t)blk * a.pv.block_bytes + ((size_t)(gr % lm.b_rpb) * a.d_out[j] + col) * 2);
+  const int lid = lo < a.n_seg && a.seg_indptr[lo] <= tok && tok < a.n_tokens ? a.lora_ids[lo] : -1, mat = a.mat_index[j], d_out = a.d_out[j];
+  const LoraEntry* en = lid < 0 || (uint32_t)lid >= a.pv.dir_cap || mat >= a.pv.dir[lid].n_mats ? nullptr : a.pv.dir + lid;
+  const int rank = en ? min(en->rank, RMAX) : 0;
+  const LoraMat lm = rank > 0 ? en->mats[mat] : LoraMat{};
+  for (int cb = 0; cb < BN; cb += 32) {
+    uint32_t o[32];
+    __syncwarp();
+    tmem_ld32(acc + cb, o);
+    tmem_wait_ld();
+    for (int r = 0; r < rank; ++r) {
+      const uint32_t gr = lm.b_row0 + r, blk = a.pv.tables[en->table_off + lm.b_tab + gr / lm.b_rpb];
+      if (blk >= a.pv.n_blocks) continue;
+      const uint4* b = reinterpret_cast<const uint4*>(a.pv.slab + (size_t)blk * a.pv.block_bytes + ((size_t)(gr % lm.b_rpb) * d_out + n0 + cb) * 2);
 #pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      if (col + 8 * h >= a.d_out[j]) break;
-      const uint4 q = b[h];
-      if (nonfinite_chunk(q) == 0u) continue;
-      float v = 0.f;
-      if (a.v16) {
-        v = __bfloat162float(a.v16[((size_t)j * a.n_tokens + tok) * RMAX + r]);
-      } else {
-        for (int sp = 0; sp < a.ksplit; ++sp) v += a.v[((size_t)(j * a.ksplit + sp) * a.n_tokens + tok) * RMAX + r];
-        v = __bfloat162float(__float2bfloat16_rn(v * a.scale));
-      }
-      const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+      for (int h = 0; h < 4; ++h) {
+        if (n0 + cb + 8 * h >= d_out) break;
+        const uint4 q = b[h];
+        if (nonfinite_chunk(q) == 0u) continue;
+        float v = 0.f;
+        if (a.v16) {
+          v = __bfloat162float(a.v16[((size_t)j * a.n_tokens + tok) * RMAX + r]);
+        } else {
+          for (int sp = 0; sp < a.ksplit; ++sp) v += a.v[((size_t)(j * a.ksplit + sp) * a.n_tokens + tok) * RMAX + r];
+          v = __bfloat162float(__float2bfloat16_rn(v * a.scale));
+        }
+        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        const float bv = __uint_as_float(c & 1 ? w[c >> 1] & 0xffff0000u : w[c >> 1] << 16);
-        if ((__float_as_uint(bv) & 0x7f800000u) == 0x7f800000u) o[8 * h + c] = __float_as_uint(fmaf(v, bv, __uint_as_float(o[8 * h + c])));
+        for (int c = 0; c < 8; ++c) {
+          const float bv = __uint_as_float(c & 1 ? w[c >> 1] & 0xffff0000u : w[c >> 1] << 16);
+          if ((__float_as_uint(bv) & 0x7f800000u) == 0x7f800000u) o[8 * h + c] = __float_as_uint(fmaf(v, bv, __uint_as_float(o[8 * h + c])));
+        }
       }
     }
+    __syncwarp();
+    tmem_st32(acc + cb, o);
   }
+  tmem_wait_st();
 }
 
 template <int BN, int RMAX, int G>
@@ -352,7 +359,8 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
       tc_fence_after();
       __nv_bfloat16* yrow = side < 0 ? a.y[t.j] + (size_t)tok * d_out + n0 : nullptr;
       const bool wide = side < 0 && a.wide[t.j];
-      const bool nonfinite = *nonfinite_slot != 0;       // (of this tile or one before or behind it: then a look at the token's own rows)
+      // (a value of this tile's stages or of those of a tile before or behind it)
+      if (__any_sync(0xffffffffu, *nonfinite_slot != 0)) add_nonfinite_terms<BN, RMAX>(a, t.j, tok, n0, lane_addr + buf * BN);
 #pragma unroll 2
       for (int cb = 0; cb < BN; cb += 32) {
         uint32_t o[32];
@@ -360,14 +368,6 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
         tmem_ld32(lane_addr + buf * BN + cb, o);
         tmem_wait_ld();
         if (tok < a.n_tokens) {
-          if (nonfinite) {
-            uint32_t f[32];
-#pragma unroll
-            for (int c = 0; c < 32; ++c) f[c] = o[c];
-            add_nonfinite_terms<RMAX>(a, t.j, tok, n0 + cb, f);
-#pragma unroll
-            for (int c = 0; c < 32; ++c) o[c] = f[c];
-          }
           uint32_t pk[16];
 #pragma unroll
           for (int c = 0; c < 16; ++c) pk[c] = pack_bf16(__uint_as_float(o[2 * c]), __uint_as_float(o[2 * c + 1]));
@@ -519,6 +519,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
           cp_async16(bs + (ch >> 3) * B_GROUP + (ER * slot + r) * 128 + (((ch & 7) ^ (r & 7)) << 4),
                      have ? reinterpret_cast<const unsigned char*>(at) + ch * 16 : a.pv.slab, have);
         }
+        cp_async_commit();
         // shrink results of this CTA's 128 rows at the stage's ranks
         const int u = 2 * e + (vch >> 1);
         const unsigned long long x = u < n_units ? list[u] : 0ull;
@@ -561,8 +562,8 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
           }
         }
         cp_async_commit();
-        cp_async_wait<0>();
-        // infinities and NaNs out of the B rows (this thread's own pieces; add_nonfinite_terms has the reason)
+        cp_async_wait<1>();                              // the B rows; v16 may still be on its way
+        // infinities and NaNs out of them (this thread's own pieces; add_nonfinite_terms has the reason)
         uint32_t found = 0;
 #pragma unroll
         for (int i = 0; i < ER * CPR / 128; ++i) {
@@ -580,6 +581,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
           *nonfinite_slot = 1;
           if (G == 2) st_cluster_u32(map_cluster_rank(smem_u32(const_cast<int*>(nonfinite_slot)), (uint32_t)(crank ^ 1)), 1u);
         }
+        cp_async_wait<0>();
         fence_async_smem();                              // the tensor core reads shared memory through the async proxy
         asm volatile("bar.sync %0, 128;" ::"r"(3 + slot) : "memory");
         if (et == 0 && ok) mbar_arrive_cluster(efull0 + 8u * slot);
