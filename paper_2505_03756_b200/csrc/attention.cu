@@ -729,7 +729,7 @@ Packed packed_slots(int n_req, int n_tbl, int n_kv, int csize, int sms) {
   const int longest = n_tbl - n_req + 1;
   if (n_req < 2 || csize >= PACK || longest <= (csize == 1 ? 100 : 150) + n_req * csize) return {0, 0};
   Packed p = {0, 0};
-  for (int pages : {16, 24, 32, 48}) {
+  for (int pages : {8, 12, 16, 24, 32, 48}) {
     p.part_pages = pages;
     p.slots = (std::min(n_req + n_tbl * 3 / (2 * pages), PACK * n_req) + PACK - 1) / PACK * PACK;
     if (p.slots * n_kv <= 4 * sms) return p;
