@@ -29,6 +29,7 @@
 #include <string.h>
 #include <algorithm>
 #include "giveup.cuh"
+#include "kv_tail.cuh"
 #include "lora_skinny.cuh"
 #include "mma_utils.cuh"
 #include "tc_ptx.cuh"
@@ -448,8 +449,8 @@ __global__ void __launch_bounds__(MAX_THREADS, 1) lora_skinny_kernel(const __gri
   const int side = a.kv_side[j];
   uint32_t kv_blk[2] = {0, 0};
   int kv_slot[2] = {-1, -1};
-  bool kv_last[2] = {false, false};
   if (epi) {
+    if (a.n_req > 0) clear_v_tails(a, (int)blockIdx.x, (int)gridDim.x, warp - 2, 4);
     if (side >= 0) {                                          // where K / V rows go
       for (int m = 0; m < mt; ++m) {
         const int t = m * 128 + lrow;
@@ -472,7 +473,6 @@ __global__ void __launch_bounds__(MAX_THREADS, 1) lora_skinny_kernel(const __gri
         }
         kv_blk[m] = b;
         kv_slot[m] = slot;
-        kv_last[m] = t == a.req_indptr[lo + 1] - 1;
       }
     }
     if (ok) ok = mbar_wait(bar(B_ACC), 0, abort_flag);
@@ -527,7 +527,7 @@ __global__ void __launch_bounds__(MAX_THREADS, 1) lora_skinny_kernel(const __gri
   if (epi && ok) {
     // The finished rows as bf16 through shared memory (behind the partial sums; pitch an odd number of 16-byte chunks), so that
     // they go out a whole row piece at a time: stored by the thread that owns the row, 16 bytes of 32 rows per instruction,
-    // the rows and the cleared V slots of a decode batch of 128 took up to 18 us.
+    // the rows of a decode batch of 128 took up to 18 us.
     const int nch = (c1 - c0) / 8, row_bytes = share * 2 + 16;
     unsigned char* out = smem + (size_t)(split - 1) * npad * pitch * 4;
     for (int m = 0; m < mt; ++m) {
@@ -557,12 +557,11 @@ __global__ void __launch_bounds__(MAX_THREADS, 1) lora_skinny_kernel(const __gri
                               pack_bf16(f[8 * h + 4], f[8 * h + 5]), pack_bf16(f[8 * h + 6], f[8 * h + 7]));
       }
       if (side >= 0 && t < a.n_tokens) {
-        // a column tile is one KV head: [K|V][kv head][slot][128] inside the block; in the top bits the V slots to clear
+        // a column tile is one KV head: [K|V][kv head][slot][128] inside the block
         unsigned long long at = 0;
         if (kv_slot[m] >= 0)
           at = reinterpret_cast<unsigned long long>(a.pv.slab + (size_t)kv_blk[m] * a.pv.block_bytes +
-                                                    ((size_t)(side * a.n_kv + n0 / FL_HEAD_DIM) * a.bt + kv_slot[m]) * (FL_HEAD_DIM * 2)) |
-               (unsigned long long)(side == 1 && kv_last[m] ? a.bt - 1 - kv_slot[m] : 0) << 48;
+                                                    ((size_t)(side * a.n_kv + n0 / FL_HEAD_DIM) * a.bt + kv_slot[m]) * (FL_HEAD_DIM * 2));
         row_ptr[t] = at;
       }
     }
@@ -574,19 +573,8 @@ __global__ void __launch_bounds__(MAX_THREADS, 1) lora_skinny_kernel(const __gri
       const int col = n0 + c0 + 8 * ch;
       if (side < 0) {
         if (col < d_out) *reinterpret_cast<uint4*>(a.y[j] + (size_t)t * d_out + col) = q;
-      } else if (const unsigned long long at = row_ptr[t] << 16 >> 16) {
+      } else if (const unsigned long long at = row_ptr[t]) {
         *reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(at) + (c0 + 8 * ch) * 2) = q;
-      }
-    }
-    if (side == 1) {             // V behind a request's last token
-      for (int t = warp - 2; t < a.n_tokens; t += 4) {
-        const unsigned long long w = row_ptr[t];
-        unsigned char* at = reinterpret_cast<unsigned char*>(w << 16 >> 16) + c0 * 2;
-        const int n = (int)(w >> 48) * nch;
-        for (int i = lane; i < n; i += 32) {
-          const int z = i / nch;
-          *reinterpret_cast<uint4*>(at + (size_t)(z + 1) * (FL_HEAD_DIM * 2) + (i - z * nch) * 16) = make_uint4(0u, 0u, 0u, 0u);
-        }
       }
     }
     tc_fence_before();
