@@ -24,6 +24,7 @@
 #include <string.h>
 #include <algorithm>
 #include "giveup.cuh"
+#include "kv_tail.cuh"
 #include "lora_skinny.cuh"
 #include "mma_utils.cuh"
 #include "pool.cuh"
@@ -332,7 +333,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
       // a K / V row belongs in its token's pool block: block and slot of the token's position, found while the
       // tile's MMAs are still running
       uint32_t kv_blk = 0;
-      int kv_slot = -1, kv_last = 0;
+      int kv_slot = -1;
       if (side >= 0 && tok < a.n_tokens) {
         int lo = 0, hi = a.n_req;
         while (hi - lo > 1) {
@@ -350,7 +351,6 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
           } else {
             kv_blk = blk;
             kv_slot = slot;
-            kv_last = tok == a.req_indptr[lo + 1] - 1;
           }
         }
       }
@@ -386,9 +386,6 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
                                      ((size_t)(side * a.n_kv + colg / FL_HEAD_DIM) * a.bt + kv_slot) * (FL_HEAD_DIM * 2) +
                                      (colg % FL_HEAD_DIM) * 2;
                 *reinterpret_cast<uint4*>(dst) = q;
-                if (side == 1 && kv_last)       // V of a request's last token: clear the slots behind it
-                  for (int z = kv_slot + 1; z < a.bt; ++z)
-                    *reinterpret_cast<uint4*>(dst + (z - kv_slot) * (FL_HEAD_DIM * 2)) = make_uint4(0u, 0u, 0u, 0u);
               }
             }
           }
@@ -411,6 +408,7 @@ __global__ void __launch_bounds__(LT_THREADS, 1) lora_linear_kernel(const __grid
     bool used = false, ok = true;
     int count = 0;                           // LoRA stages of all tiles so far
     int k = 0;
+    if (a.n_req > 0) clear_v_tails(a, (int)blockIdx.x, (int)gridDim.x, warp - 6, 8);       // while the shrink is still at work
     if (a.n_seg > 0) pdl_wait();             // v is the shrink's output
     for (int idx = first; a.n_seg > 0 && ok && idx < total; idx += step, ++k) {
       const Tile t = decode_tile(a, idx);
@@ -732,7 +730,7 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
     a.tbl_indptr = kv->tbl_indptr;
     a.tbl = kv->tbl;
     a.prefix_lens = kv->prefix_lens;
-    a.n_req = kv->n_req;
+    a.n_req = hybrid ? 0 : kv->n_req;       // (0: no row of this kernel goes into a block)
     a.n_kv = kv->n_kv;
     a.bt = (int)(p->block_bytes / per_tok);
   }
