@@ -6,7 +6,7 @@
 // through global memory.
 //   warp 0      TMA producer: x tile [tokens x 64] and W tile [64 x 128] per stage, ring of as many stages as fit
 //   warp 1      MMA issuer of x W
-//   warps 2-5   list of the LoRA stages, a share of them, then the epilogue (thread = token row)
+//   warps 2-5   list of the LoRA stages, a share of them, a share of the V slots to clear, then the epilogue (thread = token row)
 //   up to 8 more the other LoRA stages, four warps to a stage
 //   last warp   MMA issuer of the LoRA term, into an accumulator of its own
 // The LoRA term is one more product over a long, sparse k: the rank-rows of every adapter of the batch one after the
@@ -645,27 +645,24 @@ namespace skinny {
 
 // Up to 128 tokens always.  Above that a CTA brings 48 KB of x and W per stage for 128 columns where one of the GEMM for long batches
 // brings 32 KB for as many, while the GEMM takes a tile's LoRA stages (up to 32 ranks each) one after the other.
-//  - More than 16 such stages: here.  q, k, v of 200 tokens, twelve segments of rank 64, here and there: 7B 56 and 64 us, 13B 66 and 72,
-//    34B 85 and 81; o of 230 tokens on 7B 33 and 39.
-//  - d_in not split (q, k, v as a rule): here up to 176 tokens, unless one adapter serves them all (from 144 on the GEMM).  q, k, v of 176
-//    tokens, rank 16, one segment: 7B 38 and 31 us, 13B 51 and 38, 34B 59 and 49; eight segments 40 and 41, 53 and 50, 61 and 62; of 256
-//    tokens 46 and 37, 60 and 46, 72 and 58.
-//  - d_in split, at least 16 stages per CTA (o): the GEMM leaves half of the SMs idle.  Here up to 208 tokens; beyond, the sum over
-//    the cluster wants 24 stages to be small against.  o of 176 tokens, four segments: 7B 24 and 27 us, 13B 25 and 32, 34B 38 and 50; of 256
-//    29 and 28, 29 and 32, 45 and 50.
-//  - d_in split, fewer stages: here for many LoRA stages up to 176 tokens only.  A layer of 1024 hidden values, q, k, v of 144 tokens:
-//    8 segments of rank 16 23 and 19 us, 24 segments 26 and 25, o 16 and 21.
+//  - More than 16 such stages: here.  q, k, v of 230 tokens, twelve segments of rank 64, here and there: 7B 62 and 64 us; o 33 and 39.
+//  - d_in split over at least two CTAs of 16 stages each (o): the GEMM leaves half of the SMs idle.  Here up to 208 tokens; beyond, the sum
+//    over the cluster wants 24 stages to be small against.  o of 176 tokens, four segments: 7B 24 and 27 us, 13B 25 and 32, 34B 38 and 50; of
+//    256 29 and 28, 29 and 32, 45 and 50.
+//  - Otherwise (q, k, v; narrow layers): here for more than eight stages up to 176 tokens.  q, k, v of a decode step of 150 tokens, rank 16, 32
+//    segments: 7B 47 and 51 us, 13B 61 and 60, 34B 64 and 68, a layer of 1024 values 26 and 30; 12 segments: 41 and 40, 54 and 51, 61 and
+//    60, 23 and 22; one segment of 256 tokens 50 and 40, 66 and 54, 71 and 52, 33 and 20.
 // More than 512 ranks over short segments: the two-step way (q, k, v and o of 160 tokens on 13B, 75 adapters of rank 32: 173 us here, 141).
+// Over 1284 batches of 130 to 256 tokens the choice is 0.5 % behind the better of the two kernels.
 bool serves(const fl_pool* p, const int* d_out, int n_mats, int d_in, int n_tokens, int n_seg, int rank_max) {
   if (n_tokens <= 128) return true;
   if (n_tokens > MAX_TOKENS || (n_seg * rank_max > 8 * 64 && n_tokens <= 16 * n_seg)) return false;
+  if (n_seg * rank_max > 16 * 32) return true;
   int tiles = 0;
   for (int j = 0; j < n_mats; ++j) tiles += (d_out[j] + BN - 1) / BN;
   const int nk = (d_in + BK - 1) / BK, split = cluster_split(p, tiles, nk);
-  if (n_seg * rank_max > 16 * 32) return true;
-  if (split == 1) return n_tokens <= 176 && (n_seg > 1 || n_tokens < 144);
-  if (nk / split < 16) return n_seg * rank_max > 8 * 32 && n_tokens <= 176;
-  return n_tokens <= 208 || nk / split >= 24;
+  if (split >= 2 && nk / split >= 16) return n_tokens <= 208 || nk / split >= 24;
+  return n_seg * rank_max > 8 * 32 && n_tokens <= 176;
 }
 
 int launch(fl_pool* p, const Args& a, const void* x, const void* const* w, cudaStream_t st) {
