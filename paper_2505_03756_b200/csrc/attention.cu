@@ -44,7 +44,9 @@ __device__ __forceinline__ int block_excl_scan(int val, int* sh, int& total) {
 // the others, and all of them behind the prefill kernel's end.  The decode kernel is bound by the copy rate from DECODE_SMS SMs
 // on; a prefill unit's step takes STEP_US, one fifth longer beside it.  (7B, 16 x 512 new tokens behind 512 and 48 decode requests
 // of about 1400 keys: 299 us one after the other, 279, 270, 264 and 351 us with 100, 82, 70 and 50 SMs for the prefill kernel;
-// 1000 prefill tokens beside 1.2 GB of decode pages: 198 us, 194, 191 and 228 us with 90, 50 and 8.)
+// 1000 prefill tokens beside 1.2 GB of decode pages: 198 us, 194, 191 and 228 us with 90, 50 and 8.  Grouped heads, one after the other
+// and with the share chosen here, 34B: 16 decode requests of 2700 keys beside 1000 new tokens 144 and 97 us, beside 16 x 500 279 and 253,
+// 64 of 3600 keys beside 16 x 500 393 and 383; of 75 batches on 7B, 13B and 34B one is slower, by 1 %.)
 constexpr float STEP_US = 1.7f, KEY_US = 8e-5f, DECODE_SMS = 112.f;
 __device__ __forceinline__ float shared_time(int p, int sms, float unit_us, int n_units, float decode_us) {
   const float pre = unit_us * (p < sms ? 1.2f : 1.f) * ((n_units + p - 1) / p);
@@ -716,8 +718,9 @@ int cluster_size(int n_req, int n_tbl, int n_kv, int sms) {
 // A batch whose n_tbl entries may be one request's nearly all: with the same number of CTAs for every request that one would keep a warp
 // busy with more than 25 to 37 pages and some more for every other request (the plan's time grows with them too).  Then a request gets
 // CTAs as it has pages: `slots` of them per KV head (a request of p pages takes at most 1 + 1.5 p / part_pages), 0 = the same number for
-// each, -1 = a plan.  Small parts as long as all CTAs run at once or nearly so; where even the large ones take twice that, the many short
-// requests are better off with a CTA each, and from 200 pages on with a plan.
+// each, -1 = a plan.  Small parts as long as the CTAs with work run at once (three fit on an SM) and those without are not many more; where
+// even large parts take twice that, the many short requests are better off with a CTA each, and from 200 pages on with a plan.  (4 requests
+// of 1300 keys on 7B, a layer step of 41 us: in parts of eight pages 16 CTAs per head, 512 in all, it took 48.)
 // Attention with the same number of CTAs, as here, and with the plan (of the tree that had nothing else).  One request has nearly all: 7B, 5 requests,
 // 2560 keys 37, 14 and 24 us; 8, 3200 keys 30, 15, 29; 12, 2560 keys 41, 16, 26; 13B, 8, 2560 keys 42, 17, 27.  One has four times as many as the
 // others: 13B, 4 requests of 600 keys 29, 15, 23; 7B, 6 22, 15, 23.  Lengths from one to eight times the shortest: 7B, 5 of 350 keys
@@ -732,7 +735,8 @@ Packed packed_slots(int n_req, int n_tbl, int n_kv, int csize, int sms) {
   for (int pages : {8, 12, 16, 24, 32, 48}) {
     p.part_pages = pages;
     p.slots = (std::min(n_req + n_tbl * 3 / (2 * pages), PACK * n_req) + PACK - 1) / PACK * PACK;
-    if (p.slots * n_kv <= 4 * sms) return p;
+    const int alike = n_tbl <= pages * n_req ? 1 : n_tbl <= 2 * pages * n_req ? 2 : PACK;       // CTAs of a request if all are alike
+    if (p.slots * n_kv <= 4 * sms && n_req * alike * n_kv <= 3 * sms) return p;
   }
   if (p.slots * n_kv > 6 * sms) p.slots = longest > 200 ? -1 : 0;
   return p;
