@@ -233,6 +233,7 @@ int fl_lora_sgmv_static(fl_pool* pool, fl_bf16* y, const fl_bf16* x, int mat_ind
  * adapters: at least one adapter must be registered, FL_EBADID otherwise); x, seg_indptr, lora_ids as in
  * fl_lora_sgmv; y: device [n_tokens, d_out] bf16, overwritten.  fp32 accumulation over d_in and the rank, the
  * shrink result x A_i is rounded to bf16 before it meets B_i, one bf16 rounding of the result.
+ * An infinity or NaN in an adapter reaches the rows of its own tokens only.
  * n_seg = 0 is allowed (plain y = x W).  The _multi form runs up to 3 projections that share x (q, k, v) as one
  * launch: ys, ws and mat_indices are HOST arrays.  workspace: device scratch of at least
  * fl_lora_linear_workspace(n_tokens, n_mats) bytes, same sharing rule as fl_lora_sgmv.  After one ordinary call
@@ -251,8 +252,9 @@ int fl_lora_linear_multi(fl_pool* pool, fl_bf16* const* ys, const fl_bf16* x, co
  * pool blocks, at the positions and in the layout of fl_kv_append (cleared V slots behind a request's last token
  * included).  Bit for bit what fl_lora_linear_multi followed by fl_kv_append stores.  mat_k and mat_v must have
  * d_out = n_kv_heads * 128.  scratch_k, scratch_v: device [n_tokens, n_kv_heads * 128] bf16 each, needed only by
- * batches of short segments (n_tokens <= 16 * n_seg, e.g. a decode step), where x W is formed first and the segmented
- * projection then stores base + LoRA term; may be NULL otherwise (FL_EINVAL if such a batch comes without them).
+ * batches of short segments (n_tokens <= 16 * n_seg, e.g. a decode step): some of them (above 256 tokens, or above 128 with
+ * many adapters) form x W first, and the segmented projection then stores base + LoRA term; may be NULL otherwise (FL_EINVAL
+ * if such a batch comes without them).
  * workspace as fl_lora_linear_workspace(n_tokens, 3). */
 int fl_lora_linear_qkv_append(fl_pool* pool, fl_bf16* y_q, const fl_bf16* x, const fl_bf16* w_q, const fl_bf16* w_k,
                               const fl_bf16* w_v, int mat_q, int mat_k, int mat_v, const int32_t* seg_indptr,

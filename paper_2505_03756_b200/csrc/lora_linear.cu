@@ -10,10 +10,13 @@
 // summed, scaled, rounded to bf16) at the ranks of its own adapter and zeros elsewhere.  A tile thus needs no alignment with
 // the segments.  The stages are spread over the second half of the tile's main stages: their place in the order of the
 // sums is fixed, and a tile of many one-token segments fills its stages while the tensor cores work on.
+// The kernel is also built for tiles of 128 tokens x 256 columns with a CTA each (G = 1), for batches whose second tile of 256 tokens
+// would be mostly empty and cost the pairs a round.
 //   warp 0       TMA producer: x tile [128 x 64] (K-major) and W tile [64 x BN/2] (N contiguous, as stored) per stage
 //   warp 1       MMA issuer (of the pair's first CTA, for both)
 //   warps 2-5    epilogue: TMEM -> bf16 -> y, or K and V rows straight into each token's pool block
-//   warps 6-13   LoRA stages, warps 6-9 the even ones, 10-13 the odd ones
+//   warps 6-13   the V slots behind each request's last token (a share per CTA), then the LoRA stages, warps 6-9 the even ones,
+//                10-13 the odd ones
 // What bounds it: the tensor cores, and above them the power limit.  A layer step of 16 prompts (4907 tokens, 7B) went 737
 // -> 665 us, of 4 prompts of 1024 new tokens (34B, rank 64) 1727 -> 1507 us against the tiles of 128 tokens per CTA before;
 // with 28 one-token segments next to 4 prompts (7B, ranks 8 to 64) 734 -> 453 us, because a stage now takes the rank-rows of

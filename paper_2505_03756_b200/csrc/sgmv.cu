@@ -38,7 +38,7 @@ struct SgmvArgs {
   int n_seg, n_tokens;
   float scale;
   float* v;        // [n_mats][ksplit][n_tokens][RMAX]
-  __nv_bfloat16* v16;   // where the scaled bf16 sum goes instead, [n_mats][n_tokens][RMAX] (tiles of 16 tokens only), or null
+  __nv_bfloat16* v16;   // the scaled sum in bf16, [n_mats][n_tokens][RMAX], instead of v: tiles of 16 tokens, or the tcgen05 shrink with one slice; or null
   int ksplit;
   int tc_ksplit;     // slices of d_in for the tcgen05 shrink of long segments (0 = not applicable)
   int expand_cols;   // y columns one expand CTA covers

@@ -16,7 +16,8 @@ int shrink(fl_pool* p, const fl_bf16* x, const int* mat_indices, int n_mats, con
            const int32_t* lora_ids, int n_seg, int n_tokens, void* workspace, size_t workspace_bytes, fl_stream stream,
            ShrinkInfo* info);
 // The same in its final form: slices added, scaled, rounded to bf16 as the expand product takes them, [projection][token][rmax].
-// Tiles of 16 tokens whatever the segments' lengths: meant for batches of a few hundred tokens.
+// Tiles of 16 tokens whatever the segments' lengths, each of which reads its adapter's rows again: for batches of up to a few hundred
+// tokens, and beyond for short segments.
 int shrink_scaled(fl_pool* p, const fl_bf16* x, const int* mat_indices, int n_mats, const int32_t* seg_indptr,
                   const int32_t* lora_ids, int n_seg, int n_tokens, float scale, void* workspace, size_t workspace_bytes,
                   fl_stream stream, ShrinkInfo* info);
