@@ -113,3 +113,43 @@ def test_linear_of_long_segments_next_to_one_token_segments(long_tokens, n_one, 
         assert s.status()["device_flags"] == 0
     finally:
         s.close()
+
+
+@pytest.mark.parametrize("T,per_req,hidden,heads,n_adapters", [
+    (1, 1, 1024, (8, 8), 2), (40, 1, 1024, (8, 8), 12), (130, 1, 4096, (8, 8), 4), (200, 1, 1024, (8, 2), 3), (256, 1, 328, (64, 8), 4),
+    (300, 20, 328, (3, 1), 2), (330, 3, 328, (64, 8), 3)])
+def test_v_slots_behind_a_request_are_cleared(T, per_req, hidden, heads, n_adapters):
+    """K and V stored by the projection itself into blocks that hold old values behind the requests' last tokens: the same bytes as the
+    projection and the KV append, whichever kernel serves the batch and whichever CTA clears the slots."""
+    from paper_2505_03756_b200 import binding as fl, harness as H
+    wl = _workload(T, synth.LayerShape(hidden, *heads), per_req, n_adapters)
+    s = H.Session(wl)
+    try:
+        s.load_adapters()
+        s.build_batch()
+        s.fill_prefix_kv()
+        dims = dict((n, o) for n, _, o in wl.shape.mats)
+        tx = H.f32_to_dev(wl.x("q"), s.dev)
+        tw = [H.f32_to_dev(wl.weight(m), s.dev) for m in "qkv"]
+        ty = [torch.empty((T, dims[m]), dtype=torch.bfloat16, device=s.dev) for m in "qkv"]
+        s.lora_linear(ty, tx, tw, ["q", "k", "v"])
+        s.kv_append(ty[1], ty[2])
+        torch.cuda.synchronize()
+        blocks = sorted({int(b) for t in s.kv_tables for b in t})
+        stored = fl.device_block_bytes(s.pool, s.block_bytes, blocks)
+        kv, bt = wl.shape.n_kv_heads, wl.shape.block_tokens
+        for r in range(wl.n_req):
+            last = int(wl.prefix_lens[r] + wl.new_lens[r]) - 1
+            b = int(s.kv_tables[r][last // bt])
+            data = fl.fl_block_read(s.pool, b, s.block_bytes).reshape(2, kv, bt, 256).copy()
+            assert not data[1, :, last % bt + 1:].any()
+            data[1, :, last % bt:] = 0x55                       # the last token's own slot too: it is stored again
+            fl.fl_block_write(s.pool, b, data.reshape(-1))
+        y_q = torch.empty_like(ty[0])
+        s.lora_linear_qkv_append(y_q, tx, *tw)
+        torch.cuda.synchronize()
+        assert torch.equal(y_q, ty[0])
+        assert np.array_equal(fl.device_block_bytes(s.pool, s.block_bytes, blocks), stored)
+        assert s.status()["device_flags"] == 0
+    finally:
+        s.close()
