@@ -7,21 +7,22 @@
 // for 256 query rows.  CTAs take units from a counter in device memory until none is left; the loads of
 // the next unit start while the current one is still in its last tiles and its epilogue.
 //   warps 0-3   softmax of tile A (thread = query row = TMEM lane)      warp 8   TMA producer, unit fetch
-//   warps 4-7   softmax of tile B                                        warp 9   MMA issuer, TMEM owner
-//   (warps 10, 11 only complete the third warpgroup, whose registers go to the softmax warpgroups)
+//   warps 4-7   softmax of tile B                                        warp 9   MMA issuer of the scores, TMEM owner
+//                                                                        warps 10, 11   MMA issuers of P V, a tile each
 //   K_j / V_j (128 keys = 8 pool pages each, one 4 KiB TMA box per page) -> ring of 32 KiB slots, 128-byte swizzle;
 //   a page lands as [8-key group][64-value half][8 keys][64 values], so a tile's 8-key groups are 2 KiB apart
-//   S_X = Q_X K_j^T     tcgen05.mma 128x128x16 (x8) into TMEM columns of tile X
-//   P_X = exp2(S_X - m) -> bf16 pairs written back over the first half of S_X in TMEM
+//   S   = Q_X K_j^T     tcgen05.mma 128x128x16 (x8) into TMEM columns that both tiles use in turn
+//   P_X = exp2(S - m) -> bf16 pairs in TMEM columns of tile X's own
 //   O_X += P_X V_j      tcgen05.mma with the A operand read from TMEM, V MN-major as stored
+// A softmax warp takes its 128 scores into registers at once, so the next scores, the other tile's, go into the same columns while it
+// is at its exponentials: TMEM holds one S, two P and two O, and a tile's next scores are there when its softmax comes back for them.
+// Until then S_X(j+1) waited for PV_X(j), whose P lay in its columns, and one warp issued everything, which left the tensor pipe idle
+// during that warp's barrier tests (see the issuers).  A step of two tiles takes 3040 cycles, a unit's start and end included (34B,
+// 4 x 1024 new tokens behind 3072), of which the MMAs need 2048.  What bounds it is the power limit as much as the chain of hand-offs:
+// 16 x 1024 new tokens behind 3072, 34B, first launches on a cool chip 1500 -> 1450 us, run after run at 1000 W 1728 -> 1687 us (1540 MHz
+// now, 1580 before); 64 prompts of U{128..1024} tokens, half of them cached, 7B 317 -> 307 us.
 // P of a step comes in two halves of 64 keys, and PV of the first runs while the softmax is at the last quarter of its
-// exponentials: 256 cycles less of a chain of 3440 per step (34B, 16 x 1024 new tokens behind 3072: 1548 -> 1520 us).
-// (Scores in halves too, the next step's first 64 keys computed into TMEM columns that the softmax has read, take the
-// softmax off the chain altogether but cost 1840 us: an MMA of 64 columns takes as long as one of 128.)
-// The issuer alternates the tiles (PV_A, S_A, PV_B, S_B): while one tile's softmax runs, the tensor pipe
-// works for the other.  MMAs of one thread execute in issue order, so S_X(j+1) may overwrite P_X(j)
-// without a barrier, "S_X(j+1) complete" implies "PV_X(j) complete", and the first PV of a unit cannot
-// start before every softmax warp has finished the previous unit's epilogue (it waits for their P).
+// exponentials.
 // O is rescaled only when a row maximum grew by more than 2^8.  Every mbarrier wait is bounded; a wait
 // that gives up raises a sticky flag, the CTA drains its copies and frees its TMEM.
 #include <cuda.h>
@@ -39,7 +40,7 @@ namespace {
 
 using namespace tc;
 
-constexpr int T2_THREADS = 384;                        // three warpgroups: softmax A, softmax B, {TMA, MMA, 2 idle warps}
+constexpr int T2_THREADS = 384;                        // three warpgroups: softmax A, softmax B, {TMA, MMA x 3}
 constexpr int KT2 = 128;                               // keys per tile
 constexpr int NSLOT = 5;                               // ring slots; fills go K_0, V_0, K_1, V_1, ... across units
 constexpr uint32_t HALF_BYTES = 128 * 128;             // [128 rows][64 bf16], swizzled
@@ -50,12 +51,13 @@ constexpr uint32_t OFF_Q2 = 0;                         // Q_A, Q_B
 constexpr uint32_t OFF_RING = 2 * TILE_BYTES;
 constexpr uint32_t OFF_BAR2 = OFF_RING + NSLOT * TILE_BYTES;
 constexpr uint32_t T2_SMEM = OFF_BAR2 + 512;           // barriers, TMEM address, abort flag, two unit descriptors
-constexpr uint32_t T2_TMEM_COLS = 512;                 // S_A | S_B | O_A | O_B, 128 columns each
+constexpr uint32_t T2_TMEM_COLS = 512;                 // S (128 columns) | P_A | P_B (64 each) | O_A | O_B (128 each)
+constexpr uint32_t TM_P = 128, TM_O = 256;
 constexpr float RESCALE_LOG2 = 8.f;
 
-enum { C_QFULL = 0, C_QEMPTY = 1, C_FULL = 2, C_EMPTY = C_FULL + NSLOT, C_SFULL = C_EMPTY + NSLOT, C_PFULL = C_SFULL + 2,
-       C_PHALF = C_PFULL + 2, C_ODONE = C_PHALF + 2, C_UFULL = C_ODONE + 2, C_UEMPTY = C_UFULL + 2, C_IDLE = C_UEMPTY + 2, C_COUNT };
-constexpr int UNIT_READERS = 9;                        // MMA issuer + 8 softmax warps
+enum { C_QFULL = 0, C_QEMPTY = 1, C_FULL = 2, C_EMPTY = C_FULL + NSLOT, C_SFULL = C_EMPTY + NSLOT, C_SFREE = C_SFULL + 2,
+       C_PFULL = C_SFREE + 1, C_PHALF = C_PFULL + 2, C_PVDONE = C_PHALF + 2, C_UFULL = C_PVDONE + 2, C_UEMPTY = C_UFULL + 2, C_IDLE = C_UEMPTY + 2, C_COUNT };
+constexpr int UNIT_READERS = 11;                       // three MMA issuers + 8 softmax warps
 
 struct Unit {           // what a CTA works on at one time
   int tok0[2];          // first token row (in the packed q / out tensors) of each tile
@@ -125,17 +127,18 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
     mbar_init(bar(C_QEMPTY), 1);
     for (int s = 0; s < NSLOT; ++s) {
       mbar_init(bar(C_FULL + s), 1);
-      mbar_init(bar(C_EMPTY + s), 1);
+      mbar_init(bar(C_EMPTY + s), 2);      // one arrival per tile
     }
     for (int x = 0; x < 2; ++x) {
       mbar_init(bar(C_SFULL + x), 1);
       mbar_init(bar(C_PFULL + x), 4);
       mbar_init(bar(C_PHALF + x), 4);
-      mbar_init(bar(C_ODONE + x), 1);
+      mbar_init(bar(C_PVDONE + x), 1);
       mbar_init(bar(C_UFULL + x), 1);
       mbar_init(bar(C_UEMPTY + x), UNIT_READERS);
     }
-    mbar_init(bar(C_IDLE), 1);
+    mbar_init(bar(C_SFREE), 4);
+    mbar_init(bar(C_IDLE), 3);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -235,50 +238,31 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
           }
         }
       }
-    } else if (warp == 9) {
-      // ------------------------------------------------ MMA issuer
-      // The issuer's own instruction stream is on the critical path of every hand-off (it shares its scheduler with two
-      // softmax warps, and the tensor pipe's queue is an instruction or two deep), so the loop is kept lean: the whole warp
-      // runs it converged and an elected lane issues a tile's eight MMAs and their commit as one block, descriptors are a
-      // fixed high word and a low word that steps by constants, ring slot and phase are running counters, and a barrier is
-      // tested once before the bounded wait loop is entered.
+    } else {
+      // ------------------------------------------------ MMA issuers: warp 9 the scores of both tiles, warps 10 and 11 P V of one each
+      // The tensor pipe's queue is an instruction or two deep, and a barrier test takes an issuer 100 to 250 cycles even where the
+      // phase is long over, so with one warp for everything the pipe stood still for a third of a step while that warp looked at its
+      // seven barriers.  Nothing orders the three warps but the barriers.  Their loops are kept lean: the whole warp runs converged and
+      // an elected lane issues a tile's eight MMAs as one block, descriptors are a fixed high word and a low word that steps by
+      // constants, ring slot and phase are running counters, and a barrier is tested once before the bounded wait loop is entered.
       constexpr uint32_t IDESC = instr_desc(128, false);        // S: both operands K-major
       constexpr uint32_t IDESC_PV = instr_desc(D, true);        // O: V is MN-major
       constexpr uint32_t HI_Q = desc_hi(1024), HI_KV = desc_hi(GROUP_BYTES);
-      const uint32_t q_lo[2] = {desc_lo(sbase + OFF_Q2, 16), desc_lo(sbase + OFF_Q2 + TILE_BYTES, 16)};
-      const uint32_t ring_k_lo = desc_lo(sbase + OFF_RING, 16), ring_v_lo = desc_lo(sbase + OFF_RING, 1024);
       struct Cur {                     // a position in the K/V ring: slot and the parity of its current use
         int s;
         uint32_t ph;
         __device__ Cur next() const { return s + 1 == NSLOT ? Cur{0, ph ^ 1u} : Cur{s + 1, ph}; }
       };
-      Cur cur{0, 0};                   // K_0 of the next unit
-      uint32_t ph_p[2] = {0, 0};       // parity of the next P tile per tile (C_PFULL)
-      uint32_t ph_q = 0;               // parity of the next unit's Q (C_QFULL)
       auto wait_all = [&](uint32_t b, uint32_t parity) {
         if (__all_sync(0xffffffffu, mbar_try(b, parity))) return true;       // the common case: one test
         return __all_sync(0xffffffffu, mbar_wait(b, parity, abort_flag)) != 0;
       };
-      auto wait_full = [&](Cur c) { return wait_all(bar(C_FULL + c.s), c.ph); };
-      auto issue_s = [&](int x, Cur c) {
-        umma_s_tile_elect(tmem + x * 128, q_lo[x], ring_k_lo + (uint32_t)c.s * (TILE_BYTES >> 4), HI_Q, HI_KV, IDESC, bar(C_SFULL + x));
-      };
-      auto issue_pv = [&](int x, Cur c, int h, bool first) {      // keys 64 h .. of the step
-        umma_pv_half_elect(tmem + 256 + x * 128, tmem + x * 128 + 32 * h, ring_v_lo + (uint32_t)c.s * (TILE_BYTES >> 4) + h * (TILE_BYTES >> 5),
-                           HI_KV, IDESC_PV, first ? 0u : 1u);
-      };
-      // PV of a step in two halves, the first while the softmax is still at the last quarter of its exponentials
-      auto take_pv = [&](int x, Cur c, bool first, bool last) {
-        if (!wait_all(bar(C_PHALF + x), ph_p[x])) return false;
-        tc_fence_after();
-        issue_pv(x, c, 0, first);
-        if (!wait_all(bar(C_PFULL + x), ph_p[x])) return false;
-        ph_p[x] ^= 1u;
-        tc_fence_after();
-        issue_pv(x, c, 1, false);
-        if (last) umma_commit_elect(bar(C_ODONE + x));
-        return true;
-      };
+      Cur cur{0, 0};                   // K_0 of the unit, for warps 10 and 11 V_0
+      if (warp != 9) cur = cur.next();
+      const int x = warp - 10;         // the tile of warps 10 and 11
+      uint32_t ph_q = 0;               // parity of the next unit's Q (C_QFULL)
+      uint32_t ph_s = 1;               // parity of the score tile before (C_SFREE); true at once before the first one
+      uint32_t ph_p = 0;               // parity of the next P tile (C_PFULL)
       bool ok = true;
       for (int k = 0; ok; ++k) {
         if (!wait_all(bar(C_UFULL + (k & 1)), (k >> 1) & 1)) break;
@@ -288,37 +272,45 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
         if (lane == 0 && u_index >= 0) mbar_arrive(bar(C_UEMPTY + (k & 1)));
         if (u_index < 0) break;
         if (!u_valid) continue;
-        Cur ck = cur;                  // K_j; V_j and K_(j+1) follow it in the ring
-        ok = wait_all(bar(C_QFULL), ph_q) && wait_full(ck);
-        if (!ok) break;
-        ph_q ^= 1u;
-        tc_fence_after();
-        if (nA > 0) issue_s(0, ck);
-        if (nB > 0) issue_s(1, ck);
-        umma_commit_elect(bar(C_EMPTY + ck.s));
-        if (n_kt == 1) umma_commit_elect(bar(C_QEMPTY));
-        for (int j = 0; ok && j < n_kt; ++j) {
-          const bool more = j + 1 < n_kt;
-          const Cur cv = ck.next(), cn = cv.next();
-          // V_j and K_(j+1) landed long ago as a rule: both tests go first, where the tensor pipe still works on S_B or waits
-          // for tile A's softmax anyway, and not between tile A's two MMA groups
-          ok = wait_full(cv) && (!more || wait_full(cn));
-          if (ok && j < nA) {
-            ok = take_pv(0, cv, j == 0, j == nA - 1);
+        if (warp == 9) {
+          ok = wait_all(bar(C_QFULL), ph_q);
+          ph_q ^= 1u;
+          for (int j = 0; ok && j < n_kt; ++j, cur = cur.next().next()) {
+            ok = wait_all(bar(C_FULL + cur.s), cur.ph);
+            const uint32_t k_lo = desc_lo(sbase + OFF_RING, 16) + (uint32_t)cur.s * (TILE_BYTES >> 4);
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+              if (ok && j < (t == 0 ? nA : nB)) {
+                ok = wait_all(bar(C_SFREE), ph_s);       // the softmax has taken the scores before these
+                if (!ok) break;
+                ph_s ^= 1u;
+                tc_fence_after();
+                umma_s_tile_elect(tmem, desc_lo(sbase + OFF_Q2 + t * TILE_BYTES, 16), k_lo, HI_Q, HI_KV, IDESC, bar(C_SFULL + t));
+              }
+              umma_commit_elect(bar(C_EMPTY + cur.s));
+            }
+            if (j + 1 == n_kt) umma_commit_elect(bar(C_QEMPTY));
           }
-          if (!ok) break;
-          if (j + 1 < nA) issue_s(0, cn);
-          if (j < nB) {
-            ok = take_pv(1, cv, j == 0, j == nB - 1);
-            if (!ok) break;
+        } else {
+          for (int j = 0; ok && j < n_kt; ++j, cur = cur.next().next()) {
+            // (the barrier is for the tile's share in the slot's release too: without it that could be ahead by a phase)
+            ok = wait_all(bar(C_FULL + cur.s), cur.ph);
+            if (ok && j < (x == 0 ? nA : nB)) {
+              // PV of a step in two halves, the first while the softmax is still at the last quarter of its exponentials
+              const uint32_t o = tmem + TM_O + x * 128, p = tmem + TM_P + x * 64;
+              const uint32_t v_lo = desc_lo(sbase + OFF_RING, 1024) + (uint32_t)cur.s * (TILE_BYTES >> 4);
+              if (!(ok = wait_all(bar(C_PHALF + x), ph_p))) break;
+              tc_fence_after();
+              umma_pv_half_elect(o, p, v_lo, HI_KV, IDESC_PV, j == 0 ? 0u : 1u);
+              if (!(ok = wait_all(bar(C_PFULL + x), ph_p))) break;
+              ph_p ^= 1u;
+              tc_fence_after();
+              umma_pv_half_elect(o, p + 32, v_lo + (TILE_BYTES >> 5), HI_KV, IDESC_PV, 1u);
+              umma_commit_elect(bar(C_PVDONE + x));
+            }
+            umma_commit_elect(bar(C_EMPTY + cur.s));
           }
-          umma_commit_elect(bar(C_EMPTY + cv.s));
-          if (j + 1 < nB) issue_s(1, cn);
-          if (more) umma_commit_elect(bar(C_EMPTY + cn.s));
-          if (j + 2 == n_kt) umma_commit_elect(bar(C_QEMPTY));     // the unit's last S MMAs are in the pipe: Q is free after them
-          ck = cn;
         }
-        cur = ck;                      // behind V of the last key tile: K_0 of the next unit
       }
     }
   } else {
@@ -326,10 +318,9 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
     // ------------------------------------------------ softmax of tile x: thread = query row = TMEM lane
     const int x = warp >> 2, row = tid & 127;
     const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    const uint32_t s_addr = lane_addr + x * 128, o_addr = lane_addr + 256 + x * 128;
+    const uint32_t p_addr = lane_addr + TM_P + x * 64, o_addr = lane_addr + TM_O + x * 128;
     const float sl2 = a.scale_log2;
     int steps = 0;      // S tiles of this tile taken so far (phase of C_SFULL)
-    int epis = 0;       // epilogues so far (phase of C_ODONE)
     for (int k = 0;; ++k) {
       // this tile's few fields straight from the published descriptor
       if (!mbar_wait(bar(C_UFULL + (k & 1)), (k >> 1) & 1, abort_flag)) break;
@@ -344,13 +335,16 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
       float m_used = 0.f, m_run = -INFINITY, l = 0.f;
       bool ok = true;
       for (int j = 0; j < nk; ++j) {
-        ok = mbar_wait(bar(C_SFULL + x), steps++ & 1, abort_flag);
+        ok = mbar_wait(bar(C_SFULL + x), steps & 1, abort_flag);
         if (!ok) break;
         tc_fence_after();
         uint32_t s[4][32];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) tmem_ld32(s_addr + 32 * c, s[c]);
+        for (int c = 0; c < 4; ++c) tmem_ld32(lane_addr + 32 * c, s[c]);
         tmem_wait_ld();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(C_SFREE));
         const int u0 = j * KT2;
         if (u0 + KT2 - 1 > lim) {     // a tile that reaches past this row's last visible key
 #pragma unroll
@@ -375,8 +369,13 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
           alpha = ex2_approx((m_used - m_run) * sl2);
           m_used = m_run;
         }
-        // S_X(j) complete implies PV_X(j-1) complete: O may be touched here
+        // P_X and O_X may be touched once PV_X(j-1) is complete
+        bool pv_done = j == 0;
         if (__any_sync(0xffffffffu, rescale)) {
+          ok = mbar_wait(bar(C_PVDONE + x), (steps - 1) & 1, abort_flag);
+          if (!ok) break;
+          tc_fence_after();
+          pv_done = true;
 #pragma unroll
           for (int cb = 0; cb < D; cb += 32) {
             uint32_t o[32];
@@ -388,6 +387,8 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
           }
           l *= alpha;
         }
+        // (as a rule it is by the time the first P is there: the answer of a test ahead of the exponentials costs nothing, one behind them 220 cycles)
+        if (!pv_done) pv_done = mbar_test(bar(C_PVDONE + x), (steps - 1) & 1);
         const float2 sc2 = make_float2(sl2, sl2);
         const float nm = -m_used * sl2;
         const float2 nm2 = make_float2(nm, nm);
@@ -402,14 +403,21 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
             sum[e & 1] = __fadd2_rn(sum[e & 1], p);
             pk[e] = pack_bf16(p.x, p.y);
           }
+          if (c == 0 && !pv_done) {
+            ok = mbar_wait(bar(C_PVDONE + x), (steps - 1) & 1, abort_flag);
+            tc_fence_after();
+            __syncwarp();
+          }
           if (c == 2) {                    // the stores of the first 64 keys have long landed
             tmem_wait_st();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(C_PHALF + x));
           }
-          tmem_st16(s_addr + 16 * c, pk);
+          tmem_st16(p_addr + 16 * c, pk);
         }
+        if (!ok) break;
+        ++steps;
         l += (sum[0].x + sum[0].y) + (sum[1].x + sum[1].y);
         tmem_wait_st();
         tc_fence_before();
@@ -417,7 +425,7 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
         if (lane == 0) mbar_arrive(bar(C_PFULL + x));
       }
       // ---- epilogue: O / l -> bf16, each thread stores its own row (8 x 32 bytes, contiguous)
-      if (ok) ok = mbar_wait(bar(C_ODONE + x), epis++ & 1, abort_flag);
+      if (ok) ok = mbar_wait(bar(C_PVDONE + x), (steps - 1) & 1, abort_flag);
       if (!ok) break;
       tc_fence_after();
       const float inv = l > 0.f ? 1.f / l : 0.f;
@@ -449,7 +457,7 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
   if (*abort_flag) {
     if (tid == 0) atomicOr(a.pv.flags, (uint32_t)FLAG_WAIT_GAVE_UP);
     // copies and MMAs still in flight use this CTA's shared memory and TMEM
-    if (warp == 9) umma_commit_elect(bar(C_IDLE));
+    if (warp >= 9) umma_commit_elect(bar(C_IDLE));
     if (warp == 8 && lane == 0) {
       giveup::drain(kv_fills, NSLOT, [&](int s, uint32_t parity) { return mbar_try(bar(C_FULL + s), parity); });
       giveup::drain(q_fills, 1, [&](int, uint32_t parity) { return mbar_try(bar(C_QFULL), parity); });
