@@ -790,10 +790,14 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
       k.n_req = a.n_req;
       k.n_kv = a.n_kv;
       k.bt = a.bt;
-      sgmv::ShrinkInfo info = {1, 16};
+      sgmv::ShrinkInfo info = {1, 16, false};
       if (n_seg > 0) {
-        rc = sgmv::shrink_scaled(p, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace,
-                                 v_bytes, stream, &info);
+        // Above rank 16 and on wide layers the tcgen05 shrink is the faster one for segments above a few tokens (q, k, v of 128 tokens, one
+        // segment: rank 64 7B 34.0 and 27.2 us, 34B 53 and 45; rank 32 28.4 and 27.5, 46 and 44; 40 tokens 25.8 and 25.2, 43 and 42;
+        // but on a layer of 1024 values, 112 tokens, 19.4 and 20.5).
+        const bool tc = rank_max > 16 && p->sgmv_shrink_kind == 0 && n_tokens > 16 * n_seg && a.d_in >= 2048;
+        rc = (tc ? sgmv::shrink : sgmv::shrink_scaled)(p, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace,
+                                                       v_bytes, stream, &info);
         if (rc != FL_OK) break;
       }
       k.rmax = info.rmax;
@@ -816,7 +820,7 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
     }
     for (int j = n_mats; j < MAX_LIN; ++j) maps.w[j] = maps.w[0];
     if (rc != FL_OK) break;
-    sgmv::ShrinkInfo info = {1, rank_max};
+    sgmv::ShrinkInfo info = {1, rank_max, false};
     if (hybrid) {
       // y = x W from the GEMM alone, then the segmented projection adds the LoRA term to it
       a.ksplit = 1;
@@ -836,22 +840,19 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
       break;
     }
     if (n_seg > 0) {
-      // Two shrinks: in tiles of 16 tokens, whose result is final, and in tiles of 64 (rank 16) or 128 tokens, which read the adapters' rows
-      // less often but split d_in where tiles are few, and a LoRA stage that sums fp32 slices takes 5600 cycles instead of 1500.  The
-      // first one is the better one as long as a segment's x and the rows that it reads again are few (at rank 64, where it reads the
-      // most, as long as the batch is small too).  q, k, v, first and second one: rank 16, 7B, 288 tokens, 20 per segment 64 and 67 us, 72
-      // per segment 59 and 54; 1000 tokens of 1024 values, 100 per segment 23 and 25.  Rank 32, 7B, 1024 tokens, 20 per segment 116 and 162, 102
-      // 95 and 92; 1024 values, 100 26 and 29.  Rank 64, 7B, 1024 tokens, 20 per segment 158 and 294, 102 99 and 112, 8192 tokens, 128 per
-      // segment 780 and 707; 34B, 16384 tokens, 128 per segment 2570 and 2096 us.  Over 960 such batches the choice is 1 % behind the
-      // better one.
-      const double per = (double)n_tokens / n_seg * a.d_in;
-      const bool final = rank_max == 16 ? per <= 1.7e5 : rank_max == 32 ? per <= 3e5
-                       : n_tokens <= 40 * n_seg || (n_tokens <= 128 * n_seg && per * n_tokens <= 4e8);
+      // Two shrinks, in tiles of 16 tokens and of 64 or 128 tokens.  Above rank 16, where the second one runs on tcgen05, it is the better one
+      // for all but segments of a few tokens (q, k, v on 7B, rank 64: 320 tokens, 40 per segment 53 and 35 us; 512, 64 per segment 92 and 60;
+      // 1920, 80 per segment 148 and 138; rank 32, 512 tokens, 64 per segment 61 and 53; 1024 tokens and more the same).  At rank 16 the
+      // second one reads the adapters' rows less often, but where it leaves fp32 slices of d_in a LoRA stage that sums them takes 5600
+      // cycles instead of 1500: the first one is the better one as long as a segment's x and the rows that it reads again are few
+      // (7B, 288 tokens, 20 per segment 64 and 67 us, 72 per segment 59 and 54; 1000 tokens of 1024 values, 100 per segment 23 and 25).
+      const bool tc = rank_max > 16 && p->sgmv_shrink_kind == 0;
+      const bool final = n_tokens <= 16 * n_seg || (!tc && (double)n_tokens / n_seg * a.d_in <= (rank_max == 16 ? 1.7e5 : 3e5));
       rc = final ? sgmv::shrink_scaled(p, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace, v_bytes,
                                        stream, &info)
-                 : sgmv::shrink(p, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, workspace, v_bytes, stream, &info);
+                 : sgmv::shrink(p, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace, v_bytes, stream, &info);
       if (rc != FL_OK) break;
-      if (final) a.v16 = reinterpret_cast<const __nv_bfloat16*>(workspace);
+      if (info.final) a.v16 = reinterpret_cast<const __nv_bfloat16*>(workspace);
     }
     a.ksplit = info.ksplit;
     a.rmax = info.rmax;

@@ -38,7 +38,7 @@ struct SgmvArgs {
   int n_seg, n_tokens;
   float scale;
   float* v;        // [n_mats][ksplit][n_tokens][RMAX]
-  __nv_bfloat16* v16;   // the scaled sum in bf16, [n_mats][n_tokens][RMAX], instead of v: tiles of 16 tokens, or the tcgen05 shrink with one slice; or null
+  __nv_bfloat16* v16;   // the scaled sum in bf16, [n_mats][n_tokens][RMAX], instead of v: tiles of 16 tokens, or the tcgen05 shrink; or null
   int ksplit;
   int tc_ksplit;     // slices of d_in for the tcgen05 shrink of long segments (0 = not applicable)
   int expand_cols;   // y columns one expand CTA covers
@@ -891,7 +891,6 @@ int launch_pair(fl_pool* p, SgmvArgs& a, int tiles, int d_out_max, cudaStream_t 
     a.ksplit = a.tc_ksplit;
     sgmv::TcShrinkArgs t;
     t.pv = a.pv;
-    t.v = a.v;
     t.ksplit = a.ksplit;
     t.n_mats = a.n_mats;
     for (int j = 0; j < 3; ++j) t.mat_index[j] = a.mat_index[j < a.n_mats ? j : 0];
@@ -901,8 +900,7 @@ int launch_pair(fl_pool* p, SgmvArgs& a, int tiles, int d_out_max, cudaStream_t 
     t.n_tokens = a.n_tokens;
     t.d_in = p->mats[a.mat_index[0]].d_in;
     t.scale = a.scale;
-    t.v16 = nullptr;
-    if (!shrink_only && a.ksplit == 1) t.v16 = a.v16 = reinterpret_cast<__nv_bfloat16*>(a.v);      // one slice: v in its final form
+    t.v16 = a.v16 = reinterpret_cast<__nv_bfloat16*>(a.v);
     const int rc = sgmv::shrink_tc(p, t, a.x, RMAX, st);
     if (rc != FL_OK) return rc;
   } else if (TM == 64 && RMAX == 16 && a.n_mats == 3) {      // at higher ranks the three accumulators cost too many registers
@@ -1026,24 +1024,20 @@ int sgmv_common(fl_pool* p, fl_bf16* const* ys, const fl_bf16* x, const int* mat
     if (shrink_ctas < 592 && need <= workspace_bytes) a.ksplit = 2;
   }
   a.tc_ksplit = 0;
-  if (!small && n_mats <= 3 && rmax >= 32) {     // at rank 16 the mma.sync shrink is the faster one
-    // units of (128-token tile, slice of d_in) for the tcgen05 shrink: about four per SM when the scratch the caller
-    // brought has room for the slices, every slice at least 512 values deep
+  if (!small && n_mats <= 3) {
+    // At rank 16 the mma.sync shrink is the faster one for small batches, whose time is look-ups (shrink and expand, 7B: q, k, v of 512 tokens
+    // 13.8 and 15.2 us; o of 2000 tokens 12 and 17), and where the tiles of 128 tokens take more than one round (q, k, v of 19770 tokens
+    // 205 and 214); in between the tcgen05 one is (q, k, v of 3200 tokens 48 and 45, of 5600 70 and 67; on 34B 2000 tokens 32 and 28).
     const int d_in = p->mats[mat_indices[0]].d_in;
-    const long tiles = (long)n_seg + n_tokens / 128;
-    int ks = (int)std::min<long>(8, std::max<long>(1, (4L * p->sm_count + tiles - 1) / tiles));
-    ks = std::min(ks, std::max(1, d_in / 512));
-    // (measured against the size every caller has to bring, not against what this caller brought: the number of
-    // slices fixes the order of the sums, and equal calls should give equal bits)
-    const size_t room = fl_lora_sgmv_workspace(n_tokens, n_mats);
-    while (ks > 1 && (size_t)n_mats * ks * (size_t)n_tokens * rmax * sizeof(float) + 256 > room) --ks;
-    if ((size_t)n_mats * ks * (size_t)n_tokens * rmax * sizeof(float) + 256 <= room) a.tc_ksplit = ks;
+    if (rmax >= 32 || ((double)n_tokens * d_in >= (n_mats == 3 ? 8e6 : 2e7) && n_tokens / 128 + n_seg / 2 < p->sm_count))
+      a.tc_ksplit = sgmv::tc_slices(p, n_seg, n_tokens, d_in, rmax, n_mats);
   }
   int rc;
   const bool so = shrink_only != nullptr;
   if (so) {
-    shrink_only->ksplit = (!small && p->sgmv_shrink_kind == 0 && a.tc_ksplit > 0) ? a.tc_ksplit : a.ksplit;
+    shrink_only->ksplit = a.ksplit;
     shrink_only->rmax = rmax;
+    shrink_only->final = scaled || (!small && p->sgmv_shrink_kind == 0 && a.tc_ksplit > 0);
   }
   if (small) {
     const int tiles = n_seg + n_tokens / 16;
@@ -1066,10 +1060,10 @@ int sgmv_common(fl_pool* p, fl_bf16* const* ys, const fl_bf16* x, const int* mat
 
 namespace sgmv {
 int shrink(fl_pool* p, const fl_bf16* x, const int* mat_indices, int n_mats, const int32_t* seg_indptr,
-           const int32_t* lora_ids, int n_seg, int n_tokens, void* workspace, size_t workspace_bytes, fl_stream stream,
+           const int32_t* lora_ids, int n_seg, int n_tokens, float scale, void* workspace, size_t workspace_bytes, fl_stream stream,
            ShrinkInfo* info) {
   fl_bf16* none[FL_MAX_MATS] = {};
-  return sgmv_common(p, none, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, 1.f, workspace,
+  return sgmv_common(p, none, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace,
                      workspace_bytes, stream, nullptr, info);
 }
 int shrink_scaled(fl_pool* p, const fl_bf16* x, const int* mat_indices, int n_mats, const int32_t* seg_indptr,

@@ -7,15 +7,16 @@ namespace sgmv {
 struct ShrinkInfo {
   int ksplit;   // slices of d_in whose partial sums have to be added
   int rmax;     // row pitch of the partial sums (16, 32 or 64: the pool's highest rank rounded up)
+  bool final;   // slices added, scaled, rounded to bf16 as the expand product takes them, [projection][token][rmax]
 };
 
-// v = x A_i per segment for the listed projections (which share x), unscaled fp32 partial sums written to
-// workspace as [projection][slice][token][rmax]; workspace sized by fl_lora_sgmv_workspace(n_tokens, n_mats).
+// v = x A_i per segment for the listed projections (which share x): unscaled fp32 partial sums written to
+// workspace as [projection][slice][token][rmax], or the final form; workspace sized by fl_lora_sgmv_workspace(n_tokens, n_mats).
 // Rows of segments without an adapter are left untouched.
 int shrink(fl_pool* p, const fl_bf16* x, const int* mat_indices, int n_mats, const int32_t* seg_indptr,
-           const int32_t* lora_ids, int n_seg, int n_tokens, void* workspace, size_t workspace_bytes, fl_stream stream,
+           const int32_t* lora_ids, int n_seg, int n_tokens, float scale, void* workspace, size_t workspace_bytes, fl_stream stream,
            ShrinkInfo* info);
-// The same in its final form: slices added, scaled, rounded to bf16 as the expand product takes them, [projection][token][rmax].
+// The same, always in its final form.
 // Tiles of 16 tokens whatever the segments' lengths, each of which reads its adapter's rows again: for batches of up to a few hundred
 // tokens, and beyond for short segments.
 int shrink_scaled(fl_pool* p, const fl_bf16* x, const int* mat_indices, int n_mats, const int32_t* seg_indptr,
@@ -79,15 +80,45 @@ __device__ __forceinline__ const unsigned char* lora_row(const PoolView& pv, uin
   return pv.slab + (size_t)blk * pv.block_bytes + (size_t)(g % rpb) * 2 * (size_t)width;
 }
 
+// The starts of a thread's COUNT rank-rows, of one or several streams: find(i, entry, offset) gives row i's table entry and its offset in
+// the block, or false where there is no row.  All entries are asked for before any is looked at (one after the other, twelve of them took
+// 3.5 us).  ok[i] = false where there is no row, or none to be read; its start is the slab's.
+template <int COUNT, typename Find>
+__device__ __forceinline__ void lora_rows(const PoolView& pv, Find find, const unsigned char* (&start)[COUNT], bool (&ok)[COUNT]) {
+  uint32_t blk[COUNT], off[COUNT];
+#pragma unroll
+  for (int i = 0; i < COUNT; ++i) {
+    uint32_t entry = 0;
+    off[i] = 0;
+    ok[i] = find(i, entry, off[i]);
+    blk[i] = ok[i] ? pv.tables[entry] : 0u;
+  }
+  bool bad = false;
+#pragma unroll
+  for (int i = 0; i < COUNT; ++i) {
+    if (blk[i] >= pv.n_blocks) {
+      bad = true;
+      ok[i] = false;
+    }
+    start[i] = ok[i] ? pv.slab + (size_t)blk[i] * pv.block_bytes + off[i] : pv.slab;
+  }
+  if (bad) atomicOr(pv.flags, (uint32_t)FLAG_BAD_BLOCK);
+}
+// Table entry and byte offset inside the block of rank-row `row` of a stream (arguments as for lora_row).
+__device__ __forceinline__ void lora_row_at(uint32_t table_off, uint32_t tab, uint32_t row0, uint32_t rpb, int width, int row, uint32_t& entry, uint32_t& off) {
+  const uint32_t g = row0 + (uint32_t)row, q = g / rpb;
+  entry = table_off + tab + q;
+  off = (g - q * rpb) * 2u * (uint32_t)width;
+}
+
 #endif
 
 // The same shrink on the 5th-generation tensor cores for long segments (tiles of 128 tokens, x by TMA, adapter rows
-// by cp.async, accumulator in TMEM); same scratch layout.  Returns FL_EINVAL when it does not cover the case
-// (the caller then takes the mma.sync kernels).
+// by cp.async, accumulator in TMEM), always in its final form.  The slices of d_in are the CTAs of a cluster.
+constexpr int TC_MAX_SLICES = 8;
 struct TcShrinkArgs {
   PoolView pv;
-  float* v;
-  __nv_bfloat16* v16;      // one slice only: the scaled sum in bf16, [projection][token][rmax], instead of v
+  __nv_bfloat16* v16;      // [projection][token][rmax]
   float scale;
   int ksplit, n_mats;
   int mat_index[3];
@@ -95,6 +126,7 @@ struct TcShrinkArgs {
   const int32_t* lora_ids;
   int n_seg, n_tokens, d_in;
 };
+int tc_slices(const fl_pool* p, int n_seg, int n_tokens, int d_in, int rmax, int n_mats);      // slices of d_in to take
 int shrink_tc(fl_pool* p, const TcShrinkArgs& a, const void* x, int rmax, cudaStream_t st);
 
 }  // namespace sgmv

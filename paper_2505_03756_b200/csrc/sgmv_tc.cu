@@ -1,16 +1,19 @@
 // The shrink v = x A_i of the segmented LoRA projection (Eq. 1, Eq. 2; Section 2.1) for long segments, on the
 // 5th-generation tensor cores.
 //
-// At rank 32-64 and three projections per call the mma.sync shrink is bound by the legacy tensor path and by the
-// ldmatrix traffic, not by reading x.  Here a CTA takes a tile of 128 tokens of one segment and a slice of d_in:
-//   warp 0      TMA producer: x tile [128 tokens x 64] per stage (K-major, 128-byte swizzle)
-//   warp 1      MMA issuer: D[128 x (projections * RMAX)] += x tile * adapter rows^T, tcgen05.mma 128 x N x 16
-//   warps 2-5   adapter rows (row p of A is d_in contiguous values in a pool block, found through the adapter's block
-//               table) by 16-byte cp.async into the stage, in the operand's swizzled layout, a few stages in flight
-//   warps 6-9   epilogue: TMEM -> fp32 partial sums [projection][slice][token][RMAX], rows of the segment only
-// The accumulator is double buffered in TMEM, so a unit's epilogue overlaps the next unit's stages.  Units go to
-// the CTAs round robin.  Every mbarrier wait is bounded; a wait that gives up raises a sticky flag and the CTA
-// tears down (its copies drained, its TMEM freed).  No cluster launch, no multicast.
+// A CTA takes a tile of 128 tokens of one segment and a slice of d_in:
+//   warp 0       TMA producer: x tile [128 tokens x 64] per stage (K-major, 128-byte swizzle)
+//   warp 1       MMA issuer: D[128 x (projections * RMAX)] += x tile * adapter rows^T, tcgen05.mma 128 x N x 16
+//   warps 2-9    adapter rows (row p of A is d_in contiguous values in a pool block, found through the adapter's block
+//                table) by 16-byte cp.async into the stage, in the operand's swizzled layout; two groups of four warps take the stages
+//                in turn, and the copies themselves arrive on the stage's barrier when they have landed
+//   warps 10-13  epilogue: TMEM -> v in its final form, scaled and rounded to bf16, [projection][token][RMAX], rows of the segment only
+// Two ways to fill the SMs.  With one slice CTAs stay and go through the tiles, the accumulator is double buffered in TMEM and a tile's
+// epilogue overlaps the next one's stages.  With more (SLICED) the slices of a tile are the CTAs of a cluster: each leaves its sums in its
+// own shared memory, and all threads of a CTA read a share of the columns from all of them and add in the slices' order.  (Sent to the CTA
+// that adds them, by the thread that owns a row, 16 bytes of 32 rows at a time, the sums of three projections at rank 64 took 11 us of 24.)
+// Every mbarrier wait is bounded; a wait that gives up raises a sticky flag and the CTA tears down (its cluster told, its copies
+// drained, its TMEM freed).  No multicast.
 #include <cuda.h>
 #include <algorithm>
 #include "giveup.cuh"
@@ -24,10 +27,10 @@ namespace {
 
 using namespace tc;
 
-constexpr int ST_THREADS = 320;
+constexpr int COPY_GROUPS = 2;
+constexpr int ST_THREADS = 64 + 128 * COPY_GROUPS + 128;
 constexpr int TM = 128, BK = 64;
 constexpr uint32_t X_BYTES = TM * BK * 2;
-constexpr int PF = 4;                 // adapter-row stages a copy thread keeps in flight
 
 template <int N>
 struct Cfg {
@@ -40,6 +43,10 @@ struct Cfg {
   static_assert(2 * N <= 512, "two accumulators must fit in TMEM");
   static_assert(SMEM <= 227 * 1024, "shared memory");
 };
+
+// Columns of a tile that each of the `ks` CTAs of a cluster finishes; row pitch of a CTA's sums in shared memory, in floats.
+__host__ __device__ constexpr int share_of(int n, int ks) { return (n / 16 + ks - 1) / ks * 16; }
+__host__ __device__ constexpr int sum_pitch(int n) { return n + 4; }
 
 struct Unit {
   int seg, tok0, tok1, lid, kb, n_it, split;
@@ -70,13 +77,18 @@ __device__ __forceinline__ Unit decode_unit(const sgmv::TcShrinkArgs& a, int u) 
   return t;
 }
 
-template <int RMAX, int NM>
-__global__ void __launch_bounds__(ST_THREADS, 1) sgmv_shrink_tc_kernel(const sgmv::TcShrinkArgs a, const __grid_constant__ CUtensorMap xmap,
+__device__ __forceinline__ uint4 pack_scaled(const float* f, float scale) {
+  return make_uint4(pack_bf16(f[0] * scale, f[1] * scale), pack_bf16(f[2] * scale, f[3] * scale), pack_bf16(f[4] * scale, f[5] * scale),
+                    pack_bf16(f[6] * scale, f[7] * scale));
+}
+
+template <int RMAX, int NM, bool SLICED>
+__global__ void __launch_bounds__(ST_THREADS, 1) sgmv_shrink_tc_kernel(const __grid_constant__ sgmv::TcShrinkArgs a, const __grid_constant__ CUtensorMap xmap,
                                                                        int n_units) {
   constexpr int N = RMAX * NM;
   using C = Cfg<N>;
   constexpr int NS = C::NS;
-  static_assert(NS > PF, "the ring must hold more stages than a copy thread keeps in flight");
+  static_assert(TM * sum_pitch(N) * 4 <= NS * C::STAGE, "a slice's sums must fit in the ring that they reuse");
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const uint32_t sbase = smem_u32(smem);
@@ -87,11 +99,12 @@ __global__ void __launch_bounds__(ST_THREADS, 1) sgmv_shrink_tc_kernel(const sgm
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + C::OFF_BAR + 8 * B_COUNT);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_BAR + 8 * B_COUNT + 4);
   volatile int* fills_slot = reinterpret_cast<volatile int*>(smem + C::OFF_BAR + 8 * B_COUNT + 8);
-  static_assert(8 * B_COUNT + 12 <= 256, "bookkeeping area too small");
+  volatile int* missing_slot = reinterpret_cast<volatile int*>(smem + C::OFF_BAR + 8 * B_COUNT + 12);      // this CTA has no part of the sum
+  static_assert(8 * B_COUNT + 16 <= 256, "bookkeeping area too small");
 
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) {
-      mbar_init(bar(B_FULL + s), 1 + 128);     // the TMA producer's arrive (with the byte count) + the 128 copy threads
+      mbar_init(bar(B_FULL + s), 1 + 128);     // the TMA producer's arrive (with the byte count) + the 128 threads of a copy group
       mbar_init(bar(B_EMPTY + s), 1);
     }
     for (int b = 0; b < 2; ++b) {
@@ -100,6 +113,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) sgmv_shrink_tc_kernel(const sgm
     }
     mbar_init(bar(B_IDLE), 1);
     *abort_flag = 0;
+    *missing_slot = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -111,76 +125,73 @@ __global__ void __launch_bounds__(ST_THREADS, 1) sgmv_shrink_tc_kernel(const sgm
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   pdl_wait();                 // x may come from the kernel right before this one
-  pdl_launch_dependents();    // the kernel that consumes the partial sums may set itself up while this grid runs
+  pdl_launch_dependents();    // the kernel that consumes v may set itself up while this grid runs
 
-  long long fills = 0, arrived = 0;    // x copies that the producer has issued; stages that a copy thread has signalled
+  // (a sliced tile is the CTA's only one, and every warp needs it again for the sum)
+  const Unit only = SLICED ? decode_unit(a, blockIdx.x) : Unit{};
+  auto unit = [&](int u) { return SLICED ? only : decode_unit(a, u); };
+  int fills = 0;       // x copies that the producer has issued
+  int owed = 0;        // first stage that a copy thread has not signalled yet, of those of its group
+  bool ok = true;
   if (warp == 0) {
     // ------------------------------------------------ TMA producer (lane 0 issues; the warp decodes units together)
-    long long f = 0;
-    bool ok = true;
+    int s = 0;
+    uint32_t ph = 1;
     for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
-      const Unit t = decode_unit(a, u);
+      const Unit t = unit(u);
       if (!t.ok) continue;
-      for (int it = 0; it < t.n_it; ++it, ++f) {
-        if (lane == 0) {
-          const int s = (int)(f % NS);
-          const long long use = f / NS;
-          if (use > 0) ok = mbar_wait(bar(B_EMPTY + s), (uint32_t)((use - 1) & 1), abort_flag);
-          if (ok) {
-            mbar_expect_tx(bar(B_FULL + s), X_BYTES);
-            tma_load_2d(sbase + s * C::STAGE, &xmap, bar(B_FULL + s), t.kb + it * BK, t.tok0);
-            ++fills;
-          }
-        }
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-        if (!ok) break;
-      }
-    }
-  } else if (warp == 1) {
-    // ------------------------------------------------ MMA issuer
-    constexpr uint32_t IDESC = instr_desc(N, false);     // both operands K-major
-    long long f = 0;
-    bool ok = true;
-    int k = 0;       // units with work so far
-    for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
-      const Unit t = decode_unit(a, u);
-      if (!t.ok || t.n_it == 0) continue;
-      const int buf = k & 1;
       if (lane == 0) {
-        if (k >= 2) ok = mbar_wait(bar(B_ACC_EMPTY + buf), (uint32_t)(((k >> 1) - 1) & 1), abort_flag);
-        tc_fence_after();
-        const uint32_t d_tmem = tmem + buf * N;
-        for (int it = 0; ok && it < t.n_it; ++it) {
-          const long long ff = f + it;
-          const int s = (int)(ff % NS);
-          ok = mbar_wait(bar(B_FULL + s), (uint32_t)((ff / NS) & 1), abort_flag);
+        for (int it = 0; it < t.n_it; ++it) {
+          ok = mbar_wait(bar(B_EMPTY + s), ph, abort_flag);
           if (!ok) break;
-          tc_fence_after();
-          const uint32_t ab = sbase + s * C::STAGE, bb = ab + X_BYTES;
-#pragma unroll
-          for (int ks = 0; ks < BK / 16; ++ks)
-            umma_bf16(d_tmem, smem_desc(ab + ks * 32, 16, 1024), smem_desc(bb + ks * 32, 16, 1024), IDESC, (it > 0 || ks > 0) ? 1u : 0u);
-          umma_commit(bar(B_EMPTY + s));
+          mbar_expect_tx(bar(B_FULL + s), X_BYTES);
+          tma_load_2d(sbase + s * C::STAGE, &xmap, bar(B_FULL + s), t.kb + it * BK, t.tok0);
+          ++fills;
+          if (++s == NS) { s = 0; ph ^= 1u; }
         }
-        if (ok) umma_commit(bar(B_ACC_FULL + buf));
       }
       ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-      f += t.n_it;
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------ MMA issuer: the whole warp runs converged, an elected lane issues
+    constexpr uint32_t IDESC = instr_desc(N, false);     // both operands K-major
+    constexpr uint32_t HI = desc_hi(1024);
+    auto wait_all = [&](uint32_t b, uint32_t parity) {
+      if (__all_sync(0xffffffffu, mbar_try(b, parity))) return true;       // the common case: one test
+      return __all_sync(0xffffffffu, mbar_wait(b, parity, abort_flag)) != 0;
+    };
+    int s = 0, k = 0;         // k: units with work so far
+    uint32_t ph = 0;
+    for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
+      const Unit t = unit(u);
+      if (!t.ok || t.n_it == 0) continue;
+      const int buf = k & 1;
+      if (k >= 2) ok = wait_all(bar(B_ACC_EMPTY + buf), (uint32_t)(((k >> 1) - 1) & 1));
+      tc_fence_after();
+      for (int it = 0; ok && it < t.n_it; ++it) {
+        if (!(ok = wait_all(bar(B_FULL + s), ph))) break;
+        fence_async_smem();            // the adapter rows were written by the generic proxy, the tensor core reads through the async one
+        tc_fence_after();
+        const uint32_t a_lo = desc_lo(sbase + s * C::STAGE, 16), b_lo = desc_lo(sbase + s * C::STAGE + X_BYTES, 16);
+#pragma unroll
+        for (int ks = 0; ks < BK / 16; ++ks)
+          umma_ss_elect(tmem + buf * N, a_lo + 2 * ks, HI, b_lo + 2 * ks, HI, IDESC, (it > 0 || ks > 0) ? 1u : 0u);
+        umma_commit_elect(bar(B_EMPTY + s));
+        if (++s == NS) { s = 0; ph ^= 1u; }
+      }
+      if (ok) umma_commit_elect(bar(B_ACC_FULL + buf));
       ++k;
     }
-  } else if (warp < 6) {
+  } else if (warp < 2 + 4 * COPY_GROUPS) {
     // ------------------------------------------------ adapter rows: row n = projection * RMAX + rank row, 8 chunks of 16 bytes
-    const int ct = tid - 64;                      // 0..127
+    const int ct = (tid - 64) & 127, group = (warp - 2) >> 2;
     constexpr int RPT = N / 16;                   // rows per thread: n = ct / 8 + 16 i
     const int cc = ct & 7;
-    long long f = 0;                              // stages issued
-    bool ok = true;
-    auto signal = [&](long long upto) {           // the copies of stages < upto have landed: make them visible, arrive
-      fence_async_smem();
-      for (; arrived < upto; ++arrived) mbar_arrive(bar(B_FULL + (int)(arrived % NS)));
-    };
+    int f = 0, s = 0;                             // stages of this CTA so far
+    uint32_t ph = 1;
+    owed = group;
     for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
-      const Unit t = decode_unit(a, u);
+      const Unit t = unit(u);
       if (!t.ok) continue;
       const LoraEntry* e = a.pv.dir + t.lid;
       const int rank = min(e->rank, RMAX);
@@ -188,88 +199,65 @@ __global__ void __launch_bounds__(ST_THREADS, 1) sgmv_shrink_tc_kernel(const sgm
       const uint32_t table_off = e->table_off;
       const unsigned char* rowp[RPT];
       bool rok[RPT];
-#pragma unroll
-      for (int i = 0; i < RPT; ++i) {
+      sgmv::lora_rows<RPT>(a.pv, [&](int i, uint32_t& entry, uint32_t& off) {
         const int n = (ct >> 3) + 16 * i;
         const int m = n / RMAX, r = n % RMAX;
-        rok[i] = false;
-        rowp[i] = a.pv.slab;
-        if (m < a.n_mats && r < rank) {
-          const LoraMat& lm = e->mats[a.mat_index[m]];
-          rowp[i] = sgmv::lora_row(a.pv, table_off, lm.a_tab, lm.a_row0, lm.a_rpb, a.d_in, r, rok[i]);
-        }
-      }
+        if (m >= a.n_mats || r >= rank) return false;
+        const LoraMat& lm = e->mats[a.mat_index[m]];
+        sgmv::lora_row_at(table_off, lm.a_tab, lm.a_row0, lm.a_rpb, a.d_in, r, entry, off);
+        return true;
+      }, rowp, rok);
       const int ke = min(a.d_in, t.kb + ((a.d_in + a.ksplit * BK - 1) / (a.ksplit * BK)) * BK);
       for (int it = 0; it < t.n_it; ++it, ++f) {
-        const int s = (int)(f % NS);
-        const long long use = f / NS;
-        if (use > 0) ok = mbar_wait(bar(B_EMPTY + s), (uint32_t)((use - 1) & 1), abort_flag);
-        if (!ok) break;
-        const int kk = t.kb + it * BK + cc * 8;
-        const uint32_t bs = sbase + s * C::STAGE + X_BYTES;
+        if ((f & (COPY_GROUPS - 1)) == group) {
+          ok = mbar_wait(bar(B_EMPTY + s), ph, abort_flag);
+          if (!ok) break;
+          const int kk = t.kb + it * BK + cc * 8;
+          const uint32_t bs = sbase + s * C::STAGE + X_BYTES;
 #pragma unroll
-        for (int i = 0; i < RPT; ++i) {
-          const int n = (ct >> 3) + 16 * i;
-          cp_async16(bs + n * 128 + ((cc ^ (n & 7)) << 4), rowp[i] + (size_t)kk * 2, rok[i] && kk < ke);
+          for (int i = 0; i < RPT; ++i) {
+            const int n = (ct >> 3) + 16 * i;
+            cp_async16(bs + n * 128 + ((cc ^ (n & 7)) << 4), rowp[i] + (size_t)kk * 2, rok[i] && kk < ke);
+          }
+          cp_async_arrive(bar(B_FULL + s));       // when they have landed
+          owed = f + COPY_GROUPS;
         }
-        cp_async_commit();
-        if (f + 1 >= PF) {                         // once at most PF - 1 groups are pending, the stages before them have landed
-          cp_async_wait<PF - 1>();
-          signal(f + 2 - PF);
-        }
+        if (++s == NS) { s = 0; ph ^= 1u; }
       }
-      // the unit's last stages: the issuer should not wait for them until this thread has found its next unit
-      cp_async_wait<0>();
-      if (ok) signal(f);
     }
+    cp_async_commit();
     cp_async_wait<0>();
   } else {
     // ------------------------------------------------ epilogue: thread = token row = TMEM lane
     const int quarter = warp & 3;
     const int row = quarter * 32 + lane;
     const uint32_t lane_addr = tmem + ((uint32_t)(quarter * 32) << 16);
-    bool ok = true;
     int k = 0;
     for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
-      const Unit t = decode_unit(a, u);
+      const Unit t = unit(u);
       if (!t.ok) continue;
       const int tok = t.tok0 + row;
       const bool mine = tok < t.tok1;
-      if (t.n_it == 0) {          // an empty slice of d_in still owes its zeros to the sum over slices
-        if (mine)
-          for (int j = 0; j < a.n_mats; ++j) {
-            float4* dst = reinterpret_cast<float4*>(a.v + ((size_t)(j * a.ksplit + t.split) * a.n_tokens + tok) * RMAX);
-            for (int c = 0; c < RMAX / 4; ++c) dst[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-          }
-        continue;
-      }
       const int buf = k & 1;
-      ok = mbar_wait(bar(B_ACC_FULL + buf), (uint32_t)((k >> 1) & 1), abort_flag);
-      ok = __all_sync(0xffffffffu, ok);
+      ok = group_and(mbar_wait(bar(B_ACC_FULL + buf), (uint32_t)((k >> 1) & 1), abort_flag), 1, 128);
       if (!ok) break;
       tc_fence_after();
 #pragma unroll
       for (int c0 = 0; c0 < N; c0 += 16) {
         uint32_t o[16];
+        __syncwarp();
         tmem_ld16(lane_addr + buf * N + c0, o);
         tmem_wait_ld();
         const int j = c0 / RMAX, col = c0 % RMAX;
-        if (mine && j < a.n_mats && a.v16) {
-          uint4* dst = reinterpret_cast<uint4*>(a.v16 + ((size_t)j * a.n_tokens + tok) * RMAX + col);
+        if constexpr (SLICED) {        // (behind the last MMA: nobody reads the ring any more)
 #pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            const uint32_t* q = o + 8 * c;
-            dst[c] = make_uint4(pack_bf16(__uint_as_float(q[0]) * a.scale, __uint_as_float(q[1]) * a.scale),
-                                pack_bf16(__uint_as_float(q[2]) * a.scale, __uint_as_float(q[3]) * a.scale),
-                                pack_bf16(__uint_as_float(q[4]) * a.scale, __uint_as_float(q[5]) * a.scale),
-                                pack_bf16(__uint_as_float(q[6]) * a.scale, __uint_as_float(q[7]) * a.scale));
-          }
+          for (int q = 0; q < 16; q += 4)
+            st_shared_v4(sbase + (uint32_t)(row * sum_pitch(N) + c0 + q) * 4u, make_uint4(o[q], o[q + 1], o[q + 2], o[q + 3]));
         } else if (mine && j < a.n_mats) {
-          float4* dst = reinterpret_cast<float4*>(a.v + ((size_t)(j * a.ksplit + t.split) * a.n_tokens + tok) * RMAX + col);
-#pragma unroll
-          for (int c = 0; c < 4; ++c)
-            dst[c] = make_float4(__uint_as_float(o[4 * c]), __uint_as_float(o[4 * c + 1]), __uint_as_float(o[4 * c + 2]),
-                                 __uint_as_float(o[4 * c + 3]));
+          uint4* dst = reinterpret_cast<uint4*>(a.v16 + ((size_t)j * a.n_tokens + tok) * RMAX + col);
+          const float* of = reinterpret_cast<const float*>(o);
+          dst[0] = pack_scaled(of, a.scale);
+          dst[1] = pack_scaled(of + 8, a.scale);
         }
       }
       tc_fence_before();
@@ -277,6 +265,35 @@ __global__ void __launch_bounds__(ST_THREADS, 1) sgmv_shrink_tc_kernel(const sgm
       if (lane == 0) mbar_arrive(bar(B_ACC_EMPTY + buf));
       ++k;
     }
+    if (SLICED && !ok && tid == ST_THREADS - 1) *missing_slot = 1;
+  }
+  __syncwarp();
+  if (SLICED && only.ok) {       // (the CTAs of a cluster have a tile, or none, together)
+    const int ks = a.ksplit, rank = (int)cluster_ctarank();
+    cluster_sync();          // every slice's sums are there
+    const int told = lane < ks ? (int)ld_cluster_u32(map_cluster_rank(smem_u32(const_cast<int*>(missing_slot)), (uint32_t)lane)) : 0;
+    if (giveup::may_store(true, __any_sync(0xffffffffu, told != 0) ? 1 : 0)) {
+      const int share = share_of(N, ks), c0 = min(rank * share, N), quads = (min(c0 + share, N) - c0) / 4;
+      const int rows = only.tok1 - only.tok0;
+      for (int i = tid; i < rows * quads; i += ST_THREADS) {
+        const int row = i / quads, c = c0 + (i - row * quads) * 4;
+        const uint32_t at = sbase + (uint32_t)(row * sum_pitch(N) + c) * 4u;
+        float4 v[sgmv::TC_MAX_SLICES];
+#pragma unroll
+        for (int p = 0; p < sgmv::TC_MAX_SLICES; ++p)
+          if (p < ks) v[p] = ld_cluster_f32x4(map_cluster_rank(at, (uint32_t)p));
+        float4 f = v[0];
+#pragma unroll
+        for (int p = 1; p < sgmv::TC_MAX_SLICES; ++p)
+          if (p < ks) { f.x += v[p].x; f.y += v[p].y; f.z += v[p].z; f.w += v[p].w; }
+        const int j = c / RMAX, col = c % RMAX;
+        if (j < a.n_mats)
+          *reinterpret_cast<uint2*>(a.v16 + ((size_t)j * a.n_tokens + only.tok0 + row) * RMAX + col) =
+              make_uint2(pack_bf16(f.x * a.scale, f.y * a.scale), pack_bf16(f.z * a.scale, f.w * a.scale));
+      }
+    }
+    __syncwarp();
+    cluster_sync();          // nobody leaves while its sums are still being read
   }
   // ------------------------------------------------ teardown
   tc_fence_before();
@@ -284,13 +301,13 @@ __global__ void __launch_bounds__(ST_THREADS, 1) sgmv_shrink_tc_kernel(const sgm
   if (*abort_flag) {
     if (tid == 0) atomicOr(a.pv.flags, (uint32_t)FLAG_WAIT_GAVE_UP);
     // x copies and MMAs still in flight use this CTA's shared memory and TMEM (the adapter-row copies were waited for by their own
-    // threads above).  A stage's phase ends with its x copy only if the copy threads signal it too; each owes at most the last
+    // threads above).  A stage's phase ends with its x copy only if its copy threads signal it too; each owes at most the last
     // phase of a slot, since the one before it was over when the producer armed it.
-    if (tid == 0) *fills_slot = (int)fills;
+    if (tid == 0) *fills_slot = fills;
     __syncthreads();
-    if (warp >= 2 && warp < 6)
-      for (; arrived < *fills_slot; ++arrived) mbar_arrive(bar(B_FULL + (int)(arrived % NS)));
-    if (warp == 1 && lane == 0) umma_commit(bar(B_IDLE));
+    if (warp >= 2 && warp < 2 + 4 * COPY_GROUPS)
+      for (; owed < *fills_slot; owed += COPY_GROUPS) mbar_arrive(bar(B_FULL + owed % NS));
+    if (warp == 1) umma_commit_elect(bar(B_IDLE));
     if (tid == 0) {
       giveup::drain(fills, NS, [&](int s, uint32_t parity) { return mbar_try(bar(B_FULL + s), parity); });
       giveup::drain(1, 1, [&](int, uint32_t parity) { return mbar_try(bar(B_IDLE), parity); });
@@ -308,11 +325,14 @@ int launch(fl_pool* p, const sgmv::TcShrinkArgs& a, const CUtensorMap& xmap, int
   using C = Cfg<RMAX * NM>;
   static bool configured[16] = {};
   if (!configured[p->device & 15]) {
-    FL_CUDA(p, cudaFuncSetAttribute(sgmv_shrink_tc_kernel<RMAX, NM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM));
+    FL_CUDA(p, cudaFuncSetAttribute(sgmv_shrink_tc_kernel<RMAX, NM, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM));
+    FL_CUDA(p, cudaFuncSetAttribute(sgmv_shrink_tc_kernel<RMAX, NM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM));
     configured[p->device & 15] = true;
   }
-  const unsigned grid = (unsigned)std::min(n_units, p->sm_count);
-  FL_CUDA(p, launch_pdl(sgmv_shrink_tc_kernel<RMAX, NM>, dim3(grid), dim3(ST_THREADS), C::SMEM, st, a, xmap, n_units));
+  if (a.ksplit > 1)
+    FL_CUDA(p, launch_pdl_cluster(sgmv_shrink_tc_kernel<RMAX, NM, true>, dim3((unsigned)n_units), dim3((unsigned)a.ksplit), dim3(ST_THREADS), C::SMEM, st, a, xmap, n_units));
+  else
+    FL_CUDA(p, launch_pdl(sgmv_shrink_tc_kernel<RMAX, NM, false>, dim3((unsigned)std::min(n_units, p->sm_count)), dim3(ST_THREADS), C::SMEM, st, a, xmap, n_units));
   FL_CUDA(p, cudaGetLastError());
   return FL_OK;
 }
@@ -321,9 +341,27 @@ int launch(fl_pool* p, const sgmv::TcShrinkArgs& a, const CUtensorMap& xmap, int
 
 namespace sgmv {
 
+int tc_slices(const fl_pool* p, int n_seg, int n_tokens, int d_in, int rmax, int n_mats) {
+  // Rounds of tiles over the SMs times what a tile's slice takes: about 6 us of look-ups, ramp and end, 4 us more where slices are added,
+  // and per stage the fill of x and of the adapter rows at 50 bytes per clock.  Clusters of four find a place on the GPU's groups of 16 to
+  // 20 SMs about 32 times, clusters of eight 16 times; other sizes leave more SMs empty.
+  const long tiles = (n_tokens + TM - 1) / TM + n_seg / 2;
+  const int nk = (d_in + BK - 1) / BK;
+  const double stage = (X_BYTES + n_mats * rmax * 128) / 95e3;
+  int best = 1;
+  double least = 0;
+  for (int ks = 1; ks <= TC_MAX_SLICES && (ks == 1 || nk / ks >= 4); ks *= 2) {
+    const int kchunk = (nk + ks - 1) / ks;
+    if ((ks - 1) * kchunk >= nk) continue;                                       // every slice of d_in must hold something
+    const long at_once = ks <= 2 ? p->sm_count / ks : p->sm_count * 9 / 10 / ks;
+    const double cost = (double)((tiles + at_once - 1) / at_once) * (6 + (ks > 1 ? 4 : 0) + kchunk * stage);
+    if (ks == 1 || cost < least) { least = cost; best = ks; }
+  }
+  return best;
+}
+
 int shrink_tc(fl_pool* p, const TcShrinkArgs& a, const void* x, int rmax, cudaStream_t st) {
-  if (a.n_mats < 1 || a.n_mats > 3 || a.d_in % 8 != 0 || a.ksplit < 1) return FL_EINVAL;
-  if ((long long)(a.ksplit - 1) * BK >= a.d_in) return FL_EINVAL;      // every slice of d_in must hold something
+  if (a.n_mats < 1 || a.n_mats > 3 || a.d_in % 8 != 0 || a.ksplit < 1 || a.ksplit > TC_MAX_SLICES) return FL_EINVAL;
   alignas(64) CUtensorMap xmap;
   const uint64_t dims[2] = {(uint64_t)a.d_in, (uint64_t)a.n_tokens};
   const uint64_t strides[1] = {(uint64_t)a.d_in * 2};
