@@ -23,6 +23,12 @@ using sgmv::lora_row;
 constexpr int SG_THREADS = 128;
 constexpr int KS = 64;            // d_in elements per shrink pipeline stage (128-byte rows)
 constexpr int SH_STAGES = 4;
+// Tiles of 16 tokens behind which the final form is wanted: a CTA's slice is 8 to 27 stages, each 0.5 us after the one before with four in
+// flight, and the projection's CTAs that need the SM wait meanwhile.  More in flight where the CTAs all run at once: shrink and projection of
+// o, 64 tokens, 15 adapters of rank 64, 34B 42.7 -> 38.9 us (12 stages; 8: 40.1); one token of rank 16 on 7B, 46.9 -> 46.2 us a layer (8 stages;
+// with 12 there is no room for the projection's CTAs beside these, and it takes 49.0).
+constexpr int deep_stages(int rmax) { return rmax == 64 ? 12 : 8; }
+constexpr double deep_per_sm(int rmax) { return rmax == 64 ? 1.1 : rmax == 32 ? 2 : 3; }
 constexpr int NSUB = 128;         // y columns per expand sub-tile (256-byte rows)
 constexpr int EXPAND_COLS_MIN = 512, EXPAND_COLS_MAX = 2048;   // y columns per expand CTA: picked per call
 constexpr int KSPLIT_MAX = 8;
@@ -67,9 +73,9 @@ __device__ __forceinline__ uint4 add_bf16x8(uint4 a, uint4 b) {
 }
 
 // the pipeline's stages, and for short tiles (which reuse it) the sums of the four warps
-__host__ __device__ constexpr int shrink_pipe_bytes(int tm, int rmax) { return SH_STAGES * (tm + rmax) * 128; }
+__host__ __device__ constexpr int shrink_pipe_bytes(int tm, int rmax, int stages) { return stages * (tm + rmax) * 128; }
 
-template <int TM, int RMAX>
+template <int TM, int RMAX, int STAGES>
 __global__ void __launch_bounds__(SG_THREADS) sgmv_shrink_kernel(const SgmvArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   pdl_wait();                 // x may come from the kernel right before this one
@@ -112,17 +118,14 @@ __global__ void __launch_bounds__(SG_THREADS) sgmv_shrink_kernel(const SgmvArgs 
     xok[i] = t < tok1;
     xrow[i] = a.x + (size_t)(xok[i] ? t : tok0) * d_in;
   }
-  const __nv_bfloat16* arow[AR];
+  const unsigned char* arow[AR];
   bool aok[AR];
-#pragma unroll
-  for (int i = 0; i < AR; ++i) {
+  sgmv::lora_rows<AR>(a.pv, [&](int i, uint32_t& entry, uint32_t& off) {
     const int r = crow + 16 * i;
-    aok[i] = false;
-    arow[i] = reinterpret_cast<const __nv_bfloat16*>(a.pv.slab);
-    if (r < rank)
-      arow[i] = reinterpret_cast<const __nv_bfloat16*>(
-          lora_row(a.pv, table_off, lm.a_tab, lm.a_row0, lm.a_rpb, d_in, r, aok[i]));
-  }
+    if (r >= rank) return false;
+    sgmv::lora_row_at(table_off, lm.a_tab, lm.a_row0, lm.a_rpb, d_in, r, entry, off);
+    return true;
+  }, arow, aok);
   const uint32_t sbase = smem_u32(smem);
   auto load_stage = [&](int it, int st) {
     const int kk = kb + it * KS + cchunk * 8;
@@ -131,7 +134,7 @@ __global__ void __launch_bounds__(SG_THREADS) sgmv_shrink_kernel(const SgmvArgs 
 #pragma unroll
     for (int i = 0; i < XR; ++i) cp_async16(xs + swz(crow + 16 * i, cchunk, 8), xrow[i] + kk, xok[i] && kok);
 #pragma unroll
-    for (int i = 0; i < AR; ++i) cp_async16(as + swz(crow + 16 * i, cchunk, 8), arow[i] + kk, aok[i] && kok);
+    for (int i = 0; i < AR; ++i) cp_async16(as + swz(crow + 16 * i, cchunk, 8), arow[i] + (size_t)kk * 2, aok[i] && kok);
   };
 
   float acc[RMAX / 8][4];
@@ -139,17 +142,17 @@ __global__ void __launch_bounds__(SG_THREADS) sgmv_shrink_kernel(const SgmvArgs 
   for (int n = 0; n < RMAX / 8; ++n) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
 
 #pragma unroll
-  for (int s = 0; s < SH_STAGES - 1; ++s) {
+  for (int s = 0; s < STAGES - 1; ++s) {
     if (s < n_it) load_stage(s, s);
     cp_async_commit();
   }
   const int mrow = (TM == 64 ? warp * 16 : 0) + (lane & 7) + 8 * ((lane >> 3) & 1);
   for (int it = 0; it < n_it; ++it) {
-    cp_async_wait<SH_STAGES - 2>();
+    cp_async_wait<STAGES - 2>();
     __syncthreads();
-    if (it + SH_STAGES - 1 < n_it) load_stage(it + SH_STAGES - 1, (it + SH_STAGES - 1) % SH_STAGES);
+    if (it + STAGES - 1 < n_it) load_stage(it + STAGES - 1, (it + STAGES - 1) % STAGES);
     cp_async_commit();
-    const uint32_t xs = sbase + (it % SH_STAGES) * STAGE_BYTES, as = xs + TM * 128;
+    const uint32_t xs = sbase + (it % STAGES) * STAGE_BYTES, as = xs + TM * 128;
 #pragma unroll
     for (int ks = 0; ks < KS / 16; ++ks) {
       if (TM == 16 && ks != warp) continue;   // short tiles: the four warps split each stage along k
@@ -200,7 +203,7 @@ __global__ void __launch_bounds__(SG_THREADS) sgmv_shrink_kernel(const SgmvArgs 
     // through distributed shared memory.  The slices are added in order: the result does not depend on timing.  (Where an
     // expand of the same few microseconds follows, it adds the slices itself: the cluster's barrier costs 1 to 2 us more than
     // it saves there.)
-    float* all = reinterpret_cast<float*>(smem + shrink_pipe_bytes(TM, RMAX));      // first CTA: [slice][16 rows][RMAX]
+    float* all = reinterpret_cast<float*>(smem + shrink_pipe_bytes(TM, RMAX, STAGES));      // first CTA: [slice][16 rows][RMAX]
     __syncthreads();
     if (clustered) cluster_wait();
     const uint32_t dst = clustered ? map_cluster_rank(smem_u32(all + split * 16 * RMAX), 0) : 0;
@@ -877,15 +880,22 @@ int launch_expand_short(fl_pool* p, SgmvArgs& a, int tiles, int d_out_max, cudaS
   return FL_OK;
 }
 
-template <int TM, int RMAX>
-int launch_pair(fl_pool* p, SgmvArgs& a, int tiles, int d_out_max, cudaStream_t st, bool shrink_only) {
+template <int TM, int RMAX, int STAGES>
+int launch_shrink(fl_pool* p, const SgmvArgs& a, int tiles, cudaStream_t st) {
   static bool configured[16] = {};
-  const int shrink_smem_max = shrink_pipe_bytes(TM, RMAX) + (TM == 16 ? KSPLIT_MAX * 16 * RMAX * 4 : 0);
-  const int shrink_smem = a.v16 ? shrink_smem_max : shrink_pipe_bytes(TM, RMAX);      // + every slice's sums
+  const int smem_max = shrink_pipe_bytes(TM, RMAX, STAGES) + (TM == 16 ? KSPLIT_MAX * 16 * RMAX * 4 : 0);
+  const int smem = a.v16 ? smem_max : shrink_pipe_bytes(TM, RMAX, STAGES);      // + every slice's sums
   if (!configured[p->device & 15]) {
-    FL_CUDA(p, cudaFuncSetAttribute(sgmv_shrink_kernel<TM, RMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, shrink_smem_max));
+    FL_CUDA(p, cudaFuncSetAttribute(sgmv_shrink_kernel<TM, RMAX, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
     configured[p->device & 15] = true;
   }
+  FL_CUDA(p, launch_pdl_cluster(sgmv_shrink_kernel<TM, RMAX, STAGES>, dim3(tiles * a.n_mats, a.ksplit), dim3(1, a.v16 ? a.ksplit : 1),
+                                dim3(SG_THREADS), smem, st, a));
+  return FL_OK;
+}
+
+template <int TM, int RMAX>
+int launch_pair(fl_pool* p, SgmvArgs& a, int tiles, int d_out_max, cudaStream_t st, bool shrink_only) {
   if (TM == 64 && p->sgmv_shrink_kind == 0 && a.n_mats <= 3 && a.tc_ksplit > 0) {
     // long segments: the shrink on tcgen05 tensor cores, tiles of 128 tokens, its own number of d_in slices
     a.ksplit = a.tc_ksplit;
@@ -918,8 +928,9 @@ int launch_pair(fl_pool* p, SgmvArgs& a, int tiles, int d_out_max, cudaStream_t 
     else
       FL_CUDA(p, launch_pdl(sgmv_shrink3_kernel<RMAX, 4>, dim3(tiles, a.ksplit), dim3(SG_THREADS), smem_of[1], st, a));
   } else {
-    FL_CUDA(p, launch_pdl_cluster(sgmv_shrink_kernel<TM, RMAX>, dim3(tiles * a.n_mats, a.ksplit), dim3(1, a.v16 ? a.ksplit : 1),
-                                  dim3(SG_THREADS), shrink_smem, st, a));
+    const bool deep = TM == 16 && a.v16 && tiles * a.n_mats * a.ksplit <= p->sm_count * deep_per_sm(RMAX);
+    const int rc = deep ? launch_shrink<TM, RMAX, TM == 16 ? deep_stages(RMAX) : SH_STAGES>(p, a, tiles, st) : launch_shrink<TM, RMAX, SH_STAGES>(p, a, tiles, st);
+    if (rc != FL_OK) return rc;
   }
   if (shrink_only) return FL_OK;       // the caller consumes the partial sums itself
   return TM == 64 ? launch_expand_long<RMAX>(p, a, st) : launch_expand_short<RMAX>(p, a, tiles, d_out_max, st);
