@@ -584,14 +584,47 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_decode_kernel(const AttnArgs
 
 // ------------------------------------------------------------------ prefill (tensor-core tiles, mma.sync)
 // One CTA per (request, tile of 64 new tokens, query head); warp w owns rows 16w..16w+15.
+// PLANNED = false: small batches, all requests, whatever their new tokens, in one kernel.  Every warp finds its tile by itself from the
+// requests' numbers, 32 requests at a time.  What such a batch takes is the chain of look-ups and launches: plan, tcgen05 prefill kernel and
+// a decode kernel without work take 10 us for 4 requests of 32 new tokens behind 32 (8 heads), this one 5.
+__device__ __forceinline__ bool find_query_tile(const AttnArgs& a, int item, int& req, int& q0) {
+  const int lane = threadIdx.x & 31;
+  for (int r0 = 0; r0 < a.n_req; r0 += 32) {
+    const int tiles = r0 + lane < a.n_req ? (max(0, a.new_lens[r0 + lane]) + QT - 1) / QT : 0;
+    int incl = tiles;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int o = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += o;
+    }
+    const uint32_t behind = __ballot_sync(0xffffffffu, incl > item);      // the first request that ends behind the tile
+    if (behind) {
+      const int src = __ffs(behind) - 1;
+      req = r0 + src;
+      q0 = (item - __shfl_sync(0xffffffffu, incl - tiles, src)) * QT;
+      return true;
+    }
+    item -= __shfl_sync(0xffffffffu, incl, 31);
+  }
+  return false;
+}
+template <bool PLANNED>
 __global__ void __launch_bounds__(ATT_THREADS) attn_prefill_kernel(const AttnArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   const int item = blockIdx.x / a.n_q, hq = blockIdx.x % a.n_q;
-  if (item >= a.hdr->n_prefill) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t4 = lane & 3;
-  const int2 it = a.prefill_list[item];
-  const int i = it.x, q0 = it.y;
+  int i, q0;
+  if (PLANNED) {
+    if (item >= a.hdr->n_prefill) return;
+    const int2 it = a.prefill_list[item];
+    i = it.x;
+    q0 = it.y;
+  } else {
+    pdl_wait();                 // q, K and V come from the kernel right before this one
+    pdl_launch_dependents();
+    if (!find_query_tile(a, item, i, q0)) return;
+  }
   const int n_new = a.new_lens[i], prefix = a.prefix_lens[i], ctx = prefix + n_new;
   const int h = hq / (a.n_q / a.n_kv);
   const int tok0 = a.req_indptr[i] + q0;
@@ -742,6 +775,16 @@ Packed packed_slots(int n_req, int n_tbl, int n_kv, int csize, int sms) {
   return p;
 }
 
+// Batches that attn_prefill_kernel<false> serves by itself: contexts of at most eight blocks in the mean, a table that leaves little room for one
+// long context among short ones (the lengths themselves are not known here), and CTAs that run in three rounds at most.  A CTA takes 2.3 us
+// per 64 keys, so it is contexts that the line is about.  Attention, this kernel and the three of the planned way, in us, heads / KV heads
+// 8/8, 32/32, 64/8: 1 request of 32 new tokens behind 32 5.0 and 9.6, 5.1 and 10.0, 5.1 and 10.4; 4 such 5.1 and 9.9, 5.7 and 10.4, 6.1 and
+// 11.4; 16 such 5.7 and 10.4, 10.8 and 20.1, (64/8 stays planned) 19.6 and 21.7; 4 of 64 behind 64 7.3 and 10.0, 8.7 and 10.6, 9.2 and 11.9.
+// Beyond: 1 request of 64 new tokens behind 192 12.0 and 11.4, 12.1 and 11.5, 12.3 and 12.8; 1 of 128 behind 384 21 and 14, 21 and 14, 25 and 16.
+bool small_batch(int n_req, int n_tokens, int n_tbl, int n_q, int sms) {
+  return (n_tokens / QT + n_req) * (long long)n_q <= 6ll * sms && n_tbl <= 8ll * n_req && n_tbl <= 32 + 2ll * n_req;
+}
+
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct WsLayout {
@@ -823,7 +866,8 @@ int fl_paged_attention(fl_pool* p, fl_bf16* out, const fl_bf16* q, const int32_t
           cudaFuncSetAttribute(attn_decode_kernel<BESIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, DEC_SMEM) != cudaSuccess ||
           cudaFuncSetAttribute(attn_decode_kernel<CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize, DEC_SMEM) != cudaSuccess ||
           cudaFuncSetAttribute(attn_decode_kernel<PACKED>, cudaFuncAttributeMaxDynamicSharedMemorySize, DEC_SMEM) != cudaSuccess ||
-          cudaFuncSetAttribute(attn_prefill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PRE_SMEM) != cudaSuccess) {
+          cudaFuncSetAttribute(attn_prefill_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PRE_SMEM) != cudaSuccess ||
+          cudaFuncSetAttribute(attn_prefill_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PRE_SMEM) != cudaSuccess) {
         p->last_cuda = (int)cudaGetLastError();
         rc = FL_ECUDA;
         break;
@@ -855,6 +899,14 @@ int fl_paged_attention(fl_pool* p, fl_bf16* out, const fl_bf16* q, const int32_t
       }
       break;
     }
+    if (kind == 0 && small_batch(n_req, n_tokens, n_tbl, n_q_heads, p->sm_count)) {
+      const cudaError_t e = launch_pdl(attn_prefill_kernel<false>, dim3((unsigned)(w.max_prefill * n_q_heads)), dim3(ATT_THREADS), PRE_SMEM, st, a);
+      if (e != cudaSuccess) {
+        p->last_cuda = (int)e;
+        rc = FL_ECUDA;
+      }
+      break;
+    }
     // every kernel of the call is a programmatic dependent launch: it may start while the one before it drains
     // and waits inside for that kernel's results
     if (launch_pdl(attn_plan_kernel, dim3(1), dim3(256), 0, st, a, w.chunk,
@@ -869,7 +921,7 @@ int fl_paged_attention(fl_pool* p, fl_bf16* out, const fl_bf16* q, const int32_t
       if (rc != FL_OK) break;
       beside = max_items > 0;
     } else {
-      attn_prefill_kernel<<<(unsigned)w.max_prefill * n_q_heads, ATT_THREADS, PRE_SMEM, st>>>(a);
+      attn_prefill_kernel<true><<<(unsigned)w.max_prefill * n_q_heads, ATT_THREADS, PRE_SMEM, st>>>(a);
     }
     cudaError_t e = launch_pdl(beside ? attn_decode_kernel<BESIDE> : attn_decode_kernel<PLAIN>, dim3((unsigned)w.max_decode * n_kv_heads + (beside ? 1u : 0u)),
                                dim3(ATT_THREADS), DEC_SMEM, st, a, w.chunk, 0);

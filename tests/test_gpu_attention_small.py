@@ -1,0 +1,53 @@
+"""fl_paged_attention of small batches, served by one kernel without a plan: new tokens around a tile's 64 rows and a warp's 16,
+contexts around 64 keys, requests without a new token, one-token requests among prompts, more than 32 requests, grouped heads, a
+request whose table is too short, and batches on either side of the line to the planned kernels."""
+import math
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from oracle.attention import attend_request
+from paper_2505_03756_b200 import synth
+
+from _util import assert_close, oracle_context
+
+
+@pytest.mark.parametrize("heads,prefix,new", [
+    ((4, 4), [0], [64]), ((4, 4), [0], [65]), ((8, 8), [32] * 4, [32] * 4), ((2, 2), [0, 63, 1, 15], [63, 1, 17, 128]),
+    ((8, 2), [64, 0, 16], [64, 16, 33]), ((8, 1), [17, 40], [19, 3]), ((4, 4), [0, 5, 0, 30], [127, 0, 1, 18]),
+    ((2, 1), [7 * (i % 9) for i in range(40)], [1 + 5 * (i % 7) for i in range(40)]), ((4, 4), [300] + [0] * 9, [30] + [16] * 9),
+    ((16, 16), [60], [68]), ((16, 16), [61], [68]), ((32, 32), [16] * 13, [64] * 13), ((32, 32), [16] * 14, [64] * 14)])
+def test_small_batch(heads, prefix, new):
+    from paper_2505_03756_b200 import harness as H
+    wl = synth.make_workload("tiny", n_req=len(new), len_range=(0, 0), n_adapters=1, shape=synth.LayerShape(heads[0] * 128, *heads))
+    wl.prefix_lens[:], wl.new_lens[:] = prefix, new
+    wl.pool_blocks = int(np.sum((wl.prefix_lens + wl.new_lens + 15) // 16)) + 64
+    s = H.Session(wl, adapters=[])
+    try:
+        s.build_batch()
+        s.fill_prefix_kv()
+        k_new, v_new = wl.kv_new()
+        s.kv_append(H.f32_to_dev(k_new, s.dev), H.f32_to_dev(v_new, s.dev))
+        q = wl.q()
+        tq = H.f32_to_dev(q, s.dev)
+        out = torch.full(q.shape, float("nan"), dtype=torch.bfloat16, device=s.dev)
+        s.attention(out, tq)
+        got = H.dev_to_f32(out)
+        for i in range(wl.n_req):
+            lo, hi = int(wl.req_indptr[i]), int(wl.req_indptr[i + 1])
+            k, v = oracle_context(wl, i, k_new, v_new)
+            assert_close(got[lo:hi], attend_request(q[lo:hi], k, v, prefix[i], 1.0 / math.sqrt(128)), f"small {heads} request {i}")
+        assert s.status()["device_flags"] == 0
+        if len(new) > 1 and new[-1] > 0:                         # the last request's keys now end behind its table
+            s.t_prefix[-1] += 4096
+            bad = torch.full(q.shape, 3.0, dtype=torch.bfloat16, device=s.dev)
+            s.attention(bad, tq)
+            torch.cuda.synchronize()
+            n = int(wl.req_indptr[-2])
+            assert torch.equal(bad[:n], out[:n]) and bool((bad[n:] == 3.0).all())
+            assert s.status(clear=True)["device_flags"] != 0
+    finally:
+        s.close()
