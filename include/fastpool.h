@@ -102,8 +102,8 @@ int fl_pool_status(fl_pool* pool, fl_status* out, int clear);
 int fl_last_cuda_error(fl_pool* pool);
 /* Switches.  FL_OPT_PREFILL_KERNEL: 0 (default) = prefill attention on tcgen05 tensor cores with
  * TMEM accumulators and TMA-staged pages, two query tiles per CTA sharing the K/V stream; 1 = the
- * mma.sync kernel.  Same results within rounding.  The tcgen05 kernel needs sm_scale > 0; other values are
- * served by the mma.sync kernel.
+ * mma.sync kernel.  Same results within rounding.  The tcgen05 kernel needs sm_scale > 0; other values, and small
+ * batches of short contexts, are served by the mma.sync kernel.
  * FL_OPT_POISON_FREED: 1 = debugging aid that stands in for a memory checker: fl_block_free waits for the
  * device and fills every freed DEVICE block with 0xFF bytes (bf16 NaN patterns), so a block table that still
  * names a freed block turns the output of whatever reads it into NaN instead of plausible numbers.  0 (default)

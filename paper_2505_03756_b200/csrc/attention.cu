@@ -2,7 +2,8 @@
 //
 // A plan kernel sorts the requests of a batch into two work lists: requests with at most 16 query
 // rows per KV head (decode steps) are cut into chunks of keys that independent CTAs reduce
-// (split-KV, merged by the last of them); the others (prefill) are cut into tiles of 64 query rows per head.
+// (split-KV, merged by the last of them); the others (prefill) are cut into tiles of 64 query rows per head, or of 128 for the
+// tcgen05 kernel.  A few decode requests, and small batches of any kind, are served without a plan.
 // Both kernels stage KV pages (one 4 KiB contiguous piece per block, KV head and K/V side) into
 // shared memory with 16-byte cp.async through the block table and run QK^T and PV on bf16 tensor
 // cores with an fp32 online softmax.

@@ -86,7 +86,7 @@ struct fl_pool {
 // may still read), which waits for that whole grid and its memory operations.  A kernel that calls
 // pdl_launch_dependents() lets the next one start once all its CTAs are past that point: the shrinks, the attention kernels and the
 // projection of few tokens do; behind the expands, the projection of long batches and the KV append the next kernel starts when they
-// have ended.  Both instructions do nothing in a kernel launched the ordinary way, as the KV append and the mma.sync prefill kernel are.
+// have ended.  Both instructions do nothing in a kernel launched the ordinary way, as the KV append and the planned mma.sync prefill kernel are.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <typename... KArgs, typename... Args>

@@ -576,7 +576,8 @@ __global__ void __launch_bounds__(SG_THREADS, 5) sgmv_expand_kernel(const SgmvAr
 // What bounds it: reading and writing y; on the way there the instructions per piece of y and the latency of the prologue's
 // look-ups, which is why all 64 row addresses are found at once (a lane each), and so are the places of all the CTA's K / V
 // rows (a thread each; looked up tile by tile in the loop they cost 24 of 223 us for the q, k, v call of 64 prompts on 7B).
-// Shrink and expand of 16384 tokens on 34B (rank 64): o 217 -> 179 us, q, k, v with the KV store 271 -> 240 us; of 19770
+// Shrink and expand of 16384 tokens on 34B (rank 64): o 217 -> 179 us, q, k, v with the KV store 271 -> 240 us (171 and 226 with the
+// shrink of today); of 19770
 // tokens on 7B (rank 16): 98 -> 93 us and 232 -> 205 us; before, tiles of 64 tokens and 128 columns with three barriers
 // each had one tile of y per CTA in flight and read the B rows again for every 64 tokens.
 constexpr int EX_COLS = 256, EX_DEPTH = 4;
