@@ -343,8 +343,8 @@ namespace sgmv {
 
 int tc_slices(const fl_pool* p, int n_seg, int n_tokens, int d_in, int rmax, int n_mats) {
   // Rounds of tiles over the SMs times what a tile's slice takes: about 6 us of look-ups, ramp and end, 4 us more where slices are added,
-  // and per stage the fill of x and of the adapter rows at 50 bytes per clock.  Clusters of four find a place on the GPU's groups of 16 to
-  // 20 SMs about 32 times, clusters of eight 16 times; other sizes leave more SMs empty.
+  // and per stage the fill of x and of the adapter rows at 50 bytes per clock.  Clusters of four find a place on the GPU's groups of SMs
+  // 33 times, clusters of eight 15 times (as the occupancy query says for this shared memory); other sizes leave more SMs empty.
   const long tiles = (n_tokens + TM - 1) / TM + n_seg / 2;
   const int nk = (d_in + BK - 1) / BK;
   const double stage = (X_BYTES + n_mats * rmax * 128) / 95e3;
@@ -353,7 +353,7 @@ int tc_slices(const fl_pool* p, int n_seg, int n_tokens, int d_in, int rmax, int
   for (int ks = 1; ks <= TC_MAX_SLICES && (ks == 1 || nk / ks >= 4); ks *= 2) {
     const int kchunk = (nk + ks - 1) / ks;
     if ((ks - 1) * kchunk >= nk) continue;                                       // every slice of d_in must hold something
-    const long at_once = ks <= 2 ? p->sm_count / ks : p->sm_count * 9 / 10 / ks;
+    const long at_once = ks <= 2 ? p->sm_count / ks : ks == 4 ? p->sm_count * 9 / 40 : p->sm_count * 13 / 128;
     const double cost = (double)((tiles + at_once - 1) / at_once) * (6 + (ks > 1 ? 4 : 0) + kchunk * stage);
     if (ks == 1 || cost < least) { least = cost; best = ks; }
   }
