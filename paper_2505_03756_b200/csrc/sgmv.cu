@@ -26,7 +26,8 @@ constexpr int SH_STAGES = 4;
 // Tiles of 16 tokens behind which the final form is wanted: a CTA's slice is 8 to 27 stages, each 0.5 us after the one before with four in
 // flight, and the projection's CTAs that need the SM wait meanwhile.  More in flight where the CTAs all run at once: shrink and projection of
 // o, 64 tokens, 15 adapters of rank 64, 34B 42.7 -> 38.9 us (12 stages; 8: 40.1); one token of rank 16 on 7B, 46.9 -> 46.2 us a layer (8 stages;
-// with 12 there is no room for the projection's CTAs beside these, and it takes 49.0).
+// with 12 there is no room for the projection's CTAs beside these, and it takes 49.0).  Not for slices of a few stages, which only lose that
+// room (8 tokens of rank 32 on a layer of 1024 values: 37.0 -> 38.9 us a layer).
 constexpr int deep_stages(int rmax) { return rmax == 64 ? 12 : 8; }
 constexpr double deep_per_sm(int rmax) { return rmax == 64 ? 1.1 : rmax == 32 ? 2 : 3; }
 constexpr int NSUB = 128;         // y columns per expand sub-tile (256-byte rows)
@@ -929,7 +930,8 @@ int launch_pair(fl_pool* p, SgmvArgs& a, int tiles, int d_out_max, cudaStream_t 
     else
       FL_CUDA(p, launch_pdl(sgmv_shrink3_kernel<RMAX, 4>, dim3(tiles, a.ksplit), dim3(SG_THREADS), smem_of[1], st, a));
   } else {
-    const bool deep = TM == 16 && a.v16 && tiles * a.n_mats * a.ksplit <= p->sm_count * deep_per_sm(RMAX);
+    const int slice = (p->mats[a.mat_index[0]].d_in + KS * a.ksplit - 1) / (KS * a.ksplit);       // stages
+    const bool deep = TM == 16 && a.v16 && slice > SH_STAGES && tiles * a.n_mats * a.ksplit <= p->sm_count * deep_per_sm(RMAX);
     const int rc = deep ? launch_shrink<TM, RMAX, TM == 16 ? deep_stages(RMAX) : SH_STAGES>(p, a, tiles, st) : launch_shrink<TM, RMAX, SH_STAGES>(p, a, tiles, st);
     if (rc != FL_OK) return rc;
   }
