@@ -9,7 +9,7 @@
 //   warps 0-3   softmax of tile A (thread = query row = TMEM lane)      warp 8   TMA producer, unit fetch
 //   warps 4-7   softmax of tile B                                        warp 9   MMA issuer of the scores, TMEM owner
 //                                                                        warps 10, 11   MMA issuers of P V, a tile each
-//   K_j / V_j (128 keys = 8 pool pages each, one 4 KiB TMA box per page) -> ring of 32 KiB slots, 128-byte swizzle;
+//   K_j / V_j (128 keys = 8 pool pages each, one 4 KiB TMA box per page) -> two rings of 32 KiB slots, 128-byte swizzle;
 //   a page lands as [8-key group][64-value half][8 keys][64 values], so a tile's 8-key groups are 2 KiB apart
 //   S   = Q_X K_j^T     tcgen05.mma 128x128x16 (x8) into TMEM columns that both tiles use in turn
 //   P_X = exp2(S - m) -> bf16 pairs in TMEM columns of tile X's own
@@ -30,6 +30,7 @@
 #include <string.h>
 #include <algorithm>
 #include "attention.cuh"
+#include "attention_roles.cuh"
 #include "giveup.cuh"
 #include "mma_utils.cuh"
 #include "tc_ptx.cuh"
@@ -42,20 +43,21 @@ using namespace tc;
 
 constexpr int T2_THREADS = 384;                        // three warpgroups: softmax A, softmax B, {TMA, MMA x 3}
 constexpr int KT2 = 128;                               // keys per tile
-constexpr int NSLOT = 5;                               // ring slots; fills go K_0, V_0, K_1, V_1, ... across units
 constexpr uint32_t HALF_BYTES = 128 * 128;             // [128 rows][64 bf16], swizzled
 constexpr uint32_t TILE_BYTES = 2 * HALF_BYTES;        // a Q, K or V tile
 constexpr uint32_t PAGE_BYTES = BT * 128 * 2;          // K or V of one head of one block: [2 groups][2 halves][8 tokens][64 bf16]
 constexpr uint32_t GROUP_BYTES = PAGE_BYTES / 2;       // stride between 8-key groups of a K/V tile
 constexpr uint32_t OFF_Q2 = 0;                         // Q_A, Q_B
-constexpr uint32_t OFF_RING = 2 * TILE_BYTES;
-constexpr uint32_t OFF_BAR2 = OFF_RING + NSLOT * TILE_BYTES;
+constexpr uint32_t OFF_K = 2 * TILE_BYTES;
+constexpr uint32_t OFF_V = OFF_K + K_SLOTS * TILE_BYTES;
+constexpr uint32_t OFF_BAR2 = OFF_V + V_SLOTS * TILE_BYTES;
 constexpr uint32_t T2_SMEM = OFF_BAR2 + 512;           // barriers, TMEM address, abort flag, two unit descriptors
 constexpr uint32_t T2_TMEM_COLS = 512;                 // S (128 columns) | P_A | P_B (64 each) | O_A | O_B (128 each)
 constexpr uint32_t TM_P = 128, TM_O = 256;
 constexpr float RESCALE_LOG2 = 8.f;
 
-enum { C_QFULL = 0, C_QEMPTY = 1, C_FULL = 2, C_EMPTY = C_FULL + NSLOT, C_SFULL = C_EMPTY + NSLOT, C_SFREE = C_SFULL + 2,
+enum { C_QFULL = 0, C_QEMPTY = 1, C_KFULL = 2, C_KEMPTY = C_KFULL + K_SLOTS, C_VFULL = C_KEMPTY + K_SLOTS, C_VEMPTY = C_VFULL + V_SLOTS,
+       C_SFULL = C_VEMPTY + V_SLOTS, C_SFREE = C_SFULL + 2,
        C_PFULL = C_SFREE + 1, C_PHALF = C_PFULL + 2, C_PVDONE = C_PHALF + 2, C_UFULL = C_PVDONE + 2, C_UEMPTY = C_UFULL + 2, C_IDLE = C_UEMPTY + 2, C_COUNT };
 constexpr int UNIT_READERS = 11;                       // three MMA issuers + 8 softmax warps
 
@@ -125,9 +127,13 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
   if (tid == 0) {
     mbar_init(bar(C_QFULL), 1);
     mbar_init(bar(C_QEMPTY), 1);
-    for (int s = 0; s < NSLOT; ++s) {
-      mbar_init(bar(C_FULL + s), 1);
-      mbar_init(bar(C_EMPTY + s), 2);      // one arrival per tile
+    for (int s = 0; s < K_SLOTS; ++s) {
+      mbar_init(bar(C_KFULL + s), 1);
+      mbar_init(bar(C_KEMPTY + s), 1);
+    }
+    for (int s = 0; s < V_SLOTS; ++s) {
+      mbar_init(bar(C_VFULL + s), 1);
+      mbar_init(bar(C_VEMPTY + s), 2);      // one arrival per tile
     }
     for (int x = 0; x < 2; ++x) {
       mbar_init(bar(C_SFULL + x), 1);
@@ -159,7 +165,7 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
 
   // Readers take the k-th unit of this CTA from slot k & 1 (index -1 = no more work) and release the slot.
 
-  int kv_fills = 0, q_fills = 0;       // ring slots and Q buffers that the producer has armed
+  int k_fills = 0, v_fills = 0, q_fills = 0;       // ring slots and Q buffers that the producer has armed
 
   // the softmax warpgroups keep 128 scores per thread in registers: they take the registers the third
   // warpgroup does not need
@@ -169,7 +175,8 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
       // ------------------------------------------------ unit fetch + TMA producer
       // The whole warp runs the loop; lane 0 fetches units and does the waiting, lanes 0-7 each own one of a tile's eight
       // pages (their block-id loads and their TMA issues run side by side).
-      int fill = 0;                    // ring fills so far, over all units
+      RingPos<K_SLOTS> k_pos;
+      RingPos<V_SLOTS> v_pos;
       int n_valid = 0;                 // units whose Q tiles were loaded so far
       bool ok = true;
       for (int k = 0; ok; ++k) {
@@ -208,35 +215,34 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
           const int x = lane >> 1, half = lane & 1;
           tma_load_3d(sbase + OFF_Q2 + x * TILE_BYTES + half * HALF_BYTES, &q_map, bar(C_QFULL), 64 * half, up->hq[x], up->tok0[x]);
         }
-        for (int j = 0; ok && j < n_kt_max; ++j) {
-          // this lane's page of the tile (pages behind the last needed key are masked anyway: re-read the last
-          // valid page); K_j and V_j come from the same blocks
-          // lane = page: eight lanes issue one 4 KiB box each
-          uint32_t blk = 0;
-          if (lane < KT2 / BT) {
-            blk = a.tbl[tbl0 + min(j * (KT2 / BT) + lane, n_pages - 1)];
-            if (blk >= a.pv.n_blocks) {
-              atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_BLOCK);
-              blk = 0;
+        // this lane's page of the tile (pages behind the last needed key are masked anyway: re-read the last
+        // valid page); K_j and V_j come from the same blocks
+        // lane = page: eight lanes issue one 4 KiB box each
+        uint32_t blk = 0;
+        auto fill = [&](int side, uint32_t slot, uint32_t full, uint32_t empty, uint32_t parity, int& fills) {
+          if (lane == 0) {
+            ok = mbar_wait(empty, parity, abort_flag);
+            if (ok) {
+              mbar_expect_tx(full, TILE_BYTES);
+              ++fills;
             }
           }
-#pragma unroll
-          for (int side = 0; side < 2; ++side, ++fill) {
-            const int s = fill % NSLOT, use = fill / NSLOT;
-            if (lane == 0) {
-              if (use > 0) ok = mbar_wait(bar(C_EMPTY + s), (use - 1) & 1, abort_flag);
-              if (ok) {
-                mbar_expect_tx(bar(C_FULL + s), TILE_BYTES);
-                ++kv_fills;
-              }
-            }
-            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;     // the transaction count is armed before any copy is issued
-            if (!ok) break;
-            if (lane < KT2 / BT)
-              tma_load_5d(sbase + OFF_RING + s * TILE_BYTES + lane * PAGE_BYTES, &kv_map, bar(C_FULL + s), 0, 0, 0,
-                          2 * (side * a.n_kv + h), (int)blk);
-          }
-        }
+          ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;     // the transaction count is armed before any copy is issued
+          if (ok && lane < KT2 / BT) tma_load_5d(slot + lane * PAGE_BYTES, &kv_map, full, 0, 0, 0, 2 * (side * a.n_kv + h), (int)blk);
+          return ok;
+        };
+        load_tiles(n_kt_max, k_pos, v_pos,
+                   [&](int j) {
+                     if (lane < KT2 / BT) {
+                       blk = a.tbl[tbl0 + min(j * (KT2 / BT) + lane, n_pages - 1)];
+                       if (blk >= a.pv.n_blocks) {
+                         atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_BLOCK);
+                         blk = 0;
+                       }
+                     }
+                   },
+                   [&](RingPos<K_SLOTS> p) { return fill(0, sbase + OFF_K + p.s * TILE_BYTES, bar(C_KFULL + p.s), bar(C_KEMPTY + p.s), p.ph ^ 1u, k_fills); },
+                   [&](RingPos<V_SLOTS> p) { return fill(1, sbase + OFF_V + p.s * TILE_BYTES, bar(C_VFULL + p.s), bar(C_VEMPTY + p.s), p.ph ^ 1u, v_fills); });
       }
     } else {
       // ------------------------------------------------ MMA issuers: warp 9 the scores of both tiles, warps 10 and 11 P V of one each
@@ -248,17 +254,12 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
       constexpr uint32_t IDESC = instr_desc(128, false);        // S: both operands K-major
       constexpr uint32_t IDESC_PV = instr_desc(D, true);        // O: V is MN-major
       constexpr uint32_t HI_Q = desc_hi(1024), HI_KV = desc_hi(GROUP_BYTES);
-      struct Cur {                     // a position in the K/V ring: slot and the parity of its current use
-        int s;
-        uint32_t ph;
-        __device__ Cur next() const { return s + 1 == NSLOT ? Cur{0, ph ^ 1u} : Cur{s + 1, ph}; }
-      };
       auto wait_all = [&](uint32_t b, uint32_t parity) {
         if (__all_sync(0xffffffffu, mbar_try(b, parity))) return true;       // the common case: one test
         return __all_sync(0xffffffffu, mbar_wait(b, parity, abort_flag)) != 0;
       };
-      Cur cur{0, 0};                   // K_0 of the unit, for warps 10 and 11 V_0
-      if (warp != 9) cur = cur.next();
+      RingPos<K_SLOTS> k_pos;          // of warp 9
+      RingPos<V_SLOTS> v_pos;          // of warps 10 and 11
       const int x = warp - 10;         // the tile of warps 10 and 11
       uint32_t ph_q = 0;               // parity of the next unit's Q (C_QFULL)
       uint32_t ph_s = 1;               // parity of the score tile before (C_SFREE); true at once before the first one
@@ -275,41 +276,29 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
         if (warp == 9) {
           ok = wait_all(bar(C_QFULL), ph_q);
           ph_q ^= 1u;
-          for (int j = 0; ok && j < n_kt; ++j, cur = cur.next().next()) {
-            ok = wait_all(bar(C_FULL + cur.s), cur.ph);
-            const uint32_t k_lo = desc_lo(sbase + OFF_RING, 16) + (uint32_t)cur.s * (TILE_BYTES >> 4);
-#pragma unroll
-            for (int t = 0; t < 2; ++t) {
-              if (ok && j < (t == 0 ? nA : nB)) {
-                ok = wait_all(bar(C_SFREE), ph_s);       // the softmax has taken the scores before these
-                if (!ok) break;
-                ph_s ^= 1u;
-                tc_fence_after();
-                umma_s_tile_elect(tmem, desc_lo(sbase + OFF_Q2 + t * TILE_BYTES, 16), k_lo, HI_Q, HI_KV, IDESC, bar(C_SFULL + t));
-              }
-              umma_commit_elect(bar(C_EMPTY + cur.s));
-            }
-            if (j + 1 == n_kt) umma_commit_elect(bar(C_QEMPTY));
-          }
+          if (ok)
+            ok = issue_scores(n_kt, nA, nB, k_pos, ph_s,
+                              [&](RingPos<K_SLOTS> p) { return wait_all(bar(C_KFULL + p.s), p.ph); },
+                              [&](uint32_t ph) { return wait_all(bar(C_SFREE), ph); },
+                              [&](int t, RingPos<K_SLOTS> p) {
+                                tc_fence_after();
+                                umma_s_tile_elect(tmem, desc_lo(sbase + OFF_Q2 + t * TILE_BYTES, 16), desc_lo(sbase + OFF_K, 16) + (uint32_t)p.s * (TILE_BYTES >> 4),
+                                                  HI_Q, HI_KV, IDESC, bar(C_SFULL + t));
+                              },
+                              [&](RingPos<K_SLOTS> p) { umma_commit_elect(bar(C_KEMPTY + p.s)); },
+                              [&] { umma_commit_elect(bar(C_QEMPTY)); });
         } else {
-          for (int j = 0; ok && j < n_kt; ++j, cur = cur.next().next()) {
-            // (the barrier is for the tile's share in the slot's release too: without it that could be ahead by a phase)
-            ok = wait_all(bar(C_FULL + cur.s), cur.ph);
-            if (ok && j < (x == 0 ? nA : nB)) {
-              // PV of a step in two halves, the first while the softmax is still at the last quarter of its exponentials
-              const uint32_t o = tmem + TM_O + x * 128, p = tmem + TM_P + x * 64;
-              const uint32_t v_lo = desc_lo(sbase + OFF_RING, 1024) + (uint32_t)cur.s * (TILE_BYTES >> 4);
-              if (!(ok = wait_all(bar(C_PHALF + x), ph_p))) break;
-              tc_fence_after();
-              umma_pv_half_elect(o, p, v_lo, HI_KV, IDESC_PV, j == 0 ? 0u : 1u);
-              if (!(ok = wait_all(bar(C_PFULL + x), ph_p))) break;
-              ph_p ^= 1u;
-              tc_fence_after();
-              umma_pv_half_elect(o, p + 32, v_lo + (TILE_BYTES >> 5), HI_KV, IDESC_PV, 1u);
-              umma_commit_elect(bar(C_PVDONE + x));
-            }
-            umma_commit_elect(bar(C_EMPTY + cur.s));
-          }
+          ok = issue_pv(n_kt, x == 0 ? nA : nB, v_pos, ph_p,
+                        [&](RingPos<V_SLOTS> p) { return wait_all(bar(C_VFULL + p.s), p.ph); },
+                        [&](int half, uint32_t ph) { return wait_all(bar((half == 0 ? C_PHALF : C_PFULL) + x), ph); },
+                        [&](int half, RingPos<V_SLOTS> p, bool first) {
+                          tc_fence_after();
+                          umma_pv_half_elect(tmem + TM_O + x * 128, tmem + TM_P + x * 64 + 32 * half,
+                                             desc_lo(sbase + OFF_V, 1024) + (uint32_t)p.s * (TILE_BYTES >> 4) + half * (TILE_BYTES >> 5), HI_KV, IDESC_PV,
+                                             first && half == 0 ? 0u : 1u);
+                        },
+                        [&] { umma_commit_elect(bar(C_PVDONE + x)); },
+                        [&](RingPos<V_SLOTS> p) { umma_commit_elect(bar(C_VEMPTY + p.s)); });
         }
       }
     }
@@ -459,7 +448,8 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
     // copies and MMAs still in flight use this CTA's shared memory and TMEM
     if (warp >= 9) umma_commit_elect(bar(C_IDLE));
     if (warp == 8 && lane == 0) {
-      giveup::drain(kv_fills, NSLOT, [&](int s, uint32_t parity) { return mbar_try(bar(C_FULL + s), parity); });
+      giveup::drain(k_fills, K_SLOTS, [&](int s, uint32_t parity) { return mbar_try(bar(C_KFULL + s), parity); });
+      giveup::drain(v_fills, V_SLOTS, [&](int s, uint32_t parity) { return mbar_try(bar(C_VFULL + s), parity); });
       giveup::drain(q_fills, 1, [&](int, uint32_t parity) { return mbar_try(bar(C_QFULL), parity); });
       giveup::drain(1, 1, [&](int, uint32_t parity) { return mbar_try(bar(C_IDLE), parity); });
     }
