@@ -87,4 +87,14 @@ ROLE_FN bool issue_pv(int n_kt, int n, V& v, uint32_t& ph_p, Full full, Part par
   return ok;
 }
 
+// A look at a barrier, a test or a bounded wait, by all lanes of a warp that go on to tensor-memory instructions: those are aligned, so the
+// lanes have to agree (each looks for itself, and the phase may end in between), and what the phase's MMAs touched is only theirs behind a
+// tcgen05 fence.
+template <typename Look, typename Vote, typename Fence>
+ROLE_FN bool seen_by_all(Look look, Vote vote, Fence fence) {
+  if (!vote(look())) return false;
+  fence();
+  return true;
+}
+
 }  // namespace attn

@@ -310,9 +310,11 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
     const uint32_t p_addr = lane_addr + TM_P + x * 64, o_addr = lane_addr + TM_O + x * 128;
     const float sl2 = a.scale_log2;
     int steps = 0;      // S tiles of this tile taken so far (phase of C_SFULL)
+    auto vote = [](bool v) { return __all_sync(0xffffffffu, v) != 0; };
+    auto wait = [&](int k, int parity) { return seen_by_all([&] { return mbar_wait(bar(k), (uint32_t)parity, abort_flag); }, vote, tc_fence_after); };
     for (int k = 0;; ++k) {
       // this tile's few fields straight from the published descriptor
-      if (!mbar_wait(bar(C_UFULL + (k & 1)), (k >> 1) & 1, abort_flag)) break;
+      if (!vote(mbar_wait(bar(C_UFULL + (k & 1)), (k >> 1) & 1, abort_flag))) break;
       const Unit* up = unit_slot + (k & 1);
       const int u_index = up->index, u_valid = up->valid;
       const int rows = up->rows[x], nk = up->n_kt[x], lim0 = up->lim0[x], out_tok0 = up->tok0[x], out_hq = up->hq[x];
@@ -324,9 +326,8 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
       float m_used = 0.f, m_run = -INFINITY, l = 0.f;
       bool ok = true;
       for (int j = 0; j < nk; ++j) {
-        ok = mbar_wait(bar(C_SFULL + x), steps & 1, abort_flag);
+        ok = wait(C_SFULL + x, steps & 1);
         if (!ok) break;
-        tc_fence_after();
         uint32_t s[4][32];
 #pragma unroll
         for (int c = 0; c < 4; ++c) tmem_ld32(lane_addr + 32 * c, s[c]);
@@ -361,9 +362,8 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
         // P_X and O_X may be touched once PV_X(j-1) is complete
         bool pv_done = j == 0;
         if (__any_sync(0xffffffffu, rescale)) {
-          ok = mbar_wait(bar(C_PVDONE + x), (steps - 1) & 1, abort_flag);
+          ok = wait(C_PVDONE + x, (steps - 1) & 1);
           if (!ok) break;
-          tc_fence_after();
           pv_done = true;
 #pragma unroll
           for (int cb = 0; cb < D; cb += 32) {
@@ -377,7 +377,7 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
           l *= alpha;
         }
         // (as a rule it is by the time the first P is there: the answer of a test ahead of the exponentials costs nothing, one behind them 220 cycles)
-        if (!pv_done) pv_done = mbar_test(bar(C_PVDONE + x), (steps - 1) & 1);
+        if (!pv_done) pv_done = seen_by_all([&] { return mbar_test(bar(C_PVDONE + x), (steps - 1) & 1); }, vote, tc_fence_after);
         const float2 sc2 = make_float2(sl2, sl2);
         const float nm = -m_used * sl2;
         const float2 nm2 = make_float2(nm, nm);
@@ -392,11 +392,7 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
             sum[e & 1] = __fadd2_rn(sum[e & 1], p);
             pk[e] = pack_bf16(p.x, p.y);
           }
-          if (c == 0 && !pv_done) {
-            ok = mbar_wait(bar(C_PVDONE + x), (steps - 1) & 1, abort_flag);
-            tc_fence_after();
-            __syncwarp();
-          }
+          if (c == 0 && !pv_done) ok = wait(C_PVDONE + x, (steps - 1) & 1);
           if (c == 2) {                    // the stores of the first 64 keys have long landed
             tmem_wait_st();
             tc_fence_before();
@@ -414,9 +410,8 @@ attn_prefill_tc2_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap kv
         if (lane == 0) mbar_arrive(bar(C_PFULL + x));
       }
       // ---- epilogue: O / l -> bf16, each thread stores its own row (8 x 32 bytes, contiguous)
-      if (ok) ok = mbar_wait(bar(C_PVDONE + x), (steps - 1) & 1, abort_flag);
+      if (ok) ok = wait(C_PVDONE + x, (steps - 1) & 1);
       if (!ok) break;
-      tc_fence_after();
       const float inv = l > 0.f ? 1.f / l : 0.f;
       uint4* orow = reinterpret_cast<uint4*>(a.out + ((size_t)(out_tok0 + row) * a.n_q + out_hq) * D);
 #pragma unroll

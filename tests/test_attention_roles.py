@@ -266,3 +266,53 @@ int main() {
   return lone > 0 && pairs == 0 ? 0 : 1;
 }
 """)
+
+
+def test_a_softmax_warp_stores_as_one_and_behind_a_fence(tmp_path):
+    """32 lanes that look at the barrier of the step before one after the other, while its phase ends at any time, and go on to an
+    aligned store: they take one way to it, behind the phase's end and behind a fence that follows their last look.  The model sees it
+    when the lanes do not vote, or do not fence."""
+    run_model(tmp_path, """
+enum { VOTES = 1, FENCES = 2 };
+struct Meet { int here = 0; bool all = true; };
+int faults(int with) {
+  int bad = 0;
+  for (int end = 1; end < 400; end += 3) {
+    Sim sim;
+    Bar pv;
+    Meet votes[2];
+    int waited = 0, stored = 0;
+    sim.at(end, [&] { pv.arrive(); });
+    for (int lane = 0; lane < 32; ++lane)
+      sim.spawn([&, lane] {
+        bool fenced = false;
+        int round = 0;
+        auto vote = [&](bool v) {
+          if (!(with & VOTES)) return v;
+          Meet& m = votes[round++];
+          m.all &= v;
+          for (++m.here; m.here < 32;) sim.pass(1);
+          return m.all;
+        };
+        auto fence = [&] { fenced = (with & FENCES) != 0; };
+        sim.pass(1 + lane);                     // the lanes' looks are not at one time
+        bool done = attn::seen_by_all([&] { fenced = false; return pv.test(0); }, vote, fence);
+        sim.pass(100);
+        if (!done) {
+          ++waited;
+          done = attn::seen_by_all([&] { fenced = false; while (!pv.test(0)) sim.pass(1 + lane % 3); return true; }, vote, fence);
+        }
+        ++stored;
+        bad += !done || !fenced || !pv.test(0);
+      });
+    sim.run();
+    bad += stored != 32 || (waited != 0 && waited != 32);
+  }
+  return bad;
+}
+int main() {
+  const int good = faults(VOTES | FENCES), lone = faults(FENCES), open = faults(VOTES);
+  printf("%d faults, %d without the vote, %d without the fence\\n", good, lone, open);
+  return good == 0 && lone > 0 && open > 0 ? 0 : 1;
+}
+""")
