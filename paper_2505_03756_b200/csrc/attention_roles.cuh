@@ -45,24 +45,26 @@ ROLE_FN bool load_tiles(int n_kt, K& k, V& v, Pages pages, FillK fill_k, FillV f
   return true;
 }
 
+// An issuer whose wait gave up leaves at once and gives nothing back: the copies into its slots may still be on their way, and the producer
+// would arm a barrier whose phase is open, which the draining behind a wait that gave up (giveup.cuh) could not make out.
+
 // Issuer of the scores S = Q_X K_j^T of both tiles, nA and nB steps of n_kt: ph_free is the parity of the score tile before, which its
 // softmax warps have to have taken.
 template <typename K, typename Full, typename Free, typename Issue, typename Release, typename ReleaseQ>
 ROLE_FN bool issue_scores(int n_kt, int nA, int nB, K& k, uint32_t& ph_free, Full full, Free free, Issue issue, Release release, ReleaseQ release_q) {
-  bool ok = true;
-  for (int j = 0; ok && j < n_kt; ++j, k = k.next()) {
-    ok = full(k);
+  for (int j = 0; j < n_kt; ++j, k = k.next()) {
+    if (!full(k)) return false;
 #pragma unroll
     for (int x = 0; x < 2; ++x) {
-      if (!ok || j >= (x == 0 ? nA : nB)) continue;
-      if (!(ok = free(ph_free))) break;
+      if (j >= (x == 0 ? nA : nB)) continue;
+      if (!free(ph_free)) return false;
       ph_free ^= 1u;
       issue(x, k);
     }
     release(k);
-    if (j + 1 == n_kt) release_q();
   }
-  return ok;
+  release_q();
+  return true;
 }
 
 // Issuer of O_X += P_X V_j of one tile, n steps of n_kt.  P of a step comes in two halves of 64 keys, and the product of the first runs
@@ -70,13 +72,12 @@ ROLE_FN bool issue_scores(int n_kt, int nA, int nB, K& k, uint32_t& ph_free, Ful
 // in the slot's release would be ahead by a phase otherwise.
 template <typename V, typename Full, typename Part, typename Issue, typename Done, typename Release>
 ROLE_FN bool issue_pv(int n_kt, int n, V& v, uint32_t& ph_p, Full full, Part part, Issue issue, Done done, Release release) {
-  bool ok = true;
-  for (int j = 0; ok && j < n_kt; ++j, v = v.next()) {
-    ok = full(v);
-    if (ok && j < n) {
+  for (int j = 0; j < n_kt; ++j, v = v.next()) {
+    if (!full(v)) return false;
+    if (j < n) {
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        if (!(ok = part(h, ph_p))) return false;
+        if (!part(h, ph_p)) return false;
         issue(h, v, j == 0);
       }
       ph_p ^= 1u;
@@ -84,7 +85,7 @@ ROLE_FN bool issue_pv(int n_kt, int n, V& v, uint32_t& ph_p, Full full, Part par
     }
     release(v);
   }
-  return ok;
+  return true;
 }
 
 // A look at a barrier, a test or a bounded wait, by all lanes of a warp that go on to tensor-memory instructions: those are aligned, so the

@@ -72,7 +72,7 @@ struct Bar {
 struct Slot { int tile = -1, readers = 0, open = 0; };      // what has landed, MMAs under way on it, copies under way into it
 
 struct Unit { int n[2]; };
-constexpr long LIMIT = 200000, NEVER = 40 * LIMIT;
+constexpr long LIMIT = 60000, NEVER = 40 * LIMIT;
 
 // One ring: K and V take turns, as the kernel had it once.  Own rings: the kernel's.
 struct Shared5 : attn::RingPos<5> {
@@ -246,6 +246,51 @@ def test_tiles_are_there_when_they_are_read_and_stay_until_they_have_been(tmp_pa
     """Units of one and two query tiles, one to twelve key tiles, alone and with another unit behind them, and any copy late."""
     run_model(tmp_path, """
 int main() { all_units(own_rings); return wrong ? 1 : 0; }
+""")
+
+
+def test_nothing_is_given_back_behind_a_wait_that_gave_up(tmp_path):
+    """Any one copy, of K or of V, that lands long after the waits' limit: the slots whose copies are on their way are not armed again, so
+    that the drain behind the abort waits for every copy."""
+    run_model(tmp_path, """
+int main() {
+  static char text[128];
+  for (int b : {0, 1, 9})
+    for (int late = 0; late < 28; ++late)
+      for (int more = 0; more < 3; ++more) {              // the copies behind it: on time, as late, or a little late
+        snprintf(text, sizeof(text), "late copy %d, second tile %d, more %d", late, b, more);
+        where = text;
+        Cta c;
+        c.latency = [=](bool v, int t) {
+          const int n = 2 * (v ? t - 1000000 : t) + v;
+          return n == late ? NEVER : n > late && more == 1 ? NEVER + 37 * n : n > late && more == 2 ? LIMIT + 37 * n : 900;
+        };
+        own_rings(c, {{{9, b}}, {{5, 0}}}, 1800);         // ends when all events are over: the copies too
+        if (!c.abort) fault("the late copy was not missed", 0, late, 0);
+      }
+  for (int late = 0; late < 28; ++late) {                 // and what the drain sees when it starts at once
+    Cta c;
+    where = "drain";
+    c.latency = [=](bool v, int t) { return 2 * (v ? t - 1000000 : t) + v == late ? 3 * LIMIT : 900; };
+    bool stopped = false;
+    std::function<void()> watch = [&] {
+      if (!c.abort) { c.sim.at(c.sim.now + 1000, watch); return; }
+      if (!stopped) { stopped = true; c.sim.at(c.sim.now + 1000, watch); return; }       // every role has left
+      c.sim.spawn([&] {
+        auto drain = [&](int first, int n, int fills) {
+          giveup::drain(fills, n, [&](int s, uint32_t parity) { c.sim.pass(20); return c.full[first + s].test(parity); });
+        };
+        drain(0, attn::K_SLOTS, c.fills[0]);
+        drain(attn::K_SLOTS, attn::V_SLOTS, c.fills[1]);
+        for (int s = 0; s < 5; ++s)
+          if (c.slots[s].open) fault("drained beside a copy on its way", s, late, c.slots[s].open);
+      });
+    };
+    c.sim.at(0, watch);
+    own_rings(c, {{{9, 9}}, {{5, 0}}}, 1800);
+  }
+  return wrong ? 1 : 0;
+}
 """)
 
 
