@@ -609,8 +609,22 @@ __device__ __forceinline__ bool find_query_tile(const AttnArgs& a, int item, int
   }
   return false;
 }
+// Without a plan a warp of the grid's last CTA looks for what the plan would have: more tiles than the grid has, which nobody serves, and
+// contexts beyond what n_tbl covers.
+__device__ __forceinline__ void check_sizes(const AttnArgs& a, int chunk) {
+  const int lane = threadIdx.x & 31, group = a.n_q / a.n_kv;
+  int tiles = 0, chunks = 0;
+  for (int i = lane; i < a.n_req; i += 32) {
+    const int n = max(0, a.new_lens[i]);
+    tiles += (n + QT - 1) / QT;
+    if (n > 0 && n * group <= DEC_ROWS) chunks += (a.prefix_lens[i] + n + chunk - 1) / chunk;
+  }
+  tiles = __reduce_add_sync(0xffffffffu, tiles);
+  chunks = __reduce_add_sync(0xffffffffu, chunks);
+  if (lane == 0 && (tiles > a.max_prefill || chunks > a.max_decode)) atomicOr(a.pv.flags, (uint32_t)FLAG_BAD_POS);
+}
 template <bool PLANNED>
-__global__ void __launch_bounds__(ATT_THREADS) attn_prefill_kernel(const AttnArgs a) {
+__global__ void __launch_bounds__(ATT_THREADS) attn_prefill_kernel(const AttnArgs a, int chunk) {
   extern __shared__ __align__(128) unsigned char smem[];
   const int item = blockIdx.x / a.n_q, hq = blockIdx.x % a.n_q;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -624,7 +638,9 @@ __global__ void __launch_bounds__(ATT_THREADS) attn_prefill_kernel(const AttnArg
   } else {
     pdl_wait();                 // q, K and V come from the kernel right before this one
     pdl_launch_dependents();
-    if (!find_query_tile(a, item, i, q0)) return;
+    const bool found = find_query_tile(a, item, i, q0);
+    if (blockIdx.x + 1 == gridDim.x && warp == 0) check_sizes(a, chunk);       // (as a rule this CTA has no tile)
+    if (!found) return;
   }
   const int n_new = a.new_lens[i], prefix = a.prefix_lens[i], ctx = prefix + n_new;
   const int h = hq / (a.n_q / a.n_kv);
@@ -901,7 +917,7 @@ int fl_paged_attention(fl_pool* p, fl_bf16* out, const fl_bf16* q, const int32_t
       break;
     }
     if (kind == 0 && small_batch(n_req, n_tokens, n_tbl, n_q_heads, p->sm_count)) {
-      const cudaError_t e = launch_pdl(attn_prefill_kernel<false>, dim3((unsigned)(w.max_prefill * n_q_heads)), dim3(ATT_THREADS), PRE_SMEM, st, a);
+      const cudaError_t e = launch_pdl(attn_prefill_kernel<false>, dim3((unsigned)(w.max_prefill * n_q_heads)), dim3(ATT_THREADS), PRE_SMEM, st, a, w.chunk);
       if (e != cudaSuccess) {
         p->last_cuda = (int)e;
         rc = FL_ECUDA;
@@ -922,7 +938,7 @@ int fl_paged_attention(fl_pool* p, fl_bf16* out, const fl_bf16* q, const int32_t
       if (rc != FL_OK) break;
       beside = max_items > 0;
     } else {
-      attn_prefill_kernel<true><<<(unsigned)w.max_prefill * n_q_heads, ATT_THREADS, PRE_SMEM, st>>>(a);
+      attn_prefill_kernel<true><<<(unsigned)w.max_prefill * n_q_heads, ATT_THREADS, PRE_SMEM, st>>>(a, w.chunk);
     }
     cudaError_t e = launch_pdl(beside ? attn_decode_kernel<BESIDE> : attn_decode_kernel<PLAIN>, dim3((unsigned)w.max_decode * n_kv_heads + (beside ? 1u : 0u)),
                                dim3(ATT_THREADS), DEC_SMEM, st, a, w.chunk, 0);

@@ -51,3 +51,31 @@ def test_small_batch(heads, prefix, new):
             assert s.status(clear=True)["device_flags"] != 0
     finally:
         s.close()
+
+
+@pytest.mark.parametrize("prefix,new,n_tokens,n_tbl", [
+    ([0, 0, 0, 0], [200, 8, 8, 8], 100, None),               # four tiles where n_tokens leaves room for two: one kernel without a plan
+    ([0], [128], 40, None), ([0] * 40, [8] * 39 + [300], 255, None),
+    ([0, 0], [2000, 8], 100, None),                          # the planned kernels
+    ([0, 399], [17, 1], 18, 8), ([600, 399, 399], [700, 1, 1], 702, 25)])      # decode contexts that n_tbl does not cover, without and with a plan
+def test_sizes_that_are_too_small_raise_the_status(prefix, new, n_tokens, n_tbl):
+    """Too few tokens or table entries named in the call; q, out and the tables hold all the rows that the requests have."""
+    from paper_2505_03756_b200 import binding as fl, harness as H
+    wl = synth.make_workload("tiny", n_req=len(new), len_range=(0, 0), n_adapters=1, shape=synth.LayerShape(512, 4, 4))
+    wl.prefix_lens[:], wl.new_lens[:] = prefix, new
+    wl.pool_blocks = int(np.sum((wl.prefix_lens + wl.new_lens + 15) // 16)) + 64
+    s = H.Session(wl, adapters=[])
+    try:
+        s.build_batch()
+        s.fill_prefix_kv()
+        k_new, v_new = wl.kv_new()
+        s.kv_append(H.f32_to_dev(k_new, s.dev), H.f32_to_dev(v_new, s.dev))
+        q = H.f32_to_dev(wl.q(), s.dev)
+        out = torch.zeros_like(q)
+        for tokens, tbl, bad in ((wl.n_tokens, s.n_tbl, False), (n_tokens, s.n_tbl if n_tbl is None else n_tbl, True)):
+            ws = torch.empty(fl.fl_paged_attention_workspace(wl.n_req, wl.n_tokens, s.n_tbl, 4, 4), dtype=torch.uint8, device=s.dev)
+            fl.fl_paged_attention(s.pool, out, q, s.t_req_indptr, s.t_tbl_indptr, s.t_tbl, s.t_prefix, s.t_new, wl.n_req, tokens, tbl, 4, 4, 0.1, ws)
+            torch.cuda.synchronize()
+            assert (s.status(clear=True)["device_flags"] != 0) == bad
+    finally:
+        s.close()
