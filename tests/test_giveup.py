@@ -46,6 +46,36 @@ int main() {
 """ % n_ctas)
 
 
+@pytest.mark.parametrize("n_ctas", [2, 4, 8])
+def test_a_sum_whose_parts_are_fetched_is_not_stored_without_one(tmp_path, n_ctas):
+    """The tcgen05 shrink: a CTA leaves its part, or a word that it has none, in its own memory before the barrier; behind it each looks at
+    every CTA's word, a lane each, and stores its share of the sum only if none is set.  Memory without a part holds old bytes."""
+    run_model(tmp_path, """
+int main() {
+  const int n = %d;
+  int wrong = 0;
+  for (int failed = 0; failed < 1 << n; ++failed) {
+    std::vector<int> missing(n, 0);
+    std::vector<long> part(n, 1000000);
+    for (int c = 0; c < n; ++c) {
+      if (failed >> c & 1) missing[c] = 1;
+      else part[c] = 1 << c;
+    }
+    for (int c = 0; c < n; ++c) {
+      bool any = false;
+      for (int lane = 0; lane < 32; ++lane) any |= (lane < n ? missing[lane] : 0) != 0;
+      long sum = 0;
+      for (long v : part) sum += v;
+      const bool stores = giveup::may_store(true, any ? 1 : 0);
+      if (stores && sum != (1 << n) - 1) { printf("CTA %%d of %%d stores %%ld with %%x failed\\n", c, n, sum, failed); ++wrong; }
+      if (!stores && failed == 0) { printf("CTA %%d of %%d stores nothing\\n", c, n); ++wrong; }
+    }
+  }
+  return wrong ? 1 : 0;
+}
+""" % n_ctas)
+
+
 BARRIER = """
 // A ring slot's barrier: a phase ends when its arrivals and its bytes have come.  A parity test is true for every phase but the
 // current one of that parity, so also for the one before it.
