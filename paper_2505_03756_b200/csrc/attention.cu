@@ -792,14 +792,17 @@ Packed packed_slots(int n_req, int n_tbl, int n_kv, int csize, int sms) {
   return p;
 }
 
-// Batches that attn_prefill_kernel<false> serves by itself: contexts of at most eight blocks in the mean, a table that leaves little room for one
-// long context among short ones (the lengths themselves are not known here), and CTAs that run in three rounds at most.  A CTA takes 2.3 us
+// Batches that attn_prefill_kernel<false> serves by itself: contexts of at most eight blocks in the mean, 40 for the longest if the others have
+// one each (the lengths themselves are not known here), and CTAs that run in three rounds at most.  A CTA takes 2.3 us
 // per 64 keys, so it is contexts that the line is about.  Attention, this kernel and the three of the planned way, in us, heads / KV heads
 // 8/8, 32/32, 64/8: 1 request of 32 new tokens behind 32 5.0 and 9.6, 5.1 and 10.0, 5.1 and 10.4; 4 such 5.1 and 9.9, 5.7 and 10.4, 6.1 and
-// 11.4; 16 such 5.7 and 10.4, 10.8 and 20.1, (64/8 stays planned) 19.6 and 21.7; 4 of 64 behind 64 7.3 and 10.0, 8.7 and 10.6, 9.2 and 11.9.
+// 11.4; 4 of 64 behind 64 7.3 and 10.0, 8.7 and 10.6, 9.2 and 11.9.
 // Beyond: 1 request of 64 new tokens behind 192 12.0 and 11.4, 12.1 and 11.5, 12.3 and 12.8; 1 of 128 behind 384 21 and 14, 21 and 14, 25 and 16.
+// One request has nearly all of the table, a decode step's keys beside prompts of 16 tokens: 14 blocks, 6 requests 10 and 10, 11 and 15, 13 and 21;
+// 26 blocks 16 and 10, 17 and 16, 21 and 22; 40 blocks 22 and 11, 24 and 18, 28 and 24 (a prompt's keys 22 and 17, 24 and 18, 28 and 19), the
+// most that the rule lets through is lost there; among 60 requests 24 and 23 on 8 heads.  64 blocks, 16 requests, 35 to 38 and 15 to 29.
 bool small_batch(int n_req, int n_tokens, int n_tbl, int n_q, int sms) {
-  return (n_tokens / QT + n_req) * (long long)n_q <= 6ll * sms && n_tbl <= 8ll * n_req && n_tbl <= 32 + 2ll * n_req;
+  return (n_tokens / QT + n_req) * (long long)n_q <= 6ll * sms && n_tbl <= 8ll * n_req && n_tbl - n_req < 40;
 }
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }

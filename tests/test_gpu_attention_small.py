@@ -1,6 +1,6 @@
 """fl_paged_attention of small batches, served by one kernel without a plan: new tokens around a tile's 64 rows and a warp's 16,
 contexts around 64 keys, requests without a new token, one-token requests among prompts, more than 32 requests, grouped heads, a
-request whose table is too short, and batches on either side of the line to the planned kernels."""
+request whose table is too short, one long context among many short ones, and batches on either side of each line to the planned kernels."""
 import math
 
 import numpy as np
@@ -15,12 +15,33 @@ from paper_2505_03756_b200 import synth
 from _util import assert_close, oracle_context
 
 
+def without_plan(heads, prefix, new):
+    """The rule of attention.cu: CTAs of three rounds, eight blocks a request, 40 for one if the others have one each."""
+    tables = [-(-(p + n) // 16) for p, n in zip(prefix, new)]
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    return (sum(new) // 64 + len(new)) * heads[0] <= 6 * sms and sum(tables) <= 8 * len(new) and sum(tables) - len(new) < 40
+
 @pytest.mark.parametrize("heads,prefix,new", [
     ((4, 4), [0], [64]), ((4, 4), [0], [65]), ((8, 8), [32] * 4, [32] * 4), ((2, 2), [0, 63, 1, 15], [63, 1, 17, 128]),
     ((8, 2), [64, 0, 16], [64, 16, 33]), ((8, 1), [17, 40], [19, 3]), ((4, 4), [0, 5, 0, 30], [127, 0, 1, 18]),
     ((2, 1), [7 * (i % 9) for i in range(40)], [1 + 5 * (i % 7) for i in range(40)]), ((4, 4), [300] + [0] * 9, [30] + [16] * 9),
     ((16, 16), [60], [68]), ((16, 16), [61], [68]), ((32, 32), [16] * 13, [64] * 13), ((32, 32), [16] * 14, [64] * 14)])
 def test_small_batch(heads, prefix, new):
+    check_batch(heads, prefix, new)
+
+
+@pytest.mark.parametrize("heads,prefix,new,alone", [
+    ((2, 1), [7 * (i % 3) for i in range(40)], [0 if 30 <= i < 34 else 1 + 3 * (i % 5) for i in range(40)], True),      # the 33rd request and on
+    ((4, 4), [0] * 33, [16] * 32 + [150], True), ((2, 2), [0] * 70, [3] * 40 + [0] * 28 + [65, 7], True),
+    ((32, 32), [0] * 15, [48] * 15, True), ((32, 32), [0] * 16, [48] * 16, False),                                       # the grid's line
+    ((4, 4), [20] * 3, [108] * 3, True), ((4, 4), [20] * 3, [108, 108, 109], False),                                     # eight blocks each
+    ((4, 4), [0] * 99 + [623], [16] * 99 + [17], True), ((4, 4), [0] * 99 + [640], [16] * 99 + [1], False)])             # the longest one's
+def test_the_lines_to_the_planned_kernels(heads, prefix, new, alone):
+    assert without_plan(heads, prefix, new) == alone
+    check_batch(heads, prefix, new)
+
+
+def check_batch(heads, prefix, new):
     from paper_2505_03756_b200 import harness as H
     wl = synth.make_workload("tiny", n_req=len(new), len_range=(0, 0), n_adapters=1, shape=synth.LayerShape(heads[0] * 128, *heads))
     wl.prefix_lens[:], wl.new_lens[:] = prefix, new
