@@ -790,17 +790,18 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
       k.n_req = a.n_req;
       k.n_kv = a.n_kv;
       k.bt = a.bt;
-      sgmv::ShrinkInfo info = {1, 16, false};
+      k.rmax = n_seg > 0 ? rank_max : 16;
+      sgmv::ShrinkInfo info = {1, k.rmax, false};
       if (n_seg > 0) {
         // Above rank 16 and on wide layers the tcgen05 shrink is the faster one for segments above a few tokens (q, k, v of 128 tokens, one
         // segment: rank 64 7B 34.0 and 27.2 us, 34B 53 and 45; rank 32 28.4 and 27.5, 46 and 44; 40 tokens 25.8 and 25.2, 43 and 42;
         // but on a layer of 1024 values, 112 tokens, 19.4 and 20.5).
         const bool tc = rank_max > 16 && p->sgmv_shrink_kind == 0 && n_tokens > 16 * n_seg && a.d_in >= 2048;
-        rc = (tc ? sgmv::shrink : sgmv::shrink_scaled)(p, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace,
-                                                       v_bytes, stream, &info);
+        const sgmv::Follower next = skinny::footprint(p, k);
+        rc = tc ? sgmv::shrink(p, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace, v_bytes, stream, &info)
+                : sgmv::shrink_scaled(p, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace, v_bytes, stream, &info, &next);
         if (rc != FL_OK) break;
       }
-      k.rmax = info.rmax;
       rc = skinny::launch(p, k, x, reinterpret_cast<const void* const*>(ws), st);
       break;
     }
@@ -849,7 +850,7 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
       const bool tc = rank_max > 16 && p->sgmv_shrink_kind == 0;
       const bool final = n_tokens <= 16 * n_seg || (!tc && (double)n_tokens / n_seg * a.d_in <= (rank_max == 16 ? 1.7e5 : 3e5));
       rc = final ? sgmv::shrink_scaled(p, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace, v_bytes,
-                                       stream, &info)
+                                       stream, &info, nullptr)
                  : sgmv::shrink(p, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace, v_bytes, stream, &info);
       if (rc != FL_OK) break;
       if (info.final) a.v16 = reinterpret_cast<const __nv_bfloat16*>(workspace);

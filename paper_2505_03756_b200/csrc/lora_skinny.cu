@@ -665,6 +665,13 @@ bool serves(const fl_pool* p, const int* d_out, int n_mats, int d_in, int n_toke
   return n_seg * rank_max > 8 * 32 && n_tokens <= 176;
 }
 
+sgmv::Follower footprint(const fl_pool* p, const Args& a) {
+  KArgs ka;
+  uint32_t smem;
+  layout(p, a, &ka, &smem);
+  return {ka.tile_base[a.n_mats] * ka.split, ka.split, smem};
+}
+
 int launch(fl_pool* p, const Args& a, const void* x, const void* const* w, cudaStream_t st) {
   KArgs ka;
   uint32_t smem;

@@ -1,6 +1,7 @@
 // The base projection with the LoRA branch folded in, for batches of few tokens (see lora_skinny.cu).
 #pragma once
 #include "pool.cuh"
+#include "sgmv.cuh"
 
 namespace skinny {
 
@@ -26,6 +27,9 @@ struct Args {
 
 // Whether `launch` is the faster way for a call (n_seg = 0: no adapters).
 bool serves(const fl_pool* p, const int* d_out, int n_mats, int d_in, int n_tokens, int n_seg, int rank_max);
+
+// What `launch` will take for these arguments.
+sgmv::Follower footprint(const fl_pool* p, const Args& a);
 
 // y = x W + (scaled x A) B for n_tokens <= MAX_TOKENS.  With n_seg > 0 the shrink that writes v must be the launch right
 // before this one on the stream.

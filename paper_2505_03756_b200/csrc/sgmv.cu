@@ -24,12 +24,9 @@ constexpr int SG_THREADS = 128;
 constexpr int KS = 64;            // d_in elements per shrink pipeline stage (128-byte rows)
 constexpr int SH_STAGES = 4;
 // Tiles of 16 tokens behind which the final form is wanted: a CTA's slice is 8 to 27 stages, each 0.5 us after the one before with four in
-// flight, and the projection's CTAs that need the SM wait meanwhile.  More in flight where the CTAs all run at once: shrink and projection of
-// o, 64 tokens, 15 adapters of rank 64, 34B 42.7 -> 38.9 us (12 stages; 8: 40.1); one token of rank 16 on 7B, 46.9 -> 46.2 us a layer (8 stages;
-// with 12 there is no room for the projection's CTAs beside these, and it takes 49.0).  Not for slices of a few stages, which only lose that
-// room (8 tokens of rank 32 on a layer of 1024 values: 37.0 -> 38.9 us a layer).
+// flight.  With 8 or 12 in flight (rank 64) it takes half as long, but its CTAs take twice the shared memory, and the projection's CTAs, which
+// are on their way to W meanwhile, wait for the SMs: `deeper` decides.
 constexpr int deep_stages(int rmax) { return rmax == 64 ? 12 : 8; }
-constexpr double deep_per_sm(int rmax) { return rmax == 64 ? 1.1 : rmax == 32 ? 2 : 3; }
 constexpr int NSUB = 128;         // y columns per expand sub-tile (256-byte rows)
 constexpr int EXPAND_COLS_MIN = 512, EXPAND_COLS_MAX = 2048;   // y columns per expand CTA: picked per call
 constexpr int KSPLIT_MAX = 8;
@@ -882,6 +879,33 @@ int launch_expand_short(fl_pool* p, SgmvArgs& a, int tiles, int d_out_max, cudaS
   return FL_OK;
 }
 
+// Whether the kernel behind finds a place for all its CTAs while `ctas` of a shrink with `smem` bytes each are there, as many on an SM as fit.
+// (Clusters do not fill every SM; the shares are those that tell the measured sides apart.)
+constexpr int SM_SMEM = 228 * 1024, CTA_SMEM = 1024;       // an SM's shared memory, and what each CTA takes beside its own
+bool has_room(const sgmv::Follower& f, int ctas, int smem, int sms) {
+  return f.ctas <= (sms - (double)ctas / (SM_SMEM / (smem + CTA_SMEM))) * (f.cluster == 1 ? 1 : f.cluster == 2 ? 0.9255 : f.cluster == 3 ? 0.8677 : 0.91);
+}
+// Whether the shrink in tiles of 16 tokens has more of its stages in flight: where the projection's CTAs have no room beside the shallow one either,
+// or room beside the deeper one as well, on the same SMs, and where the deeper one's clusters run at once (15 of eight, one CTA per SM).
+// Decode steps (a graph of q, k, v with the KV store, attention over 512 keys, o; 13B up and down too, so that W comes from HBM), shallow everywhere,
+// deeper everywhere and with this rule, us:  rank 64, 4 requests with an adapter each, 13B 143.5, 137.1, 137; 34B 90.9, 92.0, 86; 12 of them
+// 34B 124.1, 125.1, 122; 13B 194.5, 191.0, 183; 16 of them 34B 129.9, 144.7, 130; 7B 97.0, 106.5, 97.  Rank 32, 4 of them 34B 77.3, 84.9,
+// 77; 13B 115.4, 128.6, 115; 12 13B 174.1, 164.9, 166.  Rank 16, one 7B 46.6, 45.9, 46; 8 13B 130.6, 143.2, 131; 37 7B 115.4, 112.3, 112.
+// 294 such steps: 1 % less than with a bound on the number of the deeper one's CTAs alone, 2 % less than with four stages; the worst, 16 adapters
+// of rank 64 on 13B, 2 % more than the former.  (The same calls back to back, with W in L2, order themselves quite differently.)
+bool deeper(const fl_pool* p, const SgmvArgs& a, int rmax, int tiles, const sgmv::Follower* next) {
+  const int slice = (p->mats[a.mat_index[0]].d_in + KS * a.ksplit - 1) / (KS * a.ksplit);       // stages
+  if (!a.v16 || slice <= SH_STAGES) return false;
+  // behind it a GEMM on all SMs (rank 16: shallow and deeper within 1 us of 16 to 110, but 900 tokens in 45 segments on 7B, o, 38 and 35)
+  if (!next) return tiles * a.n_mats * a.ksplit <= p->sm_count * (rmax == 64 ? 1.1 : rmax == 32 ? 2 : 3);
+  const int sums = KSPLIT_MAX * 16 * rmax * 4, shallow = shrink_pipe_bytes(16, rmax, SH_STAGES) + sums, deep = shrink_pipe_bytes(16, rmax, deep_stages(rmax)) + sums;
+  const int each = a.n_mats * a.ksplit, few = std::max(a.n_seg, (a.n_tokens + 15) / 16) * each;            // CTAs with a tile, at least
+  const int most = next->cluster == 1 ? few : (a.n_seg + std::max(0, a.n_tokens - a.n_seg) / 16) * each;      // and at most
+  if (few > p->sm_count * 13 / 16 * (SM_SMEM / (deep + CTA_SMEM))) return false;
+  if (!has_room(*next, most, shallow, p->sm_count)) return true;
+  return next->cluster > 1 && (int)next->smem + deep + 2 * CTA_SMEM <= SM_SMEM && has_room(*next, most * 3 / 2, deep, p->sm_count);
+}
+
 template <int TM, int RMAX, int STAGES>
 int launch_shrink(fl_pool* p, const SgmvArgs& a, int tiles, cudaStream_t st) {
   static bool configured[16] = {};
@@ -897,7 +921,7 @@ int launch_shrink(fl_pool* p, const SgmvArgs& a, int tiles, cudaStream_t st) {
 }
 
 template <int TM, int RMAX>
-int launch_pair(fl_pool* p, SgmvArgs& a, int tiles, int d_out_max, cudaStream_t st, bool shrink_only) {
+int launch_pair(fl_pool* p, SgmvArgs& a, int tiles, int d_out_max, cudaStream_t st, bool shrink_only, const sgmv::Follower* next) {
   if (TM == 64 && p->sgmv_shrink_kind == 0 && a.n_mats <= 3 && a.tc_ksplit > 0) {
     // long segments: the shrink on tcgen05 tensor cores, tiles of 128 tokens, its own number of d_in slices
     a.ksplit = a.tc_ksplit;
@@ -930,8 +954,7 @@ int launch_pair(fl_pool* p, SgmvArgs& a, int tiles, int d_out_max, cudaStream_t 
     else
       FL_CUDA(p, launch_pdl(sgmv_shrink3_kernel<RMAX, 4>, dim3(tiles, a.ksplit), dim3(SG_THREADS), smem_of[1], st, a));
   } else {
-    const int slice = (p->mats[a.mat_index[0]].d_in + KS * a.ksplit - 1) / (KS * a.ksplit);       // stages
-    const bool deep = TM == 16 && a.v16 && slice > SH_STAGES && tiles * a.n_mats * a.ksplit <= p->sm_count * deep_per_sm(RMAX);
+    const bool deep = TM == 16 && deeper(p, a, RMAX, tiles, next);
     const int rc = deep ? launch_shrink<TM, RMAX, TM == 16 ? deep_stages(RMAX) : SH_STAGES>(p, a, tiles, st) : launch_shrink<TM, RMAX, SH_STAGES>(p, a, tiles, st);
     if (rc != FL_OK) return rc;
   }
@@ -966,7 +989,7 @@ struct KvDest {      // where K and V results go when they are appended to the p
 int sgmv_common(fl_pool* p, fl_bf16* const* ys, const fl_bf16* x, const int* mat_indices, int n_mats,
                 const int32_t* seg_indptr, const int32_t* lora_ids, int n_seg, int n_tokens,
                 float scale, void* workspace, size_t workspace_bytes, fl_stream stream, const KvDest* kv,
-                sgmv::ShrinkInfo* shrink_only = nullptr, bool scaled = false) {
+                sgmv::ShrinkInfo* shrink_only = nullptr, bool scaled = false, const sgmv::Follower* next = nullptr) {
   if (!p || n_mats < 1 || n_mats > FL_MAX_MATS || n_seg < 0 || n_tokens < 0 || !ys || !mat_indices) return FL_EINVAL;
   if (n_seg == 0 || n_tokens == 0) return FL_OK;
   if (!x || !seg_indptr || !lora_ids || !workspace) return FL_EINVAL;
@@ -1057,14 +1080,14 @@ int sgmv_common(fl_pool* p, fl_bf16* const* ys, const fl_bf16* x, const int* mat
     const int tiles = n_seg + n_tokens / 16;
     // slices of d_in so that all CTAs run at once: at rank 64 three of them fit on an SM, below that at least five
     if (scaled) a.ksplit = std::max(1, std::min(KSPLIT_MAX, (rmax == 64 ? 3 : 4) * p->sm_count / (tiles * n_mats)));
-    rc = rmax == 16 ? launch_pair<16, 16>(p, a, tiles, d_out_max, st, so)
-       : rmax == 32 ? launch_pair<16, 32>(p, a, tiles, d_out_max, st, so)
-                    : launch_pair<16, 64>(p, a, tiles, d_out_max, st, so);
+    rc = rmax == 16 ? launch_pair<16, 16>(p, a, tiles, d_out_max, st, so, next)
+       : rmax == 32 ? launch_pair<16, 32>(p, a, tiles, d_out_max, st, so, next)
+                    : launch_pair<16, 64>(p, a, tiles, d_out_max, st, so, next);
   } else {
     const int tiles = n_seg + n_tokens / 64;
-    rc = rmax == 16 ? launch_pair<64, 16>(p, a, tiles, d_out_max, st, so)
-       : rmax == 32 ? launch_pair<64, 32>(p, a, tiles, d_out_max, st, so)
-                    : launch_pair<64, 64>(p, a, tiles, d_out_max, st, so);
+    rc = rmax == 16 ? launch_pair<64, 16>(p, a, tiles, d_out_max, st, so, next)
+       : rmax == 32 ? launch_pair<64, 32>(p, a, tiles, d_out_max, st, so, next)
+                    : launch_pair<64, 64>(p, a, tiles, d_out_max, st, so, next);
   }
   if (prev != p->device && prev >= 0) cudaSetDevice(prev);
   return rc;
@@ -1082,10 +1105,10 @@ int shrink(fl_pool* p, const fl_bf16* x, const int* mat_indices, int n_mats, con
 }
 int shrink_scaled(fl_pool* p, const fl_bf16* x, const int* mat_indices, int n_mats, const int32_t* seg_indptr,
                   const int32_t* lora_ids, int n_seg, int n_tokens, float scale, void* workspace, size_t workspace_bytes,
-                  fl_stream stream, ShrinkInfo* info) {
+                  fl_stream stream, ShrinkInfo* info, const Follower* next) {
   fl_bf16* none[FL_MAX_MATS] = {};
   return sgmv_common(p, none, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace,
-                     workspace_bytes, stream, nullptr, info, true);
+                     workspace_bytes, stream, nullptr, info, true, next);
 }
 }  // namespace sgmv
 

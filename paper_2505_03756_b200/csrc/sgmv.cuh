@@ -10,6 +10,11 @@ struct ShrinkInfo {
   bool final;   // slices added, scaled, rounded to bf16 as the expand product takes them, [projection][token][rmax]
 };
 
+struct Follower {      // the kernel that waits for v with all its CTAs: how many, in clusters of how many, and the shared memory of one
+  int ctas, cluster;
+  uint32_t smem;
+};
+
 // v = x A_i per segment for the listed projections (which share x): unscaled fp32 partial sums written to
 // workspace as [projection][slice][token][rmax], or the final form; workspace sized by fl_lora_sgmv_workspace(n_tokens, n_mats).
 // Rows of segments without an adapter are left untouched.
@@ -18,10 +23,10 @@ int shrink(fl_pool* p, const fl_bf16* x, const int* mat_indices, int n_mats, con
            ShrinkInfo* info);
 // The same, always in its final form.
 // Tiles of 16 tokens whatever the segments' lengths, each of which reads its adapter's rows again: for batches of up to a few hundred
-// tokens, and beyond for short segments.
+// tokens, and beyond for short segments.  `next` is the kernel behind, null where that one has CTAs on all SMs anyway.
 int shrink_scaled(fl_pool* p, const fl_bf16* x, const int* mat_indices, int n_mats, const int32_t* seg_indptr,
                   const int32_t* lora_ids, int n_seg, int n_tokens, float scale, void* workspace, size_t workspace_bytes,
-                  fl_stream stream, ShrinkInfo* info);
+                  fl_stream stream, ShrinkInfo* info, const Follower* next);
 
 #ifdef __CUDACC__
 // Token tile `tile` (tiles of tm tokens, counted over segments that carry an adapter, or over all segments) -> segment and

@@ -53,3 +53,35 @@ def test_shrink_of_long_segments(hidden, lens, rank):
         assert s.status()["device_flags"] == 0
     finally:
         s.close()
+
+
+# around the lines of the shrink with more stages in flight: up to 15 clusters of eight at rank 64, twelve to twenty segments and fewer, slices of five stages
+@pytest.mark.parametrize("hidden,rank,lens", [
+    (4096, 64, [4] * 12), (4096, 64, [1] * 14), (4096, 64, [1] * 15), (4104, 64, [1] * 16), (8192, 64, [3] * 16), (4096, 64, [1] * 20),
+    (2624, 64, [5, 1, 30, 2]), (2560, 32, [2] * 30), (2560, 32, [2] * 37), (2568, 16, [1] * 44), (2560, 16, [1] * 60)])
+def test_shrink_of_decode_steps(hidden, rank, lens):
+    from paper_2505_03756_b200 import harness as H
+    shape = synth.LayerShape(hidden, 2, 2, block_tokens=16)
+    n = len(lens)
+    wl = synth.make_workload("decode13b", n_req=n, len_range=(3, 20), n_adapters=n, shape=shape)
+    wl.ranks[:] = [rank - i % 3 for i in range(n)]
+    wl.lora_of_req[:] = np.arange(n)
+    wl.new_lens[:] = lens
+    wl.pool_blocks = int(np.sum((wl.prefix_lens + wl.new_lens + 15) // 16)) + 260 * n + 64
+    s = H.Session(wl)
+    try:
+        s.load_adapters()
+        s.build_batch()
+        seg, ids = wl.segments()
+        x, w = wl.x("q"), wl.weight("q")
+        tx, tw = H.f32_to_dev(x, s.dev), H.f32_to_dev(w, s.dev)
+        out = []
+        for _ in range(3):
+            y = torch.full((wl.n_tokens, 256), float("nan"), dtype=torch.bfloat16, device=s.dev)
+            s.lora_linear([y], tx, [tw], ["q"])
+            out.append(y)
+        assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
+        assert_close(H.dev_to_f32(out[0]), lora_linear(x, w, seg, ids, oracle_adapters(wl, "q"), wl.scale), f"decode {hidden} rank {rank}")
+        assert s.status()["device_flags"] == 0
+    finally:
+        s.close()
