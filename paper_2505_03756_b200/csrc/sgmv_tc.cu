@@ -342,19 +342,25 @@ int launch(fl_pool* p, const sgmv::TcShrinkArgs& a, const CUtensorMap& xmap, int
 namespace sgmv {
 
 int tc_slices(const fl_pool* p, int n_seg, int n_tokens, int d_in, int rmax, int n_mats) {
-  // Rounds of tiles over the SMs times what a tile's slice takes: about 6 us of look-ups, ramp and end, 4 us more where slices are added,
-  // and per stage the fill of x and of the adapter rows at 50 bytes per clock.  Clusters of four find a place on the GPU's groups of SMs
-  // 33 times, clusters of eight 15 times (as the occupancy query says for this shared memory); other sizes leave more SMs empty.
-  const long tiles = (n_tokens + TM - 1) / TM + n_seg / 2;
+  // Rounds of tiles over the SMs times what a tile's slice takes, in us beside what every tile does: look-ups, ramp and end, where slices are
+  // added their barriers and the sums, by rows, columns and CTAs (clusters of eight get into each other's way as well), and per stage the fill
+  // of x and of the adapter rows at 60 bytes per clock.
+  // Clusters of four find a place on the GPU's groups of SMs 33 times, clusters of eight 15 times (as the occupancy query says for this shared
+  // memory); other sizes leave more SMs empty.  Shrink and expand with two, four and eight slices, 7B, 512 tokens: one segment of rank 64, q, k, v
+  // 25.0, 21.8 and 21.9; 16 segments q, k, v 27.9, 24.5 and 33.7, o 15.5, 13.3 and 18.2; 1000 tokens in four, o 18.0, 15.8 and 16.4.  Over 356
+  // batches of 300 to 9000 tokens the choice is 0.3 % behind the best (2.6 with one price for every sum and fewer tiles than segments).
+  const long tiles = std::max<long>(n_seg, (n_tokens + TM - 1) / TM + n_seg / 2);
+  const double rows = std::min<double>(TM, (double)n_tokens / tiles) / TM;
   const int nk = (d_in + BK - 1) / BK;
-  const double stage = (X_BYTES + n_mats * rmax * 128) / 95e3;
+  const double stage = (X_BYTES + n_mats * rmax * 128) / 115e3;
   int best = 1;
   double least = 0;
   for (int ks = 1; ks <= TC_MAX_SLICES && (ks == 1 || nk / ks >= 4); ks *= 2) {
     const int kchunk = (nk + ks - 1) / ks;
     if ((ks - 1) * kchunk >= nk) continue;                                       // every slice of d_in must hold something
     const long at_once = ks <= 2 ? p->sm_count / ks : ks == 4 ? p->sm_count * 9 / 40 : p->sm_count * 13 / 128;
-    const double cost = (double)((tiles + at_once - 1) / at_once) * (6 + (ks > 1 ? 4 : 0) + kchunk * stage);
+    const double sum = ks == 1 ? 0 : 4 + 0.125 * ks + rows * (n_mats * rmax * ks / 256.0 + (ks == 8 ? 0.25 * std::max(0L, tiles - 4) : 0));
+    const double cost = (double)((tiles + at_once - 1) / at_once) * (6 + sum + kchunk * stage);
     if (ks == 1 || cost < least) { least = cost; best = ks; }
   }
   return best;

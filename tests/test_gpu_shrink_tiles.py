@@ -16,7 +16,8 @@ from _util import assert_close, oracle_adapters
 # hidden (= d_in), tokens per segment, rank
 @pytest.mark.parametrize("hidden,lens,rank", [
     (2056, [127, 128, 129, 1], 33), (2048, [257, 1], 64), (4160, [40], 32), (5120, [96, 32], 64), (4096, [300, 300, 300, 300], 17), (1096, [128] * 24, 64),
-    (328, [90, 700], 20), (2048, [128] * 60, 24), (7176, [255, 1, 1200], 16)])
+    (328, [90, 700], 20), (2048, [128] * 60, 24), (7176, [255, 1, 1200], 16),
+    (4104, [40] * 39, 64)])
 def test_shrink_of_long_segments(hidden, lens, rank):
     from paper_2505_03756_b200 import harness as H
     shape = synth.LayerShape(hidden, 2, 2, block_tokens=16)
