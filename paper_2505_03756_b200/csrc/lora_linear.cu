@@ -841,14 +841,16 @@ int linear_common(fl_pool* p, fl_bf16* const* ys_in, const fl_bf16* x, const fl_
       break;
     }
     if (n_seg > 0) {
-      // Two shrinks, in tiles of 16 tokens and of 64 or 128 tokens.  Above rank 16, where the second one runs on tcgen05, it is the better one
-      // for all but segments of a few tokens (q, k, v on 7B, rank 64: 320 tokens, 40 per segment 53 and 35 us; 512, 64 per segment 92 and 60;
-      // 1920, 80 per segment 148 and 138; rank 32, 512 tokens, 64 per segment 61 and 53; 1024 tokens and more the same).  At rank 16 the
+      // Two shrinks, in tiles of 16 tokens and of 64 or 128 tokens.  Above rank 16 and on wide layers, where the second one runs on tcgen05, it is the
+      // better one for all but segments of a few tokens (q, k, v on 7B, rank 64: 320 tokens, 40 per segment 53 and 35 us; 512, 64 per segment 92
+      // and 60; 1920, 80 per segment 148 and 138; rank 32, 512 tokens, 64 per segment 61 and 53; 1024 tokens and more the same).  At rank 16 the
       // second one reads the adapters' rows less often, but where it leaves fp32 slices of d_in a LoRA stage that sums them takes 5600
       // cycles instead of 1500: the first one is the better one as long as a segment's x and the rows that it reads again are few
       // (7B, 288 tokens, 20 per segment 64 and 67 us, 72 per segment 59 and 54; 1000 tokens of 1024 values, 100 per segment 23 and 25).
-      const bool tc = rank_max > 16 && p->sgmv_shrink_kind == 0;
-      const bool final = n_tokens <= 16 * n_seg || (!tc && (double)n_tokens / n_seg * a.d_in <= (rank_max == 16 ? 1.7e5 : 3e5));
+      // On layers of 1024 values so it is at higher ranks (a layer step, rank 32, 200 tokens in one segment 42.4 and 47.3 us, 512 in four 43.6 and
+      // 47.1; rank 64, 256 in four 50.3 and 55.4, but 512 in one 65 and 56).
+      const bool tc = rank_max > 16 && p->sgmv_shrink_kind == 0 && a.d_in >= 2048;
+      const bool final = n_tokens <= 16 * n_seg || (!tc && (double)n_tokens / n_seg * a.d_in <= (rank_max == 16 ? 1.7e5 : rank_max == 32 ? 3e5 : 1.32e5));
       rc = final ? sgmv::shrink_scaled(p, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace, v_bytes,
                                        stream, &info, nullptr)
                  : sgmv::shrink(p, x, mat_indices, n_mats, seg_indptr, lora_ids, n_seg, n_tokens, scale, workspace, v_bytes, stream, &info);
