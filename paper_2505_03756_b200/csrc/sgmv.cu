@@ -892,7 +892,7 @@ bool has_room(const sgmv::Follower& f, int ctas, int smem, int sms) {
 // 34B 124.1, 125.1, 122; 13B 194.5, 191.0, 183; 16 of them 34B 129.9, 144.7, 130; 7B 97.0, 106.5, 97.  Rank 32, 4 of them 34B 77.3, 84.9,
 // 77; 13B 115.4, 128.6, 115; 12 13B 174.1, 164.9, 166.  Rank 16, one 7B 46.6, 45.9, 46; 8 13B 130.6, 143.2, 131; 37 7B 115.4, 112.3, 112.
 // 294 such steps: 1 % less than with a bound on the number of the deeper one's CTAs alone, 2 % less than with four stages; the worst, 16 adapters
-// of rank 64 on 13B, 2 % more than the former.  (The same calls back to back, with W in L2, order themselves quite differently.)
+// of rank 64 on 13B, 2 % more than the former.  Not above 128 tokens (rank 16, 200 tokens in one segment, 13B 187 us, shallow 175; 34B 115.5, 111.4).  (The same calls back to back, with W in L2, order themselves quite differently.)
 bool deeper(const fl_pool* p, const SgmvArgs& a, int rmax, int tiles, const sgmv::Follower* next) {
   const int slice = (p->mats[a.mat_index[0]].d_in + KS * a.ksplit - 1) / (KS * a.ksplit);       // stages
   if (!a.v16 || slice <= SH_STAGES) return false;
@@ -901,7 +901,7 @@ bool deeper(const fl_pool* p, const SgmvArgs& a, int rmax, int tiles, const sgmv
   const int sums = KSPLIT_MAX * 16 * rmax * 4, shallow = shrink_pipe_bytes(16, rmax, SH_STAGES) + sums, deep = shrink_pipe_bytes(16, rmax, deep_stages(rmax)) + sums;
   const int each = a.n_mats * a.ksplit, few = std::max(a.n_seg, (a.n_tokens + 15) / 16) * each;            // CTAs with a tile, at least
   const int most = next->cluster == 1 ? few : (a.n_seg + std::max(0, a.n_tokens - a.n_seg) / 16) * each;      // and at most
-  if (few > p->sm_count * 13 / 16 * (SM_SMEM / (deep + CTA_SMEM))) return false;
+  if (few > p->sm_count * 13 / 16 * (SM_SMEM / (deep + CTA_SMEM)) || a.n_tokens > 128) return false;
   if (!has_room(*next, most, shallow, p->sm_count)) return true;
   return next->cluster > 1 && (int)next->smem + deep + 2 * CTA_SMEM <= SM_SMEM && has_room(*next, most * 3 / 2, deep, p->sm_count);
 }
